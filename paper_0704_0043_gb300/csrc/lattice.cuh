@@ -48,6 +48,91 @@ template <> struct Ar<double> {
     static __device__ __forceinline__ double sqrt(double a) { return __dsqrt_rn(a); }
 };
 
+// Hardware reciprocal approximation (one special-function instruction,
+// relative error below 2^-22).
+__device__ __forceinline__ float rcp_approx(float x)
+{
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// Correctly rounded FP64 quotients with few FP64 instructions.  This GPU's FP64
+// unit takes a warp's instruction in 64 cycles, and __ddiv_rn costs about 13 of
+// them, so the divisions of a site (20 for D2Q9, 9 for D1Q3) were half of the
+// FP64 step.  recip64 seeds 1/b from the FP32 special-function unit through
+// integer operations on b's bits (no FP64 conversion) and refines it by one
+// Newton step (relative error below 2^-42); quot64 corrects a * (1/b) once by
+// its residual and then checks the result exactly (Markstein's residual
+// argument, IBM J. Res. Dev. 34 (1990) 111): the last residual a - b q is one
+// exact FMA, and q is the correctly rounded quotient when the residual is
+// below b * ulp(q) / 2 (there are no ties in a division).  That is 2
+// instructions per denominator and 4 per quotient.  Where the check does not
+// hold (the quotient within 2^-33 ulp of a rounding boundary, a power-of-two q,
+// operands outside 2^-500 .. 2^499, zero or negative b, nonfinite values) `slow`
+// is set and the caller repeats its evaluation with __ddiv_rn.
+// With the site evaluation below (shared sub-expressions, no FP64 comparisons)
+// the 600 x 500 FP64 cavity step went from 347 to 256 us (tiled kernel with its
+// tail), and the 512 x 512 entropic FP64 step from 787 to 694 us.
+struct Recip64 {
+    double b, y;
+};
+
+__device__ __forceinline__ bool in_range64(int hi)  // 2^-500 <= x < 2^500 by the high word (x > 0)
+{
+    return (unsigned)(hi - (523 << 20)) < (1000u << 20);
+}
+
+__device__ __forceinline__ Recip64 recip64(double b, bool &slow)
+{
+    const int hi = __double2hiint(b), lo = __double2loint(b);
+    slow |= !in_range64(hi);
+    // mantissa of b in [1, 2), its reciprocal in (1/2, 1], and that as a double over 2^exponent(b)
+    const float m = __int_as_float(0x3f800000 | ((hi & 0xfffff) << 3) | (int)((unsigned)lo >> 29));
+    const int r = __float_as_int(rcp_approx(m));
+    const double y0 = __hiloint2double((r >> 3) + ((896 + 1023) << 20) - (hi & 0x7ff00000), r << 29);
+    Recip64 R;
+    R.b = b;
+    R.y = fma(y0, fma(-b, y0, 1.0), y0);
+    return R;
+}
+
+__device__ __forceinline__ double quot64(double a, const Recip64 &R, bool &slow)
+{
+    const double q0 = __dmul_rn(a, R.y);
+    const double q = fma(fma(-R.b, q0, a), R.y, q0);
+    const double r = fma(-R.b, q, a);  // exact
+    const int ah = __double2hiint(a) & 0x7fffffff, al = __double2loint(a);
+    const int qh = __double2hiint(q), rh = __double2hiint(r) & 0x7fffffff;
+    const unsigned rl = (unsigned)__double2loint(r);
+    // b * 2^(exponent(q) - 53) by its exponent field
+    const int hh = __double2hiint(R.b) + (qh & 0x7ff00000) - ((1023 + 53) << 20);
+    const unsigned hl = (unsigned)__double2loint(R.b);
+    const bool below = rh < hh || (rh == hh && rl < hl);
+    const bool exact = (rh | (int)rl) == 0;
+    const bool pow2 = ((qh & 0xfffff) | __double2loint(q)) == 0;
+    const bool zero = (ah | al) == 0;
+    slow |= !(zero || (in_range64(ah) && (exact || (below && !pow2))));
+    return zero ? a : q;
+}
+
+// Tests of FP64 values by their bits: a comparison takes the FP64 unit as long as
+// an addition does.  x > 0, x < 0 (false for NaN) and x finite.
+__device__ __forceinline__ bool gt0(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) - 1ull < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool lt0(double x)
+{
+    return (unsigned long long)__double_as_longlong(x) - 0x8000000000000001ull < 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool finite64(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x7ff00000; }
+__device__ __forceinline__ bool nan64(double x)
+{
+    return ((unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
+}
+__device__ __forceinline__ bool below_one(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x3ff00000; }  // |x| < 1
+
 template <> struct Ar<float> {
     static __device__ __forceinline__ float add(float a, float b) { return a + b; }
     static __device__ __forceinline__ float sub(float a, float b) { return a - b; }
@@ -104,6 +189,13 @@ __device__ __forceinline__ void moments9(const T f[9], T &rho, T &ux, T &uy)
     jy = A::sub(jy, f[7]);
     jy = A::sub(jy, f[8]);
     rho = r;
+    if constexpr (std::is_same<T, double>::value) {
+        bool slow = false;
+        const Recip64 R = recip64(r, slow);
+        ux = quot64(jx, R, slow);
+        uy = quot64(jy, R, slow);
+        if (!slow) return;
+    }
     ux = A::div(jx, r);
     uy = A::div(jy, r);
 }
@@ -114,8 +206,14 @@ __device__ __forceinline__ void moments3(const T f[3], T &rho, T &ux, T &uy)
     using A = Ar<T>;
     T r = A::add(A::add(f[0], f[1]), f[2]);
     rho = r;
-    ux = A::div(A::sub(f[2], f[1]), r);
     uy = T(0);
+    const T j = A::sub(f[2], f[1]);
+    if constexpr (std::is_same<T, double>::value) {
+        bool slow = false;
+        ux = quot64(j, recip64(r, slow), slow);
+        if (!slow) return;
+    }
+    ux = A::div(j, r);
 }
 
 // Eq. polyeq2d: f*_k = rho W_k (1 + 3 v_k.u + 9 (v_k.u)^2 / 2 - 3 u^2 / 2).
@@ -127,6 +225,24 @@ __device__ __forceinline__ void feq9(T rho, T ux, T uy, T fs[9])
 {
     using A = Ar<T>;
     const T usq = A::add(A::mul(ux, ux), A::mul(uy, uy));
+    if constexpr (std::is_same<T, double>::value) {
+        // the operations of the printed formula, each rounded on its own, with what
+        // opposite directions share evaluated once: 3 (-c) = -(3 c) and (-c)^2 = c^2,
+        // and the halvings (exact) taken into the following addition
+        const double t3 = A::mul(3.0, usq);
+        fs[0] = A::mul(A::mul(rho, Lat<9>::w(0)), fma(t3, -0.5, 1.0));
+        auto pair = [&](double rw, double c, double &plus, double &minus) {
+            const double c3 = A::mul(3.0, c), s9 = A::mul(9.0, A::mul(c, c));
+            plus = A::mul(rw, fma(t3, -0.5, fma(s9, 0.5, A::add(1.0, c3))));
+            minus = A::mul(rw, fma(t3, -0.5, fma(s9, 0.5, A::sub(1.0, c3))));
+        };
+        const double r1 = A::mul(rho, Lat<9>::w(1)), r5 = A::mul(rho, Lat<9>::w(5));
+        pair(r1, ux, fs[1], fs[3]);
+        pair(r1, uy, fs[2], fs[4]);
+        pair(r5, A::add(ux, uy), fs[5], fs[7]);
+        pair(r5, A::sub(uy, ux), fs[6], fs[8]);
+        return;
+    }
     const T tail = A::mul(A::mul(T(3), usq), T(0.5));
     const T c[9] = {T(0), ux, uy, -ux, -uy, A::add(ux, uy), A::sub(uy, ux), -A::add(ux, uy),
                     A::sub(ux, uy)};
@@ -149,8 +265,19 @@ __device__ __forceinline__ void feq3(T rho, T u, T fs[3])
 {
     using A = Ar<T>;
     const T uu = A::mul(u, u);
-    fs[0] = A::mul(A::div(A::mul(T(2), rho), T(3)), A::sub(T(1), A::mul(A::mul(T(3), uu), T(0.5))));
-    const T r6 = A::div(rho, T(6));
+    T r6;
+    bool slow = true;
+    if constexpr (std::is_same<T, double>::value) {
+        // 2 rho / 3 and rho / 6 are rho / 3 times powers of two: one rounding, the same values
+        slow = false;
+        const double r3 = quot64(rho, Recip64{3.0, 1.0 / 3.0}, slow);
+        fs[0] = A::mul(A::mul(2.0, r3), fma(A::mul(3.0, uu), -0.5, 1.0));
+        r6 = A::mul(0.5, r3);
+    }
+    if (slow) {
+        fs[0] = A::mul(A::div(A::mul(T(2), rho), T(3)), A::sub(T(1), A::mul(A::mul(T(3), uu), T(0.5))));
+        r6 = A::div(rho, T(6));
+    }
     fs[1] = A::mul(r6, A::add(A::sub(T(1), A::mul(T(3), u)), A::mul(T(3), uu)));
     fs[2] = A::mul(r6, A::add(A::add(T(1), A::mul(T(3), u)), A::mul(T(3), uu)));
     if constexpr (std::is_same<T, float>::value) fs[0] = rho - (fs[1] + fs[2]);  // see feq9
@@ -181,14 +308,21 @@ __device__ __forceinline__ void feq(T rho, T ux, T uy, T fs[Q])
 __device__ __forceinline__ bool feq_ent9(double rho, double ux, double uy, double fs[9])
 {
     using A = Ar<double>;
-    if (!(fabs(ux) < 1.0) || !(fabs(uy) < 1.0)) return false;
+    if (!below_one(ux) || !below_one(uy)) return false;
     const double u[2] = {ux, uy};
-    double Aj[2], Xj[2];
+    double Aj[2], Xj[2], Yj[2];  // A, X and A / X of Eq. maxwellian per axis
 #pragma unroll
     for (int j = 0; j < 2; ++j) {
         const double sq = A::sqrt(A::add(1.0, A::mul(3.0, A::mul(u[j], u[j]))));
         Aj[j] = A::sub(2.0, sq);
-        Xj[j] = A::div(A::add(A::mul(2.0, u[j]), sq), A::sub(1.0, u[j]));
+        const double num = A::add(A::mul(2.0, u[j]), sq), den = A::sub(1.0, u[j]);
+        bool slow = false;
+        Xj[j] = quot64(num, recip64(den, slow), slow);
+        Yj[j] = quot64(Aj[j], recip64(Xj[j], slow), slow);
+        if (slow) {
+            Xj[j] = A::div(num, den);
+            Yj[j] = A::div(Aj[j], Xj[j]);
+        }
     }
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
@@ -196,7 +330,7 @@ __device__ __forceinline__ bool feq_ent9(double rho, double ux, double uy, doubl
         double f = A::mul(rho, Lat<9>::w(k));
 #pragma unroll
         for (int j = 0; j < 2; ++j) {
-            const double P = v[j] == 1 ? A::mul(Aj[j], Xj[j]) : (v[j] == -1 ? A::div(Aj[j], Xj[j]) : Aj[j]);
+            const double P = v[j] == 1 ? A::mul(Aj[j], Xj[j]) : (v[j] == -1 ? Yj[j] : Aj[j]);
             f = A::mul(f, P);
         }
         fs[k] = f;
@@ -210,10 +344,12 @@ __device__ __forceinline__ bool feq_ent9(double rho, double ux, double uy, doubl
 __device__ __forceinline__ bool feq_ent3(double rho, double u, double fs[3])
 {
     using A = Ar<double>;
-    if (!(fabs(u) < 1.0)) return false;
+    if (!below_one(u)) return false;
     const double sq = A::sqrt(A::add(1.0, A::mul(3.0, A::mul(u, u))));
-    fs[0] = A::mul(A::div(A::mul(2.0, rho), 3.0), A::sub(2.0, sq));
-    const double r6 = A::div(rho, 6.0);
+    bool slow = false;
+    const double r3 = quot64(rho, Recip64{3.0, 1.0 / 3.0}, slow);
+    const double r6 = slow ? A::div(rho, 6.0) : A::mul(0.5, r3);
+    fs[0] = A::mul(slow ? A::div(A::mul(2.0, rho), 3.0) : A::mul(2.0, r3), A::sub(2.0, sq));
     fs[1] = A::mul(-r6, A::sub(A::add(A::mul(3.0, u), 1.0), A::mul(2.0, sq)));
     fs[2] = A::mul(r6, A::add(A::sub(A::mul(3.0, u), 1.0), A::mul(2.0, sq)));
     return true;
@@ -233,19 +369,22 @@ __device__ __forceinline__ bool feq_any(int eq, double rho, double ux, double uy
     return true;
 }
 
-// f ln(f / f*) for f > 0, f* > 0 (FP64).  Where f is within 2^-5 of f*
-// (almost every site of a flow) by the series of the inverse hyperbolic
-// tangent, ln(f / f*) = 2 atanh z = 2 (z + z^3/3 + z^5/5 + ...) with
-// z = (f - f*) / (f + f*): f - f* is exact there (Sterbenz), z carries two
-// roundings, and with |z| < 0.016 the terms past z^9/9 are below 1e-19 of the
-// sum, so the logarithm is within a few ulps of ln(f / f*) itself.  Elsewhere
-// the CUDA logarithm of the rounded ratio.  The series costs one division and
-// five multiply-adds instead of a division and a general logarithm.
+// f ln(f / f*) for f > 0, f* > 0 (FP64).  Where f is within about 2^-5 of f*
+// (almost every site of a flow; tested on the high words) by the series of the
+// inverse hyperbolic tangent, ln(f / f*) = 2 atanh z = 2 (z + z^3/3 + z^5/5 + ...)
+// with z = (f - f*) / (f + f*): f - f* is exact there (Sterbenz), z carries two
+// roundings (the residual-corrected quotient of quot64, which is within 2^-33 ulp
+// of the rounded one and needs no check here), and with |z| < 0.017 the terms past
+// z^9/9 are below 1e-19 of the sum, so the logarithm is within a few ulps of
+// ln(f / f*) itself.  Elsewhere the CUDA logarithm of the rounded ratio.
 __device__ __forceinline__ double f_ln_ratio(double f, double fs)
 {
-    const double d = f - fs;
-    if (!(fabs(d) < 0.03125 * fs)) return Ar<double>::mul(f, log(Ar<double>::div(f, fs)));
-    const double z = d / (f + fs);
+    const double d = f - fs, den = f + fs;
+    bool far = (__double2hiint(d) & 0x7fffffff) >= __double2hiint(fs) - (5 << 20);
+    const Recip64 R = recip64(den, far);  // den outside 2^-500 .. 2^500: the general form
+    if (far) return Ar<double>::mul(f, log(Ar<double>::div(f, fs)));
+    const double z0 = d * R.y;
+    const double z = fma(fma(-den, z0, d), R.y, z0);
     const double w = z * z;
     double p = fma(w, 1.0 / 9.0, 1.0 / 7.0);
     p = fma(p, w, 1.0 / 5.0);
@@ -264,14 +403,14 @@ __device__ __forceinline__ double rel_entropy(const double f[Q], const double fs
     bool neg = false, nan = false;
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
-        neg |= f[k] < 0.0;
-        nan |= !(f[k] >= 0.0) && !(f[k] < 0.0);
+        neg |= lt0(f[k]);
+        nan |= nan64(f[k]);
     }
     if (neg) return (double)INFINITY;
     double s = 0.0;
 #pragma unroll
     for (int k = 0; k < Q; ++k)
-        if (f[k] > 0.0) s = A::add(s, f_ln_ratio(f[k], fs[k]));
+        if (gt0(f[k])) s = A::add(s, f_ln_ratio(f[k], fs[k]));
     return nan ? (double)NAN : s;
 }
 
@@ -366,78 +505,124 @@ __device__ __forceinline__ T quad_entropy(const T g[Q], const T fs[Q])
     return s;
 }
 
+// The polynomial collision and entropies of a site with every division by
+// __ddiv_rn and every test spelled out: the general case behind site_poly64.
+// out = {f*, f', dS(f'), dS(f_in)}; returns true for a site that cannot be
+// limited.  Not inlined: rarely taken.
+template <int Q>
+__device__ __noinline__ bool site_poly64_ref(const double *fin, double a, bool collide, double *out)
+{
+    using A = Ar<double>;
+    double f[Q], fs[Q], fp[Q], rho, ux, uy;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) f[k] = fin[k];
+    moments<Q, double>(f, rho, ux, uy);
+    bool bad = !(rho > 0.0) || !isfinite(rho) || !isfinite(ux) || !isfinite(uy);
+    feq<Q, double>(rho, ux, uy, fs);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) fp[k] = collide ? A::add(fs[k], A::mul(a, A::sub(fs[k], f[k]))) : f[k];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) bad |= !(fs[k] > 0.0) || !isfinite(f[k]);
+    const double ds = quad_entropy<Q, double>(fp, fs);
+    const double ds_in = collide ? quad_entropy<Q, double>(f, fs) : 0.0;
+    bad |= !isfinite(ds) || !isfinite(ds_in);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        out[k] = fs[k];
+        out[Q + k] = fp[k];
+    }
+    out[2 * Q] = ds;
+    out[2 * Q + 1] = ds_in;
+    return bad;
+}
+
+// The polynomial collision and entropies of a site (site_collide, eq = 0) for
+// the FP64 unit: dS(f') and dS(f_in) share one reciprocal of f*_k, and
+// f* - f_in serves the collision and dS(f_in) alike ((f_in - f*)^2 is the same
+// product).  When no quotient sets `slow`, rho and every f*_k are positive and
+// finite and so are the populations and sums, so the site is good without a
+// single FP64 comparison (each would cost as much as an addition).  The results
+// are those of site_poly64_ref bit for bit.
+template <int Q>
+__device__ __forceinline__ bool site_poly64(const double fin[Q], double a, bool collide, double fs[Q], double fp[Q],
+                                            double &ds, double &ds_in, double &rho, bool need_in)
+{
+    using A = Ar<double>;
+    double ux, uy;
+    bool slow = false;
+    moments<Q, double>(fin, rho, ux, uy);
+    feq<Q, double>(rho, ux, uy, fs);
+    slow |= !in_range64(__double2hiint(rho));
+    ds = 0.0;
+    ds_in = 0.0;
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        const double n = A::sub(fs[k], fin[k]);
+        fp[k] = collide ? A::add(fs[k], A::mul(a, n)) : fin[k];
+        const Recip64 R = recip64(fs[k], slow);
+        const double d = collide ? A::sub(fp[k], fs[k]) : n;
+        const double t = quot64(A::mul(d, d), R, slow);
+        ds = k == 0 ? t : A::add(ds, t);
+        if (collide && need_in) {
+            const double ti = quot64(A::mul(n, n), R, slow);
+            ds_in = k == 0 ? ti : A::add(ds_in, ti);
+        }
+    }
+    if (!slow) return false;
+    double f[Q], out[2 * Q + 2];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) f[k] = fin[k];
+    const bool bad = site_poly64_ref<Q>(f, a, collide, out);
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        fs[k] = out[k];
+        fp[k] = out[Q + k];
+    }
+    ds = out[2 * Q];
+    ds_in = out[2 * Q + 1];
+    return bad;
+}
+
 // Collision and entropy at one site from its arriving populations f_in:
 // f*, f' = f* + a (f* - f_in) with a = 2 beta - 1 (Eq. collLBGK), dS(f'),
 // dS(f_in) and rho.  With collide = false (limiter pass on a stored state)
 // f' = f_in.  Returns true for a site that cannot be limited: rho <= 0, no f*
-// or f*_k <= 0 for some k, or a nonfinite value.  eq = 1 (FP64 only):
-// entropic f* and the exact relative entropy, which is +inf (not an error)
-// for a state with a negative population; need_in = false skips dS(f_in).
+// or f*_k <= 0 for some k, or a nonfinite value.  eq = 1: entropic f* and the
+// exact relative entropy, which is +inf (not an error) for a state with a
+// negative population; need_in = false skips dS(f_in).
 template <int Q, typename T>
 __device__ __forceinline__ bool site_collide(const T fin[Q], T a, bool collide, T fs[Q], T fp[Q],
                                              T &ds, T &ds_in, T &rho, int eq = 0, bool need_in = true,
                                              int coll = 0, double beta = 0.0)
 {
     using A = Ar<T>;
+    static_assert(std::is_same<T, double>::value, "FP32 sites take site_collide_dev");
+    if (eq != 1) return site_poly64<Q>(fin, a, collide, fs, fp, ds, ds_in, rho, need_in);
     T ux, uy;
     moments<Q, T>(fin, rho, ux, uy);
-    bool bad = !(rho > T(0)) || !isfinite(rho) || !isfinite(ux) || !isfinite(uy);
-    if constexpr (std::is_same<T, double>::value) {
-        if (eq == 1) {
-            if (!feq_any<Q>(1, rho, ux, uy, fs)) {
-                bad = true;
+    bool bad = !gt0(rho) || !finite64(rho) || !finite64(ux) || !finite64(uy);
+    if (!feq_any<Q>(1, rho, ux, uy, fs)) {
+        bad = true;
 #pragma unroll
-                for (int k = 0; k < Q; ++k) fs[k] = 0.0;
-            }
-#pragma unroll
-            for (int k = 0; k < Q; ++k) fp[k] = collide ? A::add(fs[k], A::mul(a, A::sub(fs[k], fin[k]))) : fin[k];
-#pragma unroll
-            for (int k = 0; k < Q; ++k) bad |= !(fs[k] > 0.0) || !isfinite(fs[k]) || !isfinite(fin[k]);
-            if (coll == 1 && collide && !bad) {
-                // Eq. elbm: f' = (1 - beta) f + beta f~ = f + (beta alpha)(f* - f)
-                const double ba = A::mul(beta, elbm_alpha<Q>(fin, fs));
-#pragma unroll
-                for (int k = 0; k < Q; ++k) fp[k] = A::add(fin[k], A::mul(ba, A::sub(fs[k], fin[k])));
-            }
-            ds = bad ? 0.0 : rel_entropy<Q>(fp, fs);
-            // dS(f_in) feeds only the statistics: sites that only supply a
-            // stencil value (need_in = false) skip it; with finite populations
-            // and f* > 0 it is never NaN, so the flag does not depend on it
-            ds_in = (bad || !collide || !need_in) ? 0.0 : rel_entropy<Q>(fin, fs);
-            bad |= isnan(ds) || isnan(ds_in);
-            return bad;
-        }
+        for (int k = 0; k < Q; ++k) fs[k] = 0.0;
     }
-    feq<Q, T>(rho, ux, uy, fs);
 #pragma unroll
     for (int k = 0; k < Q; ++k) fp[k] = collide ? A::add(fs[k], A::mul(a, A::sub(fs[k], fin[k]))) : fin[k];
 #pragma unroll
-    for (int k = 0; k < Q; ++k) bad |= !(fs[k] > T(0)) || !isfinite(fin[k]);
-    ds = quad_entropy<Q, T>(fp, fs);
-    ds_in = collide ? quad_entropy<Q, T>(fin, fs) : T(0);
-    bad |= !isfinite(ds) || !isfinite(ds_in);
-    return bad;
-}
-
-// FP64 dS(f') of the collision alone (the Ehrenfests' key): same operations as
-// site_collide, without dS(f_in).  Returns false for a site that cannot be limited.
-__device__ __forceinline__ bool key_dS9(const double fin[9], double a, double &ds)
-{
-    using A = Ar<double>;
-    double rho, ux, uy, fs[9];
-    moments9<double>(fin, rho, ux, uy);
-    feq9<double>(rho, ux, uy, fs);
-    bool bad = !(rho > 0.0) || !isfinite(rho) || !isfinite(ux) || !isfinite(uy);
-    double s = 0.0;
+    for (int k = 0; k < Q; ++k) bad |= !gt0(fs[k]) || !finite64(fs[k]) || !finite64(fin[k]);
+    if (coll == 1 && collide && !bad) {
+        // Eq. elbm: f' = (1 - beta) f + beta f~ = f + (beta alpha)(f* - f)
+        const double ba = A::mul(beta, elbm_alpha<Q>(fin, fs));
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        bad |= !(fs[k] > 0.0) || !isfinite(fin[k]);
-        const double fp = A::add(fs[k], A::mul(a, A::sub(fs[k], fin[k])));
-        const double d = A::sub(fp, fs[k]);
-        s = A::add(s, A::div(A::mul(d, d), fs[k]));
+        for (int k = 0; k < Q; ++k) fp[k] = A::add(fin[k], A::mul(ba, A::sub(fs[k], fin[k])));
     }
-    ds = s;
-    return !bad && isfinite(s);
+    ds = bad ? 0.0 : rel_entropy<Q>(fp, fs);
+    // dS(f_in) feeds only the statistics: sites that only supply a
+    // stencil value (need_in = false) skip it; with finite populations
+    // and f* > 0 it is never NaN, so the flag does not depend on it
+    ds_in = (bad || !collide || !need_in) ? 0.0 : rel_entropy<Q>(fin, fs);
+    bad |= nan64(ds) || nan64(ds_in);
+    return bad;
 }
 
 // Positivity rule (Sec. 3.1): largest lambda <= 1 such that f* + lambda (f' - f*) >= 0.
@@ -469,15 +654,6 @@ __device__ __forceinline__ T phi_median(T x, T med, T delta, int mode)
     }
     const T t = med > delta ? med : delta;
     return x > t ? A::sqrt(A::div(t, x)) : T(1);
-}
-
-// Hardware reciprocal approximation (one special-function instruction,
-// relative error below 2^-22): the FP32 entropy denominators.
-__device__ __forceinline__ float rcp_approx(float x)
-{
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
 }
 
 // ---------------------------------------------------------------------------
