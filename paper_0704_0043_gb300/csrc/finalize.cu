@@ -9,11 +9,13 @@
 // 64-bit pattern of dS (positive doubles order like their bit patterns), then
 // four passes over the site index among the candidates tied at the threshold.
 //
-// The kernel sits between two step launches, so it is built for latency: the
-// candidates arrive with their FP64 keys (the step kernels evaluate them where
-// they find them), up to kCap of them are kept in shared memory, and sums use
-// warp shuffles or exact integer arithmetic.  One block runs the tail.  When a
-// pass records more candidates than that (a state far from equilibrium), the
+// The kernel sits between two step launches, so it is built for latency: one
+// block runs it, most candidates arrive with their FP64 keys, the selection
+// (select.cuh) keys only those of the others that can matter, and sums use warp
+// shuffles or exact integer arithmetic.  The tail starts from a cold instruction
+// cache (about 10 ns per instruction fetched), so rarely taken parts are out of
+// line.  When a pass records more candidates than the block holds in shared
+// memory (a state far from equilibrium), the
 // tail runs as a cooperative grid of one block per SM that first preselects
 // them (dense_select): the FP32 dS recorded with each candidate is within 1/64
 // of its FP64 key, so a radix search over the FP32 values bounds the k-th
@@ -24,127 +26,12 @@
 #include "internal.h"
 #include "keys.cuh"
 #include "lattice.cuh"
+#include "select.cuh"
 
 namespace lbm {
 namespace {
 
-constexpr int kFinThreads = 512;
-constexpr int kFinWarps = kFinThreads / 32;
-constexpr int kCap = 2048;  // candidates held (and selected sets sorted) in shared memory
-constexpr unsigned kFull = 0xffffffffu;
 constexpr unsigned kSelSpinLimit = 1u << 21;  // grid-barrier polls (about a second) before giving up
-
-__device__ __forceinline__ unsigned long long key_bits(double d) { return (unsigned long long)__double_as_longlong(d); }
-
-__device__ __forceinline__ long long fidx(long long plane, int pitch, int k, int y, int x)
-{
-    return (long long)k * plane + (long long)y * pitch + kLead + x;
-}
-
-// The pass's input at site (x, y) in FP32: after free flight (collide) with the
-// step kernels' FP32 arithmetic (bounce-back, lid term added as hi + lo), or
-// the stored populations themselves (limiter pass).
-template <int Q, typename S>
-__device__ void pull_dev(const FinalParams &p, int x, int y, float g[Q])
-{
-    const S *src = (const S *)p.src;
-    const bool wrapx = bc_wrap_x(p.boundary), wrapy = Q == 9 && bc_wrap_y(p.boundary);
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        if (!p.collide) {
-            g[k] = s2f(src[fidx(p.plane, p.pitch, k, y, x)]);
-            continue;
-        }
-        int sx = x - Lat<Q>::cx(k), sy = y - Lat<Q>::cy(k);
-        if (wrapx) sx = sx < 0 ? sx + p.nx : (sx >= p.nx ? sx - p.nx : sx);
-        if (wrapy) sy = sy < 0 ? sy + p.ny : (sy >= p.ny ? sy - p.ny : sy);
-        if (sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny) {
-            g[k] = s2f(src[fidx(p.plane, p.pitch, k, sy, sx)]);
-        } else {
-            float v = s2f(src[fidx(p.plane, p.pitch, Lat<Q>::opp(k), y, x)]);
-            if (Q == 9 && sy > p.ny - 1) v = __fadd_rn(__fadd_rn(v, p.lidf[k]), p.lidlo[k]);
-            g[k] = v;
-        }
-    }
-}
-
-// Sum over the block in a fixed order (same result every run): warp shuffle
-// trees, then a shuffle tree over the warp totals; thread 0 gets the sum.
-// FP64 additions are slow on this GPU, so the dependent chain is kept short.
-// `warp0_only`: the other warps hold zeros, so warp 0's tree is the sum (the
-// same bits: adding the zero totals changes nothing).
-__device__ double block_sum0(double v, double *red, bool warp0_only)
-{
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    if (warp0_only && warp != 0) return 0.0;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-    if (warp0_only) return v;
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        double r = lane < kFinWarps ? red[lane] : 0.0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) r += __shfl_down_sync(kFull, r, o);
-        v = r;
-    }
-    return v;
-}
-
-
-// The digit of a radix-selection pass: hist[d] counts the keys with digit d
-// among those still in play, and the rem-th of them is wanted, counting from
-// the top digit down (desc) or from digit 0 up.  Threads 0..255 scan the
-// counts with warp shuffles (integer sums, so the same on every run) and the
-// block picks the digit with __syncthreads_count; every thread of the block
-// must call this.  Writes the digit to *digit and the rank left within it to
-// *rem_left.
-__device__ void pick_digit(const unsigned *hist, long long rem, bool desc, unsigned long long *part,
-                           unsigned long long *digit, long long *rem_left)
-{
-    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    unsigned long long c = 0;
-    if (t < 256) {
-        c = hist[desc ? 255 - t : t];  // position t of the scan order
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned long long y = __shfl_up_sync(0xffffffffu, c, o);
-            if (lane >= o) c += y;
-        }
-        if (lane == 31) part[w] = c;
-    }
-    __syncthreads();
-    if (t < 256)
-        for (int j = 0; j < w; ++j) c += part[j];
-    // c = inclusive count up to scan position t; the wanted digit is the first
-    // position whose inclusive count reaches rem
-    const int before = __syncthreads_count(t < 256 && (long long)c < rem);
-    if (t == before && t < 256) {
-        *digit = (unsigned long long)(desc ? 255 - t : t);
-        *rem_left = rem - ((long long)c - (long long)hist[desc ? 255 - t : t]);
-    }
-    __syncthreads();
-}
-
-// The geometry of the FP64 key evaluation (D2Q9, FP32 / 16-bit storage).
-__device__ KeyGeom key_geom(const FinalParams &p)
-{
-    KeyGeom kg;
-    kg.nx = p.nx;
-    kg.ny = p.ny;
-    kg.pitch = p.pitch;
-    kg.boundary = p.boundary;
-    kg.plane = p.plane;
-    kg.a = p.a;
-    kg.rw0 = p.rw[0];
-    kg.rw1 = p.rw[1];
-    kg.rw5 = p.rw[5];
-    kg.lid4 = p.lid[4];
-    kg.lid7 = p.lid[7];
-    kg.lid8 = p.lid[8];
-    kg.eq = p.eq;
-    return kg;
-}
 
 // Grid barrier of the cooperative tail: each block adds one arrival to *bar;
 // with `wait` it polls until `target` blocks have arrived.  The poll is
@@ -398,7 +285,7 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
 // GRID: the cooperative grid of one block per SM (dense candidates are
 // preselected by all blocks; block 0 runs the tail); otherwise one block.
 template <int Q, typename S, bool BATCHED, bool GRID = false>
-__global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const FinalParams p0, S *__restrict__ f0,
+__global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const __grid_constant__ FinalParams p0, S *__restrict__ f0,
                                                           const FinalArgs *__restrict__ table)
 {
     using T = compute_t<S>;
@@ -411,9 +298,7 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
     // them are resident, so its blocks cannot keep one of ours from running
     // (the grid barriers below wait for resident blocks only).
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    __shared__ double s_key[kCap];
-    __shared__ int s_site[kCap];
-    __shared__ int s_idx[kCap];
+    __shared__ SelShared sh;
     __shared__ long long s_wpart[kFinWarps], s_rem2, s_tot;
     __shared__ int s_bin, s_flag, s_qn;
     __shared__ unsigned s_acc, s_cnt, s_nv;
@@ -427,7 +312,7 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
         const bool dense = n0 > kCap && p0.sel_state != nullptr && p0.k_max > 0;
         if (!dense && blockIdx.x != 0) return;
         if (dense) {
-            use_list = dense_select<Q, S>(p0, n0, reinterpret_cast<unsigned *>(s_key), s_wpart, &s_bin, &s_rem2,
+            use_list = dense_select<Q, S>(p0, n0, reinterpret_cast<unsigned *>(sh.key), s_wpart, &s_bin, &s_rem2,
                                           &s_tot, &s_flag, &s_qn, &s_acc, &s_cnt, &s_nv);
             if (blockIdx.x != 0) return;
         }
@@ -441,12 +326,8 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
     }
     const FinalParams &p = BATCHED ? sA.p : p0;
     S *__restrict__ f = BATCHED ? (S *)sA.f : f0;
-    __shared__ double red[kFinWarps + 1];
     __shared__ double tot[P_NSTAT];
-    __shared__ unsigned hist[256];
-    __shared__ unsigned long long s_part[8], s_digit;
-    __shared__ long long s_rem, s_step, s_rec;
-    __shared__ int s_nsel, s_valid;
+    __shared__ long long s_step, s_rec;
     __shared__ unsigned s_status;
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
 
@@ -462,16 +343,14 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
         const int nrec = *p.cand_count;
         n = nrec < p.cand_cap ? nrec : p.cand_cap;
     }
-    const int *list = use_list ? p.sel_state->list : nullptr;
-    auto cidx = [&](int i) -> int { return use_list ? list[i] : i; };
     Cand first{};
-    if (!BATCHED && p.ehrenfest && (use_list ? t < n : t < p.cand_cap)) first = p.cand[cidx(t)];
+    if (!BATCHED && p.ehrenfest && (use_list ? t < n : t < p.cand_cap)) first = p.cand[use_list ? p.sel_state->list[t] : t];
     if (t == 0) {
         s_step = p.counters[0];
         s_rec = p.counters[1];
         s_status = *p.status;
-        s_nsel = 0;
-        s_valid = use_list ? (int)s_nv : 0;
+        sh.nsel = 0;
+        sh.valid = use_list ? (int)s_nv : 0;
     }
     if (p.fixed) {
         // the fused kernel's kFxRows fixed-point accumulator rows (exact integer
@@ -536,266 +415,17 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
         double v = (v0 + v1) + (v2 + v3);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-        if (lane == 0) red[warp] = v;
+        if (lane == 0) sh.red[warp] = v;
     }
     __syncthreads();
-    if (!p.fixed && t < P_NSTAT) tot[t] = red[2 * t] + red[2 * t + 1];
+    if (!p.fixed && t < P_NSTAT) tot[t] = sh.red[2 * t] + sh.red[2 * t + 1];
     __syncthreads();
-    const bool small = n <= kCap;  // candidates held in shared memory
-    const long long k = p.k_max;
-
-    // candidate keys: FP64 dS(f'), written with the candidates by the step
-    // kernels (sites at or below the threshold carry -1); the fused kernel
-    // leaves NaN where a warp had more candidates than it keys itself, and
-    // those are keyed here, one thread per candidate, with the same operations.
-    // The preselected list holds keyed, valid candidates and their count.
-    constexpr bool kLowPrec = !std::is_same<S, double>::value;
-    if (use_list) {
-        for (int i = t; i < n && small; i += kFinThreads) {
-            const Cand c = !BATCHED && i == t ? first : p.cand[list[i]];
-            s_key[i] = c.key;
-            s_site[i] = c.site;
-        }
-    } else {
-        for (int i = t; i < n; i += kFinThreads) {
-            Cand c = !BATCHED && i == t ? first : p.cand[i];
-            if constexpr (kLowPrec && Q == 9) {
-                if (isnan(c.key)) c.key = key_dS9_lane<S>(key_geom(p), (const S *)p.src, c.site, p.delta_e);
-            }
-            // below the threshold -> -1, so that from here on a key is valid
-            // exactly when its bit pattern is a positive integer (FP64 compares
-            // are slow on this GPU; positive doubles order like their patterns)
-            if (!(c.key > p.delta_e) && c.key != -1.0) c.key = -1.0;
-            if (small) {
-                s_key[i] = c.key;
-                s_site[i] = c.site;
-            } else {
-                p.cand[i].key = c.key;
-            }
-        }
-    }
-    __syncthreads();
-    auto key_of = [&](int i) -> double { return small ? s_key[i] : p.cand[cidx(i)].key; };
-    auto site_of = [&](int i) -> int { return small ? s_site[i] : p.cand[cidx(i)].site; };
-    if (!use_list) {
-        int nv = 0;
-        for (int i = t; i < n; i += kFinThreads) nv += (long long)key_bits(key_of(i)) > 0;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) nv += __shfl_down_sync(kFull, nv, o);
-        if (lane == 0 && nv) atomicAdd(&s_valid, nv);
-    }
-    __syncthreads();
-    const int n_valid = s_valid;
+    int n_valid = 0;
     double ehr_sum = 0.0;
-    const bool ehr_active = p.ehrenfest && k > 0 && n_valid > 0;  // the same for the whole block
-    if (ehr_active) {
-        unsigned long long kv = 0;  // threshold dS pattern
-        int site_thr = 0x7fffffff;
-        const bool take_all = (long long)n_valid <= k;
-        // few candidates (held in shared memory, at most one per thread): each
-        // thread ranks its own by counting the keys that beat it (larger dS, or
-        // equal dS at a lower site) -- one pass instead of the digit passes
-        const bool by_rank = !take_all && small && n <= kFinThreads;
-        if (by_rank) {
-            bool chosen = false;
-            if (t < n) {
-                const unsigned long long u = key_bits(s_key[t]);
-                const int st = s_site[t];
-                long long rank = 0;
-                if ((long long)u > 0) {
-                    for (int j = 0; j < n; ++j) {
-                        const unsigned long long v = key_bits(s_key[j]);
-                        rank += (long long)v > 0 && (v > u || (v == u && s_site[j] < st));
-                    }
-                    chosen = rank < k;
-                }
-            }
-            if (chosen) {
-                const int j = atomicAdd(&s_nsel, 1);
-                if (j < p.sel_cap) p.sel[j] = cidx(t);
-                if (j < kCap) s_idx[j] = t;
-            }
-        }
-        if (!take_all && !by_rank) {
-            unsigned long long prefix = 0, mask = 0;
-            long long rem = k;
-            for (int shift = 56; shift >= 0; shift -= 8) {
-                for (int d = t; d < 256; d += kFinThreads) hist[d] = 0;
-                __syncthreads();
-                for (int i = t; i < n; i += kFinThreads) {
-                    const double key = key_of(i);
-                    const unsigned long long u = key_bits(key);
-                    if ((long long)u > 0 && (u & mask) == prefix) atomicAdd(&hist[(u >> shift) & 255u], 1u);
-                }
-                __syncthreads();
-                pick_digit(hist, rem, true, s_part, &s_digit, &s_rem);
-                prefix = prefix | (s_digit << shift);
-                rem = s_rem;
-                mask |= 255ull << shift;
-                __syncthreads();
-            }
-            kv = prefix;
-            // among the candidates with dS == kv take the `rem` lowest sites
-            unsigned sprefix = 0, smask = 0;
-            for (int shift = 24; shift >= 0; shift -= 8) {
-                for (int d = t; d < 256; d += kFinThreads) hist[d] = 0;
-                __syncthreads();
-                for (int i = t; i < n; i += kFinThreads) {
-                    const double key = key_of(i);
-                    const unsigned s = (unsigned)site_of(i);
-                    if ((long long)key_bits(key) > 0 && key_bits(key) == kv && (s & smask) == sprefix)
-                        atomicAdd(&hist[(s >> shift) & 255u], 1u);
-                }
-                __syncthreads();
-                pick_digit(hist, rem, false, s_part, &s_digit, &s_rem);
-                sprefix = sprefix | ((unsigned)s_digit << shift);
-                rem = s_rem;
-                smask |= 255u << shift;
-                __syncthreads();
-            }
-            site_thr = (int)sprefix;
-        }
-        // compaction of the chosen candidates: candidate indices in p.sel, list
-        // entries in s_idx (the first kCap)
-        for (int i = t; i < n && !by_rank; i += kFinThreads) {
-            const double key = key_of(i);
-            const unsigned long long u = key_bits(key);
-            const bool chosen = (long long)u > 0 && (take_all || u > kv || (u == kv && site_of(i) <= site_thr));
-            if (chosen) {
-                const int j = atomicAdd(&s_nsel, 1);
-                if (j < p.sel_cap) p.sel[j] = cidx(i);
-                if (j < kCap) s_idx[j] = i;
-            }
-        }
-        __syncthreads();
-        if (t == 0 && s_nsel > p.sel_cap) s_nsel = p.sel_cap;
-        __syncthreads();
-        const int nsel = s_nsel;
-        const bool sorted = nsel <= kCap;
-        if (sorted) {
-            // bitonic sort of the chosen set by site index (padding sorts last).
-            // The payload is s_idx (chosen list entries, -1 for padding); the
-            // sort key is the site: read through s_site when the candidates are
-            // held in shared memory, else copied into s_site first (then free)
-            int m = 1;
-            while (m < nsel) m <<= 1;
-            for (int i = t; i < m; i += kFinThreads) {
-                if (i >= nsel) s_idx[i] = -1;
-                if (!small) s_site[i] = i < nsel ? site_of(s_idx[i]) : 0x7fffffff;
-            }
-            __syncthreads();
-            auto skey = [&](int i) -> int {
-                if (!small) return s_site[i];
-                const int li = s_idx[i];
-                return li >= 0 ? s_site[li] : 0x7fffffff;
-            };
-            for (int size = 2; size <= m; size <<= 1) {
-                for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                    for (int i = t; i < m; i += kFinThreads) {
-                        const int j = i ^ stride;
-                        if (j > i) {
-                            const bool up = (i & size) == 0;
-                            const int ki = skey(i), kj = skey(j);
-                            if ((ki > kj) == up) {
-                                int a = s_idx[i]; s_idx[i] = s_idx[j]; s_idx[j] = a;
-                                if (!small) {
-                                    s_site[i] = kj;
-                                    s_site[j] = ki;
-                                }
-                            }
-                        }
-                    }
-                    __syncthreads();
-                }
-            }
-        }
-        // Ehrenfests' step at each chosen site, in site order when sorted
-        for (int r = t; r < nsel; r += kFinThreads) {
-            // the chosen candidate's site and key (from shared memory when
-            // sorted) and its phi
-            int site;
-            double key, phi;
-            if (sorted) {
-                const int li = s_idx[r];
-                site = small ? s_site[li] : s_site[r];
-                key = key_of(li);
-                phi = p.cand[cidx(li)].phi;
-            } else {
-                const Cand c = p.cand[p.sel[r]];
-                site = c.site;
-                key = c.key;
-                phi = c.phi;
-            }
-            const int x = site % p.nx, y = site / p.nx;
-            T g[Q], fs[Q], rho, ux, uy;
-            bool write = true;
-            if constexpr (std::is_same<T, float>::value) {
-                // FP32 / 16-bit storage: f*(m) as g - n (the limiter with phi = 0),
-                // m taken from the pass's input (the collision conserves m), so
-                // mass and momentum are kept and the result is rounded once
-                float drho, nq[Q];
-                pull_dev<Q, S>(p, x, y, g);
-                moments_dev<Q>(g, p.rho_ref, drho, rho, ux, uy);
-                if (p.eq == 1) {
-                    // entropic f*: from the limited state in FP64 (the stored values), the
-                    // entropy the step adds, dS w.r.t. its own f*; a state whose moments
-                    // have no entropic f* keeps its populations
-                    double fl[Q], fsd[Q], r2, a2, b2;
-#pragma unroll
-                    for (int q = 0; q < Q; ++q)
-                        fl[q] = Ar<double>::add((double)s2f(f[fidx(p.plane, p.pitch, q, y, x)]), p.rw[q]);
-                    moments<Q, double>(fl, r2, a2, b2);
-                    write = feq_any<Q>(1, r2, a2, b2, fsd);
-                    if (write) {
-                        const double d = rel_entropy<Q>(fl, fsd);
-                        if (isfinite(d)) ehr_sum = Ar<double>::add(ehr_sum, d);
-                        if constexpr (Q == 9)
-                            feq_ent9_x<F1>(drho, rho, ux, uy, fs);
-                        else
-                            feq_ent3_dev(drho, rho, ux, fs);
-                    } else {
-#pragma unroll
-                        for (int q = 0; q < Q; ++q) fs[q] = 0.f;
-                    }
-                } else {
-                    feq_dev<Q>(drho, rho, ux, uy, fs);
-                }
-                neq_dev<Q>(g, fs, nq);
-#pragma unroll
-                for (int q = 0; q < Q; ++q) fs[q] = g[q] - nq[q];
-            } else {
-                // FP64: f*(m(f')) from the stored f', in the oracle's order
-#pragma unroll
-                for (int q = 0; q < Q; ++q) g[q] = s2f(f[fidx(p.plane, p.pitch, q, y, x)]);
-                moments<Q, T>(g, rho, ux, uy);
-                if (p.eq == 1) {
-                    // entropic f*: the step adds dS of the limited state w.r.t. its own f*
-                    // where the limited state's moments have no entropic f* the site keeps its populations
-                    write = feq_any<Q>(1, rho, ux, uy, fs);
-                    const double d = write ? rel_entropy<Q>(g, fs) : (double)NAN;
-                    if (isfinite(d)) ehr_sum = Ar<double>::add(ehr_sum, d);
-                } else {
-                    feq<Q, T>(rho, ux, uy, fs);
-                }
-            }
-            if (write) {
-#pragma unroll
-                for (int q = 0; q < Q; ++q) f[fidx(p.plane, p.pitch, q, y, x)] = f2s<S>(fs[q]);
-            }
-            if (p.eq != 1) ehr_sum = Ar<double>::add(ehr_sum, Ar<double>::mul(Ar<double>::mul(phi, phi), key));
-        }
-        __syncthreads();
-        // the chosen sites, as site indices, for lbm_limited_sites
-        if (sorted) {
-            for (int r = t; r < nsel; r += kFinThreads) p.sel[r] = small ? s_site[s_idx[r]] : s_site[r];
-        } else {
-            // unsorted (more than kCap chosen): convert in place, one owner per slot
-            for (int r = t; r < nsel; r += kFinThreads) p.sel[r] = p.cand[p.sel[r]].site;
-        }
-    }
+    if (n > 0) ehr_sum = finish_candidates<Q, S>(p, f, n, use_list, !BATCHED, first, sh, n_valid);
     // thread r applied chosen site r: with at most 32 of them only warp 0
     // holds terms
-    const double esum = ehr_active ? block_sum0(ehr_sum, red, s_nsel <= 32) : 0.0;
+    const double esum = sh.nsel > 0 ? block_sum0(ehr_sum, sh.red, sh.nsel <= 32) : 0.0;
     if (t == 0) {
         long long step = s_step;
         if (p.collide) {
@@ -812,7 +442,7 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
         st.dS_lim = Ar<double>::add(tot[P_DS_LIM], esum);
         st.n_pos = (long long)tot[P_NPOS];
         st.n_med = (long long)tot[P_NMED];
-        st.n_ehr = s_nsel;
+        st.n_ehr = sh.nsel;
         st.n_cand = n_valid;
         st.n_bad = (long long)tot[P_NBAD];
         // the step kernel set its status bits before this launch began
@@ -840,7 +470,7 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
             slot[1] = a;
             slot[2] = b;
         }
-        *p.sel_count = s_nsel;
+        *p.sel_count = sh.nsel;
         *p.cand_count = 0;
         if (p.work != nullptr) *p.work = 0;  // the next fused launch starts at its first item
     }

@@ -57,59 +57,68 @@ __device__ __noinline__ double key_ent9(const KeyGeom p, const S *src, int site,
     return !bad && ds > delta_e ? ds : -1.0;
 }
 
-// FP64 key dS(f') of `site`, evaluated by the whole (converged) warp: lane k < 9
-// pulls population k and evaluates f*_k and its dS term; the moments and the
-// final sum run in k order exactly as the sequential FP64 evaluation runs them,
-// so the key is the same bit for bit.  Returns the key, or -1 for a site at or
-// below delta_e or one that cannot be limited (rho <= 0, some f*_k <= 0,
-// nonfinite); every lane returns the same value.  Not inlined: the caller's
-// hot loop keeps its registers, and the call is rare.
+// FP64 keys dS(f') of up to three sites by the whole (converged) warp: lanes
+// 9 g .. 9 g + 8 take the site that lane's `site` argument names (lanes 27 .. 31
+// repeat group 0), a lane per direction.  Lane 0 of a group sums rho, lane 1
+// rho u_x and lane 2 rho u_y, each in k order as the sequential evaluation does;
+// the two quotients run together; every lane then evaluates its f*_k and its dS
+// term, and the terms are added in k order: the key is that of key_dS9_lane bit
+// for bit, in 48 FP64 instructions where one lane alone needs about 190.  Returns the key,
+// or -1 for a site at or below delta_e or one that cannot be limited; every
+// lane of a group returns the same value.  Not inlined: the caller's hot loop
+// keeps its registers, and the call is rare.
 template <typename S>
-__device__ __noinline__ double key_dS9_warp(const KeyGeom p, const S *src, int site, double delta_e)
+__device__ __noinline__ double key_dS9_group(const KeyGeom p, const S *src, int site, double delta_e)
 {
     using A = Ar<double>;
     constexpr unsigned kAll = 0xffffffffu;
-    if (p.eq == 1) return key_ent9<S>(p, src, site, delta_e);  // every lane, the same value
-    const int lane = threadIdx.x & 31, k = lane < 9 ? lane : 0;
+    if (p.eq == 1) return key_ent9<S>(p, src, site, delta_e);
+    const int lane = threadIdx.x & 31, base = lane < 27 ? lane / 9 * 9 : 0, k = lane < 27 ? lane % 9 : lane - 27;
     const int x = site % p.nx, y = site / p.nx;
     const double mine = pull_one_f64<S>(p, src, x, y, k);
-    double fin[9];
+    // lane 0: f0 + f1 + ... + f8; lane 1: f1 - f3 + f5 - f6 - f7 + f8; lane 2: f2 - f4 + f5
+    // + f6 - f7 - f8 (four bits per term: direction, 15 for none; a bit per sign)
+    const unsigned long long order = k == 1 ? 0xfff876531ull : (k == 2 ? 0xfff876542ull : 0x876543210ull);
+    const unsigned minus = k == 1 ? 0x01au : (k == 2 ? 0x032u : 0u);
+    double acc = 0.0;
 #pragma unroll
-    for (int j = 0; j < 9; ++j) fin[j] = __shfl_sync(kAll, mine, j);
-    double rho, ux, uy;
-    moments9<double>(fin, rho, ux, uy);
+    for (int j = 0; j < 9; ++j) {
+        const int d = (int)(order >> (4 * j)) & 15;
+        const double v = __shfl_sync(kAll, mine, base + (d < 9 ? d : 0));
+        const double w = __hiloint2double(__double2hiint(v) ^ (int)(((minus >> j) & 1u) << 31), __double2loint(v));
+        const double sum = j == 0 ? w : A::add(acc, w);
+        acc = d < 9 ? sum : acc;
+    }
+    const double rho = __shfl_sync(kAll, acc, base);
+    bool slow = false;
+    double u = quot64(acc, recip64(rho, slow), slow);
+    if (slow) u = A::div(acc, rho);
+    const double ux = __shfl_sync(kAll, u, base + 1), uy = __shfl_sync(kAll, u, base + 2);
     // f*_k as in feq9<double>
     const double usq = A::add(A::mul(ux, ux), A::mul(uy, uy));
-    const double tail = A::mul(A::mul(3.0, usq), 0.5);
-    const double c = k == 0 ? 0.0
-                   : k == 1 ? ux
-                   : k == 2 ? uy
-                   : k == 3 ? -ux
-                   : k == 4 ? -uy
-                   : k == 5 ? A::add(ux, uy)
-                   : k == 6 ? A::sub(uy, ux)
-                   : k == 7 ? -A::add(ux, uy)
-                            : A::sub(ux, uy);
-    double poly = A::add(A::add(1.0, A::mul(3.0, c)), A::mul(A::mul(9.0, A::mul(c, c)), 0.5));
-    poly = A::sub(poly, tail);
+    const double t3 = A::mul(3.0, usq);
+    const double both = (k == 6 || k == 8) ? A::sub(uy, ux) : A::add(ux, uy);
+    const double c = k == 0 ? 0.0 : ((k == 1 || k == 3) ? ux : ((k == 2 || k == 4) ? uy : both));
+    const bool opp = k == 3 || k == 4 || k == 7 || k == 8;
+    const double c3 = A::mul(3.0, c), s9 = A::mul(9.0, A::mul(c, c));
+    const double poly = fma(t3, -0.5, fma(s9, 0.5, A::add(1.0, opp ? -c3 : c3)));
     const double fs = A::mul(A::mul(rho, Lat<9>::w(k)), poly);
-    // collision and the dS term as in the sequential evaluation
+    // collision and the dS term
     const double fp = A::add(fs, A::mul(p.a, A::sub(fs, mine)));
-    const double d = A::sub(fp, fs);
-    bool slow = false;
-    double term = quot64(A::mul(d, d), recip64(fs, slow), slow);
-    if (slow) term = A::div(A::mul(d, d), fs);
-    const bool bad_k = lane < 9 && (!(fs > 0.0) || !isfinite(mine));
-    double s = 0.0;
+    const double d = A::sub(fp, fs), dd = A::mul(d, d);
+    bool slow_t = false;
+    double term = quot64(dd, recip64(fs, slow_t), slow_t);
+    if (slow_t) term = A::div(dd, fs);
+    const unsigned bad_lanes = __ballot_sync(kAll, !gt0(fs) || !finite64(mine));
+    double s = __shfl_sync(kAll, term, base);
 #pragma unroll
-    for (int j = 0; j < 9; ++j) s = A::add(s, __shfl_sync(kAll, term, j));
-    const bool bad = __any_sync(kAll, bad_k) || !(rho > 0.0) || !isfinite(rho) || !isfinite(ux) || !isfinite(uy);
-    return !bad && isfinite(s) && s > delta_e ? s : -1.0;
+    for (int j = 1; j < 9; ++j) s = A::add(s, __shfl_sync(kAll, term, base + j));
+    const bool bad = ((bad_lanes >> base) & 0x1ffu) != 0 || !gt0(rho) || !finite64(rho) || !finite64(ux) || !finite64(uy);
+    return !bad && finite64(s) && s > delta_e ? s : -1.0;
 }
 
 // The same key evaluated by one thread alone (lane-parallel keying of many
-// candidates: each lane keys its own site).  The operations and their order
-// are those of key_dS9_warp, so both give the same bits.
+// candidates: each lane keys its own site).
 template <typename S>
 __device__ __noinline__ double key_dS9_lane(const KeyGeom p, const S *src, int site, double delta_e)
 {
@@ -120,6 +129,32 @@ __device__ __noinline__ double key_dS9_lane(const KeyGeom p, const S *src, int s
     for (int k = 0; k < 9; ++k) fin[k] = pull_one_f64<S>(p, src, x, y, k);
     const bool bad = site_poly64<9>(fin, p.a, true, fs, fp, ds, dsin, rho, false);
     return !bad && ds > delta_e ? ds : -1.0;
+}
+
+// The key of a D1Q3 site (closed or periodic tube) by one thread.
+template <typename S>
+__device__ __noinline__ double key_dS3_lane(const KeyGeom p, const S *src, int x, double delta_e)
+{
+    const bool wrap = bc_wrap_x(p.boundary);
+    int r = x + 1, l = x - 1;
+    if (r >= p.nx) r = wrap ? 0 : -1;
+    if (l < 0) l = wrap ? p.nx - 1 : -1;
+    auto at = [&](int k, int xx) { return Ar<double>::add((double)s2f(src[(long long)k * p.plane + kLead + xx]), p.rw(k)); };
+    double fin[3], fs[3], fp[3], ds, dsin, rho;
+    fin[0] = at(0, x);
+    fin[1] = r >= 0 ? at(1, r) : at(2, x);
+    fin[2] = l >= 0 ? at(2, l) : at(1, x);
+    const bool bad = site_collide<3, double>(fin, p.a, true, fs, fp, ds, dsin, rho, p.eq, false);
+    return !bad && ds > delta_e ? ds : -1.0;
+}
+
+template <int Q, typename S>
+__device__ __forceinline__ double key_dS_lane(const KeyGeom &p, const S *src, int site, double delta_e)
+{
+    if constexpr (Q == 9)
+        return key_dS9_lane<S>(p, src, site, delta_e);
+    else
+        return key_dS3_lane<S>(p, src, site, delta_e);
 }
 
 }  // namespace lbm

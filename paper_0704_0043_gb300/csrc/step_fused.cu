@@ -60,7 +60,6 @@ constexpr int kStripCols = 62;   // finished columns per strip (64 computed)
 constexpr int kMinSegRows = 4;   // shortest row segment (an item costs a ring prologue and a few atomics)
 constexpr int kFoldRows = 128;   // FP32 partial sums are folded into fixed point every kFoldRows rows
 constexpr int kItemsPerWarp = 10;  // dynamic work: about this many items per resident warp
-constexpr int kLaneKeys = 3;     // candidates of an item from which each lane keys its own
 constexpr int kCandList = 32;    // candidates a warp keys itself per item (the tail keys the rest)
 constexpr unsigned kFull = 0xffffffffu;
 
@@ -270,7 +269,11 @@ __global__ void __launch_bounds__(kThreads, ENT ? 3 : (BATCHED ? kBlocksPerSMBat
         S *__restrict__ dst = (S *)A.dst;
         const int nx = p.nx, ny = p.ny, pitch = p.pitch;
         const int plane = (int)p.plane;  // 9 * plane < 2^31 is checked at launch
-        const int strip = it % A.strips, seg = it / A.strips;
+        // the rows next to the lid first: a lid-driven flow has its Ehrenfests'
+        // candidates in the lid's corners, and their FP64 keys (cold code, about 10 us;
+        // 40 us with entropic f*) then overlap the other items instead of ending the
+        // launch: the 2048 x 2048 entropic launch went from 306 to 262 us
+        const int strip = it % A.strips, seg = A.segs - 1 - it / A.strips;
         const int xa = kStripCols * strip - 1 + lane, xb = xa + 32;  // the lane's two columns
         const int ys = seg * A.seg_rows, ye = min(ys + A.seg_rows, ny);
         // The walk computes its own rows [ys, ye) only.  The median of its first
@@ -786,9 +789,8 @@ __global__ void __launch_bounds__(kThreads, ENT ? 3 : (BATCHED ? kBlocksPerSMBat
         }
         // FP64 keys dS(f') of the item's candidates, from the pre-step
         // populations with the FP64 path's operations and order (-1 when the
-        // site is at or below the threshold or cannot be limited).  A few are
-        // keyed one at a time by the whole warp (a lane per direction, the
-        // shortest latency), more lane-parallel; past kCandList the tail
+        // site is at or below the threshold or cannot be limited), a lane each;
+        // past kCandList the tail
         // kernel keys the rest.  An item with more candidates than that on a
         // lattice with the grid tail keys none: the grid keys only those that
         // can matter (near the k-th largest or near delta).
@@ -810,17 +812,9 @@ __global__ void __launch_bounds__(kThreads, ENT ? 3 : (BATCHED ? kBlocksPerSMBat
             kg.eq = p.eq;
             const int n = min(n_list, kCandList);
             __syncwarp();
-            if (n >= kLaneKeys) {
-                if (lane < n) {
-                    const int slot = list[lane];
-                    p.cand[slot].key = key_dS9_lane<S>(kg, src, p.cand[slot].site, p.delta_e);
-                }
-            } else {
-                for (int i = 0; i < n; ++i) {
-                    const int slot = list[i];
-                    const double key = key_dS9_warp<S>(kg, src, p.cand[slot].site, p.delta_e);
-                    if (lane == 0) p.cand[slot].key = key;
-                }
+            if (lane < n) {
+                const int slot = list[lane];
+                p.cand[slot].key = key_dS9_lane<S>(kg, src, p.cand[slot].site, p.delta_e);
             }
             __syncwarp();
         }
@@ -1003,7 +997,8 @@ int fused_make_args(const StepParams &p, const void *src, void *dst, int seg_row
         rows = (p.ny + segs - 1) / segs;
     }
     A->seg_rows = std::max(kMinSegRows, rows);
-    A->items = A->strips * ((p.ny + A->seg_rows - 1) / A->seg_rows);
+    A->segs = (p.ny + A->seg_rows - 1) / A->seg_rows;
+    A->items = A->strips * A->segs;
     A->blocks = (A->items + kWarps - 1) / kWarps;
     A->a = (float)p.a;
     A->b2 = (float)(1.0 + p.a);
