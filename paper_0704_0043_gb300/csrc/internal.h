@@ -233,6 +233,48 @@ struct TubeArgs {
     void *dst;
 };
 
+// Many steps of a small lattice in one cooperative launch (step_resident.cu).
+constexpr int kResRows = 4;        // steps whose block rows are kept: the tail may lag this far behind
+constexpr int kResMaxBlocks = 160;
+constexpr int kResMaxSteps = 1024;  // steps of one launch
+// Lattices up to these sizes take the resident kernel.  Measured us per step, resident
+// against launch by launch (square cavities with the median filter / with all
+// limiters; tubes with Ehrenfests' steps):
+//   D2Q9 FP32: 256^2 6.2 / 12.0 against 13.4 / 24.9, 384^2 8.1 / 14.2 against 14.2 / 25.8,
+//   512^2 14.9 / 23.2 against 14.5 / 26.7, 640^2 21.0 / 30.0 against 15.9 / 28.1 (16-bit
+//   alike): the fused kernel evaluates two sites a lane and reads each plane once;
+//   D2Q9 FP64: 512^2 149 / 155 against 225 / 235, 640^2 227 / 233 against 324 / 336;
+//   D1Q3 FP32: 2e5 13.2 against 14.5, 1e6 14.9 against 21.3, 1.5e6 28.2 against 26.4;
+//   D1Q3 FP64: 800 13.3 against 17.7, 5e5 102 against 125.
+constexpr long long kResMaxSites = 240000;      // D2Q9, FP32 and 16-bit storage
+constexpr long long kResMaxSites64 = 1ll << 19;  // FP64 storage
+constexpr long long kResMaxSites3 = 1ll << 20;   // D1Q3, FP32 storage
+struct ResRow {
+    double v[4];  // P_MASS .. P_DS_LIM of a worker block's sites
+    int c[4];     // positivity, median, flagged and own sites
+};
+struct ResState {
+    unsigned long long arrived;  // low word: worker arrivals; high word: candidates recorded (both since the launch)
+    unsigned done;               // steps whose candidates are finished
+    unsigned stats_done;         // steps whose record is written
+    unsigned rows_in[kResRows];  // worker rows written, steps of each slot
+    unsigned keyed;              // workers that keyed their share of a dense step's candidates
+    ResRow rows[kResRows][kResMaxBlocks];
+};
+struct ResArgs {
+    StepParams p;
+    FinalParams f;
+    void *buf[2];
+    int cur, nsteps;
+    int aw, gx, tiles;  // set by the launcher: warps that carry sites, tiles along x, tiles
+    double wall_rest;   // rest values of the boundary nodes' populations that stream back
+    ResState *rs;
+};
+bool resident_applies(const lbm_config &c);
+// Takes a.nsteps steps from a.buf[a.cur]; a.f as for the tail of a step.
+template <typename S>
+cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s);
+
 // Launchers (stream-ordered, no synchronisation).  Return cudaGetLastError().
 template <typename T>
 cudaError_t launch_tiled(int q, const StepParams &p, const T *src, T *dst, int *nblocks,
@@ -334,6 +376,7 @@ struct lbm_ctx {
     lbm::SelState *sel_state = nullptr;  // Ehrenfests' limiter: the cooperative tail's selection state
     int fin_grid = 0;                     // blocks of the cooperative tail (0: one-block tail only)
     bool capturing = false;               // a graph capture is in progress (one-block tail)
+    lbm::ResState *res = nullptr;         // resident steps: counters and rows (nullptr: stepped launch by launch)
     double *ens = nullptr;  // [kEnsBlocks][2] partial sums and counts of dS, then E(dS), alpha, sum, count
     void *ent_field = nullptr;   // LBM_LIM_ENTTHRESH: the pass's dS field
     lbm::EntState *ent = nullptr;  // LBM_LIM_ENTTHRESH: solve state

@@ -32,13 +32,12 @@ __device__ double pull_one_f64(const KeyGeom &p, const S *src, int x, int y, int
     int sx = x - Lat<9>::cx(k), sy = y - Lat<9>::cy(k);
     if (wrapx) sx = sx < 0 ? sx + p.nx : (sx >= p.nx ? sx - p.nx : sx);
     if (wrapy) sy = sy < 0 ? sy + p.ny : (sy >= p.ny ? sy - p.ny : sy);
-    auto at = [&](int q, int yy, int xx) {
-        return src[(long long)q * p.plane + (long long)yy * p.pitch + kLead + xx];
-    };
-    if (sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny) return Ar<double>::add((double)s2f(at(k, sy, sx)), p.rw(k));
-    const int q = Lat<9>::opp(k);
-    double v = Ar<double>::add((double)s2f(at(q, y, x)), p.rw(q));
-    if (sy > p.ny - 1) v = Ar<double>::add(v, p.lid(k));
+    const bool in = sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny;
+    const int q = in ? k : Lat<9>::opp(k);
+    // the address is selected, not the load: several pulls stay in flight together
+    const S raw = src[(long long)q * p.plane + (long long)(in ? sy : y) * p.pitch + kLead + (in ? sx : x)];
+    double v = Ar<double>::add((double)s2f(raw), p.rw(q));
+    if (!in && sy > p.ny - 1) v = Ar<double>::add(v, p.lid(k));
     return v;
 }
 
@@ -142,8 +141,8 @@ __device__ __noinline__ double key_dS3_lane(const KeyGeom p, const S *src, int x
     auto at = [&](int k, int xx) { return Ar<double>::add((double)s2f(src[(long long)k * p.plane + kLead + xx]), p.rw(k)); };
     double fin[3], fs[3], fp[3], ds, dsin, rho;
     fin[0] = at(0, x);
-    fin[1] = r >= 0 ? at(1, r) : at(2, x);
-    fin[2] = l >= 0 ? at(2, l) : at(1, x);
+    fin[1] = at(r >= 0 ? 1 : 2, r >= 0 ? r : x);
+    fin[2] = at(l >= 0 ? 2 : 1, l >= 0 ? l : x);
     const bool bad = site_collide<3, double>(fin, p.a, true, fs, fp, ds, dsin, rho, p.eq, false);
     return !bad && ds > delta_e ? ds : -1.0;
 }

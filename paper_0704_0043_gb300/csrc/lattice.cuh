@@ -131,6 +131,11 @@ __device__ __forceinline__ bool nan64(double x)
 {
     return ((unsigned long long)__double_as_longlong(x) & 0x7fffffffffffffffull) > 0x7ff0000000000000ull;
 }
+// a > b for a, b >= 0 or +inf
+__device__ __forceinline__ bool above64(double a, double b)
+{
+    return __double_as_longlong(a) > __double_as_longlong(b);
+}
 __device__ __forceinline__ bool below_one(double x) { return (__double2hiint(x) & 0x7fffffff) < 0x3ff00000; }  // |x| < 1
 
 template <> struct Ar<float> {

@@ -136,11 +136,11 @@ size_t fx_bytes() { return (size_t)kFxRows * kFxWords * sizeof(unsigned long lon
 struct Sizes {
     int q, pitch;
     long long plane;
-    size_t elem, field, cand, sel, partials, ring, ent, selstate;
+    size_t elem, field, cand, sel, partials, ring, ent, selstate, res;
     int cand_cap, sel_cap, rows, ring_len;
     int64_t total() const
     {
-        return (int64_t)(2 * field + cand + sel + partials + ring + ens_bytes() + ent + selstate +
+        return (int64_t)(2 * field + cand + sel + partials + ring + ens_bytes() + ent + selstate + res +
                          64 * sizeof(long long) +
                          (size_t)chunks_for(rows) * sizeof(unsigned) + 4096);
     }
@@ -164,6 +164,7 @@ Sizes sizes_for(const lbm_config &c)
     z.rows = tiled_blocks_for(z.q, c.nx, c.ny);
     if (z.q == 3) z.rows = std::max(z.rows, tube_blocks(c.precision == LBM_FP64, c.nx));
     z.partials = fx_bytes() + (size_t)(z.rows + chunks_for(z.rows)) * P_NSTAT * sizeof(double);
+    z.res = resident_applies(c) ? sizeof(ResState) : 0;
     z.ring_len = std::max(1, c.stats_history);
     z.ring = (size_t)z.ring_len * sizeof(DevStats);
     // Eq. EntThresh: the pass's dS field (compute precision) and the solve's state
@@ -357,6 +358,47 @@ lbm_status run_pass(lbm_ctx *c, int collide, unsigned limiters)
     return LBM_OK;
 }
 
+// `n` steps of a small lattice by the resident kernel.  *taken: the steps
+// enqueued; fewer than n (with LBM_OK) when this context does not or can no
+// longer run it (the launch needs a cooperative grid; a stream that the caller
+// is capturing keeps the launches step by step).
+lbm_status run_resident(lbm_ctx *c, int64_t n, int64_t *taken)
+{
+    *taken = 0;
+    if (!c->res || n <= 0) return LBM_OK;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(c->stream, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+        cudaGetLastError();
+        return LBM_OK;
+    }
+    while (*taken < n) {
+        const int m = (int)std::min<int64_t>(n - *taken, kResMaxSteps);
+        ResArgs a{};
+        a.p = step_params(c, 1, c->cfg.limiters);
+        a.f = final_params(c, 1, c->cfg.limiters, 1);
+        a.buf[0] = c->buf[0];
+        a.buf[1] = c->buf[1];
+        a.cur = c->cur;
+        a.nsteps = m;
+        a.rs = c->res;
+        const cudaError_t e = with_storage(c->cfg.precision, [&](auto tag) -> cudaError_t {
+            using S = STORAGE_T;
+            return launch_resident<S>(c->q, a, c->stream);
+        });
+        if (e != cudaSuccess) {
+            // no cooperative launch on this device: step launch by launch from now on
+            cudaGetLastError();
+            cudaFree(c->res);
+            c->res = nullptr;
+            return LBM_OK;
+        }
+        c->launches += 1;
+        c->cur ^= m & 1;
+        *taken += m;
+    }
+    return LBM_OK;
+}
+
 lbm_status read_status(lbm_ctx *c, bool clear)
 {
     unsigned s = 0;
@@ -440,7 +482,7 @@ void free_all(lbm_ctx *c)
     c->events.clear();
     void *ptrs[] = {c->buf[0], c->buf[1], c->cand, c->counts, c->sel, c->partials, c->chunk_cnt,
                     c->status, c->ring, c->counters, c->stage, c->ens, c->probe, c->ent_field, c->ent,
-                    c->sel_state};
+                    c->sel_state, c->res};
     for (void *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -635,6 +677,7 @@ lbm_status lbm_create(const lbm_config *cfg, void *cuda_stream, lbm_ctx **out)
         default: c->fin_grid = finalize_grid<__half>(c->q);
         }
     }
+    if (z.res) alloc((void **)&c->res, z.res);
     if (z.ent) {
         alloc(&c->ent_field, z.ent - sizeof(EntState));
         alloc((void **)&c->ent, sizeof(EntState));
@@ -693,6 +736,26 @@ lbm_status lbm_step(lbm_ctx *c, int64_t nsteps)
     if (nsteps < 0) return fail(c, LBM_ERR_INVALID_ARG, "nsteps must be >= 0");
     if (!c->ready) return fail(c, LBM_ERR_STATE, "lbm_step before lbm_init / lbm_set_populations");
     int64_t left = nsteps;
+    // a small lattice: many steps a launch, but for the steps that per-kernel timing
+    // samples (the first of every timing_every)
+    while (c->res && left > 0) {
+        int64_t m = left, taken = 0;
+        if (c->timing) {
+            const int64_t at = c->timing_pass % c->timing_every;
+            if (c->timing_every <= 1 || at == 0) {
+                lbm_status s = run_pass(c, 1, c->cfg.limiters);
+                if (s != LBM_OK) return s;
+                --left;
+                continue;
+            }
+            m = std::min<int64_t>(left, c->timing_every - at);
+        }
+        lbm_status s = run_resident(c, m, &taken);
+        if (s != LBM_OK) return s;
+        if (taken == 0) break;
+        if (c->timing) c->timing_pass += taken;
+        left -= taken;
+    }
     // graph replay (not while per-kernel timing records its events)
     const int gs = c->graph_steps;
     while (gs > 0 && !c->timing && left >= gs) {

@@ -9,6 +9,7 @@
 #include "internal.h"
 #include "keys.cuh"
 #include "lattice.cuh"
+#include "site.cuh"
 
 namespace lbm {
 namespace {
@@ -22,35 +23,29 @@ constexpr unsigned kFull = 0xffffffffu;
 
 __device__ __forceinline__ unsigned long long key_bits(double d) { return (unsigned long long)__double_as_longlong(d); }
 
-__device__ __forceinline__ long long fidx(long long plane, int pitch, int k, int y, int x)
-{
-    return (long long)k * plane + (long long)y * pitch + kLead + x;
-}
-
 // The pass's input at site (x, y) in FP32: after free flight (collide) with the
 // step kernels' FP32 arithmetic (bounce-back, lid term added as hi + lo), or
-// the stored populations themselves (limiter pass).
+// the stored populations themselves (limiter pass).  The loads do not wait for
+// one another (see pull).
 template <int Q, typename S>
-__device__ void pull_dev(const FinalParams &p, int x, int y, float g[Q])
+__device__ __forceinline__ void pull_dev(const FinalParams &p, int x, int y, float g[Q])
 {
     const S *src = (const S *)p.src;
     const bool wrapx = bc_wrap_x(p.boundary), wrapy = Q == 9 && bc_wrap_y(p.boundary);
+    const int xl = x > 0 ? x - 1 : (wrapx ? p.nx - 1 : -1), xr = x + 1 < p.nx ? x + 1 : (wrapx ? 0 : -1);
+    const int yl = y > 0 ? y - 1 : (wrapy ? p.ny - 1 : -1), yr = y + 1 < p.ny ? y + 1 : (wrapy ? 0 : -1);
+    S raw[Q];
 #pragma unroll
     for (int k = 0; k < Q; ++k) {
-        if (!p.collide) {
-            g[k] = s2f(src[fidx(p.plane, p.pitch, k, y, x)]);
-            continue;
-        }
-        int sx = x - Lat<Q>::cx(k), sy = y - Lat<Q>::cy(k);
-        if (wrapx) sx = sx < 0 ? sx + p.nx : (sx >= p.nx ? sx - p.nx : sx);
-        if (wrapy) sy = sy < 0 ? sy + p.ny : (sy >= p.ny ? sy - p.ny : sy);
-        if (sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny) {
-            g[k] = s2f(src[fidx(p.plane, p.pitch, k, sy, sx)]);
-        } else {
-            float v = s2f(src[fidx(p.plane, p.pitch, Lat<Q>::opp(k), y, x)]);
-            if (Q == 9 && sy > p.ny - 1) v = __fadd_rn(__fadd_rn(v, p.lidf[k]), p.lidlo[k]);
-            g[k] = v;
-        }
+        const int sx = Lat<Q>::cx(k) > 0 ? xl : (Lat<Q>::cx(k) < 0 ? xr : x);
+        const int sy = Lat<Q>::cy(k) > 0 ? yl : (Lat<Q>::cy(k) < 0 ? yr : y);
+        const bool own = !p.collide, out = sx < 0 || sy < 0;
+        raw[k] = src[fidx(p.plane, p.pitch, !own && out ? Lat<Q>::opp(k) : k, own || out ? y : sy, own || out ? x : sx)];
+    }
+#pragma unroll
+    for (int k = 0; k < Q; ++k) {
+        g[k] = s2f(raw[k]);
+        if (Q == 9 && Lat<Q>::cy(k) < 0 && yr < 0 && p.collide) g[k] = __fadd_rn(__fadd_rn(g[k], p.lidf[k]), p.lidlo[k]);
     }
 }
 
@@ -112,8 +107,9 @@ __device__ void pick_digit(const unsigned *hist, long long rem, bool desc, unsig
     __syncthreads();
 }
 
-// The geometry of the FP64 key evaluation (D2Q9, FP32 / 16-bit storage).
-__device__ KeyGeom key_geom(const FinalParams &p)
+// The geometry of the FP64 key evaluation (FP32 / 16-bit storage).
+template <typename P>
+__device__ __forceinline__ KeyGeom key_geom(const P &p)
 {
     KeyGeom kg;
     kg.nx = p.nx;
@@ -139,6 +135,7 @@ struct SelShared {
     float ds[kCap];  // FP32 dS the candidate was recorded on
     int site[kCap];
     int idx[kCap];
+    long long rkey[kRankCap];  // keys in play, packed
     unsigned hist[256];
     unsigned long long part[8], digit;
     double red[2 * P_NSTAT + 2 > kFinWarps + 1 ? 2 * P_NSTAT + 2 : kFinWarps + 1];
@@ -150,12 +147,16 @@ struct SelShared {
 // (1 - 1/32), T a lower bound of the k-th largest FP32 dS among the candidates
 // R that are certainly above delta (FP32 dS above delta (1 + 1/64); finite).
 // 0 when R has fewer than k.  The FP32 dS is within 1/64 of the FP64 key, so a
-// candidate below that bound cannot reach the k-th largest key.  u(i): the
-// pattern of candidate i < n.  Every thread of the block calls it.
-template <typename F>
-__device__ __forceinline__ int fp32_bound(SelShared &sh, int n, long long k, int dhi_bits, F u)
+// candidate below that bound cannot reach the k-th largest key.  `keyed`: every
+// candidate has its key and the patterns are the keys rounded, which order as the
+// keys do, so T itself is the bound.  Every thread of the block calls it.
+template <typename S>
+__device__ __noinline__ int fp32_bound(const FinalParams &p, int n, bool small, bool keyed, SelShared &sh)
 {
     const int t = threadIdx.x, lane = t & 31;
+    const long long k = p.k_max;
+    const int dhi_bits = __float_as_int((float)(p.delta_e * (1.0 + 1.0 / 64.0)));
+    auto u = [&](int i) -> int { return __float_as_int(small ? sh.ds[i] : p.cand[i].ds32); };
     auto in_r = [&](int v) { return v > dhi_bits && v < 0x7f800000; };
     if (t == 0) {
         sh.tlow = 0;
@@ -180,17 +181,18 @@ __device__ __forceinline__ int fp32_bound(SelShared &sh, int n, long long k, int
         }
         __syncthreads();
     } else {
-        // the exponent, then the upper eight bits of the mantissa
+        // the exponent, then the upper eight (all keyed: sixteen) bits of the mantissa
         int prefix = 0;
         long long rem = k;
+        const int low = keyed ? 7 : 15;
 #pragma unroll 1
-        for (int shift = 23; shift >= 15; shift -= 8) {
+        for (int shift = 23; shift >= low; shift -= 8) {
             if (t < 256) sh.hist[t] = 0;
             __syncthreads();
             for (int base = 0; base < n; base += kFinThreads) {
                 const int i = base + t;
                 const int v = i < n ? u(i) : 0;
-                const int bin = i < n && in_r(v) && (shift == 23 || (v >> 23) == (prefix >> 23)) ? (v >> shift) & 255 : -1;
+                const int bin = i < n && in_r(v) && ((v ^ prefix) >> (shift + 8)) == 0 ? (v >> shift) & 255 : -1;
                 const unsigned peers = __match_any_sync(kFull, bin);
                 if (bin >= 0 && lane == __ffs(peers) - 1) atomicAdd(&sh.hist[bin], (unsigned)__popc(peers));
             }
@@ -203,7 +205,7 @@ __device__ __forceinline__ int fp32_bound(SelShared &sh, int n, long long k, int
         if (t == 0) sh.tlow = prefix;
         __syncthreads();
     }
-    return __float_as_int(__int_as_float(sh.tlow) * 0.96875f);
+    return keyed ? sh.tlow - 1 : __float_as_int(__int_as_float(sh.tlow) * 0.96875f);
 }
 
 // The owed keys of a pass's n candidates (see finish_candidates); returns this
@@ -212,14 +214,12 @@ __device__ __forceinline__ int fp32_bound(SelShared &sh, int n, long long k, int
 // and a common path that runs straight through costs a few us less than one that
 // jumps over rarely taken blocks.
 template <int Q, typename S>
-__device__ __noinline__ int settle_owed(const FinalParams &p, int n, bool small, SelShared &sh)
+__device__ __noinline__ int settle_owed(const FinalParams &p, int n, bool small, int tlow, SelShared &sh)
 {
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const long long k = p.k_max;
     int nv = 0;
     const int dhi_bits = __float_as_int((float)(p.delta_e * (1.0 + 1.0 / 64.0)));
     auto u = [&](int i) -> int { return __float_as_int(small ? sh.ds[i] : p.cand[i].ds32); };
-    const int tlow = k > 0 ? fp32_bound(sh, n, k, dhi_bits, u) : 0x7f800001;
     const KeyGeom kg = key_geom(p);
     if (t == 0) sh.count = 0;
     __syncthreads();
@@ -259,6 +259,27 @@ __device__ __noinline__ int settle_owed(const FinalParams &p, int n, bool small,
     }
     __syncthreads();
     return nv;
+}
+
+// FP64 keys of n <= 32 candidates, into sh.key; `site`: lane i's candidate, the same
+// in every warp.  Three to a warp with a lane per direction (D2Q9, polynomial),
+// else a lane each in the first warp.  Every thread of the block calls it.
+template <int Q, typename S>
+__device__ __noinline__ void key_few(const FinalParams &p, int n, int site, SelShared &sh)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const KeyGeom kg = key_geom(p);
+    if (Q == 9 && p.eq != 1) {
+        const int g = lane < 27 ? lane / 9 : 0, i = min(3 * warp + g, n - 1);
+        const int st = __shfl_sync(kFull, site, i);
+        if (3 * warp < n) {
+            const double key = key_dS9_group<S>(kg, (const S *)p.src, st, p.delta_e);
+            if (lane < 27 && lane % 9 == 0 && 3 * warp + g < n) sh.key[i] = key;
+        }
+    } else if (threadIdx.x < n) {
+        sh.key[lane] = key_dS_lane<Q, S>(kg, (const S *)p.src, site, p.delta_e);
+    }
+    __syncthreads();
 }
 
 // The chosen candidates among more than kRankCap in play: a radix selection
@@ -376,8 +397,8 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
 // candidate p.sel_state->list[i], all keyed and valid, n_valid given.  `first`:
 // candidate of entry threadIdx.x, loaded early, when `preloaded`.  Returns this
 // thread's share of phi^2 dS over the chosen sites (entropic f*: of the entropy
-// the step adds); sh.nsel holds the chosen count.  Every thread of a block of
-// kFinThreads calls it, n > 0.
+// the step adds); sh.nsel holds the chosen count; n_valid is set in thread 0.
+// Every thread of a block of kFinThreads calls it, n > 0.
 //
 // Keys are owed (NaN) by FP32 and 16-bit passes.  Only the candidates that can
 // reach the k largest by their FP32 dS, and those within 1/64 of delta, get one:
@@ -403,97 +424,158 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
     // below the threshold -> -1, so that from here on a key is valid exactly
     // when its bit pattern is a positive integer
     auto settle = [&](double key) { return key > p.delta_e ? key : -1.0; };
-    bool owed = false;
-    if (t == 0) {
-        sh.nsel = 0;
-        if (!use_list) sh.valid = 0;
-        sh.count = 0;
-    }
-    if (small || !use_list) {
-        for (int i = t; i < n; i += kFinThreads) {
-            const Cand c = preloaded && i == t ? first : p.cand[cidx(i)];
-            owed = owed || isnan(c.key);
-            if (small) {
-                sh.key[i] = c.key;
-                sh.site[i] = c.site;
-                sh.ds[i] = c.ds32;
-            }
-        }
-    }
-    owed = __syncthreads_or(owed) != 0;
-    if (!use_list) {
-        int nv = 0;  // candidates counted as valid here without a key, then those with one
+    int nsel = 0;         // chosen sites (few: in the first warp only)
+    bool listed = false;  // the chosen list entries are in sh.idx
+    const bool few = n <= 32 && !use_list;
+    int few_site = 0;     // few: lane r's chosen site, key and phi
+    double few_key = 0.0, few_phi = 0.0;
+    if (few) {
+        // the usual case: one warp selects in registers, without a block barrier
+        Cand c{};
+        if (lane < n) c = preloaded ? first : p.cand[lane];
+        if (preloaded && warp != 0 && lane < n) c = p.cand[lane];
+        bool owed = false;
         if constexpr (kLowPrec) {
-            if (owed) nv = settle_owed<Q, S>(p, n, small, sh);
+            owed = __any_sync(kFull, lane < n && isnan(c.key));
+            if (owed) key_few<Q, S>(p, n, c.site, sh);  // every warp takes three
         }
-        for (int i = t; i < n; i += kFinThreads) {
-            const double key = settle(key_of(i));
-            if (small)
-                sh.key[i] = key;
-            else
-                p.cand[i].key = key;
-            nv += (long long)key_bits(key) > 0;
+        if (warp == 0) {
+            if (owed) c.key = lane < n ? sh.key[lane] : -1.0;
+            const bool valid = lane < n && c.key > p.delta_e;
+            n_valid = __popc(__ballot_sync(kFull, valid));
+            nsel = k < (long long)n_valid ? (int)(k > 0 ? k : 0) : n_valid;
+            const long long u = valid ? (long long)key_bits(c.key) : -1;
+            int rank = 0;
+            for (int j = 0; j < n; ++j) {
+                const long long v = __shfl_sync(kFull, u, j);
+                const int sj = __shfl_sync(kFull, c.site, j);
+                rank += v > u || (v == u && sj < c.site);
+            }
+            if (valid && rank < nsel) sh.idx[rank] = lane;
+            __syncwarp();
+            const int from = lane < nsel ? sh.idx[lane] : 0;
+            few_site = __shfl_sync(kFull, c.site, from);
+            few_key = __shfl_sync(kFull, c.key, from);
+            few_phi = __shfl_sync(kFull, c.phi, from);
+            if (lane == 0) sh.nsel = nsel;
         }
-        nv = __reduce_add_sync(kFull, nv);
-        if (lane == 0 && nv) atomicAdd(&sh.valid, nv);
-    }
-    if (t == 0) sh.count = 0;
-    __syncthreads();
-    n_valid = sh.valid;
-    if (k <= 0 || n_valid <= 0) return 0.0;  // the same for the whole block
-
-    // the entries still in play (valid, keyed), compacted: the candidates below
-    // the FP32 bound drop out here
-    int m = n;
-    bool packed = false;
-    if (small) {
-        for (int base = 0; base < n; base += kFinThreads) {
-            const int i = base + t;
-            const bool in = i < n && (long long)key_bits(sh.key[i]) > 0;
-            const unsigned b = __ballot_sync(kFull, in);
-            int at = 0;
-            if (lane == 0 && b) at = atomicAdd(&sh.count, __popc(b));
-            at = __shfl_sync(kFull, at, 0) + __popc(b & ((1u << lane) - 1u));
-            if (in) sh.idx[at] = i;
+    } else {
+        bool owed = false;
+        if (t == 0) {
+            sh.nsel = 0;
+            if (!use_list) sh.valid = 0;
+            sh.count = 0;
         }
-        __syncthreads();
-        m = sh.count;
-        packed = m <= kRankCap;
-    }
-    const bool take_all = (long long)n_valid <= k;
-    int nsel = 0;
-    if (packed) {
-        // each thread ranks its own entry by counting the keys that beat it
-        // (larger dS, or equal dS at a lower site); the rank is its place in the
-        // chosen list, so the list's order does not depend on the recording order
-        int mine = -1;
-        long long rank = 0;
-        if (t < m) {
-            mine = sh.idx[t];
-            const unsigned long long u = key_bits(sh.key[mine]);
-            const int st = sh.site[mine];
-            for (int j = 0; j < m; ++j) {
-                const int o = sh.idx[j];
-                const unsigned long long v = key_bits(sh.key[o]);
-                rank += v > u || (v == u && sh.site[o] < st);
+        if (small || !use_list) {
+            for (int i = t; i < n; i += kFinThreads) {
+                const Cand c = preloaded && i == t ? first : p.cand[cidx(i)];
+                owed = owed || isnan(c.key);
+                if (small) {
+                    sh.key[i] = c.key;
+                    sh.site[i] = c.site;
+                    sh.ds[i] = isnan(c.key) ? c.ds32 : (float)c.key;
+                }
             }
         }
-        nsel = (int)(k < (long long)m ? k : (long long)m);
+        owed = __syncthreads_or(owed) != 0;
+        if (!use_list) {
+            // FP32 dS pattern below which a candidate cannot be among the k largest
+            int tlow = 0;
+            if (k <= 0)
+                tlow = 0x7f800001;
+            else if (n > kRank32 || (owed && n > k))
+                tlow = fp32_bound<S>(p, n, small, small && !owed, sh);
+            int nv = 0;  // candidates counted as valid here without a key, then those with one
+            if constexpr (kLowPrec) {
+                if (owed) nv = settle_owed<Q, S>(p, n, small, tlow, sh);
+            }
+            for (int i = t; i < n; i += kFinThreads) {
+                double key = settle(key_of(i));
+                nv += (long long)key_bits(key) > 0;
+                if (__float_as_int(small ? sh.ds[i] : p.cand[i].ds32) < tlow) key = -1.0;  // counted, out of play
+                if (small)
+                    sh.key[i] = key;
+                else
+                    p.cand[i].key = key;
+            }
+            nv = __reduce_add_sync(kFull, nv);
+            if (lane == 0 && nv) atomicAdd(&sh.valid, nv);
+        }
         __syncthreads();
-        if (mine >= 0 && rank < nsel) sh.idx[(int)rank] = mine;
-        if (t == 0) sh.nsel = nsel;
-        __syncthreads();
-    } else {
-        nsel = choose_many<S>(p, n, use_list, small, take_all, sh);
+        n_valid = sh.valid;
+        if (k <= 0 || n_valid <= 0) return 0.0;  // the same for the whole block
+
+        // the entries still in play (valid, keyed), compacted: the candidates below
+        // the FP32 bound drop out here
+        int m = n;
+        bool packed = false;
+        if (small) {
+            // who is in play: a ballot per 32 entries (at most 64 of them), the
+            // entries' places from the ballots before theirs
+            static_assert(kCap <= 64 * 32, "two ballots per lane");
+            const int nb = (n + 31) / 32;
+            for (int b = warp; b < nb; b += kFinWarps) {
+                const int i = 32 * b + lane;
+                const unsigned w = __ballot_sync(kFull, i < n && (long long)key_bits(sh.key[i]) > 0);
+                if (lane == 0) sh.hist[b] = w;
+            }
+            __syncthreads();
+            const int c0 = lane < nb ? __popc(sh.hist[lane]) : 0, c1 = lane + 32 < nb ? __popc(sh.hist[lane + 32]) : 0;
+            m = __reduce_add_sync(kFull, c0 + c1);
+            packed = m <= kRankCap;
+            for (int b = warp; b < nb && packed; b += kFinWarps) {
+                const int before = __reduce_add_sync(kFull, (lane < b ? c0 : 0) + (lane + 32 < b ? c1 : 0));
+                const unsigned w = sh.hist[b];
+                if ((w >> lane) & 1u) {
+                    const int at = before + __popc(w & ((1u << lane) - 1u)), i = 32 * b + lane;
+                    sh.rkey[at] = (long long)key_bits(sh.key[i]);
+                    sh.idx[at] = i;
+                }
+            }
+            __syncthreads();
+        }
+        const bool take_all = (long long)n_valid <= k;
+        if (packed) {
+            // each thread ranks its own entry by counting the keys that beat it
+            // (larger dS, or equal dS at a lower site); the rank is its place in the
+            // chosen list, so the list's order does not depend on the recording order
+            int mine = -1, rank = 0;
+            if (t < m) {
+                mine = sh.idx[t];
+                const long long u = sh.rkey[t];
+                int more = 0, same = 0;
+#pragma unroll 4
+                for (int j = 0; j < m; ++j) {  // broadcast reads
+                    const long long v = sh.rkey[j];
+                    more += v > u;
+                    same += v == u;
+                }
+                if (same > 1)  // ties (other than the entry itself)
+                    for (int j = 0; j < m; ++j) more += sh.rkey[j] == u && sh.site[sh.idx[j]] < sh.site[mine];
+                rank = more;
+            }
+            nsel = (int)(k < (long long)m ? k : (long long)m);
+            __syncthreads();
+            if (mine >= 0 && rank < nsel) sh.idx[rank] = mine;
+            if (t == 0) sh.nsel = nsel;
+            __syncthreads();
+        } else {
+            nsel = choose_many<S>(p, n, use_list, small, take_all, sh);
+        }
+        listed = packed || nsel <= kCap;  // the chosen list entries are in sh.idx
     }
-    const bool listed = packed || nsel <= kCap;  // the chosen list entries are in sh.idx
     // Ehrenfests' step at each chosen site, in the list's order
     for (int r = t; r < nsel; r += kFinThreads) {
         // the chosen candidate's site and key (from shared memory when listed) and
         // its phi
         int site;
         double key, phi;
-        if (listed) {
+        if (few) {
+            site = few_site;
+            key = few_key;
+            phi = few_phi;
+            p.sel[r] = site;
+        } else if (listed) {
             const int li = sh.idx[r];
             site = small ? sh.site[li] : sh.site[r];
             key = key_of(li);
@@ -564,6 +646,7 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
     }
     __syncthreads();
     // the chosen sites, as site indices, for lbm_limited_sites
+    if (few) return ehr_sum;
     if (listed) {
         for (int r = t; r < nsel; r += kFinThreads) p.sel[r] = small ? sh.site[sh.idx[r]] : sh.site[r];
     } else {

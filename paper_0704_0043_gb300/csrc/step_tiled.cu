@@ -16,6 +16,7 @@
 
 #include "internal.h"
 #include "lattice.cuh"
+#include "site.cuh"
 
 namespace lbm {
 namespace {
@@ -23,193 +24,6 @@ namespace {
 constexpr int kTX = 32, kTY = 8;  // D2Q9 tile of computed sites; (kTX-2) x (kTY-2) finished
 constexpr int kT1 = 64;           // D1Q3 tile; kT1 - 2 finished (small tiles: a short tube spreads over
                                   // many SMs; GB300's FP64 pipe is narrow per SM)
-
-__device__ __forceinline__ long long fidx(long long plane, int pitch, int k, int y, int x)
-{
-    return (long long)k * plane + (long long)y * pitch + kLead + x;
-}
-
-// Stored value as a compute value: FP64 storage is f itself; FP32 / BF16 /
-// FP16 storage is the deviation g, read as g in FP32 or as the absolute
-// f = (double) g + rw_k in FP64.
-template <typename S, typename T>
-__device__ __forceinline__ T load_as(const StepParams &p, S v, int k)
-{
-    if constexpr (std::is_same<S, double>::value)
-        return T(v);
-    else if constexpr (std::is_same<T, double>::value)
-        return Ar<double>::add((double)s2f(v), p.rw[k]);
-    else
-        return s2f(v);
-}
-
-// Free flight in pull form at site (x, y) (Sec. 2): f_in_k(x) = f_k(x - v_k);
-// a link leaving the lattice is reflected, f_in_k(x) = f_opp(k)(x) (halfway
-// bounce-back, Sec. 4.4.1), plus the moving-wall term for links through the lid.
-// Reads storage type S, returns compute type T (see load_as).
-template <int Q, typename S, typename T>
-__device__ __forceinline__ void pull(const StepParams &p, const S *__restrict__ f, int x, int y, T fin[Q])
-{
-    using A = Ar<T>;
-    const bool wrapx = bc_wrap_x(p.boundary);
-    const bool wrapy = (Q == 9) && bc_wrap_y(p.boundary);
-#pragma unroll
-    for (int k = 0; k < Q; ++k) {
-        int sx = x - Lat<Q>::cx(k), sy = y - Lat<Q>::cy(k);
-        if (wrapx) sx = sx < 0 ? sx + p.nx : (sx >= p.nx ? sx - p.nx : sx);
-        if (wrapy) sy = sy < 0 ? sy + p.ny : (sy >= p.ny ? sy - p.ny : sy);
-        if (sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny) {
-            fin[k] = load_as<S, T>(p, f[fidx(p.plane, p.pitch, k, sy, sx)], k);
-        } else {
-            T v = load_as<S, T>(p, f[fidx(p.plane, p.pitch, Lat<Q>::opp(k), y, x)], Lat<Q>::opp(k));
-            if (Q == 9 && sy > p.ny - 1) {
-                if constexpr (std::is_same<T, double>::value)
-                    v = A::add(v, p.lid[k]);
-                else
-                    v = A::add(A::add(v, p.lidf[k]), p.lidlo[k]);
-            }
-            fin[k] = v;
-        }
-    }
-}
-
-// Free flight and the wall rule at a boundary node (x, y) of a cavity whose
-// outer ring of nodes lies on the walls (LBM_BC_NODE_WALLS, LBM_BC_DIFFUSIVE;
-// Sec. 4.4): the populations whose source is on the lattice arrive; the others
-// are supplied by the wall.  The lid is the top row without its corners and
-// moves with (u_lid, 0); the other walls and the corners are at rest.
-//   bounce-back (Sec. 4.4.1): f_k = f_opp(k) + 6 W_k rho_wall (v_k . u_wall);
-//   diffusive (Sec. 4.4.2): f_k = gamma f*_k(1, u_wall), gamma = (sum of the
-//     arrived f_opp(k)) / (sum of f*_k(1, u_wall)) over the returned
-//     directions, evaluated in FP64 for every storage type; bounce-back in the
-//     corners.
-// A corner's two missing populations whose opposite is missing too point out
-// of the lattice again; they keep their stored values.  `mass` receives the
-// populations that stream back onto the lattice (FP64, k order).
-template <typename S, typename T>
-__device__ void wall_node(const StepParams &p, const S *__restrict__ f, int x, int y, T fin[9], double &mass)
-{
-    using A = Ar<T>;
-    bool known[9];
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int sx = x - Lat<9>::cx(k), sy = y - Lat<9>::cy(k);
-        known[k] = sx >= 0 && sx < p.nx && sy >= 0 && sy < p.ny;
-        fin[k] = known[k] ? load_as<S, T>(p, f[fidx(p.plane, p.pitch, k, sy, sx)], k) : T(0);
-    }
-    const bool corner = (x == 0 || x == p.nx - 1) && (y == 0 || y == p.ny - 1);
-    const bool lid = y == p.ny - 1 && !corner;
-    if (p.boundary == 4 && !corner) {
-        const double uw = lid ? p.u_lid : 0.0;
-        double fw[9];
-        feq_any<9>(p.eq, 1.0, uw, 0.0, fw);  // density is a linear factor of f*: take 1
-        double arrived = 0.0, returned = 0.0;
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if (!known[k]) {
-                const int o = Lat<9>::opp(k);
-                arrived = Ar<double>::add(arrived, load_as<S, double>(p, f[fidx(p.plane, p.pitch, o, y - Lat<9>::cy(o), x - Lat<9>::cx(o))], o));
-                returned = Ar<double>::add(returned, fw[k]);
-            }
-        const double gamma = Ar<double>::div(arrived, returned);
-#pragma unroll
-        for (int k = 0; k < 9; ++k)
-            if (!known[k]) {
-                const double v = Ar<double>::mul(gamma, fw[k]);
-                if constexpr (std::is_same<T, double>::value)
-                    fin[k] = v;
-                else
-                    fin[k] = (T)Ar<double>::sub(v, p.rw[k]);  // the deviation, rounded once
-            }
-    } else {
-#pragma unroll
-        for (int k = 0; k < 9; ++k) {
-            if (known[k]) continue;
-            const int o = Lat<9>::opp(k);
-            if (known[o]) {
-                T v = fin[o];
-                if (lid) {
-                    if constexpr (std::is_same<T, double>::value)
-                        v = A::add(v, p.lid[k]);
-                    else
-                        v = A::add(A::add(v, p.lidf[k]), p.lidlo[k]);
-                }
-                fin[k] = v;
-            } else {
-                fin[k] = load_as<S, T>(p, f[fidx(p.plane, p.pitch, k, y, x)], k);
-            }
-        }
-    }
-    double m = 0.0;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) {
-        const int dx = x + Lat<9>::cx(k), dy = y + Lat<9>::cy(k);
-        if (dx >= 0 && dx < p.nx && dy >= 0 && dy < p.ny) {
-            if constexpr (std::is_same<T, double>::value)
-                m = Ar<double>::add(m, fin[k]);
-            else
-                m += (double)fin[k] + p.rw[k];
-        }
-    }
-    mass = m;
-}
-
-__device__ __forceinline__ bool is_wall_node(const StepParams &p, int x, int y)
-{
-    return bc_node_walls(p.boundary) && (x == 0 || x == p.nx - 1 || y == 0 || y == p.ny - 1);
-}
-
-// Median of the dS stencil of site (x, y), tile-local position (tx, ty) in a
-// shared array with row stride `ld` (Sec. 3.5; wall rules of Sec. 4.4, read for
-// walls half a link outside the lattice: a node next to one wall uses itself
-// and its two neighbours along that wall, a corner node itself and its inward
-// x and y neighbours, every other node the 3x3 block; the two end sites of a
-// closed D1Q3 tube are not filtered).  Returns false for sites the filter skips.
-template <int Q, typename T>
-__device__ __forceinline__ bool stencil_median(const StepParams &p, const T *s, int ld, int tx, int ty,
-                                               int x, int y, T &med)
-{
-#define S_(dx, dy) s[(ty + (dy)) * ld + tx + (dx)]
-    if constexpr (Q == 3) {
-        if (p.boundary == 0 && (x == 0 || x == p.nx - 1)) return false;
-        med = med3(S_(-1, 0), S_(0, 0), S_(1, 0));
-        return true;
-    } else {
-        if (bc_node_walls(p.boundary)) {
-            // boundary nodes are not filtered; their neighbours use stencils
-            // along the wall (Sec. 4.4)
-            if (x == 0 || x == p.nx - 1 || y == 0 || y == p.ny - 1) return false;
-            const bool nx1 = x == 1 || x == p.nx - 2, ny1 = y == 1 || y == p.ny - 2;
-            if (nx1 && ny1) {
-                med = med3(S_(0, 0), S_(x == 1 ? 1 : -1, 0), S_(0, y == 1 ? 1 : -1));
-            } else if (ny1) {
-                med = med3(S_(-1, 0), S_(0, 0), S_(1, 0));
-            } else if (nx1) {
-                med = med3(S_(0, -1), S_(0, 0), S_(0, 1));
-            } else {
-                med = med9(S_(-1, -1), S_(-1, 0), S_(-1, 1), S_(0, -1), S_(0, 0), S_(0, 1), S_(1, -1), S_(1, 0),
-                           S_(1, 1));
-            }
-            return true;
-        }
-        const bool wallx = p.boundary == 0, wally = p.boundary != 1;
-        const bool nearx = wallx && (x == 0 || x == p.nx - 1);
-        const bool neary = wally && (y == 0 || y == p.ny - 1);
-        if (nearx && neary) {
-            const int dx = x == 0 ? 1 : -1, dy = y == 0 ? 1 : -1;
-            med = med3(S_(0, 0), S_(dx, 0), S_(0, dy));
-        } else if (neary) {
-            med = med3(S_(-1, 0), S_(0, 0), S_(1, 0));
-        } else if (nearx) {
-            med = med3(S_(0, -1), S_(0, 0), S_(0, 1));
-        } else {
-            med = med9(S_(-1, -1), S_(-1, 0), S_(-1, 1), S_(0, -1), S_(0, 0), S_(0, 1), S_(1, -1), S_(1, 0),
-                       S_(1, 1));
-        }
-        return true;
-    }
-#undef S_
-}
 
 __device__ __forceinline__ double warp_sum(double v)
 {
@@ -269,21 +83,16 @@ __global__ void __launch_bounds__(256) k_tiled(const StepParams p0, const S *__r
     if (wall) {
         if constexpr (Q == 9) {
             if (p.collide) {
-                wall_node<S, T>(p, src, xs, ys, fin, wmass);
+                double fw[9];
+                if (p.boundary == 4) wall_star(p, wall_lid(p, xs, ys), fw);
+                S raw[9];
+                pull_raw<9, S>(p, src, xs, ys, true, true, raw);
+                wall_node<S, T>(p, raw, xs, ys, fw, fin);
             } else {
 #pragma unroll
                 for (int k = 0; k < 9; ++k) fin[k] = load_as<S, T>(p, src[fidx(p.plane, p.pitch, k, ys, xs)], k);
-#pragma unroll
-                for (int k = 0; k < 9; ++k) {
-                    const int dx = xs + Lat<9>::cx(k), dy = ys + Lat<9>::cy(k);
-                    if (dx >= 0 && dx < p.nx && dy >= 0 && dy < p.ny) {
-                        if constexpr (std::is_same<T, double>::value)
-                            wmass = Ar<double>::add(wmass, fin[k]);
-                        else
-                            wmass += (double)fin[k] + p.rw[k];
-                    }
-                }
             }
+            wmass = wall_mass<T, double, true>(p, xs, ys, fin);
         }
     } else if (valid) {
         if (p.collide) {

@@ -60,8 +60,8 @@ __device__ void tube_pull(const StepParams &p, const S *__restrict__ f, int x, T
     if (r >= p.nx) r = wrap ? 0 : -1;
     if (l < 0) l = wrap ? p.nx - 1 : -1;
     fin[0] = tload<S, T>(p, f[tidx(p, 0, x)], 0);
-    fin[1] = r >= 0 ? tload<S, T>(p, f[tidx(p, 1, r)], 1) : tload<S, T>(p, f[tidx(p, 2, x)], 2);
-    fin[2] = l >= 0 ? tload<S, T>(p, f[tidx(p, 2, l)], 2) : tload<S, T>(p, f[tidx(p, 1, x)], 1);
+    fin[1] = tload<S, T>(p, f[tidx(p, r >= 0 ? 1 : 2, r >= 0 ? r : x)], 1);  // W_1 = W_2
+    fin[2] = tload<S, T>(p, f[tidx(p, l >= 0 ? 2 : 1, l >= 0 ? l : x)], 2);
 }
 
 template <typename S, typename T>
