@@ -455,16 +455,11 @@ __global__ void __launch_bounds__(kFinThreads, BATCHED ? 2 : 1) k_finalize(const
             // are visible: the block synchronised after them), as lbm_moments
             // evaluates them
             const int x = p.probe_site % p.nx, y = p.probe_site / p.nx;
-            double g[Q], r, a, b;
+            double r, a, b;
+            S raw[Q];
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const S v = f[fidx(p.plane, p.pitch, q, y, x)];
-                if constexpr (std::is_same<S, double>::value)
-                    g[q] = v;
-                else
-                    g[q] = Ar<double>::add((double)s2f(v), p.rw[q]);
-            }
-            moments<Q, double>(g, r, a, b);
+            for (int q = 0; q < Q; ++q) raw[q] = f[fidx(p.plane, p.pitch, q, y, x)];
+            site_moments<Q, S>(p, raw, r, a, b);
             double *slot = p.probe + 3 * ((step - 1) % p.probe_cap);
             slot[0] = r;
             slot[1] = a;

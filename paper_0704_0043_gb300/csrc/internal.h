@@ -121,7 +121,16 @@ struct DevStats {  // mirrors lbm_step_stats
     int reserved;
 };
 
+// Fixed-point form of a site's moments (site_moments): FP32 / 16-bit storage.
+struct MomentFx {
+    long long rest;  // sum of rho_ref W_k in units
+    float scale;     // 2^(27 - exponent of rho_ref)
+    float lim;       // deviations below it fit (0: never)
+    int exp;         // the unit is 2^exp
+};
+
 struct StepParams {
+    MomentFx mfx;
     int nx, ny, pitch;
     long long plane;           // elements per population plane
     int boundary;              // LBM_BC_*
@@ -162,6 +171,7 @@ struct StepParams {
 };
 
 struct FinalParams {
+    MomentFx mfx;
     int nblocks;               // partial rows to reduce
     int fixed;                 // the rows are fixed-point rows of the fused kernel
     int *work;                 // work-item counter to clear for the next step, or nullptr

@@ -539,6 +539,14 @@ StepParams cfg_step_params(const lbm_config &g, int q, int pitch, long long plan
         p.rw[k] = g.rho_ref * w;
         p.rwf[k] = (float)p.rw[k];
     }
+    {
+        const int er = std::ilogb((double)p.rho_ref), shift = 58 - er;
+        p.mfx.exp = -shift;
+        p.mfx.lim = er > -90 && er < 90 ? std::ldexp(1.0f, er) : 0.0f;
+        p.mfx.scale = std::ldexp(1.0f, std::max(-110, std::min(110, 27 - er)));
+        p.mfx.rest = 0;
+        for (int k = 0; k < q && p.mfx.lim > 0.0f; ++k) p.mfx.rest += std::llrint(std::ldexp(p.rw[k], shift));
+    }
     p.ds_out = nullptr;
     p.smooth_delta = g.smooth_delta;
     p.smooth_k = g.smooth_k;
@@ -571,6 +579,7 @@ FinalParams cfg_final_params(const lbm_config &g, const StepParams &p, int colli
         f.rw[k] = p.rw[k];
     }
     f.rho_ref = p.rho_ref;
+    f.mfx = p.mfx;
     return f;
 }
 

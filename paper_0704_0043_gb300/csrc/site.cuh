@@ -18,8 +18,8 @@ __device__ __forceinline__ long long fidx(long long plane, int pitch, int k, int
 // Stored value as a compute value: FP64 storage is f itself; FP32 / BF16 /
 // FP16 storage is the deviation g, read as g in FP32 or as the absolute
 // f = (double) g + rw_k in FP64.
-template <typename S, typename T>
-__device__ __forceinline__ T load_as(const StepParams &p, S v, int k)
+template <typename S, typename T, typename P>
+__device__ __forceinline__ T load_as(const P &p, S v, int k)
 {
     if constexpr (std::is_same<S, double>::value)
         return T(v);
@@ -27,6 +27,97 @@ __device__ __forceinline__ T load_as(const StepParams &p, S v, int k)
         return Ar<double>::add((double)s2f(v), p.rw[k]);
     else
         return s2f(v);
+}
+
+// (double) v and (float) v on integers (a conversion takes the FP64 unit as long as
+// an addition does); subnormal and nonfinite values by the conversion itself, out
+// of line (inline, the compiler runs it for every value and selects).
+__device__ __noinline__ double widen_rare(float v) { return (double)v; }
+__device__ __noinline__ float narrow_rare(double v) { return (float)v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned u = __float_as_uint(v), e = (u >> 23) & 0xffu;
+    if (e - 1u >= 0xfeu && (u << 1) != 0) return widen_rare(v);
+    const unsigned hi = (u << 1) != 0 ? ((u & 0x7fffffffu) >> 3) + (896u << 20) : 0u;
+    return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
+__device__ __forceinline__ float narrow(double v)
+{
+    const unsigned h = (unsigned)__double2hiint(v), l = (unsigned)__double2loint(v);
+    const unsigned e = (h >> 20) & 0x7ffu;
+    if (e - 897u >= 253u) {  // zero, else below 2^-126, above 2^127 or nonfinite
+        if (((h << 1) | l) == 0) return __uint_as_float(h);
+        return narrow_rare(v);
+    }
+    unsigned m = (((h & 0x7fffffffu) << 3) | (l >> 29)) - (896u << 23);
+    const unsigned rest = l & 0x1fffffffu;
+    m += rest > 0x10000000u || (rest == 0x10000000u && (m & 1u));  // to nearest, ties to even
+    return __uint_as_float(m | (h & 0x80000000u));
+}
+
+// v 2^e as a double, to nearest (ties to even); the result's exponent is normal.
+__device__ __forceinline__ double fixed_value(long long v, int e)
+{
+    if (v == 0) return 0.0;
+    unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+    const int lz = __clzll((long long)m);
+    m <<= lz;
+    unsigned long long t = m >> 11;
+    const unsigned rest = (unsigned)m & 0x7ffu;
+    t += rest > 0x400u || (rest == 0x400u && (t & 1ull));
+    t += (unsigned long long)(63 - lz + e + 1022) << 52;
+    return __longlong_as_double((long long)(t | ((unsigned long long)(v < 0) << 63)));
+}
+
+// rho, u of a site's stored populations (Eq. macro_dis; lbm_moments and the control
+// point).  FP64 storage: the FP64 formula.  FP32 / 16-bit storage: the sums of the
+// deviations in fixed point, each rounded once to 2^(exponent of rho_ref - 55) and
+// held as a high and a low 32-bit part (|g| < 2^exponent: nine of them do not
+// overflow), the sums exact and added to rho_ref sum W in units of 2^(exponent - 58)
+// (every rho_ref W_k is a whole number of them); the quotients from one reciprocal,
+// corrected by their residuals.  That is eight FP64 instructions (five for D1Q3),
+// and no less exact than the FP64 sums, which round every population and every sum.
+// A site with a deviation of rho_ref or more, or rho <= 0, takes the FP64 formula.
+template <int Q, typename S, typename P>
+__device__ __forceinline__ void site_moments(const P &p, const S raw[Q], double &rho, double &ux, double &uy)
+{
+    if constexpr (!std::is_same<S, double>::value) {
+        int h[3] = {0, 0, 0}, l[3] = {0, 0, 0};  // sums of g, c_x g, c_y g
+        bool plain = true;
+#pragma unroll
+        for (int k = 0; k < Q; ++k) {
+            const float g = s2f(raw[k]);
+            plain = plain && fabsf(g) < p.mfx.lim;
+            const float x = __fmul_rn(g, p.mfx.scale);  // below 2^27, exact
+            const int hi = __float2int_rn(x);
+            const int lo = __float2int_rn(__fmul_rn(__fsub_rn(x, __int2float_rn(hi)), 268435456.0f));
+            h[0] += hi;
+            l[0] += lo;
+            h[1] += Lat<Q>::cx(k) * hi;
+            l[1] += Lat<Q>::cx(k) * lo;
+            h[2] += Lat<Q>::cy(k) * hi;
+            l[2] += Lat<Q>::cy(k) * lo;
+        }
+        auto units = [&](int j) { return (long long)h[j] * (1ll << 31) + (long long)l[j] * 8; };
+        const long long r = p.mfx.rest + units(0), jx = units(1), jy = units(2);
+        if (plain && r > 0) {
+            bool slow = false;
+            rho = fixed_value(r, p.mfx.exp);
+            const Recip64 R = recip64(rho, slow);
+            const double a = fixed_value(jx, p.mfx.exp), a0 = __dmul_rn(a, R.y);
+            ux = fma(fma(-rho, a0, a), R.y, a0);
+            uy = 0.0;
+            if constexpr (Q == 9) {
+                const double b = fixed_value(jy, p.mfx.exp), b0 = __dmul_rn(b, R.y);
+                uy = fma(fma(-rho, b0, b), R.y, b0);
+            }
+            if (!slow) return;
+        }
+    }
+    double f[Q];
+#pragma unroll
+    for (int k = 0; k < Q; ++k) f[k] = load_as<S, double>(p, raw[k], k);
+    moments<Q, double>(f, rho, ux, uy);
 }
 
 // Free flight in pull form at site (x, y) (Sec. 2): f_in_k(x) = f_k(x - v_k);

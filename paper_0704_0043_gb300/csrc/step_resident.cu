@@ -581,10 +581,11 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
             if (f.probe != nullptr) {
                 // the control point's moments after the whole step, as lbm_moments gives them
                 const int x = f.probe_site % f.nx, y = f.probe_site / f.nx;
-                double g[Q], r, u, v;
+                double r, u, v;
+                S raw[Q];
 #pragma unroll
-                for (int q = 0; q < Q; ++q) g[q] = load_as<S, double>(a.p, dst[fidx(f.plane, f.pitch, q, y, x)], q);
-                moments<Q, double>(g, r, u, v);
+                for (int q = 0; q < Q; ++q) raw[q] = dst[fidx(f.plane, f.pitch, q, y, x)];
+                site_moments<Q, S>(a.p, raw, r, u, v);
                 double *slot = f.probe + 3 * ((step - 1) % f.probe_cap);
                 slot[0] = r;
                 slot[1] = u;

@@ -1,6 +1,5 @@
 // step_tiled.cu -- one limited LBGK step with overlapping tiles, every lattice,
-// boundary kind and precision, plus the small field kernels (init, moments,
-// population transfer, dS field).
+// boundary kind and precision, and the ensemble reduction of every lattice.
 //
 // A block computes free flight, collision and dS(f') (Eq. lbgkLB, Sec. 3.6) for
 // a tile of sites and keeps the dS values in shared memory; the sites of the
@@ -522,96 +521,6 @@ __global__ void __launch_bounds__(256) k_ens_mean(const double *__restrict__ par
     }
 }
 
-template <int Q, typename S>
-__global__ void k_delta_s(StepParams p, const S *__restrict__ f, double *__restrict__ out)
-{
-    const long long n = (long long)p.nx * p.ny;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % p.nx), y = (int)(s / p.nx);
-        if (Q == 9 && is_wall_node(p, x, y)) {  // boundary nodes are not collided
-            out[s] = 0.0;
-            continue;
-        }
-        double fin[Q], fs[Q], fp[Q], ds, dsin, rho;
-        pull<Q, S, double>(p, f, x, y, fin);
-        const bool bad = site_collide<Q, double>(fin, p.a, true, fs, fp, ds, dsin, rho, p.eq, true, p.coll, p.beta);
-        out[s] = bad ? (double)INFINITY : ds;
-    }
-}
-
-template <int Q, typename S>
-__global__ void k_init(StepParams p, const double *__restrict__ rho, const double *__restrict__ ux,
-                       const double *__restrict__ uy, S *__restrict__ f)
-{
-    const long long n = (long long)p.nx * p.ny;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % p.nx), y = (int)(s / p.nx);
-        double fs[Q];
-        if (!feq_any<Q>(p.eq, rho[s], ux[s], uy ? uy[s] : 0.0, fs)) {
-#pragma unroll
-            for (int k = 0; k < Q; ++k) fs[k] = (double)NAN;  // no entropic f* for |u_j| >= 1
-        }
-#pragma unroll
-        for (int k = 0; k < Q; ++k) {
-            if constexpr (std::is_same<S, double>::value)
-                f[fidx(p.plane, p.pitch, k, y, x)] = fs[k];
-            else
-                f[fidx(p.plane, p.pitch, k, y, x)] = f2s<S>((float)Ar<double>::sub(fs[k], p.rw[k]));
-        }
-    }
-}
-
-template <int Q, typename S>
-__global__ void k_moments(StepParams p, const S *__restrict__ f, double *__restrict__ rho, double *__restrict__ ux,
-                          double *__restrict__ uy)
-{
-    const long long n = (long long)p.nx * p.ny;
-    for (long long s = blockIdx.x * (long long)blockDim.x + threadIdx.x; s < n; s += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(s % p.nx), y = (int)(s / p.nx);
-        double g[Q], r, a, b;
-#pragma unroll
-        for (int k = 0; k < Q; ++k) g[k] = load_as<S, double>(p, f[fidx(p.plane, p.pitch, k, y, x)], k);
-        moments<Q, double>(g, r, a, b);
-        rho[s] = r;
-        ux[s] = a;
-        if (uy) uy[s] = b;
-    }
-}
-
-template <typename S>
-__global__ void k_get(int q, StepParams p, const S *__restrict__ f, double *__restrict__ out)
-{
-    const long long n = (long long)p.nx * p.ny, tot = n * q;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(e / n);
-        const long long s = e % n;
-        out[e] = load_as<S, double>(p, f[fidx(p.plane, p.pitch, k, (int)(s / p.nx), (int)(s % p.nx))], k);
-    }
-}
-
-template <typename S>
-__global__ void k_set(int q, StepParams p, const double *__restrict__ in, S *__restrict__ f)
-{
-    const long long n = (long long)p.nx * p.ny, tot = n * q;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < tot; e += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(e / n);
-        const long long s = e % n;
-        S v;
-        if constexpr (std::is_same<S, double>::value)
-            v = in[e];
-        else
-            v = f2s<S>((float)Ar<double>::sub(in[e], p.rw[k]));
-        f[fidx(p.plane, p.pitch, k, (int)(s / p.nx), (int)(s % p.nx))] = v;
-    }
-}
-
-inline int grid_for(long long n, int threads)
-{
-    long long b = (n + threads - 1) / threads;
-    if (b > 152 * 32) b = 152 * 32;
-    return (int)(b < 1 ? 1 : b);
-}
-
 }  // namespace
 
 template <typename T>
@@ -648,17 +557,6 @@ cudaError_t launch_tiled_batched_f32(int q, const TiledArgs *table, const int2 *
 }
 
 template <typename T>
-cudaError_t launch_delta_s(int q, const StepParams &p, const T *f, double *out, cudaStream_t s)
-{
-    const int g = grid_for((long long)p.nx * p.ny, 256);
-    if (q == 9)
-        k_delta_s<9, T><<<g, 256, 0, s>>>(p, f, out);
-    else
-        k_delta_s<3, T><<<g, 256, 0, s>>>(p, f, out);
-    return cudaGetLastError();
-}
-
-template <typename T>
 cudaError_t launch_ens_mean(int q, const StepParams &p, const T *src, double *ens, cudaStream_t s)
 {
     if (q == 9)
@@ -669,54 +567,9 @@ cudaError_t launch_ens_mean(int q, const StepParams &p, const T *src, double *en
     return cudaGetLastError();
 }
 
-template <typename T>
-cudaError_t launch_init(int q, const StepParams &p, const double *rho, const double *ux, const double *uy, T *f,
-                        cudaStream_t s)
-{
-    const int g = grid_for((long long)p.nx * p.ny, 256);
-    if (q == 9)
-        k_init<9, T><<<g, 256, 0, s>>>(p, rho, ux, uy, f);
-    else
-        k_init<3, T><<<g, 256, 0, s>>>(p, rho, ux, nullptr, f);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_moments(int q, const StepParams &p, const T *f, double *rho, double *ux, double *uy,
-                           cudaStream_t s)
-{
-    const int g = grid_for((long long)p.nx * p.ny, 256);
-    if (q == 9)
-        k_moments<9, T><<<g, 256, 0, s>>>(p, f, rho, ux, uy);
-    else
-        k_moments<3, T><<<g, 256, 0, s>>>(p, f, rho, ux, uy);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_get(int q, const StepParams &p, const T *f, double *out, cudaStream_t s)
-{
-    k_get<T><<<grid_for((long long)p.nx * p.ny * q, 256), 256, 0, s>>>(q, p, f, out);
-    return cudaGetLastError();
-}
-
-template <typename T>
-cudaError_t launch_set(int q, const StepParams &p, const double *in, T *f, cudaStream_t s)
-{
-    k_set<T><<<grid_for((long long)p.nx * p.ny * q, 256), 256, 0, s>>>(q, p, in, f);
-    return cudaGetLastError();
-}
-
 #define LBM_INST(T)                                                                                           \
     template cudaError_t launch_tiled<T>(int, const StepParams &, const T *, T *, int *, cudaStream_t);     \
-    template cudaError_t launch_delta_s<T>(int, const StepParams &, const T *, double *, cudaStream_t);     \
-    template cudaError_t launch_ens_mean<T>(int, const StepParams &, const T *, double *, cudaStream_t);    \
-    template cudaError_t launch_init<T>(int, const StepParams &, const double *, const double *,           \
-                                        const double *, T *, cudaStream_t);                                  \
-    template cudaError_t launch_moments<T>(int, const StepParams &, const T *, double *, double *, double *, \
-                                           cudaStream_t);                                                    \
-    template cudaError_t launch_get<T>(int, const StepParams &, const T *, double *, cudaStream_t);         \
-    template cudaError_t launch_set<T>(int, const StepParams &, const double *, T *, cudaStream_t);
+    template cudaError_t launch_ens_mean<T>(int, const StepParams &, const T *, double *, cudaStream_t);
 LBM_INST(float)
 LBM_INST(double)
 LBM_INST(__nv_bfloat16)
