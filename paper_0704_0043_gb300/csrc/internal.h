@@ -261,7 +261,7 @@ constexpr long long kResMaxSites64 = 1ll << 19;  // FP64 storage
 constexpr long long kResMaxSites3 = 1ll << 20;   // D1Q3, FP32 storage
 struct ResRow {
     double v[4];  // P_MASS .. P_DS_LIM of a worker block's sites
-    int c[4];     // positivity, median, flagged and own sites
+    int c[4];     // positivity, median, flagged sites
 };
 struct ResState {
     unsigned long long arrived;  // low word: worker arrivals; high word: candidates recorded (both since the launch)
@@ -277,10 +277,19 @@ struct ResArgs {
     void *buf[2];
     int cur, nsteps;
     int aw, gx, tiles;  // set by the launcher: warps that carry sites, tiles along x, tiles
-    double wall_rest;   // rest values of the boundary nodes' populations that stream back
+    double rest;        // rest_mass
     ResState *rs;
 };
+double rest_mass(const StepParams &p);
 bool resident_applies(const lbm_config &c);
+// The smallest FP32 D2Q9 lattices without Ehrenfests' steps: one thread-block
+// cluster, populations in shared memory (step_cluster.cu).  us per step against
+// the resident kernel, median filter, boundary nodes: 32^2 4.0 / 5.9, 100^2
+// 4.4 / 6.3, 128^2 5.8 / 6.3, 150^2 7.1 / 4.9 (16 SMs against 151).
+constexpr long long kCluMaxSites = 128 * 128;
+constexpr size_t kCluMaxBytes = 200 * 1024;  // dynamic shared memory of a block
+bool cluster_applies(const lbm_config &c);
+cudaError_t launch_cluster(ResArgs a, cudaStream_t s);
 // Takes a.nsteps steps from a.buf[a.cur]; a.f as for the tail of a step.
 template <typename S>
 cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s);
@@ -386,6 +395,7 @@ struct lbm_ctx {
     lbm::SelState *sel_state = nullptr;  // Ehrenfests' limiter: the cooperative tail's selection state
     int fin_grid = 0;                     // blocks of the cooperative tail (0: one-block tail only)
     bool capturing = false;               // a graph capture is in progress (one-block tail)
+    bool cluster = false;                 // the resident steps run as one cluster
     lbm::ResState *res = nullptr;         // resident steps: counters and rows (nullptr: stepped launch by launch)
     double *ens = nullptr;  // [kEnsBlocks][2] partial sums and counts of dS, then E(dS), alpha, sum, count
     void *ent_field = nullptr;   // LBM_LIM_ENTTHRESH: the pass's dS field

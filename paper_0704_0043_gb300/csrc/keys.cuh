@@ -64,17 +64,14 @@ __device__ __noinline__ double key_ent9(const KeyGeom p, const S *src, int site,
 // term, and the terms are added in k order: the key is that of key_dS9_lane bit
 // for bit, in 48 FP64 instructions where one lane alone needs about 190.  Returns the key,
 // or -1 for a site at or below delta_e or one that cannot be limited; every
-// lane of a group returns the same value.  Not inlined: the caller's hot loop
-// keeps its registers, and the call is rare.
-template <typename S>
-__device__ __noinline__ double key_dS9_group(const KeyGeom p, const S *src, int site, double delta_e)
+// lane of a group returns the same value.  key_dS9_core: from the lane's pulled
+// population `mine` (a2b = 2 beta - 1).  The whole is not inlined: the caller's hot
+// loop keeps its registers, and the call is rare.
+__device__ __forceinline__ double key_dS9_core(double mine, double a2b, double delta_e)
 {
     using A = Ar<double>;
     constexpr unsigned kAll = 0xffffffffu;
-    if (p.eq == 1) return key_ent9<S>(p, src, site, delta_e);
     const int lane = threadIdx.x & 31, base = lane < 27 ? lane / 9 * 9 : 0, k = lane < 27 ? lane % 9 : lane - 27;
-    const int x = site % p.nx, y = site / p.nx;
-    const double mine = pull_one_f64<S>(p, src, x, y, k);
     // lane 0: f0 + f1 + ... + f8; lane 1: f1 - f3 + f5 - f6 - f7 + f8; lane 2: f2 - f4 + f5
     // + f6 - f7 - f8 (four bits per term: direction, 15 for none; a bit per sign)
     const unsigned long long order = k == 1 ? 0xfff876531ull : (k == 2 ? 0xfff876542ull : 0x876543210ull);
@@ -103,7 +100,7 @@ __device__ __noinline__ double key_dS9_group(const KeyGeom p, const S *src, int 
     const double poly = fma(t3, -0.5, fma(s9, 0.5, A::add(1.0, opp ? -c3 : c3)));
     const double fs = A::mul(A::mul(rho, Lat<9>::w(k)), poly);
     // collision and the dS term
-    const double fp = A::add(fs, A::mul(p.a, A::sub(fs, mine)));
+    const double fp = A::add(fs, A::mul(a2b, A::sub(fs, mine)));
     const double d = A::sub(fp, fs), dd = A::mul(d, d);
     bool slow_t = false;
     double term = quot64(dd, recip64(fs, slow_t), slow_t);
@@ -114,6 +111,14 @@ __device__ __noinline__ double key_dS9_group(const KeyGeom p, const S *src, int 
     for (int j = 1; j < 9; ++j) s = A::add(s, __shfl_sync(kAll, term, base + j));
     const bool bad = ((bad_lanes >> base) & 0x1ffu) != 0 || !gt0(rho) || !finite64(rho) || !finite64(ux) || !finite64(uy);
     return !bad && finite64(s) && s > delta_e ? s : -1.0;
+}
+
+template <typename S>
+__device__ __noinline__ double key_dS9_group(const KeyGeom p, const S *src, int site, double delta_e)
+{
+    if (p.eq == 1) return key_ent9<S>(p, src, site, delta_e);
+    const int lane = threadIdx.x & 31, k = lane < 27 ? lane % 9 : lane - 27;
+    return key_dS9_core(pull_one_f64<S>(p, src, site % p.nx, site / p.nx, k), p.a, delta_e);
 }
 
 // The same key evaluated by one thread alone (lane-parallel keying of many

@@ -63,14 +63,15 @@ __device__ __forceinline__ float rcp_approx(float x)
 // FP64 step.  recip64 seeds 1/b from the FP32 special-function unit through
 // integer operations on b's bits (no FP64 conversion) and refines it by one
 // Newton step (relative error below 2^-42); quot64 corrects a * (1/b) once by
-// its residual and then checks the result exactly (Markstein's residual
-// argument, IBM J. Res. Dev. 34 (1990) 111): the last residual a - b q is one
-// exact FMA, and q is the correctly rounded quotient when the residual is
-// below b * ulp(q) / 2 (there are no ties in a division).  That is 2
-// instructions per denominator and 4 per quotient.  Where the check does not
-// hold (the quotient within 2^-33 ulp of a rounding boundary, a power-of-two q,
-// operands outside 2^-500 .. 2^499, zero or negative b, nonfinite values) `slow`
-// is set and the caller repeats its evaluation with __ddiv_rn.
+// its residual, so that q is within 2^-31 ulp of half an ulp of a/b, and then
+// settles the last bit exactly (Markstein's residual argument, IBM J. Res. Dev. 34
+// (1990) 111): r = a - b q is one exact FMA; q is the correctly rounded quotient
+// when |r| < b * ulp(q) / 2, and its neighbour on r's side otherwise (there are no
+// ties in a division; quotients next to a rounding boundary are common where a
+// fluid at rest carries rounding noise of one ulp).  That is 2 instructions per
+// denominator and 4 per quotient.  For a power-of-two q with a residual, operands
+// outside 2^-500 .. 2^499, zero or negative b and nonfinite values `slow` is set and
+// the caller repeats its evaluation with __ddiv_rn.
 // With the site evaluation below (shared sub-expressions, no FP64 comparisons)
 // the 600 x 500 FP64 cavity step went from 347 to 256 us (tiled kernel with its
 // tail), and the 512 x 512 entropic FP64 step from 787 to 694 us.
@@ -112,8 +113,10 @@ __device__ __forceinline__ double quot64(double a, const Recip64 &R, bool &slow)
     const bool exact = (rh | (int)rl) == 0;
     const bool pow2 = ((qh & 0xfffff) | __double2loint(q)) == 0;
     const bool zero = (ah | al) == 0;
-    slow |= !(zero || (in_range64(ah) && (exact || (below && !pow2))));
-    return zero ? a : q;
+    slow |= !(zero || (in_range64(ah) && (exact || !pow2)));
+    // the neighbour on r's side: one more in magnitude where r and q have one sign
+    const long long step = below ? 0ll : ((__double2hiint(r) ^ qh) < 0 ? -1ll : 1ll);
+    return zero ? a : __longlong_as_double(__double_as_longlong(q) + step);
 }
 
 // Tests of FP64 values by their bits: a comparison takes the FP64 unit as long as

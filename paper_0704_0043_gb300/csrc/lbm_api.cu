@@ -383,6 +383,14 @@ lbm_status run_resident(lbm_ctx *c, int64_t n, int64_t *taken)
         a.rs = c->res;
         const cudaError_t e = with_storage(c->cfg.precision, [&](auto tag) -> cudaError_t {
             using S = STORAGE_T;
+            if constexpr (std::is_same<S, float>::value) {
+                if (c->cluster) {
+                    const cudaError_t ce = launch_cluster(a, c->stream);
+                    if (ce == cudaSuccess) return ce;
+                    cudaGetLastError();  // no such cluster on this device
+                    c->cluster = false;
+                }
+            }
             return launch_resident<S>(c->q, a, c->stream);
         });
         if (e != cudaSuccess) {
@@ -687,6 +695,7 @@ lbm_status lbm_create(const lbm_config *cfg, void *cuda_stream, lbm_ctx **out)
         }
     }
     if (z.res) alloc((void **)&c->res, z.res);
+    c->cluster = cluster_applies(c->cfg);
     if (z.ent) {
         alloc(&c->ent_field, z.ent - sizeof(EntState));
         alloc((void **)&c->ent, sizeof(EntState));

@@ -1,0 +1,180 @@
+// resident.cuh -- what the kernels that take many steps in one launch share
+// (step_resident.cu, step_cluster.cu): a site's evaluation, the sums of a block.
+#pragma once
+
+#include <type_traits>
+
+#include "internal.h"
+#include "lattice.cuh"
+#include "select.cuh"
+#include "site.cuh"
+
+namespace lbm {
+namespace {
+
+// FP32 parameters, converted once per thread.
+struct ResK {
+    float a, b2, dm, thr_e;
+};
+
+// What a site gives the finishing code.
+template <int Q, typename T>
+struct SiteState {
+    T fin[Q], fs[Q], fp[Q];
+    float nq[Q];  // FP32
+    float fa[Q];  // FP32: absolute f*
+    T ds, dsin, rho;
+    bool bad;
+};
+
+template <int Q, typename S>
+__device__ __forceinline__ void eval_site(const StepParams &p, const ResK &kk, SiteState<Q, compute_t<S>> &v, bool need_in)
+{
+    using T = compute_t<S>;
+    if constexpr (std::is_same<T, double>::value) {
+        v.bad = site_poly64<Q>(v.fin, p.a, true, v.fs, v.fp, v.ds, v.dsin, v.rho, need_in);
+    } else {
+        v.bad = site_collide_dev<Q>(v.fin, kk.a, kk.b2, true, p.rho_ref, p.rwf, v.fs, v.nq, v.fp, v.fa, v.ds, v.dsin,
+                                    v.rho, 0);
+    }
+    if (v.bad) v.ds = T(INFINITY);
+}
+
+// Sums of the worker's sites of one step (per thread).
+template <typename T>
+struct ResSums {
+    T mass = T(0), ds = T(0), din = T(0), lim = T(0);
+    int pos = 0, med = 0, bad = 0;
+};
+
+// The sums of a warp's step, into lanes 0 (mass), 8 (dS), 16 (dS_in), 24 (dS_lim):
+// a butterfly in which each level halves the sums a lane carries.
+template <typename T>
+__device__ __forceinline__ T warp_totals(const ResSums<T> &s, int lane)
+{
+    using A = Ar<T>;
+    const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
+    T a0 = hi16 ? s.din : s.mass, a1 = hi16 ? s.lim : s.ds;
+    const T b0 = hi16 ? s.mass : s.din, b1 = hi16 ? s.ds : s.lim;
+    a0 = A::add(a0, __shfl_xor_sync(kFull, b0, 16));
+    a1 = A::add(a1, __shfl_xor_sync(kFull, b1, 16));
+    T z = hi8 ? a1 : a0;
+    z = A::add(z, __shfl_xor_sync(kFull, hi8 ? a0 : a1, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) z = A::add(z, __shfl_xor_sync(kFull, z, o));
+    return z;
+}
+
+// A block's sums of one step, gathered warp by warp.
+template <int NW, typename T>
+struct BlockAcc {
+    T part[NW][4];  // the warps' sums
+    int cnt[3];     // positivity, median, flagged sites
+    int ticket;
+    __device__ void clear()
+    {
+        for (int i = 0; i < 3; ++i) cnt[i] = 0;
+        ticket = 0;
+    }
+};
+
+// Adds a warp's sums; true in the last of the block's `warps` warps to come.
+template <int NW, typename T>
+__device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &sum, int warps)
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const T z = warp_totals<T>(sum, lane);
+    if ((lane & 7) == 0) w.part[warp][lane >> 3] = z;
+    if (__any_sync(kFull, (sum.pos | sum.med | sum.bad) != 0)) {
+        const int pos = __reduce_add_sync(kFull, sum.pos), med = __reduce_add_sync(kFull, sum.med);
+        const int bad = __reduce_add_sync(kFull, sum.bad);
+        if (lane < 3) atomicAdd(&w.cnt[lane], lane == 0 ? pos : (lane == 1 ? med : bad));
+    }
+    __threadfence_block();
+    __syncwarp();
+    int last = 0;
+    if (lane == 0) last = atomicAdd(&w.ticket, 1) == warps - 1;
+    if (!__shfl_sync(kFull, last, 0)) return false;
+    __threadfence_block();
+    return true;
+}
+
+// The last warp writes the block's row and clears the sums: FP64 parts are added
+// in warp order, FP32 parts exactly (128-bit fixed point, so in any order: lane l
+// takes parts l and l + 32, lanes with one statistic are added by shuffles).
+template <int NW, typename T>
+__device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int warps, unsigned *status)
+{
+    const int lane = threadIdx.x & 31;
+    double v = 0.0;
+    if constexpr (std::is_same<T, double>::value) {
+        if (lane < 4)
+            for (int j = 0; j < warps; ++j) v = Ar<double>::add(v, w.part[j][lane]);
+    } else {
+        static_assert(NW <= 16, "two parts a lane");
+        unsigned __int128 fx = 0;
+        bool bad = false;
+        if (lane >> 2 < warps) fx_add(fx, w.part[lane >> 2][lane & 3], bad);
+        if (8 + (lane >> 2) < warps) fx_add(fx, w.part[8 + (lane >> 2)][lane & 3], bad);
+        const unsigned nonfinite = __ballot_sync(kFull, bad);
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            const unsigned long long lo = __shfl_xor_sync(kFull, (unsigned long long)fx, o);
+            const unsigned long long hi = __shfl_xor_sync(kFull, (unsigned long long)(fx >> 64), o);
+            fx += ((unsigned __int128)hi << 64) | lo;
+        }
+        if (lane < 4) v = nonfinite & (0x11111111u << lane) ? __longlong_as_double(0x7ff8000000000000LL) : fx_value(fx);
+    }
+    if (lane < 4) row->v[lane] = v;
+    if (lane < 3) {
+        const int c = w.cnt[lane];
+        row->c[lane] = c;
+        if (lane == 2 && c) atomicOr(status, kStatNonfinite);  // a site was nonfinite
+    }
+    __syncwarp();
+    if (lane == 0) w.clear();
+    __syncwarp();
+}
+
+// The sums of a step from its block rows (lane r, r + 32, ... of each of the first
+// four warps' statistic, or one warp for all four).
+__device__ __forceinline__ void sum_rows(const ResRow *rows, int n, int stat, double &v, int &c)
+{
+    const int lane = threadIdx.x & 31;
+    v = 0.0;
+    c = 0;
+    for (int r = lane; r < n; r += 32) {
+        v += __ldcg(&rows[r].v[stat]);
+        c += __ldcg(&rows[r].c[stat]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
+    c = __reduce_add_sync(kFull, c);
+}
+
+// The stats record of a step from its sums (tot: P_MASS .. P_DS_LIM, cnt: positivity,
+// median, flagged sites).
+template <bool F64>
+__device__ __forceinline__ DevStats step_record(const ResArgs &a, const double *tot, const long long *cnt,
+                                                double ehr_sum, int nsel, int n_valid, unsigned status, long long step)
+{
+    DevStats st;
+    st.step = step;
+    // FP32 storage: the rows hold sums of rho - rho_ref and of the deviations of the
+    // boundary nodes' populations; their rest values add up to `rest`
+    st.mass = F64 ? tot[P_MASS] : tot[P_MASS] + a.rest;
+    st.sum_dS = tot[P_SUM_DS];
+    st.dS_lbgk = Ar<double>::mul(a.f.one_minus_a2, tot[P_SUM_IN]);
+    st.dS_lim = Ar<double>::add(tot[P_DS_LIM], ehr_sum);
+    st.n_pos = cnt[0];
+    st.n_med = cnt[1];
+    st.n_bad = cnt[2];
+    st.n_ehr = nsel;
+    st.n_cand = n_valid;
+    st.status = (status & kStatNonfinite) ? 4 : ((status & kStatTimeout) ? 5 : 0);
+    st.reserved = 0;
+    return st;
+}
+
+}  // namespace
+}  // namespace lbm

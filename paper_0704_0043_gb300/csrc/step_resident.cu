@@ -29,6 +29,7 @@
 
 #include "internal.h"
 #include "lattice.cuh"
+#include "resident.cuh"
 #include "select.cuh"
 #include "site.cuh"
 
@@ -90,46 +91,16 @@ __device__ __forceinline__ bool wait_arrivals(const unsigned long long *p, unsig
     return false;
 }
 
-// FP32 parameters, converted once per thread.
-struct ResK {
-    float a, b2, dm, thr_e;
-};
-
 // A worker block's shared memory.
 template <typename T>
 struct WorkShared {
     T ds[2][(kResWarps + 2) * 34];  // dS of the tile (D2Q9: rows of 34 with the halo; D1Q3: 32 aw + 2)
-    double part[2][kResWarps][4];   // FP64 storage: the warps' sums
-    unsigned long long lo[2][4], hi[2][4];  // FP32 storage: the block's sums in fixed point
-    int cnt[2][4];                  // positivity, median, flagged, own sites
-    int ticket[2], ncand[2], fxbad[2];
+    BlockAcc<kResWarps, T> acc[2];     // the block's sums, steps of each parity
+    int ncand[2];
     double fw[2][9];                // diffusive wall: f*(1, u_wall) of the resting walls and of the lid
     unsigned n;                     // candidates so far (after the barrier)
     int go;                         // 0: a wait gave up
 };
-
-// What a site gives the finishing code.
-template <int Q, typename T>
-struct SiteState {
-    T fin[Q], fs[Q], fp[Q];
-    float nq[Q];  // FP32
-    float fa[Q];  // FP32: absolute f*
-    T ds, dsin, rho;
-    bool bad;
-};
-
-template <int Q, typename S>
-__device__ __forceinline__ void eval_site(const StepParams &p, const ResK &kk, SiteState<Q, compute_t<S>> &v, bool need_in)
-{
-    using T = compute_t<S>;
-    if constexpr (std::is_same<T, double>::value) {
-        v.bad = site_poly64<Q>(v.fin, p.a, true, v.fs, v.fp, v.ds, v.dsin, v.rho, need_in);
-    } else {
-        v.bad = site_collide_dev<Q>(v.fin, kk.a, kk.b2, true, p.rho_ref, p.rwf, v.fs, v.nq, v.fp, v.fa, v.ds, v.dsin,
-                                    v.rho, 0);
-    }
-    if (v.bad) v.ds = T(INFINITY);
-}
 
 // dS(f') of a site outside the tile (0 at boundary nodes and off the lattice).
 template <int Q, typename S>
@@ -144,13 +115,6 @@ __device__ __noinline__ compute_t<S> halo_ds(const StepParams &p, ResK kk, const
     eval_site<Q, S>(p, kk, v, false);
     return v.ds;
 }
-
-// Sums of the worker's sites of one step (per thread).
-template <typename T>
-struct ResSums {
-    T mass = T(0), ds = T(0), din = T(0), lim = T(0);
-    int pos = 0, med = 0, bad = 0, own = 0;
-};
 
 // One tile: aw rows of 32 sites (D2Q9; a warp per row) or 32 aw consecutive sites
 // (D1Q3).  Every site is stored, candidates recorded, sums taken.  Every thread
@@ -279,7 +243,6 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
 #pragma unroll
         for (int k = 0; k < Q; ++k) dst[fidx(p.plane, p.pitch, k, y, x)] = f2s<S>(v.fp[k]);
     }
-    ++sum.own;
     if constexpr (F64)
         sum.mass = A::add(sum.mass, v.rho);
     else
@@ -311,82 +274,18 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
     }
 }
 
-// The sums of a warp's step, into lanes 0 (mass), 8 (dS), 16 (dS_in), 24 (dS_lim):
-// a butterfly in which each level halves the sums a lane carries.
-template <typename T>
-__device__ __forceinline__ T warp_totals(const ResSums<T> &s, int lane)
-{
-    using A = Ar<T>;
-    const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
-    T a0 = hi16 ? s.din : s.mass, a1 = hi16 ? s.lim : s.ds;
-    const T b0 = hi16 ? s.mass : s.din, b1 = hi16 ? s.ds : s.lim;
-    a0 = A::add(a0, __shfl_xor_sync(kFull, b0, 16));
-    a1 = A::add(a1, __shfl_xor_sync(kFull, b1, 16));
-    T z = hi8 ? a1 : a0;
-    z = A::add(z, __shfl_xor_sync(kFull, hi8 ? a0 : a1, 8));
-#pragma unroll
-    for (int o = 4; o > 0; o >>= 1) z = A::add(z, __shfl_xor_sync(kFull, z, o));
-    return z;
-}
-
 // A worker warp's sums of step s into the block's; the block's last warp to come
 // writes the block's row and reports it (the tail reads the rows of a step when
 // every worker has reported).  Runs while the grid barrier completes.
 template <typename T>
 __device__ __forceinline__ void block_sums(const ResArgs &a, WorkShared<T> &w, const ResSums<T> &sum, int s, int aw)
 {
-    constexpr bool F64 = std::is_same<T, double>::value;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, b = s & 1;
-    const T z = warp_totals<T>(sum, lane);
-    const int pos = __reduce_add_sync(kFull, sum.pos), med = __reduce_add_sync(kFull, sum.med);
-    const int bad = __reduce_add_sync(kFull, sum.bad), own = __reduce_add_sync(kFull, sum.own);
-    if ((lane & 7) == 0) {
-        if constexpr (F64) {
-            w.part[b][warp][lane >> 3] = z;
-        } else {
-            unsigned __int128 fx = 0;
-            bool nonfinite = false;
-            fx_add(fx, z, nonfinite);
-            if (nonfinite) atomicOr(&w.fxbad[b], 1 << (lane >> 3));
-            const unsigned long long lo = (unsigned long long)fx, hi = (unsigned long long)(fx >> 64);
-            const unsigned long long old = atomicAdd(&w.lo[b][lane >> 3], lo);
-            atomicAdd(&w.hi[b][lane >> 3], hi + (old + lo < old ? 1ull : 0ull));
-        }
-    }
-    if (lane == 0) {
-        if (pos) atomicAdd(&w.cnt[b][0], pos);
-        if (med) atomicAdd(&w.cnt[b][1], med);
-        if (bad) atomicAdd(&w.cnt[b][2], bad);
-        atomicAdd(&w.cnt[b][3], own);
-    }
-    __threadfence_block();
-    __syncwarp();
-    int last = 0;
-    if (lane == 0) last = atomicAdd(&w.ticket[b], 1) == aw - 1;
-    if (!__shfl_sync(kFull, last, 0)) return;
-    __threadfence_block();
+    const int lane = threadIdx.x & 31, b = s & 1;
+    if (!add_warp(w.acc[b], sum, aw)) return;
     // the rows of step s - kResRows are read before this one takes their place
     if (s >= kResRows && lane == 0) wait_for(&a.rs->stats_done, (unsigned)(s - kResRows + 1), a.p.status);
     __syncwarp();
-    ResRow *row = &a.rs->rows[s % kResRows][blockIdx.x];
-    if (lane < 4) {
-        double v;
-        if constexpr (F64) {
-            v = 0.0;
-            for (int j = 0; j < aw; ++j) v = Ar<double>::add(v, w.part[b][j][lane]);
-        } else {
-            v = (w.fxbad[b] >> lane) & 1 ? __longlong_as_double(0x7ff8000000000000LL)
-                                          : fx_value(((unsigned __int128)w.hi[b][lane] << 64) | w.lo[b][lane]);
-        }
-        const int c = w.cnt[b][lane];
-        row->v[lane] = v;
-        row->c[lane] = c;
-        if (lane == 2 && c) atomicOr(a.p.status, kStatNonfinite);  // a site was nonfinite
-    }
-    __syncwarp();
-    if (lane < 4) w.lo[b][lane] = w.hi[b][lane] = 0ull, w.cnt[b][lane] = 0;
-    if (lane == 0) w.ticket[b] = w.fxbad[b] = 0;
-    __syncwarp();
+    take_row(w.acc[b], &a.rs->rows[s % kResRows][blockIdx.x], aw, a.p.status);
     if (lane == 0) red_release(&a.rs->rows_in[s % kResRows], 1u);
 }
 
@@ -427,12 +326,9 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
         kk.dm = (float)p.delta_m;
         kk.thr_e = (float)(p.delta_e * (1.0 - 1.0 / 64.0));
     }
-    if (t < 8) {
-        w.lo[t >> 2][t & 3] = w.hi[t >> 2][t & 3] = 0ull;
-        w.cnt[t >> 2][t & 3] = 0;
-    }
     if (t < 2) {
-        w.ticket[t] = w.ncand[t] = w.fxbad[t] = 0;
+        w.acc[t].clear();
+        w.ncand[t] = 0;
         if (Q == 9 && p.boundary == 4) wall_star(p, t == 1, w.fw[t]);
     }
     __syncthreads();
@@ -543,16 +439,9 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         __syncthreads();
         if (!h.go) break;
         if (warp < 4) {
-            const ResRow *rows = a.rs->rows[s % kResRows];
-            double v = 0.0;
-            int c = 0;
-            for (int r = lane; r < W; r += 32) {
-                v += __ldcg(&rows[r].v[warp]);
-                c += __ldcg(&rows[r].c[warp]);
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(kFull, v, o);
-            c = __reduce_add_sync(kFull, c);
+            double v;
+            int c;
+            sum_rows(a.rs->rows[s % kResRows], W, warp, v, c);
             if (lane == 0) {
                 h.tot[warp] = v;
                 h.cnt[warp] = c;
@@ -561,21 +450,7 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         __syncthreads();
         if (t == 0) {
             step += 1;
-            DevStats st;
-            st.step = step;
-            // FP32 storage: the rows hold sums of rho - rho_ref (of the deviations of the
-            // boundary nodes' populations, whose rest values add up to wall_rest)
-            st.mass = F64 ? h.tot[P_MASS] : h.tot[P_MASS] + ((double)h.cnt[3] * (double)a.p.rho_ref + a.wall_rest);
-            st.sum_dS = h.tot[P_SUM_DS];
-            st.dS_lbgk = Ar<double>::mul(f.one_minus_a2, h.tot[P_SUM_IN]);
-            st.dS_lim = Ar<double>::add(h.tot[P_DS_LIM], ehr_sum);
-            st.n_pos = h.cnt[0];
-            st.n_med = h.cnt[1];
-            st.n_bad = h.cnt[2];
-            st.n_ehr = h.sel.nsel;
-            st.n_cand = n_valid;
-            st.status = (h.status & kStatNonfinite) ? 4 : ((h.status & kStatTimeout) ? 5 : 0);
-            st.reserved = 0;
+            const DevStats st = step_record<F64>(a, h.tot, h.cnt, ehr_sum, h.sel.nsel, n_valid, h.status, step);
             f.stats_ring[rec % f.ring_len] = st;
             rec += 1;
             if (f.probe != nullptr) {
@@ -630,6 +505,22 @@ bool resident_applies(const lbm_config &c)
     return (long long)c.nx * c.ny <= most;
 }
 
+// What FP32 / 16-bit storage leaves out of the mass: rho_ref per site, and at the
+// boundary nodes of a lattice with nodes on the walls rho_ref W_k for the
+// populations that stream back.
+double rest_mass(const StepParams &p)
+{
+    if (!bc_node_walls(p.boundary)) return (double)p.rho_ref * (double)((long long)p.nx * p.ny);
+    const long long inner = (long long)(p.nx - 2) * (p.ny - 2);
+    double m = (double)p.rho_ref * (double)inner;
+    for (int k = 0; k < 9; ++k) {
+        // nodes whose neighbour in direction k is on the lattice, less the inner ones
+        const long long all = (long long)(p.nx - (Lat<9>::cx(k) != 0)) * (p.ny - (Lat<9>::cy(k) != 0));
+        m += (double)(all - inner) * p.rw[k];
+    }
+    return m;
+}
+
 template <typename S>
 cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s)
 {
@@ -648,18 +539,7 @@ cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s)
     a.aw = aw;
     a.gx = q == 3 ? 1 : (a.p.nx + 31) / 32;
     a.tiles = tiles_for(aw);
-    a.wall_rest = 0.0;
-    if (q == 9 && bc_node_walls(a.p.boundary)) {
-        // rest values of the populations that stream back from the boundary nodes
-        const int nx = a.p.nx, ny = a.p.ny;
-        for (int k = 0; k < 9; ++k) {
-            const long long cx = Lat<9>::cx(k) != 0, cy = Lat<9>::cy(k) != 0;
-            // nodes of the ring whose neighbour in direction k is on the lattice
-            const long long all = (nx - cx) * (ny - cy);
-            const long long inner = (long long)(nx - 2) * (ny - 2);
-            a.wall_rest += (double)(all - inner) * a.p.rw[k];
-        }
-    }
+    a.rest = rest_mass(a.p);
     cudaError_t e = cudaMemsetAsync(a.rs, 0, offsetof(ResState, rows), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

@@ -1,8 +1,8 @@
 """The FP64 step's shared-reciprocal quotients (csrc/lattice.cuh).
 
-A quotient is taken from a reciprocal and checked by its exact residual; where
-the check does not hold, or an operand lies outside 2^-500 .. 2^499, the site is
-evaluated again with IEEE divisions.  Both ways give the bits of the plain
+A quotient is taken from a reciprocal and settled by its exact residual; where an
+operand lies outside 2^-500 .. 2^499 (or the quotient is a power of two with a
+residual), the site is evaluated again with IEEE divisions.  Both ways give the bits of the plain
 division, so FP64 populations and dS must equal the oracle's at every scale:
 the step is homogeneous of degree one, and scaling a state by a power of two
 moves its quotients from the fast path (scale 1, 2^200) to the general one
@@ -32,6 +32,8 @@ def test_fp64_step_equals_oracle_at_every_scale(q, ny, nx, exponent):
     w = np.array([4 / 9] + [1 / 9] * 4 + [1 / 36] * 4) if q == 9 else np.array([2 / 3, 1 / 6, 1 / 6])
     f[:, :, 2:9] = (w * scale)[:, None, None]
     f[1, :, 12:18] = f[1, :, 12:18].mean()
+    # and one at rest up to an ulp or two: quotients next to rounding boundaries
+    f[:, :, 20:30] = np.nextafter(f[:, :, 2:3], [[[0.0]], [[np.inf]], [[0.0]]] * (q // 3))
     g.set_populations(f)
     for _ in range(3):
         r = oracle.step(oc, f)

@@ -91,3 +91,30 @@ def test_timed_steps_among_resident_ones():
     assert a.timing_read()[2] == 4
     b.step(13)
     np.testing.assert_array_equal(a.get_populations(), b.get_populations())
+
+
+@pytest.mark.parametrize("limiters", [0, lbm.LIM_POSITIVITY, lbm.LIM_MEDIAN, lbm.LIM_POSITIVITY | lbm.LIM_MEDIAN])
+@pytest.mark.parametrize("nx,ny", [(5, 32), (32, 33), (100, 100), (128, 128), (250, 50), (17, 300)])
+@pytest.mark.parametrize("boundary", [lbm.BC_WALLS, lbm.BC_PERIODIC, lbm.BC_CHANNEL, lbm.BC_NODE_WALLS,
+                                      lbm.BC_DIFFUSIVE])
+def test_cluster_equals_launches(boundary, nx, ny, limiters):
+    """The smallest lattices without Ehrenfests' steps run as one cluster: bands of
+    two rows and more, ragged bands, several sites a thread, medians at the bands'
+    edges (every row is out of equilibrium) and several to a thread."""
+    both(lbm.KERNEL_TILED, rand_state(9, ny, nx, 11 + nx, eps=0.05, heavy=2), 7, lattice=lbm.D2Q9, nx=nx, ny=ny,
+         boundary=boundary, precision=lbm.FP32, beta=0.97, u_lid=0.1, limiters=limiters, delta_median=1e-4, k_max=0)
+
+
+def test_cluster_records_the_control_point():
+    """Probe samples of the cluster are the moments after each step."""
+    nx, ny = 50, 40
+    g = lbm.Lattice(lattice=lbm.D2Q9, nx=nx, ny=ny, boundary=lbm.BC_DIFFUSIVE, precision=lbm.FP32, beta=0.95, u_lid=0.1,
+                    limiters=lbm.LIM_MEDIAN, delta_median=1e-4)
+    g.init(*inputs.cavity_rest(nx, ny))
+    g.probe(33 * nx + 3, 8)
+    want = []
+    for n in (1, 3, 2):
+        g.step(n)
+        want.append(tuple(a[33, 3] for a in g.moments()))
+    got = g.probe_read(8)
+    np.testing.assert_array_equal(got[[0, 3, 5]], np.array(want))
