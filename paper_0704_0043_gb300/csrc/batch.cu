@@ -1,11 +1,18 @@
 // batch.cu -- many lattices stepped by shared launches (include/lbm_batch.h).
 //
 // Each lattice is an ordinary context (lbm_ctx) created on the batch's own
-// stream.  A batched step is at most six launches whatever the number of
-// lattices: the fused kernel over every FP32 D2Q9 cavity, the tube kernel
-// over D1Q3 lattices, the tiled kernel over the rest, and the tail kernel (one
-// block per lattice) for D2Q9 and for D1Q3.  The fused launch is one wave of resident
-// warps over the work items of all its lattices (strips of 62 columns times
+// stream.  A batched step is a few launches whatever the number of lattices: the
+// fused kernel over FP32 D2Q9 cavities, the tube kernel over D1Q3 lattices, the tiled
+// kernel over the rest, each followed by the tail kernel (one block per lattice).
+// They form chains that do not depend on one another: the cavities by the limiters
+// whose code they need (a chain of its own from 2^20 sites, where a launch lasts
+// longer than it takes to enqueue: the specialised kernel keeps fewer registers;
+// the others share the general one), and the tubes.  The chains of a run of steps
+// go to streams of their own, so one chain's tails and the end of its launches
+// overlap another's work.  256 cavities of 100 to 597 a side, a third of them with
+// each limiter, 40 steps and the reads of all states: 27.3 ms in one chain of the
+// general kernel, 24.0 ms in chains.  A fused launch is one wave of resident warps
+// over the work items of all its lattices (strips of 62 columns times
 // short row segments), handed out through one device counter, so warps that
 // finish early take more work whatever lattice it belongs to; the tube launch
 // does the same over groups of 1024 sites of every tube; tiled blocks find
@@ -24,6 +31,23 @@
 
 using namespace lbm;
 
+namespace {
+constexpr int kClasses = 4;  // fused lattices by limiter code: bit 0 the positivity rule, bit 1 the median filter
+constexpr long long kOwnChain = 1ll << 20;  // sites from which a class has its own chain
+// One chain of fused lattices (class kClasses - 1: the general kernel, also for the
+// small classes and, with their tails, the D2Q9 lattices of the tiled kernel).
+struct FusedChain {
+    std::vector<FusedArgs> h_args[2];
+    std::vector<FinalArgs> h_fin[2];
+    std::vector<int2> h_map;
+    FusedArgs *args[2] = {nullptr, nullptr};
+    FinalArgs *fin[2] = {nullptr, nullptr};
+    int2 *map = nullptr;
+    int *work = nullptr;  // the launch's work-item counter
+    int items = 0, n = 0;
+};
+}  // namespace
+
 struct lbm_batch {
     cudaStream_t user = nullptr;
     cudaStream_t run = nullptr;
@@ -34,21 +58,21 @@ struct lbm_batch {
     bool dirty = true;
     int phase = 0;               // steps since the tables were built, mod 2
     std::vector<int> cur_build;  // each lattice's current buffer when built
-    std::vector<FusedArgs> h_fused[2];
+    FusedChain chain[kClasses];
+    cudaStream_t side[kClasses] = {};  // streams of the other chains (the first chain in use takes `run`)
+    cudaEvent_t fork = nullptr, join[kClasses] = {};
     std::vector<TiledArgs> h_t3[2], h_t9[2];
-    std::vector<FinalArgs> h_fin9[2], h_fin3[2];
-    std::vector<int2> h_fmap, h_t3map, h_t9map, h_tubemap;
+    std::vector<FinalArgs> h_fin3[2];
+    std::vector<int2> h_t3map, h_t9map, h_tubemap;
     std::vector<TubeArgs> h_tube[2];
     void *table_mem = nullptr;
     size_t table_bytes = 0;
-    FusedArgs *fused[2] = {nullptr, nullptr};
     TiledArgs *t3[2] = {nullptr, nullptr}, *t9[2] = {nullptr, nullptr};
-    FinalArgs *fin9[2] = {nullptr, nullptr}, *fin3[2] = {nullptr, nullptr};
-    int2 *fmap = nullptr, *t3map = nullptr, *t9map = nullptr, *tubemap = nullptr;
+    FinalArgs *fin3[2] = {nullptr, nullptr};
+    int2 *t3map = nullptr, *t9map = nullptr, *tubemap = nullptr;
     TubeArgs *tube[2] = {nullptr, nullptr};
-    int *work = nullptr;   // the fused launch's work-item counter
-    int *twork = nullptr;  // the tube launch's
-    int fitems = 0, t3blocks = 0, t9blocks = 0, titems = 0, n9 = 0, n3 = 0;
+    int *twork = nullptr;  // the tube launch's work-item counter
+    int t3blocks = 0, t9blocks = 0, titems = 0, n3 = 0;
     // shape
     int seg_rows = 0;  // rows per fused work item; 0 = automatic
     int waves = 8;     // automatic segments: about this many work items per resident warp
@@ -124,30 +148,47 @@ lbm_status leave(lbm_batch *b)
 lbm_status rebuild(lbm_batch *b)
 {
     for (int k = 0; k < 2; ++k) {
-        b->h_fused[k].clear();
         b->h_t3[k].clear();
         b->h_tube[k].clear();
         b->h_t9[k].clear();
-        b->h_fin9[k].clear();
         b->h_fin3[k].clear();
     }
-    b->h_fmap.clear();
+    for (FusedChain &f : b->chain) {
+        for (int k = 0; k < 2; ++k) {
+            f.h_args[k].clear();
+            f.h_fin[k].clear();
+        }
+        f.h_map.clear();
+    }
     b->h_t3map.clear();
     b->h_tubemap.clear();
     b->h_t9map.clear();
     b->cur_build.assign(b->slots.size(), 0);
-    int first_fused = -1;  // index in h_fin9 of the first fused lattice's tail
+    int first_fused[kClasses];  // index in each chain's tails of its first fused lattice
+    for (int &f : first_fused) f = -1;
     int first_tube = -1;   // index in h_fin3 of the first tube's tail
-    // one row-segment length for every fused lattice: about `waves` items per
+    // one row-segment length for the fused lattices of a chain: about `waves` items per
     // resident warp over the strip rows of all of them (unless fixed)
-    long long strip_rows = 0;
+    long long strip_rows[kClasses] = {}, class_sites[kClasses] = {};
+    auto fused_class = [](const lbm_ctx *c) {
+        return ((c->cfg.limiters & LBM_LIM_POSITIVITY) ? 1 : 0) | ((c->cfg.limiters & LBM_LIM_MEDIAN) ? 2 : 0);
+    };
     for (lbm_ctx *c : b->slots) {
         if (!c) continue;
         if (!c->ready) return bfail(b, LBM_ERR_STATE, "a lattice of the batch was never initialised");
-        if (ctx_uses_fused(c)) strip_rows += (long long)((c->cfg.nx + 61) / 62) * c->cfg.ny;
+        if (ctx_uses_fused(c)) {
+            strip_rows[fused_class(c)] += (long long)((c->cfg.nx + 61) / 62) * c->cfg.ny;
+            class_sites[fused_class(c)] += (long long)c->cfg.nx * c->cfg.ny;
+        }
     }
     const long long want = std::max(1LL, (long long)b->waves * fused_slots(4, true));
-    const int seg = b->seg_rows > 0 ? b->seg_rows : (int)std::max(4LL, (strip_rows + want - 1) / want);
+    int chain_of[kClasses], seg[kClasses];
+    for (int cls = 0; cls < kClasses; ++cls) {
+        chain_of[cls] = class_sites[cls] >= kOwnChain ? cls : kClasses - 1;
+        if (chain_of[cls] != cls) strip_rows[kClasses - 1] += strip_rows[cls];
+    }
+    for (int ci = 0; ci < kClasses; ++ci)
+        seg[ci] = b->seg_rows > 0 ? b->seg_rows : (int)std::max(4LL, (strip_rows[ci] + want - 1) / want);
     for (size_t i = 0; i < b->slots.size(); ++i) {
         lbm_ctx *c = b->slots[i];
         if (!c) continue;
@@ -157,19 +198,21 @@ lbm_status rebuild(lbm_batch *b)
         for (int k = 0; k < 2; ++k) {
             void *src = c->buf[c->cur ^ k], *dst = c->buf[c->cur ^ k ^ 1];
             if (ctx_uses_fused(c)) {
+                const int ci = chain_of[fused_class(c)];
+                FusedChain &f = b->chain[ci];
                 FusedArgs A;
-                const int blocks = fused_make_args(p, src, dst, seg, 1, &A);
-                b->h_fused[k].push_back(A);
+                const int blocks = fused_make_args(p, src, dst, seg[ci], 1, &A);
+                f.h_args[k].push_back(A);
                 FinalArgs F{ctx_final_params(c, 1, lim, blocks), dst};
                 F.p.src = src;
                 F.p.fixed = 1;
                 F.p.partials = ctx_fx_rows(c);  // the fused kernel's accumulator rows
-                F.p.work = nullptr;             // the first fused lattice's tail clears the counter (below)
-                if (first_fused < 0 && k == 0) first_fused = (int)b->h_fin9[0].size();
-                b->h_fin9[k].push_back(F);
+                F.p.work = nullptr;             // the chain's first fused lattice's tail clears the counter (below)
+                if (first_fused[ci] < 0 && k == 0) first_fused[ci] = (int)f.h_fin[0].size();
+                f.h_fin[k].push_back(F);
                 if (k == 0)
                     for (int it = 0; it < A.items; ++it)
-                        b->h_fmap.push_back(make_int2((int)b->h_fused[0].size() - 1, it));
+                        f.h_map.push_back(make_int2((int)f.h_args[0].size() - 1, it));
             } else if (c->q == 3 && tube_applies(c->cfg, lim)) {
                 // D1Q3: the tube kernel, groups of chunks from one counter
                 TubeArgs A{};
@@ -200,7 +243,7 @@ lbm_status rebuild(lbm_batch *b)
                 auto &tab = c->q == 9 ? b->h_t9[k] : b->h_t3[k];
                 auto &map = c->q == 9 ? b->h_t9map : b->h_t3map;
                 tab.push_back(A);
-                (c->q == 9 ? b->h_fin9[k] : b->h_fin3[k]).push_back(F);
+                (c->q == 9 ? b->chain[kClasses - 1].h_fin[k] : b->h_fin3[k]).push_back(F);
                 if (k == 0)
                     for (int lb = 0; lb < A.blocks; ++lb) map.push_back(make_int2((int)tab.size() - 1, lb));
             }
@@ -208,13 +251,15 @@ lbm_status rebuild(lbm_batch *b)
     }
     // one device allocation holds every table
     auto sz = [](size_t n, size_t e) { return ((n * e + 255) / 256) * 256; };
-    const size_t nf = b->h_fused[0].size(), nt3 = b->h_t3[0].size(), nt9 = b->h_t9[0].size();
-    const size_t nf9 = b->h_fin9[0].size(), nf3 = b->h_fin3[0].size(), ntb = b->h_tube[0].size();
-    size_t need = 2 * (sz(nf, sizeof(FusedArgs)) + sz(nt3, sizeof(TiledArgs)) + sz(nt9, sizeof(TiledArgs)) +
-                       sz(nf9, sizeof(FinalArgs)) + sz(nf3, sizeof(FinalArgs)) + sz(ntb, sizeof(TubeArgs))) +
+    const size_t nt3 = b->h_t3[0].size(), nt9 = b->h_t9[0].size();
+    const size_t nf3 = b->h_fin3[0].size(), ntb = b->h_tube[0].size();
+    size_t need = 2 * (sz(nt3, sizeof(TiledArgs)) + sz(nt9, sizeof(TiledArgs)) + sz(nf3, sizeof(FinalArgs)) +
+                       sz(ntb, sizeof(TubeArgs))) +
                   sz(b->h_tubemap.size(), sizeof(int2)) + 256 +
-                  sz(b->h_fmap.size(), sizeof(int2)) + sz(b->h_t3map.size(), sizeof(int2)) +
-                  sz(b->h_t9map.size(), sizeof(int2)) + 256 + 256;
+                  sz(b->h_t3map.size(), sizeof(int2)) + sz(b->h_t9map.size(), sizeof(int2)) + kClasses * 256;
+    for (const FusedChain &f : b->chain)
+        need += 2 * (sz(f.h_args[0].size(), sizeof(FusedArgs)) + sz(f.h_fin[0].size(), sizeof(FinalArgs))) +
+                sz(f.h_map.size(), sizeof(int2));
     if (need > b->table_bytes) {
         BCK(b, cudaStreamSynchronize(b->run));
         if (b->table_mem) cudaFree(b->table_mem);
@@ -224,12 +269,15 @@ lbm_status rebuild(lbm_batch *b)
         b->table_bytes = need;
     }
     char *m = (char *)b->table_mem;
-    b->work = (int *)m;
-    m += 256;
+    int *const counters = (int *)m;
     b->twork = (int *)m;
     m += 256;
-    if (first_fused >= 0)
-        for (int k = 0; k < 2; ++k) b->h_fin9[k][(size_t)first_fused].p.work = b->work;
+    for (int ci = 0; ci < kClasses; ++ci) {
+        b->chain[ci].work = (int *)m;
+        m += 256;
+        if (first_fused[ci] >= 0)
+            for (int k = 0; k < 2; ++k) b->chain[ci].h_fin[k][(size_t)first_fused[ci]].p.work = b->chain[ci].work;
+    }
     if (first_tube >= 0)
         for (int k = 0; k < 2; ++k) b->h_fin3[k][(size_t)first_tube].p.work = b->twork;
     auto put = [&](const void *h, size_t n, size_t e, void **d) -> cudaError_t {
@@ -238,24 +286,27 @@ lbm_status rebuild(lbm_batch *b)
         return n ? cudaMemcpyAsync(*d, h, n * e, cudaMemcpyHostToDevice, b->run) : cudaSuccess;
     };
     for (int k = 0; k < 2; ++k) {
-        BCK(b, put(b->h_fused[k].data(), nf, sizeof(FusedArgs), (void **)&b->fused[k]));
+        for (FusedChain &f : b->chain) {
+            BCK(b, put(f.h_args[k].data(), f.h_args[k].size(), sizeof(FusedArgs), (void **)&f.args[k]));
+            BCK(b, put(f.h_fin[k].data(), f.h_fin[k].size(), sizeof(FinalArgs), (void **)&f.fin[k]));
+        }
         BCK(b, put(b->h_t3[k].data(), nt3, sizeof(TiledArgs), (void **)&b->t3[k]));
         BCK(b, put(b->h_t9[k].data(), nt9, sizeof(TiledArgs), (void **)&b->t9[k]));
-        BCK(b, put(b->h_fin9[k].data(), nf9, sizeof(FinalArgs), (void **)&b->fin9[k]));
         BCK(b, put(b->h_fin3[k].data(), nf3, sizeof(FinalArgs), (void **)&b->fin3[k]));
         BCK(b, put(b->h_tube[k].data(), ntb, sizeof(TubeArgs), (void **)&b->tube[k]));
     }
-    BCK(b, put(b->h_fmap.data(), b->h_fmap.size(), sizeof(int2), (void **)&b->fmap));
+    for (FusedChain &f : b->chain) {
+        BCK(b, put(f.h_map.data(), f.h_map.size(), sizeof(int2), (void **)&f.map));
+        f.items = (int)f.h_map.size();
+        f.n = (int)f.h_fin[0].size();
+    }
     BCK(b, put(b->h_t3map.data(), b->h_t3map.size(), sizeof(int2), (void **)&b->t3map));
     BCK(b, put(b->h_t9map.data(), b->h_t9map.size(), sizeof(int2), (void **)&b->t9map));
     BCK(b, put(b->h_tubemap.data(), b->h_tubemap.size(), sizeof(int2), (void **)&b->tubemap));
-    BCK(b, cudaMemsetAsync(b->work, 0, sizeof(int), b->run));
-    BCK(b, cudaMemsetAsync(b->twork, 0, sizeof(int), b->run));
-    b->fitems = (int)b->h_fmap.size();
+    BCK(b, cudaMemsetAsync(counters, 0, (kClasses + 1) * 256, b->run));
     b->t3blocks = (int)b->h_t3map.size();
     b->titems = (int)b->h_tubemap.size();
     b->t9blocks = (int)b->h_t9map.size();
-    b->n9 = (int)nf9;
     b->n3 = (int)nf3;
     b->dirty = false;
     b->phase = 0;
@@ -265,19 +316,61 @@ lbm_status rebuild(lbm_batch *b)
 
 int launches_per_step(const lbm_batch *b)
 {
-    return (b->fitems > 0) + (b->t3blocks > 0) + (b->t9blocks > 0) + (b->titems > 0) + (b->n9 > 0) + (b->n3 > 0);
+    int n = (b->t3blocks > 0) + (b->t9blocks > 0) + (b->titems > 0) + (b->n3 > 0);
+    for (const FusedChain &f : b->chain) n += (f.items > 0) + (f.n > 0);
+    return n;
 }
 
-// One batched step on the batch stream (table set `k`).
-cudaError_t one_step(lbm_batch *b, int k)
+// One step (table set `k`) of chain ci, 0 .. kClasses - 1 the fused lattices' and
+// (the last) the D2Q9 lattices of the tiled kernel, kClasses the tubes'.
+cudaError_t chain_step(lbm_batch *b, int ci, int k, cudaStream_t s)
 {
     cudaError_t e = cudaSuccess;
-    if (b->fitems && e == cudaSuccess) e = launch_fused_batched(b->fused[k], b->fmap, b->fitems, b->work, b->run);
-    if (b->t3blocks && e == cudaSuccess) e = launch_tiled_batched_f32(3, b->t3[k], b->t3map, b->t3blocks, b->run);
-    if (b->titems && e == cudaSuccess) e = launch_tube_batched(b->tube[k], b->tubemap, b->titems, b->twork, b->run);
-    if (b->t9blocks && e == cudaSuccess) e = launch_tiled_batched_f32(9, b->t9[k], b->t9map, b->t9blocks, b->run);
-    if (b->n9 && e == cudaSuccess) e = launch_finalize_batched_f32(9, b->fin9[k], b->n9, b->run);
-    if (b->n3 && e == cudaSuccess) e = launch_finalize_batched_f32(3, b->fin3[k], b->n3, b->run);
+    if (ci == kClasses) {
+        if (b->t3blocks) e = launch_tiled_batched_f32(3, b->t3[k], b->t3map, b->t3blocks, s);
+        if (b->titems && e == cudaSuccess) e = launch_tube_batched(b->tube[k], b->tubemap, b->titems, b->twork, s);
+        if (b->n3 && e == cudaSuccess) e = launch_finalize_batched_f32(3, b->fin3[k], b->n3, s);
+        return e;
+    }
+    const FusedChain &f = b->chain[ci];
+    if (f.items) e = launch_fused_batched(f.args[k], f.map, f.items, f.work, (ci & 2) != 0, (ci & 1) != 0, s);
+    if (ci == kClasses - 1 && b->t9blocks && e == cudaSuccess)
+        e = launch_tiled_batched_f32(9, b->t9[k], b->t9map, b->t9blocks, s);
+    if (f.n && e == cudaSuccess) e = launch_finalize_batched_f32(9, f.fin[k], f.n, s);
+    return e;
+}
+
+bool chain_used(const lbm_batch *b, int ci) { return ci == kClasses ? b->n3 > 0 : b->chain[ci].n > 0; }
+
+// `n` steps from table set `k` on, the chains side by side: the first in use on the
+// batch stream, the others on their own, forked from it and joined to it again.
+cudaError_t chains_run(lbm_batch *b, int k, int64_t n)
+{
+    cudaStream_t st[kClasses + 1] = {};
+    int side = 0;
+    bool first = true;
+    cudaError_t e = cudaSuccess;
+    for (int ci = 0; ci <= kClasses; ++ci) {
+        if (!chain_used(b, ci)) continue;
+        if (first) {
+            st[ci] = b->run;
+            first = false;
+            continue;
+        }
+        if (side == 0 && (e = cudaEventRecord(b->fork, b->run)) != cudaSuccess) return e;
+        st[ci] = b->side[side++];
+        if ((e = cudaStreamWaitEvent(st[ci], b->fork, 0)) != cudaSuccess) return e;
+    }
+    for (int64_t i = 0; i < n && e == cudaSuccess; ++i)
+        for (int ci = 0; ci <= kClasses && e == cudaSuccess; ++ci)
+            if (st[ci]) e = chain_step(b, ci, k ^ (int)(i & 1), st[ci]);
+    // joined also after an error: a capture ends with its streams joined, and what was
+    // enqueued is ordered before the batch stream's later work
+    for (int j = 0; j < side; ++j) {
+        cudaError_t je = cudaEventRecord(b->join[j], b->side[j]);
+        if (je == cudaSuccess) je = cudaStreamWaitEvent(b->run, b->join[j], 0);
+        if (e == cudaSuccess) e = je;
+    }
     return e;
 }
 
@@ -291,21 +384,19 @@ lbm_status run_steps(lbm_batch *b, int64_t n)
     int64_t left = n;
     if (b->graph_steps > 0 && left >= b->graph_steps) {
         if (b->phase == 1) {  // graphs start on even steps
-            BCK(b, one_step(b, 1));
+            BCK(b, chains_run(b, 1, 1));
             b->phase = 0;
             b->launches += lps;
             --left;
         }
         if (!b->exec && left >= b->graph_steps) {
             // the kernels' one-time attribute set-up happens outside the capture
-            BCK(b, one_step(b, 0));
-            BCK(b, one_step(b, 1));
+            BCK(b, chains_run(b, 0, 2));
             b->launches += 2 * lps;
             left -= 2;
             cudaGraph_t g = nullptr;
             BCK(b, cudaStreamBeginCapture(b->run, cudaStreamCaptureModeThreadLocal));
-            cudaError_t ce = cudaSuccess;
-            for (int i = 0; i < b->graph_steps && ce == cudaSuccess; ++i) ce = one_step(b, i & 1);
+            const cudaError_t ce = chains_run(b, 0, b->graph_steps);
             cudaError_t ee = cudaStreamEndCapture(b->run, &g);
             if (ce != cudaSuccess || ee != cudaSuccess) {
                 if (g) cudaGraphDestroy(g);
@@ -325,10 +416,10 @@ lbm_status run_steps(lbm_batch *b, int64_t n)
             left -= b->graph_steps;
         }
     }
-    for (int64_t i = 0; i < left; ++i) {
-        BCK(b, one_step(b, b->phase));
-        b->phase ^= 1;
-        b->launches += lps;
+    if (left > 0) {
+        BCK(b, chains_run(b, b->phase, left));
+        b->phase ^= (int)(left & 1);
+        b->launches += left * lps;
     }
     return LBM_OK;
 }
@@ -346,7 +437,14 @@ lbm_status lbm_batch_create(void *cuda_stream, lbm_batch **out)
     if (cudaStreamCreateWithFlags(&b->run, cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev_in, cudaEventDisableTiming) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->ev_out, cudaEventDisableTiming) != cudaSuccess ||
-        cudaEventCreate(&b->t0) != cudaSuccess || cudaEventCreate(&b->t1) != cudaSuccess) {
+        cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreate(&b->t0) != cudaSuccess || cudaEventCreate(&b->t1) != cudaSuccess || [&] {
+            for (int i = 0; i < kClasses; ++i)
+                if (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess ||
+                    cudaEventCreateWithFlags(&b->join[i], cudaEventDisableTiming) != cudaSuccess)
+                    return true;
+            return false;
+        }()) {
         cudaGetLastError();
         lbm_batch_destroy(b);
         return LBM_ERR_CUDA;
@@ -363,9 +461,13 @@ lbm_status lbm_batch_destroy(lbm_batch *b)
         if (c) lbm_destroy(c);
     drop_graph(b);
     if (b->table_mem) cudaFree(b->table_mem);
-    cudaEvent_t evs[] = {b->ev_in, b->ev_out, b->t0, b->t1};
+    cudaEvent_t evs[] = {b->ev_in, b->ev_out, b->t0, b->t1, b->fork};
     for (cudaEvent_t e : evs)
         if (e) cudaEventDestroy(e);
+    for (int i = 0; i < kClasses; ++i) {
+        if (b->join[i]) cudaEventDestroy(b->join[i]);
+        if (b->side[i]) cudaStreamDestroy(b->side[i]);
+    }
     if (b->run) cudaStreamDestroy(b->run);
     delete b;
     return LBM_OK;

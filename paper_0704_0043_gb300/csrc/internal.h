@@ -357,7 +357,9 @@ int fused_make_args(const StepParams &p, const void *src, void *dst, int seg_row
 // being item map[i].y of instance map[i].x, handed out dynamically through
 // the counter *work (cleared by the tail after the launch).  Tiled: `blocks`
 // blocks, block b running instance map[b].x as its block map[b].y.
-cudaError_t launch_fused_batched(const FusedArgs *table, const int2 *map, int items, int *work, cudaStream_t s);
+// med / pos: the lattices' median / positivity code is needed (a smaller kernel otherwise).
+cudaError_t launch_fused_batched(const FusedArgs *table, const int2 *map, int items, int *work, bool med, bool pos,
+                                 cudaStream_t s);
 cudaError_t launch_tiled_batched_f32(int q, const TiledArgs *table, const int2 *map, int blocks, cudaStream_t s);
 cudaError_t launch_finalize_batched_f32(int q, const FinalArgs *table, int n, cudaStream_t s);
 // D1Q3 streaming step (FP32 / FP64 storage): *chunked is false when the grid

@@ -51,7 +51,9 @@ namespace {
 constexpr int kWarps = 4;  // independent work items per block
 constexpr int kThreads = 32 * kWarps;
 constexpr int kBlocksPerSM = 5;         // resident blocks per SM
-constexpr int kBlocksPerSMBatched = 4;  // batched launches (the arguments in shared memory take registers)
+// Batched launches (the arguments in shared memory take registers): four blocks, but
+// three for the kernel with both limiters' code, which spills at four.
+constexpr int batched_blocks(bool med, bool pos) { return med && pos ? 3 : 4; }
 constexpr int kRing = 2;         // FP32: rows in each warp's shared-memory load ring
 constexpr int kWin = 72;         // FP32: columns of each plane copied per row (16-byte aligned window)
 constexpr int kWin16 = 80;       // 16-bit storage: the same window, 8-column aligned
@@ -147,7 +149,7 @@ __device__ __forceinline__ Sides sides(float a, float b, int lane)
 // single instance A0.
 // S: storage type of the deviations (float, __nv_bfloat16 or __half).
 template <typename S, bool MED, bool POS, bool BATCHED, bool ENS = false, bool ENT = false, bool EP = false>
-__global__ void __launch_bounds__(kThreads, ENT ? 3 : (BATCHED ? kBlocksPerSMBatched : kBlocksPerSM))
+__global__ void __launch_bounds__(kThreads, ENT ? 3 : (BATCHED ? batched_blocks(MED, POS) : kBlocksPerSM))
     k_fused(const FusedArgs A0, const FusedArgs *__restrict__ table, const int2 *__restrict__ map)
 {
     using O = F2;
@@ -968,7 +970,7 @@ cudaError_t launch_lim(const FusedArgs &A, int blocks, cudaStream_t s)
 int fused_slots(int elem_bytes, bool batched)
 {
     (void)elem_bytes;  // every storage type runs kBlocksPerSM blocks per SM
-    const int per_sm = batched ? kBlocksPerSMBatched : kBlocksPerSM;  // as in the launch bounds
+    const int per_sm = batched ? batched_blocks(true, false) : kBlocksPerSM;  // as in the launch bounds
     return per_sm * kWarps * sm_count();
 }
 
@@ -1095,14 +1097,18 @@ cudaError_t launch_fused_epass(const StepParams &p, const S *src, cudaStream_t s
 
 template cudaError_t launch_fused_epass<float>(const StepParams &, const float *, cudaStream_t);
 
-cudaError_t launch_fused_batched(const FusedArgs *table, const int2 *map, int items, int *work, cudaStream_t s)
+cudaError_t launch_fused_batched(const FusedArgs *table, const int2 *map, int items, int *work, bool med, bool pos,
+                                 cudaStream_t s)
 {
     if (items <= 0) return cudaSuccess;
     FusedArgs A0{};
     A0.items = items;
     A0.p.work = work;
-    const int blocks = std::min((items + kWarps - 1) / kWarps, fused_slots(4, true) / kWarps);
-    return launch_k<float, true, true, true>(A0, table, map, blocks, s);
+    const int blocks = std::min((items + kWarps - 1) / kWarps, batched_blocks(med, pos) * sm_count());
+    if (med && pos) return launch_k<float, true, true, true>(A0, table, map, blocks, s);
+    if (med) return launch_k<float, true, false, true>(A0, table, map, blocks, s);
+    if (pos) return launch_k<float, false, true, true>(A0, table, map, blocks, s);
+    return launch_k<float, false, false, true>(A0, table, map, blocks, s);
 }
 
 }  // namespace lbm
