@@ -22,9 +22,12 @@
 //     tube runs one site per lane (V = 1) and one warp per block, so its warps
 //     land on separate SM sub-partitions and the step lasts one site's chain;
 //   * FP32 storage with four sites a lane evaluates them as two pairs with the
-//     paired FP32 instructions and finishes a pair at once when no limiter
-//     acts on it; any other site is finished by an out-of-line function, so
-//     the walk's registers hold only what the common case needs.
+//     paired FP32 instructions.  A chunk of 128 sites on which no limiter acts
+//     is finished there; any other, and the two chunks with the tube's ends, go
+//     to an out-of-line function, so the walk's registers hold only what the
+//     common case needs.  The kernel is bound by its
+//     dependent chains at 16 warps an SM (1e7 sites: 67 -> 54 us in 323 instead of
+//     490 warp instructions a chunk; 24 warps at 80 registers spill: 62 us);
 // Ensemble-dependent limiters and 16-bit storage stay on the tiled kernel.
 #include <type_traits>
 
@@ -268,96 +271,241 @@ __device__ __forceinline__ double wsum(double v)
 constexpr int kTubeRing = 3;
 constexpr int kTubeWarps = 8;  // the most warps a block has
 constexpr int kTubeGroup = 8;  // chunks of a batched work item
-// The statistics a warp gathers: FP64 storage sums FP64 terms per lane; FP32
-// storage sums a chunk's FP32 terms per lane, adds the lanes in FP32 (a fixed
-// butterfly that leaves the four totals in lanes 0, 8, 16, 24) and the chunk
-// totals exactly, as 128-bit fixed point (integer instructions: FP64 adds per
-// chunk kept this GPU's FP64 units a third busy).
+constexpr int kTubeBlocks = 2;  // FP32 storage, four sites a lane: resident blocks per SM
+// The statistics a warp gathers.  FP64 storage sums FP64 terms per lane.  FP32
+// storage: each lane sums its FP32 terms over the whole walk with Kahan's
+// compensation (sums s - c; two interleaved chains of a paired instruction for
+// mass, dS and dS_in), no lane exchange and no conversion per chunk (FP64 adds
+// kept this GPU's FP64 units a third busy; a butterfly and a 128-bit addition a
+// chunk were 70 of its 490 instructions).
 struct TubeAcc {
     double t_mass, t_ds, t_in, t_lim;
+    float2 s_mass, c_mass, s_ds, c_ds, s_in, c_in;
+    float s_lim, c_lim;
     int c_pos, c_med, c_bad, c_own;
-    unsigned __int128 fx;  // FP32 storage: lane 0 mass, lane 8 dS, lane 16 dS_in, lane 24 dS_lim
-    bool fx_bad;
 };
 
-// FP32 storage: the four totals of acc (after the walk), in every lane.
-__device__ __forceinline__ void tube_totals(const TubeAcc &acc, double &mass, double &ds, double &din, double &lim)
+// One compensated addition (Kahan 1965): s - c += v.
+__device__ __forceinline__ void kahan2(float2 &s, float2 &c, float2 v)
 {
-    const double v = acc.fx_bad ? __longlong_as_double(0x7ff8000000000000LL) : fx_value(acc.fx);
-    mass = __shfl_sync(0xffffffffu, v, 0);
-    ds = __shfl_sync(0xffffffffu, v, 8);
-    din = __shfl_sync(0xffffffffu, v, 16);
-    lim = __shfl_sync(0xffffffffu, v, 24);
+    const float2 y = F2::sub(v, c), t = F2::add(s, y);
+    c = F2::sub(F2::sub(t, s), y);
+    s = t;
 }
 
-// a ring slot: the three planes of a chunk of 32 V sites, then f_2 left of it
-// and f_1 right of it
+// Sum of two unevaluated pairs (hi, lo): Knuth's two-sum of the high parts, the
+// low parts and the error renormalised.
+__device__ __forceinline__ float2 df_add(float2 a, float2 b)
+{
+    const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
+    float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
+    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
+    const float hi = __fadd_rn(s, e);
+    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+}
+
+// FP32 storage: the four totals of the warp's walk, in every lane: a butterfly over
+// the lanes' pairs (each of its first two levels halves the sums a lane carries:
+// lane 0 ends with mass, 8 dS, 16 dS_in, 24 dS_lim), then one conversion.  V = 1:
+// the walk is a single chunk, a site per lane, and plain FP32 additions add it.
+template <int V>
+__device__ __forceinline__ void tube_totals(const TubeAcc &acc, double &mass, double &ds, double &din, double &lim)
+{
+    constexpr unsigned kAll = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    auto add = [](float2 a, float2 b) { return V == 1 ? make_float2(__fadd_rn(a.x, b.x), 0.f) : df_add(a, b); };
+    auto both = [&](float2 s, float2 c) { return add(make_float2(s.x, -c.x), make_float2(s.y, -c.y)); };
+    auto swap = [](float2 v, int o) { return make_float2(__shfl_xor_sync(kAll, v.x, o), __shfl_xor_sync(kAll, v.y, o)); };
+    const float2 m = both(acc.s_mass, acc.c_mass), d = both(acc.s_ds, acc.c_ds), i = both(acc.s_in, acc.c_in);
+    const float2 l = make_float2(acc.s_lim, -acc.c_lim);
+    const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
+    const float2 x0 = add(hi16 ? i : m, swap(hi16 ? m : i, 16));
+    const float2 x1 = add(hi16 ? l : d, swap(hi16 ? d : l, 16));
+    float2 z = add(hi8 ? x1 : x0, swap(hi8 ? x0 : x1, 8));
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) z = add(z, swap(z, o));
+    const double v = (double)z.x + (double)z.y;
+    mass = __shfl_sync(kAll, v, 0);
+    ds = __shfl_sync(kAll, v, 8);
+    din = __shfl_sync(kAll, v, 16);
+    lim = __shfl_sync(kAll, v, 24);
+}
+
+// a ring slot: the three planes of a chunk of 32 V sites, f_1 with the site right of
+// the chunk after it, f_2 with the site left of it in front (padded to 16 bytes)
 template <typename S, int V>
 struct alignas(16) TubeSlot {
-    S f[3][32 * V];
-    S e[2];
+    static constexpr int kPad = 16 / (int)sizeof(S);
+    S f0[32 * V], f1[32 * V + kPad], f2[kPad + 32 * V];
 };
+
+// An Ehrenfests' candidate into the context's list.
+__device__ __forceinline__ void tube_record(const StepParams &p, int x, double key, double phi)
+{
+    const int slot = atomicAdd(p.cand_count, 1);
+    if (slot < p.cand_cap) {
+        Cand cd;
+        cd.key = key;
+        cd.site = x;
+        cd.phi = phi;
+        cd.ds32 = (float)key;
+        p.cand[slot] = cd;
+    } else {
+        atomicOr(p.status, kStatCandOverflow);
+    }
+}
+
+// The FP64 keys of a chunk's listed candidates (FP32 storage; the whole warp), a lane
+// each: a chunk holding many of them costs one FP64 evaluation per 32, not one per
+// site a lane carries.  Empties the list.
+__device__ __noinline__ void tube_keys(const StepParams &p, const float *__restrict__ src, int2 *klist, int *kcount)
+{
+    __syncwarp();
+    const int nk = *kcount;
+    for (int i = threadIdx.x & 31; i < nk; i += 32) {
+        const int2 e = klist[i];
+        double fin[3], fs[3], fp[3], ds, din, rho;
+        if (p.collide)
+            tube_pull<float, double>(p, src, e.x, fin);
+        else
+            tube_read<float, double>(p, src, e.x, fin);
+        const bool bad = site_collide<3, double>(fin, p.a, p.collide != 0, fs, fp, ds, din, rho, p.eq, false);
+        if (!bad && ds > p.delta_e) tube_record(p, e.x, ds, (double)__int_as_float(e.y));
+    }
+    __syncwarp();
+    if ((threadIdx.x & 31) == 0) *kcount = 0;
+    __syncwarp();
+}
+
+// A chunk that the paired path of tube_walk32 leaves (the whole warp; FP32 storage):
+// dS of every site, then each finished by tube_site32, then the keys of its
+// candidates.  Returns the lane's sums; the counts are four bits each (bad, pos, med).
+struct ChunkSums {
+    float mass, ds, din, lim;
+    unsigned counts;
+};
+template <int V>
+__device__ __noinline__ ChunkSums tube_chunk32(const StepParams &p, const TubeK kk, const float *__restrict__ src,
+                                               float *__restrict__ dst, int c, int2 *klist, int *kcount)
+{
+    using S = float;
+    const int lane = threadIdx.x & 31, nx = p.nx, xl = c * 32 * V + lane * V;
+    ChunkSums r{0.f, 0.f, 0.f, 0.f, 0u};
+    // the lane's pulls: whole vectors (the row's padding follows its last site), the
+    // neighbours' values, the tube's ends
+    float f0[V], f1[V], f2[V], ds[V];
+#pragma unroll
+    for (int j = 0; j < V; ++j) f0[j] = f1[j] = f2[j] = ds[j] = 0.f;
+    if (xl < nx) {
+        const float *const at = src + tidx(p, 0, xl);
+        float a0[V], a1[V + 1], a2[V + 1];
+        a1[V] = at[p.plane + V];
+        a2[0] = at[2 * p.plane - 1];
+        if constexpr (V == 4) {
+            const float4 v0 = *reinterpret_cast<const float4 *>(at);
+            const float4 v1 = *reinterpret_cast<const float4 *>(at + p.plane);
+            const float4 v2 = *reinterpret_cast<const float4 *>(at + 2 * p.plane);
+            a0[0] = v0.x, a0[1] = v0.y, a0[2] = v0.z, a0[3] = v0.w;
+            a1[0] = v1.x, a1[1] = v1.y, a1[2] = v1.z, a1[3] = v1.w;
+            a2[1] = v2.x, a2[2] = v2.y, a2[3] = v2.z, a2[4] = v2.w;
+        } else {
+#pragma unroll
+            for (int j = 0; j < V; ++j) {
+                a0[j] = at[j];
+                a1[j] = at[p.plane + j];
+                a2[j + 1] = at[2 * p.plane + j];
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < V; ++j) {
+            const int x = xl + j;
+            f0[j] = a0[j];
+            f1[j] = p.collide ? a1[j + 1] : a1[j];
+            f2[j] = p.collide ? a2[j] : a2[j + 1];
+            if (p.collide && x == nx - 1)  // right end: reflect or wrap
+                f1[j] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : a2[j + 1];
+            if (p.collide && x == 0)  // left end
+                f2[j] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : a1[j];
+        }
+    }
+    // dS of the lane's sites (the site's values are selected, not indexed: they stay in registers)
+    auto pick = [&](const float *v, int j) {
+        float w = v[0];
+#pragma unroll
+        for (int i = 1; i < V; ++i) w = i == j ? v[i] : w;
+        return w;
+    };
+#pragma unroll 1
+    for (int j = 0; j < V && xl + j < nx; ++j) {
+        const float f3[3] = {pick(f0, j), pick(f1, j), pick(f2, j)};
+        float fs3[3], fp3[3], fa3[3], nq3[3], d, din, rho;
+        tube_eval<float>(p, kk, f3, fs3, fp3, fa3, nq3, d, din, rho, false);
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (i == j) ds[i] = d;
+    }
+    __syncwarp();
+    // the median's neighbours: dS of the adjacent lanes' edge sites
+    const float dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
+    const float dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
+#pragma unroll 1
+    for (int j = 0; j < V && xl + j < nx; ++j) {
+        const int x = xl + j;
+        // the neighbours' dS, or the site to evaluate (outside the chunk)
+        const float dl = j > 0 ? pick(ds, j - 1) : dl_lane, dr = j + 1 < V ? pick(ds, j + 1) : dr_lane;
+        int xlo = -1, xro = -1;
+        if (x == 0)
+            xlo = nx - 1;
+        else if (j == 0 && lane == 0)
+            xlo = x - 1;
+        if (x == nx - 1)
+            xro = 0;
+        else if (j == V - 1 && lane == 31)
+            xro = x + 1;
+        const SiteSums q = tube_site32<S>(p, kk, src, dst, x, pick(f0, j), pick(f1, j), pick(f2, j), dl, dr, xlo, xro,
+                                          klist, kcount);
+        r.mass = __fadd_rn(r.mass, q.mass);
+        r.ds = __fadd_rn(r.ds, q.ds);
+        r.din = __fadd_rn(r.din, q.din);
+        r.lim = __fadd_rn(r.lim, q.lim);
+        r.counts += (unsigned)q.bad | (unsigned)q.pos << 4 | (unsigned)q.med << 8;
+    }
+    __syncwarp();
+    if (*kcount > 0) tube_keys(p, src, klist, kcount);
+    return r;
+}
 
 // One warp's walk over chunks c0, c0 + stride, ... (< c_end) of lattice p:
 // a1-a9 at every site, the Ehrenfests' candidates, the sums into acc.  `my`:
-// the warp's ring; klist / kcount: the warp's candidate list (FP32 storage).
-// Every lane of the warp takes part.
-template <typename S, int V, bool FAST = true>
-__device__ __forceinline__ void tube_walk(const StepParams &p, const S *__restrict__ src, S *__restrict__ dst,
-                                          int c0, int stride, int c_end, TubeSlot<S, V> *my, int2 *klist,
-                                          int *kcount, TubeAcc &acc)
+// the warp's ring.  Every lane of the warp takes part.  FP64 storage.
+template <int V>
+__device__ __forceinline__ void tube_walk64(const StepParams &p, const double *__restrict__ src,
+                                            double *__restrict__ dst, int c0, int stride, int c_end,
+                                            TubeSlot<double, V> *my, TubeAcc &acc)
 {
-    using T = compute_t<S>;
-    using A = Ar<T>;
+    using S = double;
+    using A = Ar<double>;
     using Slot = TubeSlot<S, V>;
-    constexpr bool F64 = std::is_same<T, double>::value;
-    constexpr int CW = 32 * V;  // sites of a chunk
-    const int lane = threadIdx.x & 31;
-    const int nx = p.nx;
-    TubeK kk{};
-    if constexpr (!F64) {
-        kk.a = (float)p.a;
-        kk.b2 = (float)(1.0 + p.a);
-        kk.dm = (float)p.delta_m;
-        kk.thr_e = (float)(p.delta_e * (1.0 - 1.0 / 64.0));
-    }
-    T dm;
-    if constexpr (F64)
-        dm = p.delta_m;
-    else
-        dm = kk.dm;
-
+    const int lane = threadIdx.x & 31, nx = p.nx;
+    const TubeK kk{};  // FP32 storage only
+    const bool lim_pos = (p.limiters & 1u) != 0, lim_ehr = (p.limiters & 2u) != 0, lim_med = (p.limiters & 4u) != 0;
     // copies of chunk c into slot `sl` (nothing past the last chunk; the group
     // is committed either way).  The chunk's window lies inside the padded row
     // (kTail zero elements follow the lattice), so whole vectors may be copied
     // past its end.
     auto issue = [&](int c, int sl) {
         if (c < c_end) {
-            const int x0 = c * CW, xl = x0 + lane * V;
+            const int x0 = c * 32 * V, xl = x0 + lane * V;
+            const S *const at = src + tidx(p, 0, xl);
             if (xl < nx) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k) tcopy<(int)sizeof(S) * V>(&my[sl].f[k][lane * V], src + tidx(p, k, xl));
+                tcopy<(int)sizeof(S) * V>(&my[sl].f0[lane * V], at);
+                tcopy<(int)sizeof(S) * V>(&my[sl].f1[lane * V], at + p.plane);
+                tcopy<(int)sizeof(S) * V>(&my[sl].f2[Slot::kPad + lane * V], at + 2 * p.plane);
             }
-            if (lane == 0 && x0 > 0) tcopy<(int)sizeof(S)>(&my[sl].e[0], src + tidx(p, 2, x0 - 1));
-            if (lane == 31 && xl + V < nx) tcopy<(int)sizeof(S)>(&my[sl].e[1], src + tidx(p, 1, xl + V));
+            if (lane == 0 && x0 > 0) tcopy<(int)sizeof(S)>(&my[sl].f2[Slot::kPad - 1], at + 2 * p.plane - 1);
+            if (lane == 31 && xl + V < nx) tcopy<(int)sizeof(S)>(&my[sl].f1[32 * V], at + p.plane + V);
         }
         tcommit();
-    };
-
-
-    // an Ehrenfests' candidate into the context's list
-    auto record = [&](int x, double key, double phi) {
-        const int slot = atomicAdd(p.cand_count, 1);
-        if (slot < p.cand_cap) {
-            Cand cd;
-            cd.key = key;
-            cd.site = x;
-            cd.phi = phi;
-            cd.ds32 = (float)key;
-            p.cand[slot] = cd;
-        } else {
-            atomicOr(p.status, kStatCandOverflow);
-        }
     };
 #pragma unroll
     for (int i = 0; i < kTubeRing - 1; ++i) issue(c0 + i * stride, i);
@@ -369,353 +517,254 @@ __device__ __forceinline__ void tube_walk(const StepParams &p, const S *__restri
         __syncwarp();                                                   // and so have the other lanes'
         const Slot &sl = my[get];
         get = get + 1 == kTubeRing ? 0 : get + 1;
-        const int x0 = c * CW, xl = x0 + lane * V;
-        S v0[V], v1[V], v2[V];
+        const int xl = c * 32 * V + lane * V;
+        const S r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
+        double ds[V], fin[V][3], fs[V][3], fp[V][3], dsin[V], rho[V];
+        double s_mass = 0.0, s_ds = 0.0, s_in = 0.0, s_lim = 0.0;
+        bool bad[V];
 #pragma unroll
         for (int j = 0; j < V; ++j) {
-            v0[j] = sl.f[0][lane * V + j];
-            v1[j] = sl.f[1][lane * V + j];
-            v2[j] = sl.f[2][lane * V + j];
-        }
-        // f_1 of the site right of the lane's last site, f_2 left of its first
-        // (the next lane's first and the previous lane's last, or the slot's edges)
-        const S r1 = lane == 31 ? sl.e[1] : sl.f[1][lane * V + V];
-        const S l2 = lane == 0 ? sl.e[0] : sl.f[2][lane * V - 1];
-
-        // the lane's pull of its site j (free flight with the tube's ends, or
-        // the stored values of a limiter pass)
-        auto build_fin = [&](int j, T f3[3]) {
-            const int x = xl + j;
+            const int x = xl + j, i = lane * V + j;
+            ds[j] = 0.0;
+            dsin[j] = 0.0;
+            rho[j] = 0.0;
+            bad[j] = false;
+            if (x >= nx) continue;
+            fin[j][0] = sl.f0[i];
             if (p.collide) {
-                f3[0] = tload<S, T>(p, v0[j], 0);
-                f3[1] = tload<S, T>(p, j + 1 < V ? v1[j + 1] : r1, 1);
-                f3[2] = tload<S, T>(p, j > 0 ? v2[j - 1] : l2, 2);
+                fin[j][1] = j + 1 < V ? sl.f1[i + 1] : r1;
+                fin[j][2] = j > 0 ? sl.f2[Slot::kPad + i - 1] : l2;
                 if (x == nx - 1)  // right end: reflect or wrap
-                    f3[1] = bc_wrap_x(p.boundary) ? tload<S, T>(p, src[tidx(p, 1, 0)], 1) : tload<S, T>(p, v2[j], 2);
+                    fin[j][1] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : sl.f2[Slot::kPad + i];
                 if (x == 0)  // left end
-                    f3[2] = bc_wrap_x(p.boundary) ? tload<S, T>(p, src[tidx(p, 2, nx - 1)], 2) : tload<S, T>(p, v1[j], 1);
+                    fin[j][2] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : sl.f1[i];
             } else {
-                f3[0] = tload<S, T>(p, v0[j], 0);
-                f3[1] = tload<S, T>(p, v1[j], 1);
-                f3[2] = tload<S, T>(p, v2[j], 2);
+                fin[j][1] = sl.f1[i];
+                fin[j][2] = sl.f2[Slot::kPad + i];
             }
-        };
-        T ds[V];
-        T s_mass = T(0), s_ds = T(0), s_in = T(0), s_lim = T(0);
-        if constexpr (!F64 && FAST) {
-            // FP32: a lane inside the tube in a colliding polynomial pass (four sites
-            // a lane) evaluates its sites as two pairs (0, 1), (2, 3) with paired
-            // instructions, and a pair on which no limiter acts (no bad site, no
-            // negative f', no dS above the median filter's delta) is finished here.
-            // Every other site keeps only its dS until the neighbours' dS are known
-            // and is then finished one at a time by tube_site32.
-            bool fastp[2] = {false, false}, paired = false;
-            if constexpr (V == 4) {
-                paired = p.collide && p.eq == 0 && xl >= 1 && xl + V <= nx - 1;
-                if (paired) {
-                    // the finished pairs' sums, added pairwise (paired instructions)
-                    float2 m2 = F2::s(0.f), d2s = F2::s(0.f), i2s = F2::s(0.f), dmax = F2::s(0.f);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const float2 g[3] = {make_float2(v0[2 * h], v0[2 * h + 1]),
-                                             make_float2(v1[2 * h + 1], h == 0 ? v1[2] : r1),
-                                             make_float2(h == 0 ? l2 : v2[1], v2[2 * h])};
-                        float2 gp[3], d2, i2, r2;
-                        bool bx, by;
-                        tube_pair_eval(kk, p.rho_ref, p.rwf, g, gp, d2, i2, r2, bx, by);
-                        bool act = bx || by;
-                        if (p.limiters & 1u) {
-#pragma unroll
-                            for (int k = 0; k < 3; ++k)
-                                act = act || (p.rwf[k] + gp[k].x < 0.f) || (p.rwf[k] + gp[k].y < 0.f);
-                        }
-                        if (p.limiters & 4u) act = act || d2.x > dm || d2.y > dm;
-                        // a site that cannot be limited has dS = +inf (as tube_eval gives it)
-                        ds[2 * h] = bx ? T(INFINITY) : d2.x;
-                        ds[2 * h + 1] = by ? T(INFINITY) : d2.y;
-                        if (act) continue;
-                        // f' stored as one 8-byte vector a plane (xl + 2h is even)
-                        fastp[h] = true;
-                        const int x = xl + 2 * h;
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) *reinterpret_cast<float2 *>(dst + tidx(p, k, x)) = gp[k];
-                        m2 = F2::add(m2, F2::sub(r2, F2::s(p.rho_ref)));  // each term exact
-                        d2s = F2::add(d2s, d2);
-                        i2s = F2::add(i2s, i2);
-                        dmax = make_float2(fmaxf(dmax.x, d2.x), fmaxf(dmax.y, d2.y));
-                    }
-                    if (fastp[0] || fastp[1]) {
-                        s_mass = __fadd_rn(m2.x, m2.y);
-                        s_ds = __fadd_rn(d2s.x, d2s.y);
-                        s_in = __fadd_rn(i2s.x, i2s.y);
-                        acc.c_own += 2 * ((int)fastp[0] + (int)fastp[1]);
-                        // Ehrenfests' candidates among the finished sites (rare: one
-                        // test a lane), and the dS field when it is asked for
-                        if ((p.limiters & 2u) && fmaxf(dmax.x, dmax.y) > kk.thr_e) {
-#pragma unroll
-                            for (int j = 0; j < V; ++j)
-                                if (fastp[j >> 1] && ds[j] > kk.thr_e)
-                                    klist[atomicAdd(kcount, 1)] = make_int2(xl + j, __float_as_int(1.f));
-                        }
-                        if (p.ds_out) {
-#pragma unroll
-                            for (int j = 0; j < V; ++j)
-                                if (fastp[j >> 1]) p.ds_out[xl + j] = (double)ds[j];
-                        }
-                    }
-                }
-            }
-            if (!paired) {
-#pragma unroll
-                for (int j = 0; j < V; ++j) {
-                    ds[j] = T(0);
-                    if (xl + j >= nx) continue;
-                    float f3[3], fs3[3], fp3[3], fa3[3], nq3[3], din, r;
-                    build_fin(j, f3);
-                    tube_eval<float>(p, kk, f3, fs3, fp3, fa3, nq3, ds[j], din, r, false);
-                }
-            }
-            // the median's neighbours: dS of the adjacent lanes' edge sites
-            const T dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
-            const T dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
-#pragma unroll
-            for (int j = 0; j < V; ++j) {
-                const int x = xl + j;
-                if (fastp[j >> 1] || x >= nx) continue;
-                float f3[3];
-                build_fin(j, f3);
-                // the neighbours' dS, or the site to evaluate (outside the chunk)
-                int xlo = -1, xro = -1;
-                float dl = 0.f, dr = 0.f;
-                if (x == 0)
-                    xlo = nx - 1;
-                else if (j > 0)
-                    dl = ds[j - 1];
-                else if (lane > 0)
-                    dl = dl_lane;
-                else
-                    xlo = x - 1;
-                if (x == nx - 1)
-                    xro = 0;
-                else if (j + 1 < V)
-                    dr = ds[j + 1];
-                else if (lane < 31)
-                    dr = dr_lane;
-                else
-                    xro = x + 1;
-                const SiteSums r =
-                    tube_site32<S>(p, kk, src, dst, x, f3[0], f3[1], f3[2], dl, dr, xlo, xro, klist, kcount);
-                s_lim = __fadd_rn(s_lim, r.lim);
-                s_mass = __fadd_rn(s_mass, r.mass);
-                s_ds = __fadd_rn(s_ds, r.ds);
-                s_in = __fadd_rn(s_in, r.din);
-                acc.c_own += 1;
-                acc.c_bad += r.bad;
-                acc.c_pos += r.pos;
-                acc.c_med += r.med;
-            }
-        } else {
-            T fin[V][3], fs[V][3], fp[V][3], fa[V][3], dsin[V], rho[V];
-            float nq[V][3];
-            bool bad[V];
-#pragma unroll
-            for (int j = 0; j < V; ++j) {
-                const int x = xl + j;
-                ds[j] = T(0);
-                dsin[j] = T(0);
-                rho[j] = T(0);
-                bad[j] = false;
-                if (x >= nx) continue;
-                if (p.collide) {
-                    fin[j][0] = tload<S, T>(p, v0[j], 0);
-                    fin[j][1] = tload<S, T>(p, j + 1 < V ? v1[j + 1] : r1, 1);
-                    fin[j][2] = tload<S, T>(p, j > 0 ? v2[j - 1] : l2, 2);
-                    if (x == nx - 1)  // right end: reflect or wrap
-                        fin[j][1] = bc_wrap_x(p.boundary) ? tload<S, T>(p, src[tidx(p, 1, 0)], 1) : tload<S, T>(p, v2[j], 2);
-                    if (x == 0)  // left end
-                        fin[j][2] =
-                            bc_wrap_x(p.boundary) ? tload<S, T>(p, src[tidx(p, 2, nx - 1)], 2) : tload<S, T>(p, v1[j], 1);
-                } else {
-                    fin[j][0] = tload<S, T>(p, v0[j], 0);
-                    fin[j][1] = tload<S, T>(p, v1[j], 1);
-                    fin[j][2] = tload<S, T>(p, v2[j], 2);
-                }
-                bad[j] = tube_eval<T>(p, kk, fin[j], fs[j], fp[j], fa[j], nq[j], ds[j], dsin[j], rho[j], true);
-            }
+            bad[j] = site_collide<3, double>(fin[j], p.a, p.collide != 0, fs[j], fp[j], ds[j], dsin[j], rho[j],
+                                             p.eq, true, p.coll, p.beta);
+            if (bad[j]) ds[j] = INFINITY;
+        }
 
-            // the median's neighbours: dS of the adjacent lanes' edge sites
-            const T dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
-            const T dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
+        // the median's neighbours: dS of the adjacent lanes' edge sites
+        const double dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
+        const double dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
 
 #pragma unroll
-            for (int j = 0; j < V; ++j) {
-                const int x = xl + j;
-                if (x >= nx) continue;
-                ++acc.c_own;
-                T phi_pos = T(1), phi_med = T(1);
-                if (!bad[j]) {
-                    if (p.limiters & 1u) {
-                        if constexpr (F64) {
-                            phi_pos = phi_positivity<3, T>(fs[j], fp[j]);
-                        } else {
-#pragma unroll
-                            for (int k = 0; k < 3; ++k) {
-                                const float fpa = p.rwf[k] + fp[j][k];  // absolute f'
-                                if (fpa < 0.f) phi_pos = fminf(phi_pos, fa[j][k] / (fa[j][k] - fpa));
-                            }
-                        }
-                    }
-                    // three-point median (the two end sites of a closed tube are not
-                    // filtered; a periodic tube's end sites wrap around to each other)
-                    const bool end = p.boundary == 0 && (x == 0 || x == nx - 1);
-                    if ((p.limiters & 4u) && ds[j] > dm && !end) {
-                        T left, right;
-                        if (x == 0)
-                            left = tube_ds<S>(p, kk, src, nx - 1);
-                        else if (j > 0)
-                            left = ds[j - 1];
-                        else if (lane > 0)
-                            left = dl_lane;
-                        else
-                            left = tube_ds<S>(p, kk, src, x - 1);
-                        if (x == nx - 1)
-                            right = tube_ds<S>(p, kk, src, 0);
-                        else if (j + 1 < V)
-                            right = ds[j + 1];
-                        else if (lane < 31)
-                            right = dr_lane;
-                        else
-                            right = tube_ds<S>(p, kk, src, x + 1);
-                        const T med = med3(left, ds[j], right);
-                        if constexpr (F64) {
-                            phi_med = (p.phi_rule == 1 && p.eq == 1)
-                                          ? phi_median_entropy<3>(fp[j], fs[j], ds[j], med, dm, p.median_mode)
-                                          : phi_median<T>(ds[j], med, dm, p.median_mode);
-                        } else {
-                            phi_med = phi_median<T>(ds[j], med, dm, p.median_mode);
-                        }
-                    }
+        for (int j = 0; j < V; ++j) {
+            const int x = xl + j;
+            if (x >= nx) continue;
+            ++acc.c_own;
+            double phi_pos = 1.0, phi_med = 1.0;
+            if (!bad[j]) {
+                if (lim_pos) phi_pos = phi_positivity<3, double>(fs[j], fp[j]);
+                // three-point median (the two end sites of a closed tube are not
+                // filtered; a periodic tube's end sites wrap around to each other)
+                const bool end = p.boundary == 0 && (x == 0 || x == nx - 1);
+                if (lim_med && ds[j] > p.delta_m && !end) {
+                    double left, right;
+                    if (x == 0)
+                        left = tube_ds<S>(p, kk, src, nx - 1);
+                    else if (j > 0)
+                        left = ds[j - 1];
+                    else if (lane > 0)
+                        left = dl_lane;
+                    else
+                        left = tube_ds<S>(p, kk, src, x - 1);
+                    if (x == nx - 1)
+                        right = tube_ds<S>(p, kk, src, 0);
+                    else if (j + 1 < V)
+                        right = ds[j + 1];
+                    else if (lane < 31)
+                        right = dr_lane;
+                    else
+                        right = tube_ds<S>(p, kk, src, x + 1);
+                    const double med = med3(left, ds[j], right);
+                    phi_med = (p.phi_rule == 1 && p.eq == 1)
+                                  ? phi_median_entropy<3>(fp[j], fs[j], ds[j], med, p.delta_m, p.median_mode)
+                                  : phi_median<double>(ds[j], med, p.delta_m, p.median_mode);
                 }
-                const T phi = phi_pos < phi_med ? phi_pos : phi_med;
-                T lim = T(0);
-                if (phi < T(1)) {
-                    if constexpr (F64) {
-                        double fo[3];
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) {
-                            fo[k] = A::add(fs[j][k], A::mul(phi, A::sub(fp[j][k], fs[j][k])));
-                            dst[tidx(p, k, x)] = fo[k];
-                        }
-                        if (p.eq == 1) {
-                            const double dout = rel_entropy<3>(fo, fs[j]);
-                            if (isfinite(ds[j]) && isfinite(dout)) lim = A::sub(ds[j], dout);
-                        } else {
-                            lim = A::mul(A::sub(1.0, A::mul(phi, phi)), ds[j]);
-                        }
-                    } else {
-                        const float cw = limit_weight(phi, kk.a, p.collide != 0);
-#pragma unroll
-                        for (int k = 0; k < 3; ++k) dst[tidx(p, k, x)] = fmaf(-cw, nq[j][k], fin[j][k]);
-                        if (p.eq == 1) {
-                            float dout[3];
-                            const float m = p.collide ? __fmul_rn(-phi, kk.a) : phi;
-#pragma unroll
-                            for (int k = 0; k < 3; ++k) dout[k] = __fmul_rn(m, nq[j][k]);
-                            const float so = rel_entropy_dev<3>(dout, fa[j]);
-                            if (isfinite(ds[j]) && isfinite(so)) lim = __fsub_rn(ds[j], so);
-                        } else {
-                            lim = __fmul_rn(__fsub_rn(1.f, __fmul_rn(phi, phi)), ds[j]);
-                        }
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) dst[tidx(p, k, x)] = f2s<S>(fp[j][k]);
-                }
-                s_lim = A::add(s_lim, lim);
-                if constexpr (F64)
-                    s_mass = A::add(s_mass, rho[j]);
-                else
-                    s_mass = __fadd_rn(s_mass, __fsub_rn(rho[j], p.rho_ref));  // each term exact
-                if (!bad[j]) {
-                    T tds = T(0), tin = T(0);
-                    if (p.eq == 1) {
-                        if (isfinite(ds[j])) tds = ds[j];
-                        if (isfinite(ds[j]) && isfinite(dsin[j])) tin = A::sub(dsin[j], ds[j]);
-                    } else {
-                        tds = ds[j];
-                        tin = dsin[j];
-                    }
-                    s_ds = A::add(s_ds, tds);
-                    s_in = A::add(s_in, tin);
-                } else {
-                    ++acc.c_bad;
-                    atomicOr(p.status, kStatNonfinite);
-                }
-                acc.c_pos += phi_pos < T(1);
-                acc.c_med += phi_med < T(1);
-                if ((p.limiters & 2u) && !bad[j]) {
-                    // Ehrenfests' candidates on an FP64 dS(f').  FP64 storage: ds itself.
-                    // FP32 storage: sites near and above the threshold go to the warp's list
-                    // and are keyed after the chunk, a lane each (below)
-                    if constexpr (F64) {
-                        if (ds[j] > p.delta_e) record(x, ds[j], (double)phi);
-                    } else {
-                        if (ds[j] > kk.thr_e) klist[atomicAdd(kcount, 1)] = make_int2(x, __float_as_int(phi));
-                    }
-                }
-                if (p.ds_out) p.ds_out[x] = (double)ds[j];
             }
-        }
-        if constexpr (!F64) {
-            __syncwarp();
-            const int nk = *kcount;
-            for (int i = lane; i < nk; i += 32) {
-                const int2 e = klist[i];
-                double fin64[3], fs64[3], fp64[3], d64, din64, r64;
-                if (p.collide)
-                    tube_pull<S, double>(p, src, e.x, fin64);
-                else
-                    tube_read<S, double>(p, src, e.x, fin64);
-                const bool b64 =
-                    site_collide<3, double>(fin64, p.a, p.collide != 0, fs64, fp64, d64, din64, r64, p.eq, false);
-                if (!b64 && d64 > p.delta_e) record(e.x, d64, (double)__int_as_float(e.y));
-            }
-            __syncwarp();
-            if (lane == 0) *kcount = 0;
-            __syncwarp();
-        }
-        if constexpr (F64) {
-            acc.t_mass = A::add(acc.t_mass, s_mass);
-            acc.t_ds = A::add(acc.t_ds, s_ds);
-            acc.t_in = A::add(acc.t_in, s_in);
-            acc.t_lim = A::add(acc.t_lim, s_lim);
-        } else {
-            // butterfly: each level halves the sums a lane carries
-            const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
-            float x0 = hi16 ? s_in : s_mass, x1 = hi16 ? s_lim : s_ds;
-            const float y0 = hi16 ? s_mass : s_in, y1 = hi16 ? s_ds : s_lim;
-            x0 = __fadd_rn(x0, __shfl_xor_sync(0xffffffffu, y0, 16));
-            x1 = __fadd_rn(x1, __shfl_xor_sync(0xffffffffu, y1, 16));
-            float z = hi8 ? x1 : x0;
-            z = __fadd_rn(z, __shfl_xor_sync(0xffffffffu, hi8 ? x0 : x1, 8));
+            const double phi = phi_pos < phi_med ? phi_pos : phi_med;
+            double lim = 0.0;
+            if (phi < 1.0) {
+                double fo[3];
 #pragma unroll
-            for (int o = 4; o > 0; o >>= 1) z = __fadd_rn(z, __shfl_xor_sync(0xffffffffu, z, o));
-            if ((lane & 7) == 0) fx_add(acc.fx, z, acc.fx_bad);
+                for (int k = 0; k < 3; ++k) {
+                    fo[k] = A::add(fs[j][k], A::mul(phi, A::sub(fp[j][k], fs[j][k])));
+                    dst[tidx(p, k, x)] = fo[k];
+                }
+                if (p.eq == 1) {
+                    const double dout = rel_entropy<3>(fo, fs[j]);
+                    if (isfinite(ds[j]) && isfinite(dout)) lim = A::sub(ds[j], dout);
+                } else {
+                    lim = A::mul(A::sub(1.0, A::mul(phi, phi)), ds[j]);
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 3; ++k) dst[tidx(p, k, x)] = fp[j][k];
+            }
+            s_lim = A::add(s_lim, lim);
+            s_mass = A::add(s_mass, rho[j]);
+            if (!bad[j]) {
+                double tds = 0.0, tin = 0.0;
+                if (p.eq == 1) {
+                    if (isfinite(ds[j])) tds = ds[j];
+                    if (isfinite(ds[j]) && isfinite(dsin[j])) tin = A::sub(dsin[j], ds[j]);
+                } else {
+                    tds = ds[j];
+                    tin = dsin[j];
+                }
+                s_ds = A::add(s_ds, tds);
+                s_in = A::add(s_in, tin);
+            } else {
+                ++acc.c_bad;
+                atomicOr(p.status, kStatNonfinite);
+            }
+            acc.c_pos += phi_pos < 1.0;
+            acc.c_med += phi_med < 1.0;
+            // Ehrenfests' candidates on dS(f') itself
+            if (lim_ehr && !bad[j] && ds[j] > p.delta_e) tube_record(p, x, ds[j], phi);
+            if (p.ds_out) p.ds_out[x] = ds[j];
         }
+        acc.t_mass = A::add(acc.t_mass, s_mass);
+        acc.t_ds = A::add(acc.t_ds, s_ds);
+        acc.t_in = A::add(acc.t_in, s_in);
+        acc.t_lim = A::add(acc.t_lim, s_lim);
     }
     twait<0>();
 }
 
+// FP32 storage: the chunks c0, c0 + stride, ... (< c_end, none with an end of the
+// tube), after those of `ends` (bit 0: chunk 0, bit 1: the last).  klist / kcount: the
+// warp's candidate list.  An entropic or limiter pass, or one site a lane, leaves every
+// chunk to tube_chunk32.
+template <int V>
+__device__ __forceinline__ void tube_walk32(const StepParams &p, const float *__restrict__ src,
+                                            float *__restrict__ dst, int c0, int stride, int c_end, unsigned ends,
+                                            TubeSlot<float, V> *my, int2 *klist, int *kcount, TubeAcc &acc)
+{
+    using S = float;
+    using Slot = TubeSlot<S, V>;
+    constexpr int CW = 32 * V;  // sites of a chunk
+    const int lane = threadIdx.x & 31, nx = p.nx;
+    TubeK kk;
+    kk.a = (float)p.a;
+    kk.b2 = (float)(1.0 + p.a);
+    kk.dm = (float)p.delta_m;
+    kk.thr_e = (float)(p.delta_e * (1.0 - 1.0 / 64.0));
+    auto leave = [&](int c) {
+        const ChunkSums r = tube_chunk32<V>(p, kk, src, dst, c, klist, kcount);
+        kahan2(acc.s_mass, acc.c_mass, make_float2(r.mass, 0.f));
+        kahan2(acc.s_ds, acc.c_ds, make_float2(r.ds, 0.f));
+        kahan2(acc.s_in, acc.c_in, make_float2(r.din, 0.f));
+        const float y = __fsub_rn(r.lim, acc.c_lim), t = __fadd_rn(acc.s_lim, y);
+        acc.c_lim = __fsub_rn(__fsub_rn(t, acc.s_lim), y);
+        acc.s_lim = t;
+        acc.c_bad += (int)(r.counts & 15u);
+        acc.c_pos += (int)(r.counts >> 4 & 15u);
+        acc.c_med += (int)(r.counts >> 8 & 15u);
+        acc.c_own += max(0, min(V, nx - c * CW - lane * V));
+    };
+    const bool paired = V == 4 && p.collide && p.eq == 0 && !p.ds_out;
+    // the ends first (their code is cold: an instruction fetch costs about 10 ns), then,
+    // when nothing is paired, the rest
+    for (int c = c0; ends || (!paired && c < c_end);) {
+        const bool end = ends != 0;
+        leave(!end ? c : (ends & 1u ? 0 : (nx - 1) / CW));
+        if (end)
+            ends &= ends - 1u;
+        else
+            c += stride;
+    }
+    if (!paired) return;
+    if constexpr (V == 4) {
+        // the flags and constants in registers (the batched kernel's lie in shared memory)
+        const bool lim_pos = (p.limiters & 1u) != 0;
+        const float rho_ref = p.rho_ref, rwf[3] = {p.rwf[0], p.rwf[1], p.rwf[2]};
+        const float d_act = (p.limiters & 4u) ? kk.dm : INFINITY, d_cand = (p.limiters & 2u) ? kk.thr_e : INFINITY;
+        const long long plane = p.plane;
+        const float *const from = src + tidx(p, 0, lane * V);
+        float *const to = dst + tidx(p, 0, lane * V);
+        // copies of chunk c into slot `sl` (nothing past the last chunk; the group is
+        // committed either way)
+        auto issue = [&](int c, int sl) {
+            if (c < c_end) {
+                const float *const at = from + (long long)c * CW;
+                tcopy<16>(&my[sl].f0[lane * V], at);
+                tcopy<16>(&my[sl].f1[lane * V], at + plane);
+                tcopy<16>(&my[sl].f2[Slot::kPad + lane * V], at + 2 * plane);
+                if (lane == 0) tcopy<4>(&my[sl].f2[Slot::kPad - 1], at + 2 * plane - 1);
+                if (lane == 31) tcopy<4>(&my[sl].f1[CW], at + plane + V);
+            }
+            tcommit();
+        };
+#pragma unroll
+        for (int i = 0; i < kTubeRing - 1; ++i) issue(c0 + i * stride, i);
+        int get = 0;
+        for (int c = c0; c < c_end; c += stride) {
+            __syncwarp();  // every lane is done with the slot refilled now
+            issue(c + (kTubeRing - 1) * stride, get == 0 ? kTubeRing - 1 : get - 1);
+            twait<kTubeRing - 1>();  // this lane's copies of chunk c have landed
+            __syncwarp();            // and so have the other lanes'
+            const Slot &sl = my[get];
+            get = get + 1 == kTubeRing ? 0 : get + 1;
+            const float4 f0 = *reinterpret_cast<const float4 *>(&sl.f0[lane * V]);
+            const float4 f1 = *reinterpret_cast<const float4 *>(&sl.f1[lane * V]);
+            const float4 f2 = *reinterpret_cast<const float4 *>(&sl.f2[Slot::kPad + lane * V]);
+            const float r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
+            const float2 ga[3] = {make_float2(f0.x, f0.y), make_float2(f1.y, f1.z), make_float2(l2, f2.x)};
+            const float2 gb[3] = {make_float2(f0.z, f0.w), make_float2(f1.w, r1), make_float2(f2.y, f2.z)};
+            float2 pa[3], pb[3], da, db, ia, ib, ra, rb;
+            bool ba, bb, bc, bd;
+            tube_pair_eval(kk, rho_ref, rwf, ga, pa, da, ia, ra, ba, bb);
+            tube_pair_eval(kk, rho_ref, rwf, gb, pb, db, ib, rb, bc, bd);
+            // does a limiter act: a bad site, dS above the median filter's delta, a
+            // negative f' of the positivity rule?
+            const float dmax = fmaxf(fmaxf(da.x, da.y), fmaxf(db.x, db.y));
+            bool act = ba || bb || bc || bd || dmax > d_act;
+            if (lim_pos) {
+#pragma unroll
+                for (int k = 0; k < 3; ++k)
+                    act = act || rwf[k] + fminf(fminf(pa[k].x, pb[k].x), fminf(pa[k].y, pb[k].y)) < 0.f;
+            }
+            if (__any_sync(0xffffffffu, act)) {
+                leave(c);
+                continue;
+            }
+            float *const at = to + (long long)c * CW;
+#pragma unroll
+            for (int k = 0; k < 3; ++k)
+                *reinterpret_cast<float4 *>(at + k * plane) = make_float4(pa[k].x, pa[k].y, pb[k].x, pb[k].y);
+            const float2 ma = F2::sub(ra, F2::s(rho_ref)), mb = F2::sub(rb, F2::s(rho_ref));  // exact
+            kahan2(acc.s_mass, acc.c_mass, F2::add(ma, mb));
+            kahan2(acc.s_ds, acc.c_ds, F2::add(da, db));
+            kahan2(acc.s_in, acc.c_in, F2::add(ia, ib));
+            acc.c_own += V;
+            // Ehrenfests' candidates: sites near or above the threshold (rare)
+            if (__any_sync(0xffffffffu, dmax > d_cand)) {
+                const float d4[4] = {da.x, da.y, db.x, db.y};
+#pragma unroll
+                for (int j = 0; j < V; ++j)
+                    if (d4[j] > d_cand)
+                        klist[atomicAdd(kcount, 1)] = make_int2(c * CW + lane * V + j, __float_as_int(1.f));
+                tube_keys(p, src, klist, kcount);
+            }
+        }
+        twait<0>();
+    }
+}
+
 template <typename S, int V>
-__global__ void __launch_bounds__(256, V > 1 ? 2 : 1)
+__global__ void __launch_bounds__(256, V == 4 ? kTubeBlocks : (V > 1 ? 2 : 1))
     k_tube(const __grid_constant__ StepParams p, const S *__restrict__ src, S *__restrict__ dst, int chunked)
 {
     constexpr bool F64 = std::is_same<compute_t<S>, double>::value;
-    __shared__ TubeSlot<S, V> ring[kTubeWarps][kTubeRing];
-    // FP32 storage: the chunk's sites whose FP32 dS(f') lies near or above the
-    // threshold (site, phi), keyed in FP64 after the chunk with one lane each:
-    // a chunk holding many of them costs one FP64 evaluation per 32, not one per
-    // site a lane carries
+    constexpr bool RING = F64 || V == 4;
+    __shared__ TubeSlot<S, V> ring[RING ? kTubeWarps : 1][RING ? kTubeRing : 1];
+    // FP32 storage: the chunk's sites whose FP32 dS(f') lies near or above the threshold
+    // (site, phi)
     __shared__ int2 klist[kTubeWarps][F64 ? 1 : 32 * V];
     __shared__ int kcount[kTubeWarps];
     // the tail of the previous pass may still run (programmatic launch)
@@ -725,14 +774,21 @@ __global__ void __launch_bounds__(256, V > 1 ? 2 : 1)
     if (lane == 0) kcount[warp] = 0;
     __syncwarp();
     TubeAcc acc{};
-    tube_walk<S, V>(p, src, dst, blockIdx.x * nw + warp, (int)gridDim.x * nw, (p.nx + 32 * V - 1) / (32 * V),
-                    ring[warp], klist[warp], &kcount[warp], acc);
+    const int w = blockIdx.x * nw + warp, stride = (int)gridDim.x * nw, chunks = (p.nx + 32 * V - 1) / (32 * V);
+    if constexpr (F64) {
+        tube_walk64<V>(p, src, dst, w, stride, chunks, ring[warp], acc);
+    } else {
+        // the two chunks with the tube's ends to the last warps, which have fewer others
+        const unsigned ends = (chunks > 1 && w == max(stride - 2, 0) ? 1u : 0u) | (w == stride - 1 ? 2u : 0u);
+        tube_walk32<V>(p, src, dst, 1 + w, stride, chunks - 1, ends, RING ? ring[warp] : ring[0], klist[warp],
+                       &kcount[warp], acc);
+    }
     double t_mass = acc.t_mass, t_ds = acc.t_ds, t_in = acc.t_in, t_lim = acc.t_lim;
-    if constexpr (!F64) tube_totals(acc, t_mass, t_ds, t_in, t_lim);
+    if constexpr (!F64) tube_totals<V>(acc, t_mass, t_ds, t_in, t_lim);
     int c_pos = acc.c_pos, c_med = acc.c_med, c_bad = acc.c_bad, c_own = acc.c_own;
 
     // block partial row: warp sums, then the warps in order; counts as integers
-    __shared__ double sred[8][P_NSTAT];
+    __shared__ double sred[kTubeWarps][P_NSTAT];
     if constexpr (F64) {
         t_mass = wsum(t_mass);
         t_ds = wsum(t_ds);
@@ -792,7 +848,7 @@ __global__ void __launch_bounds__(256, V > 1 ? 2 : 1)
 // writes each item's sums into the tube's partial row of that group (a fixed
 // evaluation order per item, so the sums do not depend on which warp ran it).
 template <int V>
-__global__ void __launch_bounds__(256, 2) k_tube_batched(const TubeArgs *__restrict__ table,
+__global__ void __launch_bounds__(256, kTubeBlocks) k_tube_batched(const TubeArgs *__restrict__ table,
                                                          const int2 *__restrict__ map, int items, int *work)
 {
     using S = float;
@@ -819,11 +875,12 @@ __global__ void __launch_bounds__(256, 2) k_tube_batched(const TubeArgs *__restr
         const int nch = (p.nx + 32 * V - 1) / (32 * V);
         const int c0 = m.y * kTubeGroup, c1 = min(c0 + kTubeGroup, nch);
         TubeAcc acc{};
-        tube_walk<S, V, false>(p, (const S *)sA[warp].src, (S *)sA[warp].dst, c0, 1, c1, ring[warp], klist[warp],
-                               &kcount[warp], acc);
+        const unsigned ends = (c0 == 0 && nch > 1 ? 1u : 0u) | (c1 == nch ? 2u : 0u);
+        tube_walk32<V>(p, (const S *)sA[warp].src, (S *)sA[warp].dst, max(c0, 1), 1, min(c1, nch - 1), ends,
+                       ring[warp], klist[warp], &kcount[warp], acc);
         // the item's totals; the counts are per lane
         double t_mass, t_ds, t_in, t_lim;
-        tube_totals(acc, t_mass, t_ds, t_in, t_lim);
+        tube_totals<V>(acc, t_mass, t_ds, t_in, t_lim);
         const int c_pos = __reduce_add_sync(0xffffffffu, acc.c_pos), c_med = __reduce_add_sync(0xffffffffu, acc.c_med);
         const int c_bad = __reduce_add_sync(0xffffffffu, acc.c_bad), c_own = __reduce_add_sync(0xffffffffu, acc.c_own);
         if (lane == 0) {
