@@ -22,12 +22,15 @@
 //     tube runs one site per lane (V = 1) and one warp per block, so its warps
 //     land on separate SM sub-partitions and the step lasts one site's chain;
 //   * FP32 storage with four sites a lane evaluates them as two pairs with the
-//     paired FP32 instructions.  A chunk of 128 sites on which no limiter acts
-//     is finished there; any other, and the two chunks with the tube's ends, go
-//     to an out-of-line function, so the walk's registers hold only what the
-//     common case needs.  The kernel is bound by its
-//     dependent chains at 16 warps an SM (1e7 sites: 67 -> 54 us in 323 instead of
-//     490 warp instructions a chunk; 24 warps at 80 registers spill: 62 us);
+//     paired FP32 instructions.  A chunk of 128 sites on which nothing acts (no
+//     limiter, no end of the tube, no Ehrenfests' candidate) is finished there
+//     with three vector stores; in any other, the pairs on which nothing acts
+//     are, and an out-of-line function takes the rest, so the walk's registers
+//     hold little more than the common case needs.  Bound by its dependent chains
+//     at 16 warps an SM: 1e7 sites 72 -> 62 us a step; 3e6 sites with all three
+//     limiters 42 -> 37 us, with 0.5 % of the sites limited 63 -> 62 us; 24 warps at
+//     80 registers spill, 1e7 sites 82 us.  Leaving whole chunks to the function:
+//     62 us, but 72 us with 0.5 % of 3e6 sites limited.
 // Ensemble-dependent limiters and 16-bit storage stay on the tiled kernel.
 #include <type_traits>
 
@@ -355,104 +358,81 @@ __device__ __forceinline__ void tube_record(const StepParams &p, int x, double k
     }
 }
 
-// The FP64 keys of a chunk's listed candidates (FP32 storage; the whole warp), a lane
-// each: a chunk holding many of them costs one FP64 evaluation per 32, not one per
-// site a lane carries.  Empties the list.
-__device__ __noinline__ void tube_keys(const StepParams &p, const float *__restrict__ src, int2 *klist, int *kcount)
-{
-    __syncwarp();
-    const int nk = *kcount;
-    for (int i = threadIdx.x & 31; i < nk; i += 32) {
-        const int2 e = klist[i];
-        double fin[3], fs[3], fp[3], ds, din, rho;
-        if (p.collide)
-            tube_pull<float, double>(p, src, e.x, fin);
-        else
-            tube_read<float, double>(p, src, e.x, fin);
-        const bool bad = site_collide<3, double>(fin, p.a, p.collide != 0, fs, fp, ds, din, rho, p.eq, false);
-        if (!bad && ds > p.delta_e) tube_record(p, e.x, ds, (double)__int_as_float(e.y));
-    }
-    __syncwarp();
-    if ((threadIdx.x & 31) == 0) *kcount = 0;
-    __syncwarp();
-}
-
-// A chunk that the paired path of tube_walk32 leaves (the whole warp; FP32 storage):
-// dS of every site, then each finished by tube_site32, then the keys of its
-// candidates.  Returns the lane's sums; the counts are four bits each (bad, pos, med).
+// The chunk's sites that the paired fast path of tube_walk did not finish (FP32
+// storage; the whole warp).  done: bits 0 and 1, the lane's pairs already finished;
+// bit 2, ds_ holds dS of its sites (otherwise evaluated here: a lane that holds an
+// end of the tube, or a pass that is not a polynomial collision).  Then the FP64 keys
+// of all of the chunk's candidates, a lane each: a chunk holding many of them costs
+// one FP64 evaluation per 32, not one per site a lane carries.  Returns the sums of
+// the sites finished here; the counts are four bits each (bad, pos, med).
 struct ChunkSums {
     float mass, ds, din, lim;
     unsigned counts;
 };
 template <int V>
 __device__ __noinline__ ChunkSums tube_chunk32(const StepParams &p, const TubeK kk, const float *__restrict__ src,
-                                               float *__restrict__ dst, int c, int2 *klist, int *kcount)
+                                               float *__restrict__ dst, const TubeSlot<float, V> *slot, int c,
+                                               unsigned done, float4 ds_, int2 *klist, int *kcount)
 {
     using S = float;
+    const TubeSlot<S, V> &sl = *slot;
     const int lane = threadIdx.x & 31, nx = p.nx, xl = c * 32 * V + lane * V;
     ChunkSums r{0.f, 0.f, 0.f, 0.f, 0u};
-    // the lane's pulls: whole vectors (the row's padding follows its last site), the
-    // neighbours' values, the tube's ends
-    float f0[V], f1[V], f2[V], ds[V];
+    float ds[V];
 #pragma unroll
-    for (int j = 0; j < V; ++j) f0[j] = f1[j] = f2[j] = ds[j] = 0.f;
-    if (xl < nx) {
-        const float *const at = src + tidx(p, 0, xl);
-        float a0[V], a1[V + 1], a2[V + 1];
-        a1[V] = at[p.plane + V];
-        a2[0] = at[2 * p.plane - 1];
-        if constexpr (V == 4) {
-            const float4 v0 = *reinterpret_cast<const float4 *>(at);
-            const float4 v1 = *reinterpret_cast<const float4 *>(at + p.plane);
-            const float4 v2 = *reinterpret_cast<const float4 *>(at + 2 * p.plane);
-            a0[0] = v0.x, a0[1] = v0.y, a0[2] = v0.z, a0[3] = v0.w;
-            a1[0] = v1.x, a1[1] = v1.y, a1[2] = v1.z, a1[3] = v1.w;
-            a2[1] = v2.x, a2[2] = v2.y, a2[3] = v2.z, a2[4] = v2.w;
+    for (int j = 0; j < V; ++j) ds[j] = j == 0 ? ds_.x : (j == 1 ? ds_.y : (j == 2 ? ds_.z : ds_.w));
+    // the lane's pull of its site j (free flight with the tube's ends, or the stored
+    // values of a limiter pass)
+    auto build_fin = [&](int j, float f3[3]) {
+        const int x = xl + j, i = lane * V + j;
+        f3[0] = sl.f0[i];
+        if (p.collide) {
+            f3[1] = sl.f1[i + 1];
+            f3[2] = sl.f2[TubeSlot<S, V>::kPad + i - 1];
+            if (x == nx - 1)  // right end: reflect or wrap
+                f3[1] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : sl.f2[TubeSlot<S, V>::kPad + i];
+            if (x == 0)  // left end
+                f3[2] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : sl.f1[i];
         } else {
-#pragma unroll
-            for (int j = 0; j < V; ++j) {
-                a0[j] = at[j];
-                a1[j] = at[p.plane + j];
-                a2[j + 1] = at[2 * p.plane + j];
-            }
+            f3[1] = sl.f1[i];
+            f3[2] = sl.f2[TubeSlot<S, V>::kPad + i];
         }
-#pragma unroll
-        for (int j = 0; j < V; ++j) {
-            const int x = xl + j;
-            f0[j] = a0[j];
-            f1[j] = p.collide ? a1[j + 1] : a1[j];
-            f2[j] = p.collide ? a2[j] : a2[j + 1];
-            if (p.collide && x == nx - 1)  // right end: reflect or wrap
-                f1[j] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : a2[j + 1];
-            if (p.collide && x == 0)  // left end
-                f2[j] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : a1[j];
-        }
-    }
-    // dS of the lane's sites (the site's values are selected, not indexed: they stay in registers)
-    auto pick = [&](const float *v, int j) {
-        float w = v[0];
-#pragma unroll
-        for (int i = 1; i < V; ++i) w = i == j ? v[i] : w;
-        return w;
     };
+    if (!(done & 4u)) {
 #pragma unroll 1
-    for (int j = 0; j < V && xl + j < nx; ++j) {
-        const float f3[3] = {pick(f0, j), pick(f1, j), pick(f2, j)};
-        float fs3[3], fp3[3], fa3[3], nq3[3], d, din, rho;
-        tube_eval<float>(p, kk, f3, fs3, fp3, fa3, nq3, d, din, rho, false);
+        for (int j = 0; j < V; ++j) {
+            float d = 0.f;
+            if (xl + j < nx) {
+                float f3[3], fs3[3], fp3[3], fa3[3], nq3[3], din, rho;
+                build_fin(j, f3);
+                tube_eval<float>(p, kk, f3, fs3, fp3, fa3, nq3, d, din, rho, false);
+            }
 #pragma unroll
-        for (int i = 0; i < V; ++i)
-            if (i == j) ds[i] = d;
+            for (int i = 0; i < V; ++i)
+                if (i == j) ds[i] = d;
+        }
     }
     __syncwarp();
     // the median's neighbours: dS of the adjacent lanes' edge sites
     const float dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
     const float dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
 #pragma unroll 1
-    for (int j = 0; j < V && xl + j < nx; ++j) {
+    for (int j = 0; j < V; ++j) {
         const int x = xl + j;
-        // the neighbours' dS, or the site to evaluate (outside the chunk)
-        const float dl = j > 0 ? pick(ds, j - 1) : dl_lane, dr = j + 1 < V ? pick(ds, j + 1) : dr_lane;
+        if (x >= nx) break;
+        // this site's dS and its neighbours', or the site to evaluate (outside the chunk)
+        float d = ds[0], dl = dl_lane, dr = dr_lane;
+#pragma unroll
+        for (int i = 0; i < V; ++i)
+            if (i == j) {
+                d = ds[i];
+                if (i > 0) dl = ds[i - 1];
+                if (i + 1 < V) dr = ds[i + 1];
+            }
+        if ((done >> (j >> 1)) & 1u) {
+            if ((p.limiters & 2u) && d > kk.thr_e) klist[atomicAdd(kcount, 1)] = make_int2(x, __float_as_int(1.f));
+            continue;
+        }
         int xlo = -1, xro = -1;
         if (x == 0)
             xlo = nx - 1;
@@ -462,8 +442,9 @@ __device__ __noinline__ ChunkSums tube_chunk32(const StepParams &p, const TubeK 
             xro = 0;
         else if (j == V - 1 && lane == 31)
             xro = x + 1;
-        const SiteSums q = tube_site32<S>(p, kk, src, dst, x, pick(f0, j), pick(f1, j), pick(f2, j), dl, dr, xlo, xro,
-                                          klist, kcount);
+        float f3[3];
+        build_fin(j, f3);
+        const SiteSums q = tube_site32<S>(p, kk, src, dst, x, f3[0], f3[1], f3[2], dl, dr, xlo, xro, klist, kcount);
         r.mass = __fadd_rn(r.mass, q.mass);
         r.ds = __fadd_rn(r.ds, q.ds);
         r.din = __fadd_rn(r.din, q.din);
@@ -471,42 +452,71 @@ __device__ __noinline__ ChunkSums tube_chunk32(const StepParams &p, const TubeK 
         r.counts += (unsigned)q.bad | (unsigned)q.pos << 4 | (unsigned)q.med << 8;
     }
     __syncwarp();
-    if (*kcount > 0) tube_keys(p, src, klist, kcount);
+    const int nk = *kcount;
+    for (int i = lane; i < nk; i += 32) {
+        const int2 e = klist[i];
+        double fin64[3], fs64[3], fp64[3], d64, din64, r64;
+        if (p.collide)
+            tube_pull<S, double>(p, src, e.x, fin64);
+        else
+            tube_read<S, double>(p, src, e.x, fin64);
+        const bool b64 = site_collide<3, double>(fin64, p.a, p.collide != 0, fs64, fp64, d64, din64, r64, p.eq, false);
+        if (!b64 && d64 > p.delta_e) tube_record(p, e.x, d64, (double)__int_as_float(e.y));
+    }
+    __syncwarp();
+    if (lane == 0) *kcount = 0;
+    __syncwarp();
     return r;
 }
 
 // One warp's walk over chunks c0, c0 + stride, ... (< c_end) of lattice p:
 // a1-a9 at every site, the Ehrenfests' candidates, the sums into acc.  `my`:
-// the warp's ring.  Every lane of the warp takes part.  FP64 storage.
-template <int V>
-__device__ __forceinline__ void tube_walk64(const StepParams &p, const double *__restrict__ src,
-                                            double *__restrict__ dst, int c0, int stride, int c_end,
-                                            TubeSlot<double, V> *my, TubeAcc &acc)
+// the warp's ring; klist / kcount: the warp's candidate list (FP32 storage).
+// Every lane of the warp takes part.
+template <typename S, int V>
+__device__ __forceinline__ void tube_walk(const StepParams &p, const S *__restrict__ src, S *__restrict__ dst,
+                                          int c0, int stride, int c_end, TubeSlot<S, V> *my, int2 *klist,
+                                          int *kcount, TubeAcc &acc)
 {
-    using S = double;
-    using A = Ar<double>;
+    using T = compute_t<S>;
+    using A = Ar<T>;
     using Slot = TubeSlot<S, V>;
-    const int lane = threadIdx.x & 31, nx = p.nx;
-    const TubeK kk{};  // FP32 storage only
+    constexpr bool F64 = std::is_same<T, double>::value;
+    constexpr int CW = 32 * V;  // sites of a chunk
+    const int lane = threadIdx.x & 31;
+    const int nx = p.nx;
+    TubeK kk{};
+    if constexpr (!F64) {
+        kk.a = (float)p.a;
+        kk.b2 = (float)(1.0 + p.a);
+        kk.dm = (float)p.delta_m;
+        kk.thr_e = (float)(p.delta_e * (1.0 - 1.0 / 64.0));
+    }
+    // the fast path's flags and constants in registers (the batched kernel's lie in
+    // shared memory)
+    const bool fast = V == 4 && !F64 && p.collide && p.eq == 0 && !p.ds_out;
     const bool lim_pos = (p.limiters & 1u) != 0, lim_ehr = (p.limiters & 2u) != 0, lim_med = (p.limiters & 4u) != 0;
+    const float rho_ref = p.rho_ref, rwf[3] = {p.rwf[0], p.rwf[1], p.rwf[2]};
+    const float d_act = lim_med ? kk.dm : INFINITY, d_cand = lim_ehr ? kk.thr_e : INFINITY;
+
     // copies of chunk c into slot `sl` (nothing past the last chunk; the group
     // is committed either way).  The chunk's window lies inside the padded row
     // (kTail zero elements follow the lattice), so whole vectors may be copied
     // past its end.
     auto issue = [&](int c, int sl) {
         if (c < c_end) {
-            const int x0 = c * 32 * V, xl = x0 + lane * V;
-            const S *const at = src + tidx(p, 0, xl);
+            const int x0 = c * CW, xl = x0 + lane * V;
             if (xl < nx) {
-                tcopy<(int)sizeof(S) * V>(&my[sl].f0[lane * V], at);
-                tcopy<(int)sizeof(S) * V>(&my[sl].f1[lane * V], at + p.plane);
-                tcopy<(int)sizeof(S) * V>(&my[sl].f2[Slot::kPad + lane * V], at + 2 * p.plane);
+                tcopy<(int)sizeof(S) * V>(&my[sl].f0[lane * V], src + tidx(p, 0, xl));
+                tcopy<(int)sizeof(S) * V>(&my[sl].f1[lane * V], src + tidx(p, 1, xl));
+                tcopy<(int)sizeof(S) * V>(&my[sl].f2[Slot::kPad + lane * V], src + tidx(p, 2, xl));
             }
-            if (lane == 0 && x0 > 0) tcopy<(int)sizeof(S)>(&my[sl].f2[Slot::kPad - 1], at + 2 * p.plane - 1);
-            if (lane == 31 && xl + V < nx) tcopy<(int)sizeof(S)>(&my[sl].f1[32 * V], at + p.plane + V);
+            if (lane == 0 && x0 > 0) tcopy<(int)sizeof(S)>(&my[sl].f2[Slot::kPad - 1], src + tidx(p, 2, x0 - 1));
+            if (lane == 31 && xl + V < nx) tcopy<(int)sizeof(S)>(&my[sl].f1[32 * V], src + tidx(p, 1, xl + V));
         }
         tcommit();
     };
+
 #pragma unroll
     for (int i = 0; i < kTubeRing - 1; ++i) issue(c0 + i * stride, i);
     int get = 0;
@@ -517,243 +527,206 @@ __device__ __forceinline__ void tube_walk64(const StepParams &p, const double *_
         __syncwarp();                                                   // and so have the other lanes'
         const Slot &sl = my[get];
         get = get + 1 == kTubeRing ? 0 : get + 1;
-        const int xl = c * 32 * V + lane * V;
-        const S r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
-        double ds[V], fin[V][3], fs[V][3], fp[V][3], dsin[V], rho[V];
-        double s_mass = 0.0, s_ds = 0.0, s_in = 0.0, s_lim = 0.0;
-        bool bad[V];
+        const int x0 = c * CW, xl = x0 + lane * V;
+        if constexpr (!F64) {
+            // the chunk's sums: the pairs' interleaved terms; the sites finished by tube_chunk32
+            float2 m2 = F2::s(0.f), d2s = F2::s(0.f), i2s = F2::s(0.f);
+            unsigned done = 0u;
+            bool rest = true;
+            float4 ds = make_float4(0.f, 0.f, 0.f, 0.f);
+            if constexpr (V == 4) {
+                if (fast) {
+                    const float4 f0 = *reinterpret_cast<const float4 *>(&sl.f0[lane * V]);
+                    const float4 f1 = *reinterpret_cast<const float4 *>(&sl.f1[lane * V]);
+                    const float4 f2 = *reinterpret_cast<const float4 *>(&sl.f2[Slot::kPad + lane * V]);
+                    const float r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
+                    const float2 ga[3] = {make_float2(f0.x, f0.y), make_float2(f1.y, f1.z), make_float2(l2, f2.x)};
+                    const float2 gb[3] = {make_float2(f0.z, f0.w), make_float2(f1.w, r1), make_float2(f2.y, f2.z)};
+                    float2 pa[3], pb[3], da, db, ia, ib, ra, rb;
+                    bool ba, bb, bc, bd;
+                    tube_pair_eval(kk, rho_ref, rwf, ga, pa, da, ia, ra, ba, bb);
+                    tube_pair_eval(kk, rho_ref, rwf, gb, pb, db, ib, rb, bc, bd);
+                    // a pair on which something acts: a bad site, a negative f' of the
+                    // positivity rule, dS above the median filter's delta
+                    bool act_a = ba || bb || fmaxf(da.x, da.y) > d_act, act_b = bc || bd || fmaxf(db.x, db.y) > d_act;
+                    if (lim_pos) {
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-            const int x = xl + j, i = lane * V + j;
-            ds[j] = 0.0;
-            dsin[j] = 0.0;
-            rho[j] = 0.0;
-            bad[j] = false;
-            if (x >= nx) continue;
-            fin[j][0] = sl.f0[i];
-            if (p.collide) {
-                fin[j][1] = j + 1 < V ? sl.f1[i + 1] : r1;
-                fin[j][2] = j > 0 ? sl.f2[Slot::kPad + i - 1] : l2;
-                if (x == nx - 1)  // right end: reflect or wrap
-                    fin[j][1] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : sl.f2[Slot::kPad + i];
-                if (x == 0)  // left end
-                    fin[j][2] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : sl.f1[i];
-            } else {
-                fin[j][1] = sl.f1[i];
-                fin[j][2] = sl.f2[Slot::kPad + i];
-            }
-            bad[j] = site_collide<3, double>(fin[j], p.a, p.collide != 0, fs[j], fp[j], ds[j], dsin[j], rho[j],
-                                             p.eq, true, p.coll, p.beta);
-            if (bad[j]) ds[j] = INFINITY;
-        }
-
-        // the median's neighbours: dS of the adjacent lanes' edge sites
-        const double dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
-        const double dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
-
+                        for (int k = 0; k < 3; ++k) {
+                            act_a = act_a || fminf(rwf[k] + pa[k].x, rwf[k] + pa[k].y) < 0.f;
+                            act_b = act_b || fminf(rwf[k] + pb[k].x, rwf[k] + pb[k].y) < 0.f;
+                        }
+                    }
+                    const bool inside = xl >= 1 && xl + V <= nx - 1;
+                    const bool cand = fmaxf(fmaxf(da.x, da.y), fmaxf(db.x, db.y)) > d_cand;
+                    rest = __any_sync(0xffffffffu, act_a || act_b || cand || !inside);
+                    const float2 ma = F2::sub(ra, F2::s(rho_ref)), mb = F2::sub(rb, F2::s(rho_ref));  // exact
+                    float *const to = dst + tidx(p, 0, xl);
+                    if (!rest) {
 #pragma unroll
-        for (int j = 0; j < V; ++j) {
-            const int x = xl + j;
-            if (x >= nx) continue;
-            ++acc.c_own;
-            double phi_pos = 1.0, phi_med = 1.0;
-            if (!bad[j]) {
-                if (lim_pos) phi_pos = phi_positivity<3, double>(fs[j], fp[j]);
-                // three-point median (the two end sites of a closed tube are not
-                // filtered; a periodic tube's end sites wrap around to each other)
-                const bool end = p.boundary == 0 && (x == 0 || x == nx - 1);
-                if (lim_med && ds[j] > p.delta_m && !end) {
-                    double left, right;
-                    if (x == 0)
-                        left = tube_ds<S>(p, kk, src, nx - 1);
-                    else if (j > 0)
-                        left = ds[j - 1];
-                    else if (lane > 0)
-                        left = dl_lane;
-                    else
-                        left = tube_ds<S>(p, kk, src, x - 1);
-                    if (x == nx - 1)
-                        right = tube_ds<S>(p, kk, src, 0);
-                    else if (j + 1 < V)
-                        right = ds[j + 1];
-                    else if (lane < 31)
-                        right = dr_lane;
-                    else
-                        right = tube_ds<S>(p, kk, src, x + 1);
-                    const double med = med3(left, ds[j], right);
-                    phi_med = (p.phi_rule == 1 && p.eq == 1)
-                                  ? phi_median_entropy<3>(fp[j], fs[j], ds[j], med, p.delta_m, p.median_mode)
-                                  : phi_median<double>(ds[j], med, p.delta_m, p.median_mode);
+                        for (int k = 0; k < 3; ++k)
+                            *reinterpret_cast<float4 *>(to + k * p.plane) =
+                                make_float4(pa[k].x, pa[k].y, pb[k].x, pb[k].y);
+                        m2 = F2::add(ma, mb);
+                        d2s = F2::add(da, db);
+                        i2s = F2::add(ia, ib);
+                    } else if (inside) {
+                        // a site that cannot be limited has dS = +inf (as tube_eval gives it)
+                        ds = make_float4(ba ? INFINITY : da.x, bb ? INFINITY : da.y, bc ? INFINITY : db.x,
+                                         bd ? INFINITY : db.y);
+                        done = 4u;
+                        if (!act_a) {
+                            done |= 1u;
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) *reinterpret_cast<float2 *>(to + k * p.plane) = pa[k];
+                            m2 = ma;
+                            d2s = da;
+                            i2s = ia;
+                        }
+                        if (!act_b) {
+                            done |= 2u;
+#pragma unroll
+                            for (int k = 0; k < 3; ++k) *reinterpret_cast<float2 *>(to + k * p.plane + 2) = pb[k];
+                            m2 = F2::add(m2, mb);
+                            d2s = F2::add(d2s, db);
+                            i2s = F2::add(i2s, ib);
+                        }
+                    }
                 }
             }
-            const double phi = phi_pos < phi_med ? phi_pos : phi_med;
-            double lim = 0.0;
-            if (phi < 1.0) {
-                double fo[3];
+            if (rest) {
+                const ChunkSums r = tube_chunk32<V>(p, kk, src, dst, &sl, c, done, ds, klist, kcount);
+                m2.x = __fadd_rn(m2.x, r.mass);
+                d2s.x = __fadd_rn(d2s.x, r.ds);
+                i2s.x = __fadd_rn(i2s.x, r.din);
+                const float y = __fsub_rn(r.lim, acc.c_lim), t = __fadd_rn(acc.s_lim, y);
+                acc.c_lim = __fsub_rn(__fsub_rn(t, acc.s_lim), y);
+                acc.s_lim = t;
+                acc.c_bad += (int)(r.counts & 15u);
+                acc.c_pos += (int)(r.counts >> 4 & 15u);
+                acc.c_med += (int)(r.counts >> 8 & 15u);
+            }
+            kahan2(acc.s_mass, acc.c_mass, m2);
+            kahan2(acc.s_ds, acc.c_ds, d2s);
+            kahan2(acc.s_in, acc.c_in, i2s);
+            acc.c_own += max(0, min(V, nx - xl));
+        } else {
+            const S r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
+            double ds[V], fin[V][3], fs[V][3], fp[V][3], dsin[V], rho[V];
+            double s_mass = 0.0, s_ds = 0.0, s_in = 0.0, s_lim = 0.0;
+            bool bad[V];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    fo[k] = A::add(fs[j][k], A::mul(phi, A::sub(fp[j][k], fs[j][k])));
-                    dst[tidx(p, k, x)] = fo[k];
-                }
-                if (p.eq == 1) {
-                    const double dout = rel_entropy<3>(fo, fs[j]);
-                    if (isfinite(ds[j]) && isfinite(dout)) lim = A::sub(ds[j], dout);
+            for (int j = 0; j < V; ++j) {
+                const int x = xl + j, i = lane * V + j;
+                ds[j] = 0.0;
+                dsin[j] = 0.0;
+                rho[j] = 0.0;
+                bad[j] = false;
+                if (x >= nx) continue;
+                fin[j][0] = sl.f0[i];
+                if (p.collide) {
+                    fin[j][1] = j + 1 < V ? sl.f1[i + 1] : r1;
+                    fin[j][2] = j > 0 ? sl.f2[Slot::kPad + i - 1] : l2;
+                    if (x == nx - 1)  // right end: reflect or wrap
+                        fin[j][1] = bc_wrap_x(p.boundary) ? src[tidx(p, 1, 0)] : sl.f2[Slot::kPad + i];
+                    if (x == 0)  // left end
+                        fin[j][2] = bc_wrap_x(p.boundary) ? src[tidx(p, 2, nx - 1)] : sl.f1[i];
                 } else {
-                    lim = A::mul(A::sub(1.0, A::mul(phi, phi)), ds[j]);
+                    fin[j][1] = sl.f1[i];
+                    fin[j][2] = sl.f2[Slot::kPad + i];
                 }
-            } else {
+                bad[j] = site_collide<3, double>(fin[j], p.a, p.collide != 0, fs[j], fp[j], ds[j], dsin[j], rho[j],
+                                                 p.eq, true, p.coll, p.beta);
+                if (bad[j]) ds[j] = INFINITY;
+            }
+
+            // the median's neighbours: dS of the adjacent lanes' edge sites
+            const double dl_lane = __shfl_up_sync(0xffffffffu, ds[V - 1], 1);
+            const double dr_lane = __shfl_down_sync(0xffffffffu, ds[0], 1);
+
 #pragma unroll
-                for (int k = 0; k < 3; ++k) dst[tidx(p, k, x)] = fp[j][k];
-            }
-            s_lim = A::add(s_lim, lim);
-            s_mass = A::add(s_mass, rho[j]);
-            if (!bad[j]) {
-                double tds = 0.0, tin = 0.0;
-                if (p.eq == 1) {
-                    if (isfinite(ds[j])) tds = ds[j];
-                    if (isfinite(ds[j]) && isfinite(dsin[j])) tin = A::sub(dsin[j], ds[j]);
-                } else {
-                    tds = ds[j];
-                    tin = dsin[j];
+            for (int j = 0; j < V; ++j) {
+                const int x = xl + j;
+                if (x >= nx) continue;
+                ++acc.c_own;
+                double phi_pos = 1.0, phi_med = 1.0;
+                if (!bad[j]) {
+                    if (lim_pos) phi_pos = phi_positivity<3, double>(fs[j], fp[j]);
+                    // three-point median (the two end sites of a closed tube are not
+                    // filtered; a periodic tube's end sites wrap around to each other)
+                    const bool end = p.boundary == 0 && (x == 0 || x == nx - 1);
+                    if (lim_med && ds[j] > p.delta_m && !end) {
+                        double left, right;
+                        if (x == 0)
+                            left = tube_ds<S>(p, kk, src, nx - 1);
+                        else if (j > 0)
+                            left = ds[j - 1];
+                        else if (lane > 0)
+                            left = dl_lane;
+                        else
+                            left = tube_ds<S>(p, kk, src, x - 1);
+                        if (x == nx - 1)
+                            right = tube_ds<S>(p, kk, src, 0);
+                        else if (j + 1 < V)
+                            right = ds[j + 1];
+                        else if (lane < 31)
+                            right = dr_lane;
+                        else
+                            right = tube_ds<S>(p, kk, src, x + 1);
+                        const double med = med3(left, ds[j], right);
+                        phi_med = (p.phi_rule == 1 && p.eq == 1)
+                                      ? phi_median_entropy<3>(fp[j], fs[j], ds[j], med, p.delta_m, p.median_mode)
+                                      : phi_median<double>(ds[j], med, p.delta_m, p.median_mode);
+                    }
                 }
-                s_ds = A::add(s_ds, tds);
-                s_in = A::add(s_in, tin);
-            } else {
-                ++acc.c_bad;
-                atomicOr(p.status, kStatNonfinite);
+                const double phi = phi_pos < phi_med ? phi_pos : phi_med;
+                double lim = 0.0;
+                if (phi < 1.0) {
+                    double fo[3];
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) {
+                        fo[k] = A::add(fs[j][k], A::mul(phi, A::sub(fp[j][k], fs[j][k])));
+                        dst[tidx(p, k, x)] = fo[k];
+                    }
+                    if (p.eq == 1) {
+                        const double dout = rel_entropy<3>(fo, fs[j]);
+                        if (isfinite(ds[j]) && isfinite(dout)) lim = A::sub(ds[j], dout);
+                    } else {
+                        lim = A::mul(A::sub(1.0, A::mul(phi, phi)), ds[j]);
+                    }
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 3; ++k) dst[tidx(p, k, x)] = fp[j][k];
+                }
+                s_lim = A::add(s_lim, lim);
+                s_mass = A::add(s_mass, rho[j]);
+                if (!bad[j]) {
+                    double tds = 0.0, tin = 0.0;
+                    if (p.eq == 1) {
+                        if (isfinite(ds[j])) tds = ds[j];
+                        if (isfinite(ds[j]) && isfinite(dsin[j])) tin = A::sub(dsin[j], ds[j]);
+                    } else {
+                        tds = ds[j];
+                        tin = dsin[j];
+                    }
+                    s_ds = A::add(s_ds, tds);
+                    s_in = A::add(s_in, tin);
+                } else {
+                    ++acc.c_bad;
+                    atomicOr(p.status, kStatNonfinite);
+                }
+                acc.c_pos += phi_pos < 1.0;
+                acc.c_med += phi_med < 1.0;
+                // Ehrenfests' candidates on dS(f') itself
+                if (lim_ehr && !bad[j] && ds[j] > p.delta_e) tube_record(p, x, ds[j], phi);
+                if (p.ds_out) p.ds_out[x] = ds[j];
             }
-            acc.c_pos += phi_pos < 1.0;
-            acc.c_med += phi_med < 1.0;
-            // Ehrenfests' candidates on dS(f') itself
-            if (lim_ehr && !bad[j] && ds[j] > p.delta_e) tube_record(p, x, ds[j], phi);
-            if (p.ds_out) p.ds_out[x] = ds[j];
+            acc.t_mass = A::add(acc.t_mass, s_mass);
+            acc.t_ds = A::add(acc.t_ds, s_ds);
+            acc.t_in = A::add(acc.t_in, s_in);
+            acc.t_lim = A::add(acc.t_lim, s_lim);
         }
-        acc.t_mass = A::add(acc.t_mass, s_mass);
-        acc.t_ds = A::add(acc.t_ds, s_ds);
-        acc.t_in = A::add(acc.t_in, s_in);
-        acc.t_lim = A::add(acc.t_lim, s_lim);
     }
     twait<0>();
-}
-
-// FP32 storage: the chunks c0, c0 + stride, ... (< c_end, none with an end of the
-// tube), after those of `ends` (bit 0: chunk 0, bit 1: the last).  klist / kcount: the
-// warp's candidate list.  An entropic or limiter pass, or one site a lane, leaves every
-// chunk to tube_chunk32.
-template <int V>
-__device__ __forceinline__ void tube_walk32(const StepParams &p, const float *__restrict__ src,
-                                            float *__restrict__ dst, int c0, int stride, int c_end, unsigned ends,
-                                            TubeSlot<float, V> *my, int2 *klist, int *kcount, TubeAcc &acc)
-{
-    using S = float;
-    using Slot = TubeSlot<S, V>;
-    constexpr int CW = 32 * V;  // sites of a chunk
-    const int lane = threadIdx.x & 31, nx = p.nx;
-    TubeK kk;
-    kk.a = (float)p.a;
-    kk.b2 = (float)(1.0 + p.a);
-    kk.dm = (float)p.delta_m;
-    kk.thr_e = (float)(p.delta_e * (1.0 - 1.0 / 64.0));
-    auto leave = [&](int c) {
-        const ChunkSums r = tube_chunk32<V>(p, kk, src, dst, c, klist, kcount);
-        kahan2(acc.s_mass, acc.c_mass, make_float2(r.mass, 0.f));
-        kahan2(acc.s_ds, acc.c_ds, make_float2(r.ds, 0.f));
-        kahan2(acc.s_in, acc.c_in, make_float2(r.din, 0.f));
-        const float y = __fsub_rn(r.lim, acc.c_lim), t = __fadd_rn(acc.s_lim, y);
-        acc.c_lim = __fsub_rn(__fsub_rn(t, acc.s_lim), y);
-        acc.s_lim = t;
-        acc.c_bad += (int)(r.counts & 15u);
-        acc.c_pos += (int)(r.counts >> 4 & 15u);
-        acc.c_med += (int)(r.counts >> 8 & 15u);
-        acc.c_own += max(0, min(V, nx - c * CW - lane * V));
-    };
-    const bool paired = V == 4 && p.collide && p.eq == 0 && !p.ds_out;
-    // the ends first (their code is cold: an instruction fetch costs about 10 ns), then,
-    // when nothing is paired, the rest
-    for (int c = c0; ends || (!paired && c < c_end);) {
-        const bool end = ends != 0;
-        leave(!end ? c : (ends & 1u ? 0 : (nx - 1) / CW));
-        if (end)
-            ends &= ends - 1u;
-        else
-            c += stride;
-    }
-    if (!paired) return;
-    if constexpr (V == 4) {
-        // the flags and constants in registers (the batched kernel's lie in shared memory)
-        const bool lim_pos = (p.limiters & 1u) != 0;
-        const float rho_ref = p.rho_ref, rwf[3] = {p.rwf[0], p.rwf[1], p.rwf[2]};
-        const float d_act = (p.limiters & 4u) ? kk.dm : INFINITY, d_cand = (p.limiters & 2u) ? kk.thr_e : INFINITY;
-        const long long plane = p.plane;
-        const float *const from = src + tidx(p, 0, lane * V);
-        float *const to = dst + tidx(p, 0, lane * V);
-        // copies of chunk c into slot `sl` (nothing past the last chunk; the group is
-        // committed either way)
-        auto issue = [&](int c, int sl) {
-            if (c < c_end) {
-                const float *const at = from + (long long)c * CW;
-                tcopy<16>(&my[sl].f0[lane * V], at);
-                tcopy<16>(&my[sl].f1[lane * V], at + plane);
-                tcopy<16>(&my[sl].f2[Slot::kPad + lane * V], at + 2 * plane);
-                if (lane == 0) tcopy<4>(&my[sl].f2[Slot::kPad - 1], at + 2 * plane - 1);
-                if (lane == 31) tcopy<4>(&my[sl].f1[CW], at + plane + V);
-            }
-            tcommit();
-        };
-#pragma unroll
-        for (int i = 0; i < kTubeRing - 1; ++i) issue(c0 + i * stride, i);
-        int get = 0;
-        for (int c = c0; c < c_end; c += stride) {
-            __syncwarp();  // every lane is done with the slot refilled now
-            issue(c + (kTubeRing - 1) * stride, get == 0 ? kTubeRing - 1 : get - 1);
-            twait<kTubeRing - 1>();  // this lane's copies of chunk c have landed
-            __syncwarp();            // and so have the other lanes'
-            const Slot &sl = my[get];
-            get = get + 1 == kTubeRing ? 0 : get + 1;
-            const float4 f0 = *reinterpret_cast<const float4 *>(&sl.f0[lane * V]);
-            const float4 f1 = *reinterpret_cast<const float4 *>(&sl.f1[lane * V]);
-            const float4 f2 = *reinterpret_cast<const float4 *>(&sl.f2[Slot::kPad + lane * V]);
-            const float r1 = sl.f1[lane * V + V], l2 = sl.f2[Slot::kPad + lane * V - 1];
-            const float2 ga[3] = {make_float2(f0.x, f0.y), make_float2(f1.y, f1.z), make_float2(l2, f2.x)};
-            const float2 gb[3] = {make_float2(f0.z, f0.w), make_float2(f1.w, r1), make_float2(f2.y, f2.z)};
-            float2 pa[3], pb[3], da, db, ia, ib, ra, rb;
-            bool ba, bb, bc, bd;
-            tube_pair_eval(kk, rho_ref, rwf, ga, pa, da, ia, ra, ba, bb);
-            tube_pair_eval(kk, rho_ref, rwf, gb, pb, db, ib, rb, bc, bd);
-            // does a limiter act: a bad site, dS above the median filter's delta, a
-            // negative f' of the positivity rule?
-            const float dmax = fmaxf(fmaxf(da.x, da.y), fmaxf(db.x, db.y));
-            bool act = ba || bb || bc || bd || dmax > d_act;
-            if (lim_pos) {
-#pragma unroll
-                for (int k = 0; k < 3; ++k)
-                    act = act || rwf[k] + fminf(fminf(pa[k].x, pb[k].x), fminf(pa[k].y, pb[k].y)) < 0.f;
-            }
-            if (__any_sync(0xffffffffu, act)) {
-                leave(c);
-                continue;
-            }
-            float *const at = to + (long long)c * CW;
-#pragma unroll
-            for (int k = 0; k < 3; ++k)
-                *reinterpret_cast<float4 *>(at + k * plane) = make_float4(pa[k].x, pa[k].y, pb[k].x, pb[k].y);
-            const float2 ma = F2::sub(ra, F2::s(rho_ref)), mb = F2::sub(rb, F2::s(rho_ref));  // exact
-            kahan2(acc.s_mass, acc.c_mass, F2::add(ma, mb));
-            kahan2(acc.s_ds, acc.c_ds, F2::add(da, db));
-            kahan2(acc.s_in, acc.c_in, F2::add(ia, ib));
-            acc.c_own += V;
-            // Ehrenfests' candidates: sites near or above the threshold (rare)
-            if (__any_sync(0xffffffffu, dmax > d_cand)) {
-                const float d4[4] = {da.x, da.y, db.x, db.y};
-#pragma unroll
-                for (int j = 0; j < V; ++j)
-                    if (d4[j] > d_cand)
-                        klist[atomicAdd(kcount, 1)] = make_int2(c * CW + lane * V + j, __float_as_int(1.f));
-                tube_keys(p, src, klist, kcount);
-            }
-        }
-        twait<0>();
-    }
 }
 
 template <typename S, int V>
@@ -761,10 +734,11 @@ __global__ void __launch_bounds__(256, V == 4 ? kTubeBlocks : (V > 1 ? 2 : 1))
     k_tube(const __grid_constant__ StepParams p, const S *__restrict__ src, S *__restrict__ dst, int chunked)
 {
     constexpr bool F64 = std::is_same<compute_t<S>, double>::value;
-    constexpr bool RING = F64 || V == 4;
-    __shared__ TubeSlot<S, V> ring[RING ? kTubeWarps : 1][RING ? kTubeRing : 1];
-    // FP32 storage: the chunk's sites whose FP32 dS(f') lies near or above the threshold
-    // (site, phi)
+    __shared__ TubeSlot<S, V> ring[kTubeWarps][kTubeRing];
+    // FP32 storage: the chunk's sites whose FP32 dS(f') lies near or above the
+    // threshold (site, phi), keyed in FP64 after the chunk with one lane each:
+    // a chunk holding many of them costs one FP64 evaluation per 32, not one per
+    // site a lane carries
     __shared__ int2 klist[kTubeWarps][F64 ? 1 : 32 * V];
     __shared__ int kcount[kTubeWarps];
     // the tail of the previous pass may still run (programmatic launch)
@@ -774,15 +748,8 @@ __global__ void __launch_bounds__(256, V == 4 ? kTubeBlocks : (V > 1 ? 2 : 1))
     if (lane == 0) kcount[warp] = 0;
     __syncwarp();
     TubeAcc acc{};
-    const int w = blockIdx.x * nw + warp, stride = (int)gridDim.x * nw, chunks = (p.nx + 32 * V - 1) / (32 * V);
-    if constexpr (F64) {
-        tube_walk64<V>(p, src, dst, w, stride, chunks, ring[warp], acc);
-    } else {
-        // the two chunks with the tube's ends to the last warps, which have fewer others
-        const unsigned ends = (chunks > 1 && w == max(stride - 2, 0) ? 1u : 0u) | (w == stride - 1 ? 2u : 0u);
-        tube_walk32<V>(p, src, dst, 1 + w, stride, chunks - 1, ends, RING ? ring[warp] : ring[0], klist[warp],
-                       &kcount[warp], acc);
-    }
+    tube_walk<S, V>(p, src, dst, blockIdx.x * nw + warp, (int)gridDim.x * nw, (p.nx + 32 * V - 1) / (32 * V),
+                    ring[warp], klist[warp], &kcount[warp], acc);
     double t_mass = acc.t_mass, t_ds = acc.t_ds, t_in = acc.t_in, t_lim = acc.t_lim;
     if constexpr (!F64) tube_totals<V>(acc, t_mass, t_ds, t_in, t_lim);
     int c_pos = acc.c_pos, c_med = acc.c_med, c_bad = acc.c_bad, c_own = acc.c_own;
@@ -875,9 +842,8 @@ __global__ void __launch_bounds__(256, kTubeBlocks) k_tube_batched(const TubeArg
         const int nch = (p.nx + 32 * V - 1) / (32 * V);
         const int c0 = m.y * kTubeGroup, c1 = min(c0 + kTubeGroup, nch);
         TubeAcc acc{};
-        const unsigned ends = (c0 == 0 && nch > 1 ? 1u : 0u) | (c1 == nch ? 2u : 0u);
-        tube_walk32<V>(p, (const S *)sA[warp].src, (S *)sA[warp].dst, max(c0, 1), 1, min(c1, nch - 1), ends,
-                       ring[warp], klist[warp], &kcount[warp], acc);
+        tube_walk<S, V>(p, (const S *)sA[warp].src, (S *)sA[warp].dst, c0, 1, c1, ring[warp], klist[warp],
+                               &kcount[warp], acc);
         // the item's totals; the counts are per lane
         double t_mass, t_ds, t_in, t_lim;
         tube_totals<V>(acc, t_mass, t_ds, t_in, t_lim);

@@ -1,9 +1,9 @@
 """FP32 tubes around the edges of the tube kernel's chunks of 128 sites.
 
-A chunk on which no limiter acts is finished at once, its candidates keyed after
-it; the chunks with the tube's ends and those where a limiter acts take another
-way.  Both, alone and batched (groups of 8 chunks), give the populations and
-counts of the tiled kernel bit for bit.
+A chunk on which nothing acts is finished at once; the chunks with the tube's
+ends, with limited sites or with candidates take another way for those sites.
+Both, alone and batched (groups of 8 chunks), give the populations and counts
+of the tiled kernel bit for bit.
 """
 import numpy as np
 import pytest
