@@ -31,6 +31,7 @@
 namespace lbm {
 namespace {
 
+constexpr int kSelLoads = 4;  // candidates a thread reads at once in dense_select
 constexpr unsigned kSelSpinLimit = 1u << 21;  // grid-barrier polls (about a second) before giving up
 
 // Grid barrier of the cooperative tail: each block adds one arrival to *bar;
@@ -148,14 +149,17 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
     };
     for (int b = t; b < kSelBins; b += kFinThreads) sh[b] = 0;
     __syncthreads();
-    for (long long base = base0; base < n; base += stride) {  // whole warps per round
-        const long long i = base + t;
-        int bin = -1;
-        if (i < n) {
-            const int u = __float_as_int(p.cand[i].ds32);
-            if (in_r(u)) bin = u >> 19;
+    // kSelLoads candidates of a thread are read together: 16 warps an SM do not hide
+    // the latency of one read each
+    for (long long base = base0; base < n; base += kSelLoads * stride) {  // whole warps per round
+        int u[kSelLoads];
+#pragma unroll
+        for (int j = 0; j < kSelLoads; ++j) {
+            const long long i = base + j * stride + t;
+            u[j] = i < n ? __float_as_int(p.cand[i].ds32) : 0x7f800000;  // not in R
         }
-        count_bin(bin);
+#pragma unroll
+        for (int j = 0; j < kSelLoads; ++j) count_bin(in_r(u[j]) ? u[j] >> 19 : -1);
     }
     __syncthreads();
     for (int b = t; b < kSelBins; b += kFinThreads)
@@ -170,14 +174,16 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
     for (int b = t; b < kSelBins; b += kFinThreads) sh[b] = 0;
     __syncthreads();
     if (!all) {
-        for (long long base = base0; base < n; base += stride) {
-            const long long i = base + t;
-            int bin = -1;
-            if (i < n) {
-                const int u = __float_as_int(p.cand[i].ds32);
-                if (in_r(u) && (u >> 19) == b1) bin = (u >> 7) & (kSelBins - 1);
+        for (long long base = base0; base < n; base += kSelLoads * stride) {
+            int u[kSelLoads];
+#pragma unroll
+            for (int j = 0; j < kSelLoads; ++j) {
+                const long long i = base + j * stride + t;
+                u[j] = i < n ? __float_as_int(p.cand[i].ds32) : 0x7f800000;
             }
-            count_bin(bin);
+#pragma unroll
+            for (int j = 0; j < kSelLoads; ++j)
+                count_bin(in_r(u[j]) && (u[j] >> 19) == b1 ? (u[j] >> 7) & (kSelBins - 1) : -1);
         }
         __syncthreads();
         for (int b = t; b < kSelBins; b += kFinThreads)
@@ -228,32 +234,41 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
         }
         append(listed, i);
     };
-    for (long long base = base0; base < n; base += stride) {  // whole blocks per round
-        const long long i = base + t;
-        bool valid = false, listed = false, need = false;
-        if (i < n) {
-            const Cand c = p.cand[i];
-            const int u = __float_as_int(c.ds32);
-            const bool top = u >= tlow_bits;
-            need = kKeyHere && isnan(c.key) && (top || u <= dhi_bits);
-            valid = !need && (isnan(c.key) ? in_r(u) : c.key > p.delta_e);
-            listed = top && valid;
+    for (long long base = base0; base < n; base += kSelLoads * stride) {  // whole blocks per round
+        Cand cs[kSelLoads];
+#pragma unroll
+        for (int j = 0; j < kSelLoads; ++j) {
+            const long long i = base + j * stride + t;
+            if (i < n) cs[j] = p.cand[i];
         }
-        append(listed, i);
-        nv += valid;
-        if constexpr (kKeyHere) {
-            const unsigned m = __ballot_sync(kFull, need);
-            int at = 0;
-            if (lane == 0 && m) at = atomicAdd(s_qn, __popc(m));
-            at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
-            if (need) queue[at] = (int)i;
-            __syncthreads();
-            const int qn = *s_qn;  // the same for the whole block
-            if (qn >= kFinThreads) {
-                drain(qn - kFinThreads, kFinThreads);
-                __syncthreads();  // the entries are read before new ones overwrite them
-                if (t == 0) *s_qn = qn - kFinThreads;
+#pragma unroll
+        for (int j = 0; j < kSelLoads; ++j) {
+            if (base + j * stride >= n) break;  // the same for the whole block
+            const long long i = base + j * stride + t;
+            bool valid = false, listed = false, need = false;
+            if (i < n) {
+                const int u = __float_as_int(cs[j].ds32);
+                const bool top = u >= tlow_bits;
+                need = kKeyHere && isnan(cs[j].key) && (top || u <= dhi_bits);
+                valid = !need && (isnan(cs[j].key) ? in_r(u) : cs[j].key > p.delta_e);
+                listed = top && valid;
+            }
+            append(listed, i);
+            nv += valid;
+            if constexpr (kKeyHere) {
+                const unsigned m = __ballot_sync(kFull, need);
+                int at = 0;
+                if (lane == 0 && m) at = atomicAdd(s_qn, __popc(m));
+                at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
+                if (need) queue[at] = (int)i;
                 __syncthreads();
+                const int qn = *s_qn;  // the same for the whole block
+                if (qn >= kFinThreads) {
+                    drain(qn - kFinThreads, kFinThreads);
+                    __syncthreads();  // the entries are read before new ones overwrite them
+                    if (t == 0) *s_qn = qn - kFinThreads;
+                    __syncthreads();
+                }
             }
         }
     }
