@@ -42,9 +42,9 @@ struct EntState {
     unsigned long long prefix;   // determined high bits (in place)
     double t;                    // result: dS_t = max(dS_0, threshold_delta)
     int done;                    // the solve ended early (no value, rhs <= 0, or dS_0 = 0)
-    int pad;
+    unsigned ticket;             // FP32 fields: blocks of the level that are done
     unsigned long long cnt[256];  // histogram of the current level: counts
-    double sum[256];              // and sums
+    double sum[256];              // and sums (FP32 fields: 64-bit integers in the bin's unit)
 };
 
 // Sticky device status bits.
