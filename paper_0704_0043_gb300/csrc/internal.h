@@ -390,6 +390,7 @@ struct lbm_ctx {
     long long plane = 0;
     size_t elem = 4;
     size_t field_bytes = 0;
+    void *arena = nullptr;  // the one allocation behind the arrays below (but stage and probe)
     void *buf[2] = {nullptr, nullptr};
     int cur = 0;
     lbm::Cand *cand = nullptr;
