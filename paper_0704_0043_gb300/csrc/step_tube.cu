@@ -26,8 +26,10 @@
 //     limiter, no end of the tube, no Ehrenfests' candidate) is finished there
 //     with three vector stores; in any other, the pairs on which nothing acts
 //     are, and an out-of-line function takes the rest, so the walk's registers
-//     hold little more than the common case needs.  Bound by its dependent chains
-//     at 16 warps an SM: 1e7 sites 72 -> 62 us a step; 3e6 sites with all three
+//     hold little more than the common case needs.  Bound by HBM at 1e8
+//     sites (523 -> 414 us, 86 % of the copy rate); at 1e7 (72 -> 62 us a step, 493 ->
+//     331 warp instructions a chunk) by the warps that meet the front's chunks, whose
+//     cold code makes them end later than the others; 3e6 sites with all three
 //     limiters 42 -> 37 us, with 0.5 % of the sites limited 63 -> 62 us; 24 warps at
 //     80 registers spill, 1e7 sites 82 us.  Leaving whole chunks to the function:
 //     62 us, but 72 us with 0.5 % of 3e6 sites limited.
