@@ -2,11 +2,11 @@
  * lbm_batch.h -- many independent lattices stepped together (C ABI of liblbm).
  *
  * A batch holds lattices of different kinds and sizes (D2Q9 cavities, D1Q3
- * tubes; FP32 storage) and advances all of them with one launch of each step
- * kernel per step: every block of the launch looks up which lattice it serves
- * in a device table, so a single grid covers all cavities (the fused kernel)
- * and a second one all other lattices (the tiled kernel), followed by one tail
- * launch with a block per lattice (Ehrenfests' step, FP64 sums).  Each lattice
+ * tubes; FP32 storage) and advances all of them with a few launches per step,
+ * whatever their number: every block of a launch looks up which lattice it serves
+ * in a device table, so one grid covers all cavities with the same limiter code
+ * (the fused kernel), another all tubes and a third all other lattices, each
+ * followed by one tail launch with a block per lattice (Ehrenfests' step, FP64 sums).  Each lattice
  * evolves exactly as it would alone (same per-site arithmetic, bit for bit).
  * Runs of steps can be captured once into a CUDA graph and replayed.  The
  * paper has no batching; the step itself is the one of include/lbm.h
@@ -91,8 +91,8 @@ lbm_status lbm_batch_tune(lbm_batch *b, int32_t trial_steps, double *best_ms);
 
 /* Fixes the fused kernel's work split: seg_rows = rows per work item (a warp
  * walking a strip of 62 columns; 0: automatic, else >= 4), waves 1 .. 64 (with
- * automatic segments: about this many work items per resident warp over the
- * fused lattices together; the items are handed out dynamically).  The split
+ * automatic segments: about this many work items per resident warp of a fused
+ * launch; the items are handed out dynamically).  The split
  * changes the speed only, never a result.  Errors: LBM_ERR_INVALID_ARG. */
 lbm_status lbm_batch_set_shape(lbm_batch *b, int32_t seg_rows, int32_t waves);
 

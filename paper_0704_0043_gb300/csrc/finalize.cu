@@ -31,7 +31,9 @@
 namespace lbm {
 namespace {
 
-constexpr int kSelLoads = 4;  // candidates a thread reads at once in dense_select
+// candidates a thread reads at once in dense_select (2.2 M of a 2048^2 lattice: four steps
+// with set and get 1562 us at one, 1490 at four, 1530 at eight)
+constexpr int kSelLoads = 4;
 constexpr unsigned kSelSpinLimit = 1u << 21;  // grid-barrier polls (about a second) before giving up
 
 // Grid barrier of the cooperative tail: each block adds one arrival to *bar;
