@@ -245,6 +245,12 @@ struct TubeArgs {
 
 // Many steps of a small lattice in one cooperative launch (step_resident.cu).
 constexpr int kResRows = 4;        // steps whose block rows are kept: the tail may lag this far behind
+// Arrival words, a step each in turn.  A word is used again kResSlots steps later.
+// Its readers have then read it: a worker reads step s before it arrives at s + 1,
+// and a worker arrives at step s only when the tail has recorded step
+// s - kResRows - 1 (the row wait of step s - 1), so kResRows + 1 words do.
+constexpr int kResSlots = 8;
+static_assert(kResSlots > kResRows, "an arrival word's readers are done before it is used again");
 constexpr int kResMaxBlocks = 160;
 constexpr int kResMaxSteps = 1024;  // steps of one launch
 // Lattices up to these sizes take the resident kernel.  Measured us per step, resident
@@ -264,7 +270,11 @@ struct ResRow {
     int c[4];     // positivity, median, flagged sites
 };
 struct ResState {
-    unsigned long long arrived;  // low word: worker arrivals; high word: candidates recorded (both since the launch)
+    // low word: worker arrivals, high word: candidates recorded, both of all the
+    // steps of this slot since the launch.  A word per step, because a reader may
+    // be late: a worker by one step, the tail by kResRows.  In one word for all
+    // steps, the candidates of workers that are ahead would count as the step's.
+    unsigned long long arrived[kResSlots];
     unsigned done;               // steps whose candidates are finished
     unsigned stats_done;         // steps whose record is written
     unsigned rows_in[kResRows];  // worker rows written, steps of each slot

@@ -15,8 +15,8 @@
 //  * The last block is the tail: sums, stats record, control point, Ehrenfests'
 //    selection and step (select.cuh).  It works on step s while the workers
 //    already take step s + 1; only a step that recorded candidates makes them
-//    wait for its selection (the arrival counter carries the candidate count, so
-//    a step without any costs no further read).  FP32 / 16-bit storage: the FP64
+//    wait for its selection (the step's arrival counter carries its candidate count,
+//    so a step without any costs no further read).  FP32 / 16-bit storage: the FP64
 //    keys of more than a few candidates are evaluated by all blocks first.
 // The per-site operations are those of the fused, tube and tiled kernels, so the
 // populations are the same bit for bit.  Sums: FP32 storage adds a warp's FP32
@@ -76,14 +76,18 @@ __device__ __forceinline__ bool wait_for(const unsigned *p, unsigned target, uns
     atomicOr(status, kStatTimeout);
     return false;
 }
-// The same on the arrival counter (low word); *cands receives its high word.
-__device__ __forceinline__ bool wait_arrivals(const unsigned long long *p, unsigned target, unsigned *cands,
+// Waits for all W workers' arrivals at step s; *n receives the candidates of the step.
+// seen: the caller's candidate totals of the slots so far.
+__device__ __forceinline__ bool wait_arrivals(const ResState *rs, int s, int W, unsigned *seen, unsigned *n,
                                               unsigned *status)
 {
+    const int slot = s % kResSlots;
+    const unsigned target = (unsigned)W * (unsigned)(s / kResSlots + 1);
     for (unsigned i = 0; i < kResSpin; ++i) {
-        const unsigned long long v = ld_acquire(p);
+        const unsigned long long v = ld_acquire(&rs->arrived[slot]);
         if ((unsigned)v >= target) {
-            *cands = (unsigned)(v >> 32);
+            *n = (unsigned)(v >> 32) - seen[slot];
+            seen[slot] = (unsigned)(v >> 32);
             return true;
         }
     }
@@ -98,7 +102,8 @@ struct WorkShared {
     BlockAcc<kResWarps, T> acc[2];     // the block's sums, steps of each parity
     int ncand[2];
     double fw[2][9];                // diffusive wall: f*(1, u_wall) of the resting walls and of the lid
-    unsigned n;                     // candidates so far (after the barrier)
+    unsigned n;                     // candidates of the step (after the barrier)
+    unsigned seen[kResSlots];       // the waiting thread's: see wait_arrivals
     int go;                         // 0: a wait gave up
 };
 
@@ -331,8 +336,8 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
         w.ncand[t] = 0;
         if (Q == 9 && p.boundary == 4) wall_star(p, t == 1, w.fw[t]);
     }
+    if (t < kResSlots) w.seen[t] = 0;
     __syncthreads();
-    unsigned seen = 0;  // candidates of the steps before
     int tile_no = 0;
     for (int s = 0; s < a.nsteps; ++s) {
         const S *src = (const S *)a.buf[(a.cur + s) & 1];
@@ -342,21 +347,16 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
             do_tile<Q, S>(p, kk, src, dst, tile, a.gx, aw, w.ds[tile_no++ & 1], w.fw, &w.ncand[s & 1], sum);
         __syncthreads();  // the block's sites are stored and its candidates counted
         if (t == 0) {
-            red_release(&a.rs->arrived, 1ull | ((unsigned long long)(unsigned)w.ncand[s & 1] << 32));
+            red_release(&a.rs->arrived[s % kResSlots], 1ull | ((unsigned long long)(unsigned)w.ncand[s & 1] << 32));
             w.ncand[s & 1] = 0;
         }
         if (warp < aw) block_sums<T>(a, w, sum, s, aw);
         const bool end = s + 1 == a.nsteps;
         if (end && !ehr) return;
-        if (t == kPoller) {
-            unsigned total = seen;
-            w.go = wait_arrivals(&a.rs->arrived, (unsigned)W * (unsigned)(s + 1), &total, p.status);
-            w.n = total;
-        }
+        if (t == kPoller) w.go = wait_arrivals(a.rs, s, W, w.seen, &w.n, p.status);
         __syncthreads();
         if (!w.go) return;
-        const unsigned n = w.n - seen;
-        seen = w.n;
+        const unsigned n = w.n;
         if (n > kTailKeys && !std::is_same<S, double>::value) {
             key_share<Q, S>(p, src, (int)n, W);
             __syncthreads();
@@ -380,7 +380,7 @@ struct TailShared {
     FinalParams f;
     double tot[4];
     long long cnt[4];
-    unsigned n;
+    unsigned n, seen[kResSlots];
     int go;
     unsigned status;
 };
@@ -397,22 +397,20 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         for (int i = t; i < (int)(sizeof(FinalParams) / 4); i += kResThreads) to[i] = from[i];
     }
     long long step = a.f.counters[0], rec = a.f.counters[1];
-    unsigned seen = 0, dense = 0;
+    unsigned dense = 0;
+    if (t < kResSlots) h.seen[t] = 0;
     __syncthreads();
     const FinalParams &f = h.f;
     for (int s = 0; s < a.nsteps; ++s) {
         S *dst = (S *)a.buf[(a.cur + s + 1) & 1];
         if (t == 0) {
-            unsigned total = seen;
-            h.go = wait_arrivals(&a.rs->arrived, (unsigned)W * (unsigned)(s + 1), &total, a.p.status);
-            h.n = total;
+            h.go = wait_arrivals(a.rs, s, W, h.seen, &h.n, a.p.status);
             h.f.src = a.buf[(a.cur + s) & 1];
             h.sel.nsel = 0;
         }
         __syncthreads();
         if (!h.go) break;
-        const unsigned n = h.n - seen;
-        seen = h.n;
+        const unsigned n = h.n;
         int n_valid = 0;
         double ehr_sum = 0.0;
         if (n > 0) {
