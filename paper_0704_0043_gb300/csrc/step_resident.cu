@@ -105,6 +105,7 @@ struct WorkShared {
     unsigned n;                     // candidates of the step (after the barrier)
     unsigned seen[kResSlots];       // the waiting thread's: see wait_arrivals
     int go;                         // 0: a wait gave up
+    int stop;                       // 1: the wait for a row's place gave up
 };
 
 // dS(f') of a site outside the tile (0 at boundary nodes and off the lattice).
@@ -268,13 +269,17 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
             is = v.ds > kk.thr_e;
         if (is) {
             atomicAdd(ncand, 1);
-            const int slot = atomicAdd(p.cand_count, 1);  // at most one per site: the list has room
-            Cand c;
-            c.key = F64 ? (double)v.ds : __longlong_as_double(0x7ff8000000000000LL);
-            c.phi = (double)phi;
-            c.site = y * p.nx + x;
-            c.ds32 = (float)v.ds;
-            p.cand[slot] = c;
+            const int slot = atomicAdd(p.cand_count, 1);
+            if (slot < p.cand_cap) {  // at most one per site: always, but after a launch that gave up
+                Cand c;
+                c.key = F64 ? (double)v.ds : __longlong_as_double(0x7ff8000000000000LL);
+                c.phi = (double)phi;
+                c.site = y * p.nx + x;
+                c.ds32 = (float)v.ds;
+                p.cand[slot] = c;
+            } else {
+                atomicOr(p.status, kStatCandOverflow);
+            }
         }
     }
 }
@@ -288,7 +293,8 @@ __device__ __forceinline__ void block_sums(const ResArgs &a, WorkShared<T> &w, c
     const int lane = threadIdx.x & 31, b = s & 1;
     if (!add_warp(w.acc[b], sum, aw)) return;
     // the rows of step s - kResRows are read before this one takes their place
-    if (s >= kResRows && lane == 0) wait_for(&a.rs->stats_done, (unsigned)(s - kResRows + 1), a.p.status);
+    if (s >= kResRows && lane == 0 && !wait_for(&a.rs->stats_done, (unsigned)(s - kResRows + 1), a.p.status))
+        w.stop = 1;  // the block leaves at its next barrier
     __syncwarp();
     take_row(w.acc[b], &a.rs->rows[s % kResRows][blockIdx.x], aw, a.p.status);
     if (lane == 0) red_release(&a.rs->rows_in[s % kResRows], 1u);
@@ -337,6 +343,7 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
         if (Q == 9 && p.boundary == 4) wall_star(p, t == 1, w.fw[t]);
     }
     if (t < kResSlots) w.seen[t] = 0;
+    if (t == 0) w.stop = 0;
     __syncthreads();
     int tile_no = 0;
     for (int s = 0; s < a.nsteps; ++s) {
@@ -355,8 +362,8 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
         if (end && !ehr) return;
         if (t == kPoller) w.go = wait_arrivals(a.rs, s, W, w.seen, &w.n, p.status);
         __syncthreads();
-        if (!w.go) return;
-        const unsigned n = w.n;
+        if (!w.go || w.stop) return;
+        const unsigned n = min(w.n, (unsigned)p.cand_cap);
         if (n > kTailKeys && !std::is_same<S, double>::value) {
             key_share<Q, S>(p, src, (int)n, W);
             __syncthreads();
@@ -410,7 +417,7 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         }
         __syncthreads();
         if (!h.go) break;
-        const unsigned n = h.n;
+        const unsigned n = min(h.n, (unsigned)f.cand_cap);
         int n_valid = 0;
         double ehr_sum = 0.0;
         if (n > 0) {
