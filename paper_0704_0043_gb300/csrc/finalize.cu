@@ -236,6 +236,7 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
         }
         append(listed, i);
     };
+    int queued = 0;  // queue entries, the same in every thread: each counts them itself
     for (long long base = base0; base < n; base += kSelLoads * stride) {  // whole blocks per round
         Cand cs[kSelLoads];
 #pragma unroll
@@ -263,18 +264,19 @@ __device__ __noinline__ bool dense_select(const FinalParams &p, int n, unsigned 
                 if (lane == 0 && m) at = atomicAdd(s_qn, __popc(m));
                 at = __shfl_sync(kFull, at, 0) + __popc(m & ((1u << lane) - 1u));
                 if (need) queue[at] = (int)i;
-                __syncthreads();
-                const int qn = *s_qn;  // the same for the whole block
-                if (qn >= kFinThreads) {
-                    drain(qn - kFinThreads, kFinThreads);
+                // (the count is not read from s_qn: a warp that is ahead adds to it again)
+                queued += __syncthreads_count(need);
+                if (queued >= kFinThreads) {
+                    queued -= kFinThreads;
+                    drain(queued, kFinThreads);
                     __syncthreads();  // the entries are read before new ones overwrite them
-                    if (t == 0) *s_qn = qn - kFinThreads;
+                    if (t == 0) *s_qn = queued;
                     __syncthreads();
                 }
             }
         }
     }
-    if constexpr (kKeyHere) drain(0, *s_qn);
+    if constexpr (kKeyHere) drain(0, queued);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) nv += __shfl_down_sync(kFull, nv, o);
     if (lane == 0 && nv) atomicAdd(s_acc, nv);
