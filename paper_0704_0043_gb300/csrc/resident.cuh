@@ -103,7 +103,7 @@ __device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &s
 // in warp order, FP32 parts exactly (128-bit fixed point, so in any order: lane l
 // takes parts l and l + 32, lanes with one statistic are added by shuffles).
 template <int NW, typename T>
-__device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int warps, unsigned *status)
+__device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int warps)
 {
     const int lane = threadIdx.x & 31;
     double v = 0.0;
@@ -126,11 +126,7 @@ __device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int wa
         if (lane < 4) v = nonfinite & (0x11111111u << lane) ? __longlong_as_double(0x7ff8000000000000LL) : fx_value(fx);
     }
     if (lane < 4) row->v[lane] = v;
-    if (lane < 3) {
-        const int c = w.cnt[lane];
-        row->c[lane] = c;
-        if (lane == 2 && c) atomicOr(status, kStatNonfinite);  // a site was nonfinite
-    }
+    if (lane < 3) row->c[lane] = w.cnt[lane];
     __syncwarp();
     if (lane == 0) w.clear();
     __syncwarp();
@@ -153,11 +149,18 @@ __device__ __forceinline__ void sum_rows(const ResRow *rows, int n, int stat, do
 }
 
 // The stats record of a step from its sums (tot: P_MASS .. P_DS_LIM, cnt: positivity,
-// median, flagged sites).
+// median, flagged sites).  `status`: the recorder's copy of the status word, read
+// when the launch begins and brought on with each step's own flagged sites.  A read of
+// the word itself would see those of later steps: the other blocks are ahead of the
+// record by one step and more.  So only the recorder sets kStatNonfinite there.
 template <bool F64>
 __device__ __forceinline__ DevStats step_record(const ResArgs &a, const double *tot, const long long *cnt,
-                                                double ehr_sum, int nsel, int n_valid, unsigned status, long long step)
+                                                double ehr_sum, int nsel, int n_valid, unsigned &status, long long step)
 {
+    if (cnt[2] != 0 && !(status & kStatNonfinite)) {  // a site was nonfinite
+        status |= kStatNonfinite;
+        atomicOr(a.p.status, kStatNonfinite);
+    }
     DevStats st;
     st.step = step;
     // FP32 storage: the rows hold sums of rho - rho_ref and of the deviations of the

@@ -135,7 +135,8 @@ struct Band {
 };
 
 // The stats record of step s by one warp of the first block.
-__device__ __noinline__ void record_step(const ResArgs &a, const CluShared &sh, int s, long long step0, long long rec0)
+__device__ __noinline__ void record_step(const ResArgs &a, const CluShared &sh, int s, long long step0, long long rec0,
+                                         unsigned &status)
 {
     const int lane = threadIdx.x & 31, slot = s % kCluSlots;
     double tot[4];
@@ -158,7 +159,7 @@ __device__ __noinline__ void record_step(const ResArgs &a, const CluShared &sh, 
         }
     }
     if (lane == 0) {
-        const DevStats st = step_record<false>(a, tot, cnt, 0.0, 0, 0, __ldcg(a.p.status), step0 + s + 1);
+        const DevStats st = step_record<false>(a, tot, cnt, 0.0, 0, 0, status, step0 + s + 1);
         a.f.stats_ring[(rec0 + s) % a.f.ring_len] = st;
         *a.f.sel_count = 0;
     }
@@ -197,6 +198,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
     // threads that carry sites, in whole warps
     const int warps = min(kCluWarps, (sites + 31) / 32);
     const long long step0 = bd.rank == 0 ? a.f.counters[0] : 0, rec0 = bd.rank == 0 ? a.f.counters[1] : 0;
+    unsigned status = *p.status;  // brought on in the recording lane
 
     // the band and its neighbours' edge rows
     {
@@ -343,11 +345,11 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
         }
         cluster_arrive();
         if (warp < warps && add_warp(sh.acc[b], sum, warps))
-            take_row(sh.acc[b], &lead->rows[slot][bd.rank], warps, p.status);
+            take_row(sh.acc[b], &lead->rows[slot][bd.rank], warps);
         cluster_wait();
         if (bd.rank == 0 && warp == kCluWarps - 1) {
             // the rows of the step before are complete since this step's barrier
-            if (s > 0) record_step(a, sh, s - 1, step0, rec0);
+            if (s > 0) record_step(a, sh, s - 1, step0, rec0, status);
             if (a.f.probe != nullptr && lane == 0) {
                 // the control point's moments after the whole step, as lbm_moments gives them
                 float raw[9];
@@ -366,7 +368,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
     }
     cluster_barrier();  // the last rows, and every access to another block's memory
     if (bd.rank == 0 && warp == kCluWarps - 1) {
-        record_step(a, sh, a.nsteps - 1, step0, rec0);
+        record_step(a, sh, a.nsteps - 1, step0, rec0, status);
         if (lane == 0) {
             a.f.counters[0] = step0 + a.nsteps;
             a.f.counters[1] = rec0 + a.nsteps;

@@ -296,7 +296,7 @@ __device__ __forceinline__ void block_sums(const ResArgs &a, WorkShared<T> &w, c
     if (s >= kResRows && lane == 0 && !wait_for(&a.rs->stats_done, (unsigned)(s - kResRows + 1), a.p.status))
         w.stop = 1;  // the block leaves at its next barrier
     __syncwarp();
-    take_row(w.acc[b], &a.rs->rows[s % kResRows][blockIdx.x], aw, a.p.status);
+    take_row(w.acc[b], &a.rs->rows[s % kResRows][blockIdx.x], aw);
     if (lane == 0) red_release(&a.rs->rows_in[s % kResRows], 1u);
 }
 
@@ -389,7 +389,6 @@ struct TailShared {
     long long cnt[4];
     unsigned n, seen[kResSlots];
     int go;
-    unsigned status;
 };
 
 template <int Q, typename S>
@@ -404,7 +403,7 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         for (int i = t; i < (int)(sizeof(FinalParams) / 4); i += kResThreads) to[i] = from[i];
     }
     long long step = a.f.counters[0], rec = a.f.counters[1];
-    unsigned dense = 0;
+    unsigned dense = 0, status = *a.p.status;
     if (t < kResSlots) h.seen[t] = 0;
     __syncthreads();
     const FinalParams &f = h.f;
@@ -437,10 +436,8 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
             ehr_sum = h.sel.nsel > 0 ? block_sum0(ehr_sum, h.sel.red, h.sel.nsel <= 32) : 0.0;
         }
         // the step's sums: every worker's row, in block order
-        if (t == 0) {
+        if (t == 0)
             h.go = wait_for(&a.rs->rows_in[s % kResRows], (unsigned)W * (unsigned)(s / kResRows + 1), a.p.status);
-            h.status = __ldcg(a.p.status);
-        }
         __syncthreads();
         if (!h.go) break;
         if (warp < 4) {
@@ -455,7 +452,7 @@ __device__ __noinline__ void tail_block(const ResArgs &a, TailShared &h)
         __syncthreads();
         if (t == 0) {
             step += 1;
-            const DevStats st = step_record<F64>(a, h.tot, h.cnt, ehr_sum, h.sel.nsel, n_valid, h.status, step);
+            const DevStats st = step_record<F64>(a, h.tot, h.cnt, ehr_sum, h.sel.nsel, n_valid, status, step);
             f.stats_ring[rec % f.ring_len] = st;
             rec += 1;
             if (f.probe != nullptr) {
