@@ -40,35 +40,84 @@ __device__ __forceinline__ void eval_site(const StepParams &p, const ResK &kk, S
     if (v.bad) v.ds = T(INFINITY);
 }
 
+// A sum.  FP64: plain additions.  FP32: the rounding error of each addition is kept
+// beside the sum (Knuth's two-sum) up to the block's row, which is FP64: a thread sums
+// several sites and a boundary node's populations, and the sums are to be no less
+// accurate than those of the kernels that take one step a launch, which go to FP64
+// after one site a lane.  The additions cost a site 20 FP32 instructions.
+template <typename T>
+struct SumOf {
+    T v = T(0);
+    using Total = T;
+    __device__ __forceinline__ void add(T x) { v = Ar<T>::add(v, x); }
+    __device__ __forceinline__ Total total() const { return v; }
+    static __device__ __forceinline__ Total plus(Total a, Total b, bool) { return Ar<T>::add(a, b); }
+    static __device__ __forceinline__ Total from(Total a, int o) { return __shfl_xor_sync(kFull, a, o); }
+};
+template <>
+struct SumOf<float> {
+    float v = 0.f, c = 0.f;
+    using Total = float2;
+    __device__ __forceinline__ void add(float x)
+    {
+        const float t = __fadd_rn(v, x), b = __fsub_rn(t, v);
+        c = __fadd_rn(c, __fadd_rn(__fsub_rn(v, __fsub_rn(t, b)), __fsub_rn(x, b)));
+        v = t;
+    }
+    __device__ __forceinline__ Total total() const { return make_float2(v, c); }
+    static __device__ __forceinline__ Total plus(Total a, Total b, bool plain)
+    {
+        return plain ? make_float2(__fadd_rn(a.x, b.x), 0.f) : df_add(a, b);
+    }
+    static __device__ __forceinline__ Total from(Total a, int o)
+    {
+        return make_float2(__shfl_xor_sync(kFull, a.x, o), __shfl_xor_sync(kFull, a.y, o));
+    }
+};
+
 // Sums of the worker's sites of one step (per thread).
 template <typename T>
 struct ResSums {
-    T mass = T(0), ds = T(0), din = T(0), lim = T(0);
+    SumOf<T> mass, ds, din, lim;
     int pos = 0, med = 0, bad = 0;
 };
 
-// The sums of a warp's step, into lanes 0 (mass), 8 (dS), 16 (dS_in), 24 (dS_lim):
-// a butterfly in which each level halves the sums a lane carries.
+// A boundary node's share of the mass (FP32: of the deviations; see rest_mass).
 template <typename T>
-__device__ __forceinline__ T warp_totals(const ResSums<T> &s, int lane)
+__device__ __forceinline__ void add_wall_mass(const StepParams &p, int x, int y, const T fin[9], SumOf<T> &mass)
 {
-    using A = Ar<T>;
-    const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
-    T a0 = hi16 ? s.din : s.mass, a1 = hi16 ? s.lim : s.ds;
-    const T b0 = hi16 ? s.mass : s.din, b1 = hi16 ? s.ds : s.lim;
-    a0 = A::add(a0, __shfl_xor_sync(kFull, b0, 16));
-    a1 = A::add(a1, __shfl_xor_sync(kFull, b1, 16));
-    T z = hi8 ? a1 : a0;
-    z = A::add(z, __shfl_xor_sync(kFull, hi8 ? a0 : a1, 8));
+    if constexpr (std::is_same<T, double>::value) {
+        mass.add(wall_mass<T>(p, x, y, fin));
+    } else {
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) z = A::add(z, __shfl_xor_sync(kFull, z, o));
+        for (int k = 0; k < 9; ++k)
+            if (wall_counts(p, x, y, k)) mass.add(fin[k]);
+    }
+}
+
+// The sums of a warp's step, into lanes 0 (mass), 8 (dS), 16 (dS_in), 24 (dS_lim):
+// a butterfly in which each level halves the sums a lane carries.  `plain` (FP32): plain
+// additions, for tubes with one site a lane, whose sums are then rounded as those of the
+// kernels that take one step a launch are.
+template <typename T>
+__device__ __forceinline__ typename SumOf<T>::Total warp_totals(const ResSums<T> &s, int lane, bool plain)
+{
+    using O = SumOf<T>;
+    using V = typename O::Total;
+    const V mass = s.mass.total(), ds = s.ds.total(), din = s.din.total(), lim = s.lim.total();
+    const bool hi16 = (lane & 16) != 0, hi8 = (lane & 8) != 0;
+    const V a0 = O::plus(hi16 ? din : mass, O::from(hi16 ? mass : din, 16), plain);
+    const V a1 = O::plus(hi16 ? lim : ds, O::from(hi16 ? ds : lim, 16), plain);
+    V z = O::plus(hi8 ? a1 : a0, O::from(hi8 ? a0 : a1, 8), plain);
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) z = O::plus(z, O::from(z, o), plain);
     return z;
 }
 
 // A block's sums of one step, gathered warp by warp.
 template <int NW, typename T>
 struct BlockAcc {
-    T part[NW][4];  // the warps' sums
+    typename SumOf<T>::Total part[NW][4];  // the warps' sums
     int cnt[3];     // positivity, median, flagged sites
     int ticket;
     __device__ void clear()
@@ -80,10 +129,10 @@ struct BlockAcc {
 
 // Adds a warp's sums; true in the last of the block's `warps` warps to come.
 template <int NW, typename T>
-__device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &sum, int warps)
+__device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &sum, int warps, bool plain)
 {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const T z = warp_totals<T>(sum, lane);
+    const typename SumOf<T>::Total z = warp_totals<T>(sum, lane, plain);
     if ((lane & 7) == 0) w.part[warp][lane >> 3] = z;
     if (__any_sync(kFull, (sum.pos | sum.med | sum.bad) != 0)) {
         const int pos = __reduce_add_sync(kFull, sum.pos), med = __reduce_add_sync(kFull, sum.med);
@@ -99,9 +148,9 @@ __device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &s
     return true;
 }
 
-// The last warp writes the block's row and clears the sums: FP64 parts are added
-// in warp order, FP32 parts exactly (128-bit fixed point, so in any order: lane l
-// takes parts l and l + 32, lanes with one statistic are added by shuffles).
+// The last warp writes the block's row and clears the sums.  FP64 additions in a fixed
+// order: FP64 parts in warp order, FP32 parts (their two halves first) by a tree: lane l
+// takes parts l and l + 32, lanes with one statistic are added by shuffles.
 template <int NW, typename T>
 __device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int warps)
 {
@@ -112,18 +161,12 @@ __device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int wa
             for (int j = 0; j < warps; ++j) v = Ar<double>::add(v, w.part[j][lane]);
     } else {
         static_assert(NW <= 16, "two parts a lane");
-        unsigned __int128 fx = 0;
-        bool bad = false;
-        if (lane >> 2 < warps) fx_add(fx, w.part[lane >> 2][lane & 3], bad);
-        if (8 + (lane >> 2) < warps) fx_add(fx, w.part[8 + (lane >> 2)][lane & 3], bad);
-        const unsigned nonfinite = __ballot_sync(kFull, bad);
+        const float2 none = make_float2(0.f, 0.f);
+        const float2 a = lane >> 2 < warps ? w.part[lane >> 2][lane & 3] : none;
+        const float2 b = 8 + (lane >> 2) < warps ? w.part[8 + (lane >> 2)][lane & 3] : none;
+        v = Ar<double>::add(Ar<double>::add(widen(a.x), widen(a.y)), Ar<double>::add(widen(b.x), widen(b.y)));
 #pragma unroll
-        for (int o = 4; o < 32; o <<= 1) {
-            const unsigned long long lo = __shfl_xor_sync(kFull, (unsigned long long)fx, o);
-            const unsigned long long hi = __shfl_xor_sync(kFull, (unsigned long long)(fx >> 64), o);
-            fx += ((unsigned __int128)hi << 64) | lo;
-        }
-        if (lane < 4) v = nonfinite & (0x11111111u << lane) ? __longlong_as_double(0x7ff8000000000000LL) : fx_value(fx);
+        for (int o = 4; o < 32; o <<= 1) v = Ar<double>::add(v, __shfl_xor_sync(kFull, v, o));
     }
     if (lane < 4) row->v[lane] = v;
     if (lane < 3) row->c[lane] = w.cnt[lane];

@@ -253,21 +253,24 @@ __device__ __forceinline__ void wall_node(const StepParams &p, const S raw[9], i
     }
 }
 
-// The populations of a boundary node that stream back onto the lattice, summed in
-// k order: FP64 storage f itself, FP32 / 16-bit storage the absolute f (W = true)
-// or the deviations alone.
-template <typename T, typename R, bool W>
-__device__ __forceinline__ R wall_mass(const StepParams &p, int x, int y, const T fin[9])
+// Population k of a boundary node streams back onto the lattice, so the mass counts it.
+__device__ __forceinline__ bool wall_counts(const StepParams &p, int x, int y, int k)
 {
-    R m = R(0);
+    const int dx = x + Lat<9>::cx(k), dy = y + Lat<9>::cy(k);
+    return dx >= 0 && dx < p.nx && dy >= 0 && dy < p.ny;
+}
+// Their sum in k order: FP64 storage f itself, FP32 / 16-bit storage the absolute f.
+template <typename T>
+__device__ __forceinline__ double wall_mass(const StepParams &p, int x, int y, const T fin[9])
+{
+    double m = 0.0;
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const int dx = x + Lat<9>::cx(k), dy = y + Lat<9>::cy(k);
-        if (dx >= 0 && dx < p.nx && dy >= 0 && dy < p.ny) {
-            if constexpr (W && std::is_same<T, float>::value)
-                m += (R)fin[k] + p.rw[k];
+        if (wall_counts(p, x, y, k)) {
+            if constexpr (std::is_same<T, float>::value)
+                m += (double)fin[k] + p.rw[k];
             else
-                m = Ar<R>::add(m, (R)fin[k]);
+                m = Ar<double>::add(m, fin[k]);
         }
     }
     return m;

@@ -232,19 +232,19 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
                 const float c = limit_weight(phi, kk.a, true);
 #pragma unroll
                 for (int k = 0; k < 9; ++k) out[k] = fmaf(-c, v.nq[k], v.fin[k]);
-                sum.lim = __fadd_rn(sum.lim, __fmul_rn(__fsub_rn(1.f, __fmul_rn(phi, phi)), v.ds));
+                sum.lim.add(__fmul_rn(__fsub_rn(1.f, __fmul_rn(phi, phi)), v.ds));
             } else {
 #pragma unroll
                 for (int k = 0; k < 9; ++k) out[k] = v.fp[k];
             }
             bd.store(b ^ 1, r, x, out);
-            sum.mass = __fadd_rn(sum.mass, __fsub_rn(v.rho, p.rho_ref));  // each term exact
+            sum.mass.add(__fsub_rn(v.rho, p.rho_ref));  // each term exact
             if (v.bad) {
                 ++sum.bad;
                 return;
             }
-            sum.ds = __fadd_rn(sum.ds, v.ds);
-            sum.din = __fadd_rn(sum.din, v.dsin);
+            sum.ds.add(v.ds);
+            sum.din.add(v.dsin);
         };
         // dS of a site for the medians (its column's copy beyond the other end where the columns wrap)
         auto put_ds = [&](int r, int x, float ds) {
@@ -291,7 +291,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
                 for (int k = 0; k < 9; ++k) raw[k] = at[bd.source(e, k, true)];
                 wall_node<float, float>(p, raw, x, j, sh.fw[wall_lid(p, x, j) ? 1 : 0], fin);
                 bd.store(b ^ 1, r, x, fin);
-                sum.mass = __fadd_rn(sum.mass, wall_mass<float, float, false>(p, x, j, fin));
+                add_wall_mass<float>(p, x, j, fin, sum.mass);
             } else {
                 SiteState<9, float> v;
                 const float phi_pos = evaluate(v, r, x);
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(kCluThreads, 1) k_cluster(const __grid_constan
             }
         }
         cluster_arrive();
-        if (warp < warps && add_warp(sh.acc[b], sum, warps))
+        if (warp < warps && add_warp(sh.acc[b], sum, warps, false))
             take_row(sh.acc[b], &lead->rows[slot][bd.rank], warps);
         cluster_wait();
         if (bd.rank == 0 && warp == kCluWarps - 1) {

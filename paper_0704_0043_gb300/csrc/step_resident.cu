@@ -19,9 +19,9 @@
 //    so a step without any costs no further read).  FP32 / 16-bit storage: the FP64
 //    keys of more than a few candidates are evaluated by all blocks first.
 // The per-site operations are those of the fused, tube and tiled kernels, so the
-// populations are the same bit for bit.  Sums: FP32 storage adds a warp's FP32
-// terms in a fixed order and the warps' totals exactly (128-bit fixed point);
-// FP64 storage adds in FP64 in a fixed order; block rows in block order.
+// populations are the same bit for bit.  Sums, in a fixed order: a thread's and a
+// warp's in the storage's compute type (FP32 with the rounding errors kept beside the
+// sums, see SumOf), block rows in FP64 and in block order.
 // Every wait is bounded (kResSpin polls, over a second); a block that gives up
 // sets kStatTimeout and leaves, and the others follow when their own waits end.
 #include <algorithm>
@@ -224,7 +224,7 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
     if (wall) {
 #pragma unroll
         for (int k = 0; k < Q; ++k) dst[fidx(p.plane, p.pitch, k, y, x)] = f2s<S>(v.fin[k]);
-        if constexpr (Q == 9) sum.mass = A::add(sum.mass, wall_mass<T, T, false>(p, x, y, v.fin));
+        if constexpr (Q == 9) add_wall_mass<T>(p, x, y, v.fin, sum.mass);
         return;
     }
     T phi = T(1);
@@ -238,27 +238,27 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
 #pragma unroll
             for (int k = 0; k < Q; ++k)
                 dst[fidx(p.plane, p.pitch, k, y, x)] = A::add(v.fs[k], A::mul(phi, A::sub(v.fp[k], v.fs[k])));
-            sum.lim = A::add(sum.lim, A::mul(A::sub(1.0, A::mul(phi, phi)), v.ds));
+            sum.lim.add(A::mul(A::sub(1.0, A::mul(phi, phi)), v.ds));
         } else {
             const float c = limit_weight(phi, kk.a, true);
 #pragma unroll
             for (int k = 0; k < Q; ++k) dst[fidx(p.plane, p.pitch, k, y, x)] = f2s<S>(fmaf(-c, v.nq[k], v.fin[k]));
-            sum.lim = __fadd_rn(sum.lim, __fmul_rn(__fsub_rn(1.f, __fmul_rn(phi, phi)), v.ds));
+            sum.lim.add(__fmul_rn(__fsub_rn(1.f, __fmul_rn(phi, phi)), v.ds));
         }
     } else {
 #pragma unroll
         for (int k = 0; k < Q; ++k) dst[fidx(p.plane, p.pitch, k, y, x)] = f2s<S>(v.fp[k]);
     }
     if constexpr (F64)
-        sum.mass = A::add(sum.mass, v.rho);
+        sum.mass.add(v.rho);
     else
-        sum.mass = __fadd_rn(sum.mass, __fsub_rn(v.rho, p.rho_ref));  // each term exact
+        sum.mass.add(__fsub_rn(v.rho, p.rho_ref));  // each term exact
     if (v.bad) {
         ++sum.bad;
         return;
     }
-    sum.ds = A::add(sum.ds, v.ds);
-    sum.din = A::add(sum.din, v.dsin);
+    sum.ds.add(v.ds);
+    sum.din.add(v.dsin);
     if (p.limiters & 2u) {
         // Ehrenfests' candidate: FP64 storage with its key; FP32 / 16-bit storage near
         // or above the threshold, keyed by the tail where it can matter
@@ -287,11 +287,11 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
 // A worker warp's sums of step s into the block's; the block's last warp to come
 // writes the block's row and reports it (the tail reads the rows of a step when
 // every worker has reported).  Runs while the grid barrier completes.
-template <typename T>
+template <int Q, typename T>
 __device__ __forceinline__ void block_sums(const ResArgs &a, WorkShared<T> &w, const ResSums<T> &sum, int s, int aw)
 {
     const int lane = threadIdx.x & 31, b = s & 1;
-    if (!add_warp(w.acc[b], sum, aw)) return;
+    if (!add_warp(w.acc[b], sum, aw, Q == 3 && a.tiles < (int)gridDim.x)) return;
     // the rows of step s - kResRows are read before this one takes their place
     if (s >= kResRows && lane == 0 && !wait_for(&a.rs->stats_done, (unsigned)(s - kResRows + 1), a.p.status))
         w.stop = 1;  // the block leaves at its next barrier
@@ -357,7 +357,7 @@ __device__ __forceinline__ void work_block(const ResArgs &a, WorkShared<compute_
             red_release(&a.rs->arrived[s % kResSlots], 1ull | ((unsigned long long)(unsigned)w.ncand[s & 1] << 32));
             w.ncand[s & 1] = 0;
         }
-        if (warp < aw) block_sums<T>(a, w, sum, s, aw);
+        if (warp < aw) block_sums<Q, T>(a, w, sum, s, aw);
         const bool end = s + 1 == a.nsteps;
         if (end && !ehr) return;
         if (t == kPoller) w.go = wait_arrivals(a.rs, s, W, w.seen, &w.n, p.status);

@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(256) k_tiled(const StepParams p0, const S *__r
 #pragma unroll
                 for (int k = 0; k < 9; ++k) fin[k] = load_as<S, T>(p, src[fidx(p.plane, p.pitch, k, ys, xs)], k);
             }
-            wmass = wall_mass<T, double, true>(p, xs, ys, fin);
+            wmass = wall_mass<T>(p, xs, ys, fin);
         }
     } else if (valid) {
         if (p.collide) {
