@@ -1075,17 +1075,6 @@ __device__ __forceinline__ T med9(T a0, T a1, T a2, T b0, T b1, T b2, T c0, T c1
     return med3(lo, mid, hi);
 }
 
-// Sum of two unevaluated pairs (hi, lo): Knuth's two-sum of the high parts, the
-// low parts and the error renormalised.
-__device__ __forceinline__ float2 df_add(float2 a, float2 b)
-{
-    const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
-    float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
-    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
-    const float hi = __fadd_rn(s, e);
-    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
-}
-
 // Adds the FP32 value v exactly to acc, a 128-bit two's-complement fixed-point
 // number in units of 2^-64 (bits of v below 2^-64 are dropped, truncating
 // toward zero).  A nonfinite v, or |v| >= 2^63, sets `bad` instead.

@@ -44,7 +44,10 @@ __device__ __forceinline__ void eval_site(const StepParams &p, const ResK &kk, S
 // beside the sum (Knuth's two-sum) up to the block's row, which is FP64: a thread sums
 // several sites and a boundary node's populations, and the sums are to be no less
 // accurate than those of the kernels that take one step a launch, which go to FP64
-// after one site a lane.  The additions cost a site 20 FP32 instructions.
+// after one site a lane.  The errors are added apart and not renormalised into the
+// sum, so a level of a tree waits for one addition, not for eight (100 x 100
+// cavity with boundary nodes: 3.8 us a step, 3.9 with renormalised pairs, 3.5 with no
+// errors kept).
 template <typename T>
 struct SumOf {
     T v = T(0);
@@ -60,14 +63,16 @@ struct SumOf<float> {
     using Total = float2;
     __device__ __forceinline__ void add(float x)
     {
-        const float t = __fadd_rn(v, x), b = __fsub_rn(t, v);
-        c = __fadd_rn(c, __fadd_rn(__fsub_rn(v, __fsub_rn(t, b)), __fsub_rn(x, b)));
-        v = t;
+        const Total t = plus(total(), make_float2(x, 0.f), false);
+        v = t.x;
+        c = t.y;
     }
     __device__ __forceinline__ Total total() const { return make_float2(v, c); }
     static __device__ __forceinline__ Total plus(Total a, Total b, bool plain)
     {
-        return plain ? make_float2(__fadd_rn(a.x, b.x), 0.f) : df_add(a, b);
+        const float t = __fadd_rn(a.x, b.x), z = __fsub_rn(t, a.x);
+        const float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(t, z)), __fsub_rn(b.x, z));
+        return make_float2(t, plain ? 0.f : __fadd_rn(__fadd_rn(a.y, b.y), e));
     }
     static __device__ __forceinline__ Total from(Total a, int o)
     {
@@ -148,9 +153,9 @@ __device__ __forceinline__ bool add_warp(BlockAcc<NW, T> &w, const ResSums<T> &s
     return true;
 }
 
-// The last warp writes the block's row and clears the sums.  FP64 additions in a fixed
-// order: FP64 parts in warp order, FP32 parts (their two halves first) by a tree: lane l
-// takes parts l and l + 32, lanes with one statistic are added by shuffles.
+// The last warp writes the block's row and clears the sums, added in a fixed order: FP64
+// parts in warp order, FP32 parts as pairs by a tree (lane l takes parts l and l + 32,
+// lanes with one statistic are added by shuffles), whose two halves FP64 then adds.
 template <int NW, typename T>
 __device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int warps)
 {
@@ -161,12 +166,13 @@ __device__ __forceinline__ void take_row(BlockAcc<NW, T> &w, ResRow *row, int wa
             for (int j = 0; j < warps; ++j) v = Ar<double>::add(v, w.part[j][lane]);
     } else {
         static_assert(NW <= 16, "two parts a lane");
+        using O = SumOf<float>;
         const float2 none = make_float2(0.f, 0.f);
-        const float2 a = lane >> 2 < warps ? w.part[lane >> 2][lane & 3] : none;
-        const float2 b = 8 + (lane >> 2) < warps ? w.part[8 + (lane >> 2)][lane & 3] : none;
-        v = Ar<double>::add(Ar<double>::add(widen(a.x), widen(a.y)), Ar<double>::add(widen(b.x), widen(b.y)));
+        float2 z = O::plus(lane >> 2 < warps ? w.part[lane >> 2][lane & 3] : none,
+                           8 + (lane >> 2) < warps ? w.part[8 + (lane >> 2)][lane & 3] : none, false);
 #pragma unroll
-        for (int o = 4; o < 32; o <<= 1) v = Ar<double>::add(v, __shfl_xor_sync(kFull, v, o));
+        for (int o = 4; o < 32; o <<= 1) z = O::plus(z, O::from(z, o), false);
+        v = Ar<double>::add(widen(z.x), widen(z.y));
     }
     if (lane < 4) row->v[lane] = v;
     if (lane < 3) row->c[lane] = w.cnt[lane];

@@ -298,6 +298,17 @@ __device__ __forceinline__ void kahan2(float2 &s, float2 &c, float2 v)
     s = t;
 }
 
+// Sum of two unevaluated pairs (hi, lo): Knuth's two-sum of the high parts, the
+// low parts and the error renormalised.
+__device__ __forceinline__ float2 df_add(float2 a, float2 b)
+{
+    const float s = __fadd_rn(a.x, b.x), bb = __fsub_rn(s, a.x);
+    float e = __fadd_rn(__fsub_rn(a.x, __fsub_rn(s, bb)), __fsub_rn(b.x, bb));
+    e = __fadd_rn(e, __fadd_rn(a.y, b.y));
+    const float hi = __fadd_rn(s, e);
+    return make_float2(hi, __fsub_rn(e, __fsub_rn(hi, s)));
+}
+
 // FP32 storage: the four totals of the warp's walk, in every lane: a butterfly over
 // the lanes' pairs (each of its first two levels halves the sums a lane carries:
 // lane 0 ends with mass, 8 dS, 16 dS_in, 24 dS_lim), then one conversion.  V = 1:
