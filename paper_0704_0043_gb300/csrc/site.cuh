@@ -71,18 +71,21 @@ __device__ __forceinline__ double fixed_value(long long v, int e)
 
 // rho, u of a site's stored populations (Eq. macro_dis; lbm_moments and the control
 // point).  FP64 storage: the FP64 formula.  FP32 / 16-bit storage: the sums of the
-// deviations in fixed point, each rounded once to 2^(exponent of rho_ref - 55) and
-// held as a high and a low 32-bit part (|g| < 2^exponent: nine of them do not
-// overflow), the sums exact and added to rho_ref sum W in units of 2^(exponent - 58)
-// (every rho_ref W_k is a whole number of them); the quotients from one reciprocal,
-// corrected by their residuals.  That is eight FP64 instructions (five for D1Q3),
-// and no less exact than the FP64 sums, which round every population and every sum.
+// deviations in fixed point, in units of 2^(exponent of rho_ref - 58): a deviation below
+// 2^exponent in size as a high part of 28 bits and a low part of 31, rounded once, so
+// exact for deviations of at least 2^(exponent - 35) and off by at most half a unit
+// below.  (The FP64 sum rounds a population to its own last place: half a unit on the
+// diagonals of D2Q9 at rho_ref = 1, two units on the axes.)  The sums are exact and added
+// to rho_ref sum W (every rho_ref W_k is a whole number of units); the quotients from one
+// reciprocal, corrected by their residuals.  That is eight FP64 instructions (five for
+// D1Q3), and no less exact than the FP64 sums, which round every sum too.
 // A site with a deviation of rho_ref or more, or rho <= 0, takes the FP64 formula.
 template <int Q, typename S, typename P>
 __device__ __forceinline__ void site_moments(const P &p, const S raw[Q], double &rho, double &ux, double &uy)
 {
     if constexpr (!std::is_same<S, double>::value) {
-        int h[3] = {0, 0, 0}, l[3] = {0, 0, 0};  // sums of g, c_x g, c_y g
+        int h[3] = {0, 0, 0};  // sums of g, c_x g, c_y g: at most nine of 2^27,
+        long long l[3] = {0, 0, 0};  // and of 2^30
         bool plain = true;
 #pragma unroll
         for (int k = 0; k < Q; ++k) {
@@ -90,15 +93,15 @@ __device__ __forceinline__ void site_moments(const P &p, const S raw[Q], double 
             plain = plain && fabsf(g) < p.mfx.lim;
             const float x = __fmul_rn(g, p.mfx.scale);  // below 2^27, exact
             const int hi = __float2int_rn(x);
-            const int lo = __float2int_rn(__fmul_rn(__fsub_rn(x, __int2float_rn(hi)), 268435456.0f));
+            const int lo = __float2int_rn(__fmul_rn(__fsub_rn(x, __int2float_rn(hi)), 2147483648.0f));
             h[0] += hi;
             l[0] += lo;
             h[1] += Lat<Q>::cx(k) * hi;
-            l[1] += Lat<Q>::cx(k) * lo;
+            l[1] += (long long)Lat<Q>::cx(k) * lo;
             h[2] += Lat<Q>::cy(k) * hi;
-            l[2] += Lat<Q>::cy(k) * lo;
+            l[2] += (long long)Lat<Q>::cy(k) * lo;
         }
-        auto units = [&](int j) { return (long long)h[j] * (1ll << 31) + (long long)l[j] * 8; };
+        auto units = [&](int j) { return (long long)h[j] * (1ll << 31) + l[j]; };
         const long long r = p.mfx.rest + units(0), jx = units(1), jy = units(2);
         if (plain && r > 0) {
             bool slow = false;
