@@ -143,20 +143,29 @@ struct SelShared {
     int nsel, valid, count, tlow;
 };
 
-// FP32 dS bit pattern from which a candidate can be among the k largest: T
-// (1 - 1/32), T a lower bound of the k-th largest FP32 dS among the candidates
-// R that are certainly above delta (FP32 dS above delta (1 + 1/64); finite).
-// 0 when R has fewer than k.  The FP32 dS is within 1/64 of the FP64 key, so a
-// candidate below that bound cannot reach the k-th largest key.  `keyed`: every
-// candidate has its key and the patterns are the keys rounded, which order as the
-// keys do, so T itself is the bound.  Every thread of the block calls it.
+// The FP32 bit pattern that candidate i is placed by: of its key rounded, or, with the key
+// owed, of the FP32 dS it was recorded on.
+__device__ __forceinline__ int cand_pattern(const FinalParams &p, int i, bool small, const SelShared &sh)
+{
+    if (small) return __float_as_int(sh.ds[i]);
+    const double key = p.cand[i].key;
+    return __float_as_int(isnan(key) ? p.cand[i].ds32 : narrow(key));
+}
+
+// Pattern from which a candidate can be among the k largest: of T (1 - 1/32), T a lower
+// bound of the k-th largest among the candidates R that are certainly above delta
+// (pattern above that of delta (1 + 1/64); finite).  0 when R has fewer than k.  The FP32
+// dS is within 1/64 of the FP64 key (the caller sees to that: mark_unsure), so a
+// candidate below that bound cannot reach the k-th largest key.  `keyed`: every candidate
+// has its key, and rounded they order as the keys do, so T itself is the bound.  Every
+// thread of the block calls it.
 template <typename S>
 __device__ __noinline__ int fp32_bound(const FinalParams &p, int n, bool small, bool keyed, SelShared &sh)
 {
     const int t = threadIdx.x, lane = t & 31;
     const long long k = p.k_max;
     const int dhi_bits = __float_as_int((float)(p.delta_e * (1.0 + 1.0 / 64.0)));
-    auto u = [&](int i) -> int { return __float_as_int(small ? sh.ds[i] : p.cand[i].ds32); };
+    auto u = [&](int i) -> int { return cand_pattern(p, i, small, sh); };
     auto in_r = [&](int v) { return v > dhi_bits && v < 0x7f800000; };
     if (t == 0) {
         sh.tlow = 0;
@@ -206,6 +215,42 @@ __device__ __noinline__ int fp32_bound(const FinalParams &p, int n, bool small, 
         __syncthreads();
     }
     return keyed ? sh.tlow - 1 : __float_as_int(__int_as_float(sh.tlow) * 0.96875f);
+}
+
+// Where the FP32 dS stands for the key: within 1/64 of it.  dS is the square of a norm of
+// n = f - f*, whose FP32 error is a few 2^-24 of the largest f*, over sqrt(f*_k) in the
+// norm: with every f*_k at least rho_ref / 256 and rho at most 2 rho_ref, below
+// 3e-5 sqrt(rho_ref), so dS of 1e-5 rho_ref and more is within 1/64 (delta of at least
+// kSureDelta rho_ref leaves a margin of six).  Entropic f*: the exact dS of a population
+// near zero may be finite in FP32 and +inf in the key, so it never stands for it.
+// Elsewhere every owed key is evaluated.
+constexpr double kSureDelta = 1.0 / 16384.0;
+constexpr float kSureFeq = 1.0f / 256.0f, kSureRho = 2.0f;
+__device__ __forceinline__ bool sure_delta(const FinalParams &p)
+{
+    return p.eq != 1 && p.delta_e >= kSureDelta * (double)p.rho_ref;
+}
+// Owed candidates outside those limits of f* and rho get an FP32 dS of +inf: no member of
+// R (see fp32_bound), and above every bound, so they are keyed.
+template <int Q, typename S>
+__device__ __noinline__ void mark_unsure(const FinalParams &p, int n, bool small, SelShared &sh)
+{
+    for (int i = threadIdx.x; i < n; i += kFinThreads) {
+        if (!isnan(small ? sh.key[i] : p.cand[i].key)) continue;
+        const int site = small ? sh.site[i] : p.cand[i].site;
+        float g[Q], gs[Q], drho, rho, ux, uy, least = 3.4e38f;
+        pull_dev<Q, S>(p, site % p.nx, site / p.nx, g);
+        moments_dev<Q>(g, p.rho_ref, drho, rho, ux, uy);
+        feq_dev<Q>(drho, rho, ux, uy, gs);
+#pragma unroll
+        for (int k = 0; k < Q; ++k) least = fminf(least, (float)p.rw[k] + gs[k]);
+        if (least >= kSureFeq * p.rho_ref && rho <= kSureRho * p.rho_ref) continue;
+        if (small)
+            sh.ds[i] = INFINITY;
+        else
+            p.cand[i].ds32 = INFINITY;
+    }
+    __syncthreads();
 }
 
 // The owed keys of a pass's n candidates (see finish_candidates); returns this
@@ -401,7 +446,8 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
 // Every thread of a block of kFinThreads calls it, n > 0.
 //
 // Keys are owed (NaN) by FP32 and 16-bit passes.  Only the candidates that can
-// reach the k largest by their FP32 dS, and those within 1/64 of delta, get one:
+// reach the k largest by their FP32 dS, those within 1/64 of delta and those whose FP32
+// dS is not sure get one:
 // FP64 is slow on this GPU (one block keying every candidate of a 517 x 389
 // cavity, several hundred with k = 20, took 25 us a step), and the others' count
 // is certain without it.  A few are keyed three to a warp (a lane per
@@ -479,20 +525,27 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
         }
         owed = __syncthreads_or(owed) != 0;
         if (!use_list) {
-            // FP32 dS pattern below which a candidate cannot be among the k largest
+            // FP32 dS pattern below which a candidate cannot be among the k largest; 0
+            // where the FP32 dS of owed keys does not stand for them
             int tlow = 0;
-            if (k <= 0)
-                tlow = 0x7f800001;
-            else if (n > kRank32 || (owed && n > k))
-                tlow = fp32_bound<S>(p, n, small, small && !owed, sh);
+            if (!owed || sure_delta(p)) {
+                if constexpr (kLowPrec) {
+                    if (owed) mark_unsure<Q, S>(p, n, small, sh);
+                }
+                if (k <= 0)
+                    tlow = 0x7f800000;
+                else if (n > kRank32 || (owed && n > k))
+                    tlow = fp32_bound<S>(p, n, small, !owed, sh);
+            }
             int nv = 0;  // candidates counted as valid here without a key, then those with one
             if constexpr (kLowPrec) {
                 if (owed) nv = settle_owed<Q, S>(p, n, small, tlow, sh);
             }
             for (int i = t; i < n; i += kFinThreads) {
+                const int v = cand_pattern(p, i, small, sh);  // every candidate is keyed or counted (-1) now
                 double key = settle(key_of(i));
                 nv += (long long)key_bits(key) > 0;
-                if (__float_as_int(small ? sh.ds[i] : p.cand[i].ds32) < tlow) key = -1.0;  // counted, out of play
+                if (v < tlow) key = -1.0;  // counted, out of play
                 if (small)
                     sh.key[i] = key;
                 else
