@@ -298,10 +298,12 @@ lbm_status lbm_probe(lbm_ctx *ctx, int64_t site, int64_t capacity);
  * Errors: LBM_ERR_STATE (no probe set), LBM_ERR_INVALID_ARG. */
 lbm_status lbm_probe_read(lbm_ctx *ctx, double *out, int64_t cap, int64_t *n);
 
-/* CUDA-graph replay for lbm_step: runs of `steps_per_graph` steps (an even
- * number >= 2; 0 turns replay off) are captured once per starting buffer into a
- * CUDA graph on a stream of the context's own and replayed on the context's
- * stream, which removes the per-launch host cost of small lattices.  The steps
+/* CUDA-graph replay for lbm_step, for lattices that are stepped launch by launch
+ * (those that LBM_KERNEL_AUTO steps many at a time in one launch are not
+ * captured: they have no launches to save): runs of `steps_per_graph` steps (an
+ * even number >= 2; 0 turns replay off) are captured once per starting buffer into
+ * a CUDA graph on a stream of the context's own and replayed on the context's
+ * stream, which removes the per-launch host cost.  The steps
  * and their results are those of plain lbm_step calls.  While per-kernel timing
  * (lbm_timing) is on, lbm_step launches plainly.  The first replay of each
  * starting buffer captures its graph; make it before any stream capture of the
@@ -309,7 +311,7 @@ lbm_status lbm_probe_read(lbm_ctx *ctx, double *out, int64_t cap, int64_t *n);
 lbm_status lbm_set_graph(lbm_ctx *ctx, int32_t steps_per_graph);
 
 /* Per-kernel timing with CUDA events recorded on the context's stream.  While
- * enabled, a timed step records an event before its step kernel, one between
+ * enabled, a timed step is launched on its own and records an event before its step kernel, one between
  * the step kernel and its one-block tail kernel, and one after the tail.
  * enable = 0 turns timing off, 1 times every step, N > 1 times one step in N
  * (the first, then every N-th: events between the kernels also delay the
@@ -320,8 +322,11 @@ lbm_status lbm_set_graph(lbm_ctx *ctx, int32_t steps_per_graph);
 lbm_status lbm_timing(lbm_ctx *ctx, int32_t enable);
 lbm_status lbm_timing_read(lbm_ctx *ctx, double *step_kernel_ms, double *tail_kernel_ms, int64_t *steps);
 
-/* The step kernel lbm_step launches for this context: LBM_KERNEL_TILED,
- * LBM_KERNEL_FUSED or LBM_KERNEL_TUBE (-1 for a NULL context). */
+/* The step kernel of this context's single steps: LBM_KERNEL_TILED,
+ * LBM_KERNEL_FUSED or LBM_KERNEL_TUBE (-1 for a NULL context).  lbm_step launches
+ * it for each step, but for the small lattices whose steps LBM_KERNEL_AUTO takes
+ * many at a time: there it is the kernel of the steps that lbm_timing samples, of
+ * those under a stream capture and of batches. */
 int32_t lbm_step_kernel(const lbm_ctx *ctx);
 
 /* Number of kernel launches the context has enqueued so far. */
