@@ -143,13 +143,31 @@ struct SelShared {
     int nsel, valid, count, tlow;
 };
 
+// use(i, load(i)) for this thread's entries i of 0 .. n - 1, four loads at a time: on a
+// list that shared memory does not hold, the block's 16 warps do not hide the latency of
+// one load each (10^6 keyed candidates of a tube, set and four steps: 16.3 ms one at a
+// time, 6.3 four at a time).
+template <typename Load, typename Use>
+__device__ __forceinline__ void over_entries(int n, Load load, Use use)
+{
+    constexpr int kLoads = 4;
+    for (int b = threadIdx.x; b < n; b += kLoads * kFinThreads) {
+        decltype(load(0)) v[kLoads];
+#pragma unroll
+        for (int j = 0; j < kLoads; ++j) v[j] = load(min(b + j * kFinThreads, n - 1));
+#pragma unroll
+        for (int j = 0; j < kLoads; ++j)
+            if (b + j * kFinThreads < n) use(b + j * kFinThreads, v[j]);
+    }
+}
+
 // The FP32 bit pattern that candidate i is placed by: of its key rounded, or, with the key
 // owed, of the FP32 dS it was recorded on.
 __device__ __forceinline__ int cand_pattern(const FinalParams &p, int i, bool small, const SelShared &sh)
 {
     if (small) return __float_as_int(sh.ds[i]);
     const double key = p.cand[i].key;
-    return __float_as_int(isnan(key) ? p.cand[i].ds32 : narrow(key));
+    return __float_as_int(nan64(key) ? p.cand[i].ds32 : narrow(key));
 }
 
 // Pattern from which a candidate can be among the k largest: of T (1 - 1/32), T a lower
@@ -236,7 +254,7 @@ template <int Q, typename S>
 __device__ __noinline__ void mark_unsure(const FinalParams &p, int n, bool small, SelShared &sh)
 {
     for (int i = threadIdx.x; i < n; i += kFinThreads) {
-        if (!isnan(small ? sh.key[i] : p.cand[i].key)) continue;
+        if (!nan64(small ? sh.key[i] : p.cand[i].key)) continue;
         const int site = small ? sh.site[i] : p.cand[i].site;
         float g[Q], gs[Q], drho, rho, ux, uy, least = 3.4e38f;
         pull_dev<Q, S>(p, site % p.nx, site / p.nx, g);
@@ -270,7 +288,7 @@ __device__ __noinline__ int settle_owed(const FinalParams &p, int n, bool small,
     __syncthreads();
     for (int i = t; i < n; i += kFinThreads) {
         const double key = small ? sh.key[i] : p.cand[i].key;
-        if (!isnan(key)) continue;
+        if (!nan64(key)) continue;
         const int v = u(i);
         if (v >= tlow || v <= dhi_bits) {
             if (small) {
@@ -335,11 +353,12 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
                                         SelShared &sh)
 {
     const int t = threadIdx.x;
-    const int *list = use_list ? p.sel_state->list : nullptr;
+    const int *const list = use_list ? p.sel_state->list : nullptr;
+    const Cand *const cand = p.cand;
     const long long k = p.k_max;
     auto cidx = [&](int i) -> int { return use_list ? list[i] : i; };
-    auto key_of = [&](int i) -> double { return small ? sh.key[i] : p.cand[cidx(i)].key; };
-    auto site_of = [&](int i) -> int { return small ? sh.site[i] : p.cand[cidx(i)].site; };
+    auto key_of = [&](int i) -> double { return small ? sh.key[i] : cand[cidx(i)].key; };
+    auto site_of = [&](int i) -> int { return small ? sh.site[i] : cand[cidx(i)].site; };
     unsigned long long kv = 0;  // threshold dS pattern
     int site_thr = 0x7fffffff;
     if (!take_all) {
@@ -348,11 +367,10 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
         for (int shift = 56; shift >= 0; shift -= 8) {
             for (int d = t; d < 256; d += kFinThreads) sh.hist[d] = 0;
             __syncthreads();
-            for (int i = t; i < n; i += kFinThreads) {
-                const double key = key_of(i);
+            over_entries(n, key_of, [&](int, double key) {
                 const unsigned long long u = key_bits(key);
                 if ((long long)u > 0 && (u & mask) == prefix) atomicAdd(&sh.hist[(u >> shift) & 255u], 1u);
-            }
+            });
             __syncthreads();
             pick_digit(sh.hist, rem, true, sh.part, &sh.digit, &sh.rem);
             prefix = prefix | (sh.digit << shift);
@@ -366,12 +384,11 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
         for (int shift = 24; shift >= 0; shift -= 8) {
             for (int d = t; d < 256; d += kFinThreads) sh.hist[d] = 0;
             __syncthreads();
-            for (int i = t; i < n; i += kFinThreads) {
-                const double key = key_of(i);
+            over_entries(n, key_of, [&](int i, double key) {
+                if ((long long)key_bits(key) <= 0 || key_bits(key) != kv) return;
                 const unsigned s = (unsigned)site_of(i);
-                if ((long long)key_bits(key) > 0 && key_bits(key) == kv && (s & smask) == sprefix)
-                    atomicAdd(&sh.hist[(s >> shift) & 255u], 1u);
-            }
+                if ((s & smask) == sprefix) atomicAdd(&sh.hist[(s >> shift) & 255u], 1u);
+            });
             __syncthreads();
             pick_digit(sh.hist, rem, false, sh.part, &sh.digit, &sh.rem);
             sprefix = sprefix | ((unsigned)sh.digit << shift);
@@ -384,15 +401,15 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
     // compaction of the chosen candidates: candidate indices in p.sel, list
     // entries in sh.idx (the first kCap)
     __syncthreads();
-    for (int i = t; i < n; i += kFinThreads) {
-        const unsigned long long u = key_bits(key_of(i));
+    over_entries(n, key_of, [&](int i, double key) {
+        const unsigned long long u = key_bits(key);
         const bool chosen = (long long)u > 0 && (take_all || u > kv || (u == kv && site_of(i) <= site_thr));
         if (chosen) {
             const int j = atomicAdd(&sh.nsel, 1);
             if (j < p.sel_cap) p.sel[j] = cidx(i);
             if (j < kCap) sh.idx[j] = i;
         }
-    }
+    });
     __syncthreads();
     if (t == 0 && sh.nsel > p.sel_cap) sh.nsel = p.sel_cap;
     __syncthreads();
@@ -436,6 +453,29 @@ __device__ __noinline__ int choose_many(const FinalParams &p, int n, bool use_li
     return nsel;
 }
 
+// More candidates than shared memory holds: whether this thread's have one without its
+// key; and, all keyed or counted (-1), those above delta counted and the others, and
+// those below the bound, put out of play.  Out of line, as settle_owed is.
+__device__ __noinline__ bool any_owed(const FinalParams &p, int n)
+{
+    const Cand *const cand = p.cand;
+    bool owed = false;
+    over_entries(n, [&](int i) { return cand[i].key; }, [&](int, double key) { owed = owed || nan64(key); });
+    return owed;
+}
+__device__ __noinline__ int settle_many(const FinalParams &p, int n, int tlow)
+{
+    Cand *const cand = p.cand;
+    const double delta = p.delta_e;
+    int nv = 0;
+    over_entries(n, [&](int i) { return cand[i].key; }, [&](int i, double key) {
+        const bool valid = above64(key, delta);
+        nv += valid && (long long)key_bits(key) > 0;
+        if (!valid || (tlow > 0 && __float_as_int(narrow(key)) < tlow)) cand[i].key = -1.0;
+    });
+    return nv;
+}
+
 // The candidates of a pass: FP64 keys where they are owed, the count n_valid of
 // candidates above delta, the k with the largest keys (ties to the lower site),
 // Ehrenfests' step at those.  List entry i < n is candidate i, or with use_list
@@ -469,7 +509,9 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
     auto site_of = [&](int i) -> int { return small ? sh.site[i] : p.cand[cidx(i)].site; };
     // below the threshold -> -1, so that from here on a key is valid exactly
     // when its bit pattern is a positive integer
-    auto settle = [&](double key) { return key > p.delta_e ? key : -1.0; };
+    // (compared as integers, as everywhere below: an FP64 comparison takes the FP64 unit
+    // as long as an addition does, and a keyed candidate is no NaN)
+    auto settle = [&](double key) { return above64(key, p.delta_e) ? key : -1.0; };
     int nsel = 0;         // chosen sites (few: in the first warp only)
     bool listed = false;  // the chosen list entries are in sh.idx
     const bool few = n <= 32 && !use_list;
@@ -482,12 +524,12 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
         if (preloaded && warp != 0 && lane < n) c = p.cand[lane];
         bool owed = false;
         if constexpr (kLowPrec) {
-            owed = __any_sync(kFull, lane < n && isnan(c.key));
+            owed = __any_sync(kFull, lane < n && nan64(c.key));
             if (owed) key_few<Q, S>(p, n, c.site, sh);  // every warp takes three
         }
         if (warp == 0) {
             if (owed) c.key = lane < n ? sh.key[lane] : -1.0;
-            const bool valid = lane < n && c.key > p.delta_e;
+            const bool valid = lane < n && above64(c.key, p.delta_e);
             n_valid = __popc(__ballot_sync(kFull, valid));
             nsel = k < (long long)n_valid ? (int)(k > 0 ? k : 0) : n_valid;
             const long long u = valid ? (long long)key_bits(c.key) : -1;
@@ -512,21 +554,24 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
             if (!use_list) sh.valid = 0;
             sh.count = 0;
         }
-        if (small || !use_list) {
+        if (small) {
             for (int i = t; i < n; i += kFinThreads) {
                 const Cand c = preloaded && i == t ? first : p.cand[cidx(i)];
-                owed = owed || isnan(c.key);
-                if (small) {
-                    sh.key[i] = c.key;
-                    sh.site[i] = c.site;
-                    sh.ds[i] = isnan(c.key) ? c.ds32 : (float)c.key;
-                }
+                owed = owed || (kLowPrec && nan64(c.key));
+                sh.key[i] = c.key;
+                sh.site[i] = c.site;
+                sh.ds[i] = nan64(c.key) ? c.ds32 : narrow(c.key);
             }
+        } else if (kLowPrec && !use_list) {
+            owed = any_owed(p, n);
         }
         owed = __syncthreads_or(owed) != 0;
         if (!use_list) {
             // FP32 dS pattern below which a candidate cannot be among the k largest; 0
-            // where the FP32 dS of owed keys does not stand for them
+            // where the FP32 dS of owed keys does not stand for them, and where it would
+            // spare nothing: choose_many goes over all entries of a list that shared
+            // memory does not hold, dropped or not (10^6 keyed candidates of a tube, set
+            // and four steps: 23.6 ms with the bound's passes, 17.1 without)
             int tlow = 0;
             if (!owed || sure_delta(p)) {
                 if constexpr (kLowPrec) {
@@ -534,22 +579,23 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
                 }
                 if (k <= 0)
                     tlow = 0x7f800000;
-                else if (n > kRank32 || (owed && n > k))
+                else if ((small && n > kRank32) || (owed && n > k))
                     tlow = fp32_bound<S>(p, n, small, !owed, sh);
             }
             int nv = 0;  // candidates counted as valid here without a key, then those with one
             if constexpr (kLowPrec) {
                 if (owed) nv = settle_owed<Q, S>(p, n, small, tlow, sh);
             }
-            for (int i = t; i < n; i += kFinThreads) {
-                const int v = cand_pattern(p, i, small, sh);  // every candidate is keyed or counted (-1) now
-                double key = settle(key_of(i));
-                nv += (long long)key_bits(key) > 0;
-                if (v < tlow) key = -1.0;  // counted, out of play
-                if (small)
+            // every candidate is keyed or counted (-1) now
+            if (small) {
+                for (int i = t; i < n; i += kFinThreads) {
+                    double key = settle(sh.key[i]);
+                    nv += (long long)key_bits(key) > 0;
+                    if (__float_as_int(sh.ds[i]) < tlow) key = -1.0;  // counted, out of play
                     sh.key[i] = key;
-                else
-                    p.cand[i].key = key;
+                }
+            } else {
+                nv += settle_many(p, n, tlow);
             }
             nv = __reduce_add_sync(kFull, nv);
             if (lane == 0 && nv) atomicAdd(&sh.valid, nv);
