@@ -523,20 +523,39 @@ double rest_mass(const StepParams &p)
     return m;
 }
 
+// Time of one round of a worker, a tile of `rows` rows of 32 sites, in units that only
+// compare.  FP64: its units bound a round, 12.5 / 20 / 37.3 us for 4 / 8 / 16 rows of
+// D2Q9 (tubes: a third, in the same proportion).  FP32 and 16-bit: latency does, 1.4 us
+// and 0.06 a row.  us a step at 4 / 8 / 16 rows:
+//   FP32 cavities 100^2 12.4 / 12.1 / 12.3, 200^2 15.7 / 14.3 / 12.1, 400^2 24.6 / 18.4 /
+//   16.9, 2000 x 100 28.4 / 20.7 / 16.8, boundary nodes 150^2 8.2 / 5.1 / 5.6;
+//   FP64 cavities 100^2 30.8 / 31.6 / 46.1, 200^2 55 / 59 / 46, 400^2 123 / 117 / 133,
+//   700^2 317 / 266 / 276;
+//   tubes FP32 2e5 13.1 / 11.1 / 9.8, 7e5 26.9 / 18.2 / 13.3; FP64 5e5 124 / 100 / 106.
+int round_cost(bool fp64, int rows)
+{
+    if (!fp64) return rows + 22;
+    if (rows <= 4) return 250;
+    if (rows <= 8) return 250 + (rows - 4) * 150 / 4;
+    return 400 + (rows - 8) * 346 / 8;
+}
+
 template <typename S>
 cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s)
 {
-    // warps that carry sites (rows of a tile): the least work of the busiest SM,
-    // rounds x warps, and of those the fewest rounds
+    // warps that carry sites (rows of a tile): the least time of the busiest SM, its rounds
+    // times the time of one (see round_cost), rows beyond the lattice left out
     const int workers = std::min(sm_count(), kResMaxBlocks) - 1;
     auto tiles_for = [&](int aw) {
         if (q == 3) return (a.p.nx + 32 * aw - 1) / (32 * aw);
         return ((a.p.nx + 31) / 32) * ((a.p.ny + aw - 1) / aw);
     };
-    int aw = 4, best = 1 << 30;
+    int aw = 4;
+    long long best = -1;
     for (int w = 4; w <= kResWarps; w *= 2) {
-        const int cost = (tiles_for(w) + workers - 1) / workers * w;
-        if (cost <= best) aw = w, best = cost;
+        const long long rounds = (tiles_for(w) + workers - 1) / workers;
+        const long long cost = rounds * round_cost(std::is_same<S, double>::value, q == 3 ? w : std::min(w, a.p.ny));
+        if (best < 0 || cost < best) aw = w, best = cost;
     }
     a.aw = aw;
     a.gx = q == 3 ? 1 : (a.p.nx + 31) / 32;
