@@ -239,30 +239,31 @@ __device__ __noinline__ int fp32_bound(const FinalParams &p, int n, bool small, 
 // n = f - f*, whose FP32 error is a few 2^-24 of the largest f*, over sqrt(f*_k) in the
 // norm: with every f*_k at least rho_ref / 256 and rho at most 2 rho_ref, below
 // 3e-5 sqrt(rho_ref), so dS of 1e-5 rho_ref and more is within 1/64 (delta of at least
-// kSureDelta rho_ref leaves a margin of six).  Entropic f*: the exact dS of a population
-// near zero may be finite in FP32 and +inf in the key, so it never stands for it.
-// Elsewhere every owed key is evaluated.
+// kSureDelta rho_ref leaves a margin of six).  As f*_k >= rho W_k (1 - 3 u^2) / 2 (D1Q3:
+// rho W_k / 4), rho (1 - 3 u^2) of at least kSureFlow rho_ref suffices.  Entropic f*: the
+// exact dS of a population near zero may be finite in FP32 and +inf in the key, so it
+// never stands for it.  Elsewhere every owed key is evaluated.
 constexpr double kSureDelta = 1.0 / 16384.0;
-constexpr float kSureFeq = 1.0f / 256.0f, kSureRho = 2.0f;
+constexpr float kSureFlow = 72.0f / 256.0f, kSureRho = 2.0f;
 __device__ __forceinline__ bool sure_delta(const FinalParams &p)
 {
     return p.eq != 1 && p.delta_e >= kSureDelta * (double)p.rho_ref;
 }
-// Owed candidates outside those limits of f* and rho get an FP32 dS of +inf: no member of
-// R (see fp32_bound), and above every bound, so they are keyed.
+// Owed candidates outside those limits of rho and u get an FP32 dS of +inf: no member of
+// R (see fp32_bound), and above every bound, so they are keyed.  (Tested at the candidates
+// and not where they are recorded: a test there cost the step kernel registers, 256
+// batched cavities 1.3 %.)
 template <int Q, typename S>
 __device__ __noinline__ void mark_unsure(const FinalParams &p, int n, bool small, SelShared &sh)
 {
     for (int i = threadIdx.x; i < n; i += kFinThreads) {
         if (!nan64(small ? sh.key[i] : p.cand[i].key)) continue;
         const int site = small ? sh.site[i] : p.cand[i].site;
-        float g[Q], gs[Q], drho, rho, ux, uy, least = 3.4e38f;
+        float g[Q], drho, rho, ux, uy;
         pull_dev<Q, S>(p, site % p.nx, site / p.nx, g);
         moments_dev<Q>(g, p.rho_ref, drho, rho, ux, uy);
-        feq_dev<Q>(drho, rho, ux, uy, gs);
-#pragma unroll
-        for (int k = 0; k < Q; ++k) least = fminf(least, (float)p.rw[k] + gs[k]);
-        if (least >= kSureFeq * p.rho_ref && rho <= kSureRho * p.rho_ref) continue;
+        const float flow = rho * (1.0f - 3.0f * (ux * ux + uy * uy));
+        if (flow >= kSureFlow * p.rho_ref && rho <= kSureRho * p.rho_ref) continue;
         if (small)
             sh.ds[i] = INFINITY;
         else
@@ -524,12 +525,12 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
         if (preloaded && warp != 0 && lane < n) c = p.cand[lane];
         bool owed = false;
         if constexpr (kLowPrec) {
-            owed = __any_sync(kFull, lane < n && nan64(c.key));
+            owed = __any_sync(kFull, lane < n && isnan(c.key));
             if (owed) key_few<Q, S>(p, n, c.site, sh);  // every warp takes three
         }
         if (warp == 0) {
             if (owed) c.key = lane < n ? sh.key[lane] : -1.0;
-            const bool valid = lane < n && above64(c.key, p.delta_e);
+            const bool valid = lane < n && c.key > p.delta_e;
             n_valid = __popc(__ballot_sync(kFull, valid));
             nsel = k < (long long)n_valid ? (int)(k > 0 ? k : 0) : n_valid;
             const long long u = valid ? (long long)key_bits(c.key) : -1;
