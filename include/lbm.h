@@ -281,7 +281,9 @@ lbm_status lbm_get_config(const lbm_ctx *ctx, lbm_config *out);
 /* Bytes of device memory the context holds (for admission by HBM footprint). */
 int64_t lbm_device_bytes(const lbm_ctx *ctx);
 
-/* Device bytes lbm_create would allocate for cfg (0 if cfg is invalid). */
+/* Device bytes a lattice of cfg takes in a batch, and by itself (0 if cfg is invalid);
+ * a lone small lattice whose steps are taken many in one launch holds up to 32 KB more
+ * (lbm_device_bytes has them). */
 int64_t lbm_footprint_bytes(const lbm_config *cfg);
 
 /* Control-point record (the monitoring point of Sec. 4.4.2): after every

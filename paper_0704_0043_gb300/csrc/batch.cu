@@ -482,7 +482,7 @@ lbm_status lbm_batch_add(lbm_batch *b, const lbm_config *cfg, int32_t *slot)
     if (cfg->limiters & kLimEnsemble)
         return bfail(b, LBM_ERR_INVALID_ARG, "the ensemble-dependent limiters are not available in batches");
     lbm_ctx *c = nullptr;
-    lbm_status s = lbm_create(cfg, (void *)b->run, &c);
+    lbm_status s = create_ctx(cfg, (void *)b->run, true, &c);
     if (s != LBM_OK) return bfail(b, s, lbm_last_error(nullptr));
     invalidate(b);
     b->slot_status.resize(b->slots.size(), LBM_OK);

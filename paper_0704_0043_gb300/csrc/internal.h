@@ -462,5 +462,7 @@ StepParams ctx_step_params(lbm_ctx *c, int collide, unsigned limiters);
 // The fused kernel's accumulator rows of a context (the tail's partials when fixed = 1).
 double *ctx_fx_rows(lbm_ctx *c);
 FinalParams ctx_final_params(lbm_ctx *c, int collide, unsigned limiters, int nblocks);
+// lbm_create; `batched`: without what only lone lattices use.
+lbm_status create_ctx(const lbm_config *cfg, void *cuda_stream, bool batched, lbm_ctx **out);
 bool ctx_uses_fused(const lbm_ctx *c);
 }  // namespace lbm

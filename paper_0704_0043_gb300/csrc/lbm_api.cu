@@ -136,11 +136,11 @@ size_t fx_bytes() { return (size_t)kFxRows * kFxWords * sizeof(unsigned long lon
 struct Sizes {
     int q, pitch;
     long long plane;
-    size_t elem, field, cand, sel, partials, ring, ent, selstate, res;
+    size_t elem, field, cand, sel, partials, ring, ent, selstate;
     int cand_cap, sel_cap, rows, ring_len;
     int64_t total() const
     {
-        return (int64_t)(2 * field + cand + sel + partials + ring + ens_bytes() + ent + selstate + res +
+        return (int64_t)(2 * field + cand + sel + partials + ring + ens_bytes() + ent + selstate +
                          64 * sizeof(long long) +
                          (size_t)chunks_for(rows) * sizeof(unsigned) + 4096);
     }
@@ -164,7 +164,6 @@ Sizes sizes_for(const lbm_config &c)
     z.rows = tiled_blocks_for(z.q, c.nx, c.ny);
     if (z.q == 3) z.rows = std::max(z.rows, tube_blocks(c.precision == LBM_FP64, c.nx));
     z.partials = fx_bytes() + (size_t)(z.rows + chunks_for(z.rows)) * P_NSTAT * sizeof(double);
-    z.res = resident_applies(c) ? sizeof(ResState) : 0;
     z.ring_len = std::max(1, c.stats_history);
     z.ring = (size_t)z.ring_len * sizeof(DevStats);
     // Eq. EntThresh: the pass's dS field (compute precision) and the solve's state
@@ -646,6 +645,14 @@ int64_t lbm_footprint_bytes(const lbm_config *cfg)
 
 lbm_status lbm_create(const lbm_config *cfg, void *cuda_stream, lbm_ctx **out)
 {
+    return create_ctx(cfg, cuda_stream, false, out);
+}
+
+}  // extern "C"
+
+namespace lbm {
+lbm_status create_ctx(const lbm_config *cfg, void *cuda_stream, bool batched, lbm_ctx **out)
+{
     if (!out) return fail(nullptr, LBM_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     std::string v = validate(cfg);
@@ -693,8 +700,10 @@ lbm_status lbm_create(const lbm_config *cfg, void *cuda_stream, lbm_ctx **out)
         default: c->fin_grid = finalize_grid<__half>(c->q);
         }
     }
-    if (z.res) part(&c->res, z.res);
-    c->cluster = cluster_applies(c->cfg);
+    // the state of the kernels that take many steps in one launch: a batch never runs them
+    const size_t res = !batched && resident_applies(c->cfg) ? sizeof(ResState) : 0;
+    if (res) part(&c->res, res);
+    c->cluster = res && cluster_applies(c->cfg);
     if (z.ent) {
         part(&c->ent_field, z.ent - sizeof(EntState));
         part(&c->ent, sizeof(EntState));
@@ -718,10 +727,13 @@ lbm_status lbm_create(const lbm_config *cfg, void *cuda_stream, lbm_ctx **out)
         delete c;
         return fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, m);
     }
-    c->device_bytes = z.total();
+    c->device_bytes = z.total() + (int64_t)res;
     *out = c;
     return LBM_OK;
 }
+}  // namespace lbm
+
+extern "C" {
 
 lbm_status lbm_destroy(lbm_ctx *c)
 {
