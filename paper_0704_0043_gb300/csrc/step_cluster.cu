@@ -22,6 +22,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "internal.h"
@@ -404,10 +405,19 @@ cudaLaunchConfig_t cluster_config(size_t bytes, cudaStream_t s, cudaLaunchAttrib
     return cfg;
 }
 
-// Whether the device runs the cluster (16 blocks of this size), asked once.
+// Whether the current device runs the cluster (16 blocks of this size): asked once for each
+// device, as the kernel's attributes are set for each.  Two threads that ask at once set the
+// same.
 bool cluster_runs()
 {
-    static const bool runs = [] {
+    constexpr int kDevices = 64;
+    static std::atomic<int> known[kDevices];  // 0: not asked, 1: it does not, 2: it does
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) {
+        cudaGetLastError();
+        return false;
+    }
+    if (known[dev].load() == 0) {
         cudaLaunchAttribute attr;
         const cudaLaunchConfig_t cfg = cluster_config(kCluMaxBytes, nullptr, &attr);
         int fit = 0;
@@ -416,9 +426,9 @@ bool cluster_runs()
             cudaFuncSetAttribute(k_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
             cudaOccupancyMaxActiveClusters(&fit, k_cluster, &cfg) == cudaSuccess && fit > 0;
         if (!ok) cudaGetLastError();
-        return ok;
-    }();
-    return runs;
+        known[dev].store(ok ? 2 : 1);
+    }
+    return known[dev].load() == 2;
 }
 
 }  // namespace
