@@ -192,7 +192,7 @@ __device__ __forceinline__ void do_tile(const StepParams &p, const ResK &kk, con
         // the stencils of the tile's edge sites reach outside it: evaluate dS there
         // only when one of them forms its median
         const bool edge = Q == 9 ? (lane == 0 || lane == 31 || warp == 0 || warp == aw - 1) : (t == 0 || t == 32 * aw - 1);
-        const bool part = x == p.nx - 1 || y == p.ny - 1;  // sites beyond the lattice's end (periodic lattices)
+        const bool part = x == p.nx - 1 || (Q == 9 && y == p.ny - 1);  // sites beyond the lattice's end (periodic lattices)
         if (__syncthreads_or(need && (edge || part))) {
             if constexpr (Q == 9) {
                 const int w = min(32, p.nx - x0), h = min(aw, p.ny - y0);
