@@ -286,12 +286,27 @@ struct ResArgs {
     FinalParams f;
     void *buf[2];
     int cur, nsteps;
-    int aw, gx, tiles;  // set by the launcher: warps that carry sites, tiles along x, tiles
+    int aw, gx, tiles, blocks;  // see ResGrid
     double rest;        // rest_mass
     ResState *rs;
 };
 double rest_mass(const StepParams &p);
 bool resident_applies(const lbm_config &c);
+// The grid of a resident launch: warps that carry sites, tiles along x, tiles, blocks, and
+// the most steps a launch takes (it holds its SMs for all of them: kResLaunchUs).
+struct ResGrid {
+    int aw, gx, tiles, blocks, most_steps;
+};
+// False: the lattice is stepped launch by launch.  A resident block fills its SM, so grids
+// that do not fit beside one another run one after the other, and what waits for the tail
+// or the barrier in one of them is lost to the others.  With lattices on several streams
+// the grid takes at most its share of the SMs, one round of tiles, or there is none.
+// us for a step of all of 1 / 2 / 4 / 8 lattices on their own streams (Ehrenfests' steps
+// and median): 300^2 FP32 resident on all SMs 15 / 30 / 60 / 120, launch by launch 27 / 29 /
+// 33 / 39; 100^2 FP32 on all SMs 12 / 23 / 46 / 93, on its share 12 / 12 / 13 and, where it
+// does not fit, launch by launch 34; 200^2 FP64 launch by launch 71 / 126 / 243 for 2 / 4 / 8.
+bool resident_grid(const lbm_config &c, int streams, ResGrid *g);
+constexpr double kResLaunchUs = 8000.0;  // about the longest launch
 // The smallest FP32 D2Q9 lattices without Ehrenfests' steps: one thread-block
 // cluster, populations in shared memory (step_cluster.cu).  us per step against
 // the resident kernel, median filter, boundary nodes: 32^2 4.0 / 5.9, 100^2
@@ -409,6 +424,7 @@ struct lbm_ctx {
     int fin_grid = 0;                     // blocks of the cooperative tail (0: one-block tail only)
     bool capturing = false;               // a graph capture is in progress (one-block tail)
     bool cluster = false;                 // the resident steps run as one cluster
+    bool listed = false;                  // the stream is in the list of live contexts' streams
     lbm::ResState *res = nullptr;         // resident steps: counters and rows (nullptr: stepped launch by launch)
     double *ens = nullptr;  // [kEnsBlocks][2] partial sums and counts of dS, then E(dS), alpha, sum, count
     void *ent_field = nullptr;   // LBM_LIM_ENTTHRESH: the pass's dS field

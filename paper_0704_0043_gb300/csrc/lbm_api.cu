@@ -10,6 +10,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <type_traits>
 #include <vector>
@@ -46,6 +47,61 @@ lbm_status cuda_fail(lbm_ctx *c, cudaError_t e, const char *what)
     } while (0)
 
 int lattice_q(int lattice) { return lattice == LBM_D1Q3 ? 3 : 9; }
+
+// The streams that live contexts are on, for resident_grid: contexts on one stream take
+// turns anyway, those on several may overlap.  Entered at create, left at destroy.
+class StreamBook {
+  public:
+    // Enter: whether the stream is listed (the caller keeps it for leave); contexts beyond
+    // the list count as a stream each.
+    bool enter(int device, cudaStream_t s)
+    {
+        std::lock_guard<std::mutex> hold(mu_);
+        Entry *at = nullptr;
+        for (Entry &e : list_) {
+            if (e.users > 0 && e.device == device && e.stream == s) {
+                ++e.users;
+                return true;
+            }
+            if (e.users == 0 && !at) at = &e;
+        }
+        if (at)
+            *at = {device, 1, s};
+        else
+            ++unlisted_;
+        return at != nullptr;
+    }
+    void leave(int device, cudaStream_t s, bool listed)
+    {
+        std::lock_guard<std::mutex> hold(mu_);
+        if (!listed) {
+            --unlisted_;
+            return;
+        }
+        for (Entry &e : list_)
+            if (e.users > 0 && e.device == device && e.stream == s) {
+                --e.users;
+                return;
+            }
+    }
+    int streams(int device)
+    {
+        std::lock_guard<std::mutex> hold(mu_);
+        int n = unlisted_;
+        for (const Entry &e : list_) n += e.users > 0 && e.device == device;
+        return std::max(n, 1);
+    }
+
+  private:
+    struct Entry {
+        int device, users;
+        cudaStream_t stream;
+    };
+    std::mutex mu_;
+    Entry list_[64] = {};
+    int unlisted_ = 0;
+};
+StreamBook g_streams;
 
 // Calls fn with a null pointer of the context's storage type.
 template <typename F>
@@ -370,8 +426,10 @@ lbm_status run_resident(lbm_ctx *c, int64_t n, int64_t *taken)
         cudaGetLastError();
         return LBM_OK;
     }
+    ResGrid g{};
+    if (!c->cluster && !resident_grid(c->cfg, g_streams.streams(c->device), &g)) return LBM_OK;
     while (*taken < n) {
-        const int m = (int)std::min<int64_t>(n - *taken, kResMaxSteps);
+        const int m = (int)std::min<int64_t>(n - *taken, c->cluster ? kResMaxSteps : g.most_steps);
         ResArgs a{};
         a.p = step_params(c, 1, c->cfg.limiters);
         a.f = final_params(c, 1, c->cfg.limiters, 1);
@@ -379,19 +437,24 @@ lbm_status run_resident(lbm_ctx *c, int64_t n, int64_t *taken)
         a.buf[1] = c->buf[1];
         a.cur = c->cur;
         a.nsteps = m;
+        a.aw = g.aw;
+        a.gx = g.gx;
+        a.tiles = g.tiles;
+        a.blocks = g.blocks;
         a.rs = c->res;
         const cudaError_t e = with_storage(c->cfg.precision, [&](auto tag) -> cudaError_t {
             using S = STORAGE_T;
             if constexpr (std::is_same<S, float>::value) {
-                if (c->cluster) {
-                    const cudaError_t ce = launch_cluster(a, c->stream);
-                    if (ce == cudaSuccess) return ce;
-                    cudaGetLastError();  // no such cluster on this device
-                    c->cluster = false;
-                }
+                if (c->cluster) return launch_cluster(a, c->stream);
             }
             return launch_resident<S>(c->q, a, c->stream);
         });
+        if (e != cudaSuccess && c->cluster) {
+            cudaGetLastError();
+            c->cluster = false;  // no such cluster on this device: the resident kernel from now on
+            if (!resident_grid(c->cfg, g_streams.streams(c->device), &g)) return LBM_OK;
+            continue;
+        }
         if (e != cudaSuccess) {
             // no cooperative launch on this device: step launch by launch from now on
             cudaGetLastError();
@@ -728,6 +791,7 @@ lbm_status create_ctx(const lbm_config *cfg, void *cuda_stream, bool batched, lb
         return fail(nullptr, e == cudaErrorMemoryAllocation ? LBM_ERR_OOM : LBM_ERR_CUDA, m);
     }
     c->device_bytes = z.total() + (int64_t)res;
+    c->listed = g_streams.enter(c->device, c->stream);
     *out = c;
     return LBM_OK;
 }
@@ -739,6 +803,7 @@ lbm_status lbm_destroy(lbm_ctx *c)
 {
     if (!c) return LBM_OK;
     cudaStreamSynchronize(c->stream);
+    g_streams.leave(c->device, c->stream, c->listed);
     free_all(c);
     delete c;
     return LBM_OK;

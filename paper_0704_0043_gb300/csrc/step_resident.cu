@@ -540,31 +540,38 @@ int round_cost(bool fp64, int rows)
     return 400 + (rows - 8) * 346 / 8;
 }
 
+bool resident_grid(const lbm_config &c, int streams, ResGrid *g)
+{
+    const bool fp64 = c.precision == LBM_FP64, tube = c.lattice == LBM_D1Q3;
+    const int sms = std::min(sm_count(), kResMaxBlocks), workers = sms - 1;
+    // warps that carry sites (rows of a tile): the least time of the busiest SM, its rounds
+    // times the time of one, rows beyond the lattice left out
+    long long best = -1;
+    for (int w = 4; w <= kResWarps; w *= 2) {
+        const int gx = tube ? 1 : (c.nx + 31) / 32;
+        const int tiles = tube ? (c.nx + 32 * w - 1) / (32 * w) : gx * ((c.ny + w - 1) / w);
+        const long long rounds = (tiles + workers - 1) / workers;
+        const long long cost = rounds * round_cost(fp64, tube ? w : std::min(w, c.ny));
+        if (streams > 1 && tiles + 1 > sms / streams) continue;
+        if (best >= 0 && cost >= best) continue;
+        best = cost;
+        *g = {w, gx, tiles, std::min(workers, tiles) + 1, 0};
+    }
+    if (best < 0) return false;
+    // units of round_cost: 1/20 us in FP64 (tubes a third), 1/16 us otherwise
+    const double us = 8.0 + (double)best * (fp64 ? (tube ? 1.0 / 60 : 1.0 / 20) : 1.0 / 16);
+    g->most_steps = std::max(16, std::min(kResMaxSteps, (int)(kResLaunchUs / us)));
+    return true;
+}
+
 template <typename S>
 cudaError_t launch_resident(int q, ResArgs a, cudaStream_t s)
 {
-    // warps that carry sites (rows of a tile): the least time of the busiest SM, its rounds
-    // times the time of one (see round_cost), rows beyond the lattice left out
-    const int workers = std::min(sm_count(), kResMaxBlocks) - 1;
-    auto tiles_for = [&](int aw) {
-        if (q == 3) return (a.p.nx + 32 * aw - 1) / (32 * aw);
-        return ((a.p.nx + 31) / 32) * ((a.p.ny + aw - 1) / aw);
-    };
-    int aw = 4;
-    long long best = -1;
-    for (int w = 4; w <= kResWarps; w *= 2) {
-        const long long rounds = (tiles_for(w) + workers - 1) / workers;
-        const long long cost = rounds * round_cost(std::is_same<S, double>::value, q == 3 ? w : std::min(w, a.p.ny));
-        if (best < 0 || cost < best) aw = w, best = cost;
-    }
-    a.aw = aw;
-    a.gx = q == 3 ? 1 : (a.p.nx + 31) / 32;
-    a.tiles = tiles_for(aw);
     a.rest = rest_mass(a.p);
     cudaError_t e = cudaMemsetAsync(a.rs, 0, offsetof(ResState, rows), s);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((unsigned)std::min(workers, a.tiles) + 1);
+    cfg.gridDim = dim3((unsigned)a.blocks);
     cfg.blockDim = dim3(kResThreads);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
