@@ -741,8 +741,9 @@ lbm_status create_ctx(const lbm_config *cfg, void *cuda_stream, bool batched, lb
         void **at;
         size_t bytes;
     };
-    std::vector<Part> parts;
-    auto part = [&](void *at, size_t bytes) { parts.push_back({(void **)at, (bytes + 255) / 256 * 256}); };
+    Part parts[16];  // (an array: what throws must not pass through a C function)
+    int nparts = 0;
+    auto part = [&](void *at, size_t bytes) { parts[nparts++] = {(void **)at, (bytes + 255) / 256 * 256}; };
     part(&c->buf[0], z.field);
     part(&c->buf[1], z.field);
     part(&c->cand, z.cand);
@@ -772,14 +773,14 @@ lbm_status create_ctx(const lbm_config *cfg, void *cuda_stream, bool batched, lb
         part(&c->ent, sizeof(EntState));
     }
     size_t all = 0;
-    for (const Part &q : parts) all += q.bytes;
+    for (int i = 0; i < nparts; ++i) all += parts[i].bytes;
     if (e == cudaSuccess) e = cudaMalloc(&c->arena, all);
     if (e == cudaSuccess) {
         e = cudaMemsetAsync(c->arena, 0, all, c->stream);
         char *m = (char *)c->arena;
-        for (const Part &q : parts) {
-            *q.at = m;
-            m += q.bytes;
+        for (int i = 0; i < nparts; ++i) {
+            *parts[i].at = m;
+            m += parts[i].bytes;
         }
     }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
