@@ -607,7 +607,10 @@ StepParams cfg_step_params(const lbm_config &g, int q, int pitch, long long plan
         p.rwf[k] = (float)p.rw[k];
     }
     {
-        const int er = std::ilogb((double)p.rho_ref), shift = 58 - er;
+        // rho_ref of any size is accepted; beyond FP32's it becomes 0 or inf here, which
+        // have no exponent (the FP64 formula then)
+        const int er = p.rho_ref > 0.0f && std::isfinite(p.rho_ref) ? std::ilogb((double)p.rho_ref) : 1000;
+        const int shift = 58 - er;
         p.mfx.exp = -shift;
         p.mfx.lim = er > -90 && er < 90 ? std::ldexp(1.0f, er) : 0.0f;
         p.mfx.scale = std::ldexp(1.0f, std::max(-110, std::min(110, 27 - er)));
