@@ -477,6 +477,140 @@ __device__ __noinline__ int settle_many(const FinalParams &p, int n, int tlow)
     return nv;
 }
 
+// The chosen candidates of a pass with more than a few (see finish_candidates): their list
+// entries in sh.idx (the first kCap), their count returned and in sh.nsel, and in sh.valid
+// that of the candidates above delta.  Out of line: the usual few candidates then run
+// straight through a cold instruction cache (2048 x 2048 entropic FP32 282 -> 276 us a
+// step, tube of 1e7 sites 68.0 -> 67.0).
+template <int Q, typename S>
+__device__ __noinline__ int choose(const FinalParams &p, int n, bool use_list, bool preloaded, Cand first, SelShared &sh)
+{
+    constexpr bool kLowPrec = !std::is_same<S, double>::value;
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int *list = use_list ? p.sel_state->list : nullptr;
+    auto cidx = [&](int i) -> int { return use_list ? list[i] : i; };
+    const bool small = n <= kCap;  // candidates held in shared memory
+    const long long k = p.k_max;
+    // below the threshold -> -1, so that from here on a key is valid exactly
+    // when its bit pattern is a positive integer (compared as integers, as everywhere
+    // below: an FP64 comparison takes the FP64 unit as long as an addition does, and a
+    // keyed candidate is no NaN)
+    auto settle = [&](double key) { return above64(key, p.delta_e) ? key : -1.0; };
+    bool owed = false;
+    if (t == 0) {
+        sh.nsel = 0;
+        if (!use_list) sh.valid = 0;
+        sh.count = 0;
+    }
+    if (small) {
+        for (int i = t; i < n; i += kFinThreads) {
+            const Cand c = preloaded && i == t ? first : p.cand[cidx(i)];
+            owed = owed || (kLowPrec && nan64(c.key));
+            sh.key[i] = c.key;
+            sh.site[i] = c.site;
+            sh.ds[i] = nan64(c.key) ? c.ds32 : narrow(c.key);
+        }
+    } else if (kLowPrec && !use_list) {
+        owed = any_owed(p, n);
+    }
+    owed = __syncthreads_or(owed) != 0;
+    if (!use_list) {
+        // FP32 dS pattern below which a candidate cannot be among the k largest; 0
+        // where the FP32 dS of owed keys does not stand for them, and where it would
+        // spare nothing: choose_many goes over all entries of a list that shared
+        // memory does not hold, dropped or not (10^6 keyed candidates of a tube, set
+        // and four steps: 23.6 ms with the bound's passes, 17.1 without)
+        int tlow = 0;
+        if (!owed || sure_delta(p)) {
+            if constexpr (kLowPrec) {
+                if (owed) mark_unsure<Q, S>(p, n, small, sh);
+            }
+            if (k <= 0)
+                tlow = 0x7f800000;
+            else if ((small && n > kRank32) || (owed && n > k))
+                tlow = fp32_bound<S>(p, n, small, !owed, sh);
+        }
+        int nv = 0;  // candidates counted as valid here without a key, then those with one
+        if constexpr (kLowPrec) {
+            if (owed) nv = settle_owed<Q, S>(p, n, small, tlow, sh);
+        }
+        // every candidate is keyed or counted (-1) now
+        if (small) {
+            for (int i = t; i < n; i += kFinThreads) {
+                double key = settle(sh.key[i]);
+                nv += (long long)key_bits(key) > 0;
+                if (__float_as_int(sh.ds[i]) < tlow) key = -1.0;  // counted, out of play
+                sh.key[i] = key;
+            }
+        } else {
+            nv += settle_many(p, n, tlow);
+        }
+        nv = __reduce_add_sync(kFull, nv);
+        if (lane == 0 && nv) atomicAdd(&sh.valid, nv);
+    }
+    __syncthreads();
+    const int n_valid = sh.valid;
+    if (k <= 0 || n_valid <= 0) return 0;  // the same for the whole block
+
+    // the entries still in play (valid, keyed), compacted: the candidates below
+    // the FP32 bound drop out here
+    int m = n;
+    bool packed = false;
+    if (small) {
+        // who is in play: a ballot per 32 entries (at most 64 of them), the
+        // entries' places from the ballots before theirs
+        static_assert(kCap <= 64 * 32, "two ballots per lane");
+        const int nb = (n + 31) / 32;
+        for (int b = warp; b < nb; b += kFinWarps) {
+            const int i = 32 * b + lane;
+            const unsigned w = __ballot_sync(kFull, i < n && (long long)key_bits(sh.key[i]) > 0);
+            if (lane == 0) sh.hist[b] = w;
+        }
+        __syncthreads();
+        const int c0 = lane < nb ? __popc(sh.hist[lane]) : 0, c1 = lane + 32 < nb ? __popc(sh.hist[lane + 32]) : 0;
+        m = __reduce_add_sync(kFull, c0 + c1);
+        packed = m <= kRankCap;
+        for (int b = warp; b < nb && packed; b += kFinWarps) {
+            const int before = __reduce_add_sync(kFull, (lane < b ? c0 : 0) + (lane + 32 < b ? c1 : 0));
+            const unsigned w = sh.hist[b];
+            if ((w >> lane) & 1u) {
+                const int at = before + __popc(w & ((1u << lane) - 1u)), i = 32 * b + lane;
+                sh.rkey[at] = (long long)key_bits(sh.key[i]);
+                sh.idx[at] = i;
+            }
+        }
+        __syncthreads();
+    }
+    const bool take_all = (long long)n_valid <= k;
+    if (packed) {
+        // each thread ranks its own entry by counting the keys that beat it
+        // (larger dS, or equal dS at a lower site); the rank is its place in the
+        // chosen list, so the list's order does not depend on the recording order
+        int mine = -1, rank = 0;
+        if (t < m) {
+            mine = sh.idx[t];
+            const long long u = sh.rkey[t];
+            int more = 0, same = 0;
+#pragma unroll 4
+            for (int j = 0; j < m; ++j) {  // broadcast reads
+                const long long v = sh.rkey[j];
+                more += v > u;
+                same += v == u;
+            }
+            if (same > 1)  // ties (other than the entry itself)
+                for (int j = 0; j < m; ++j) more += sh.rkey[j] == u && sh.site[sh.idx[j]] < sh.site[mine];
+            rank = more;
+        }
+        const int nsel = (int)(k < (long long)m ? k : (long long)m);
+        __syncthreads();
+        if (mine >= 0 && rank < nsel) sh.idx[rank] = mine;
+        if (t == 0) sh.nsel = nsel;
+        __syncthreads();
+        return nsel;
+    }
+    return choose_many<S>(p, n, use_list, small, take_all, sh);
+}
+
 // The candidates of a pass: FP64 keys where they are owed, the count n_valid of
 // candidates above delta, the k with the largest keys (ties to the lower site),
 // Ehrenfests' step at those.  List entry i < n is candidate i, or with use_list
@@ -486,10 +620,9 @@ __device__ __noinline__ int settle_many(const FinalParams &p, int n, int tlow)
 // the step adds); sh.nsel holds the chosen count; n_valid is set in thread 0.
 // Every thread of a block of kFinThreads calls it, n > 0.
 //
-// Keys are owed (NaN) by FP32 and 16-bit passes.  Only the candidates that can
-// reach the k largest by their FP32 dS, those within 1/64 of delta and those whose FP32
-// dS is not sure get one:
-// FP64 is slow on this GPU (one block keying every candidate of a 517 x 389
+// Keys are owed (NaN) by FP32 and 16-bit passes.  Only the candidates that can reach the
+// k largest by their FP32 dS, those within 1/64 of delta and those whose FP32 dS does not
+// stand for the key get one: FP64 is slow on this GPU (one block keying every candidate of a 517 x 389
 // cavity, several hundred with k = 20, took 25 us a step), and the others' count
 // is certain without it.  A few are keyed three to a warp (a lane per
 // direction), more a lane each.
@@ -507,12 +640,6 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
     double ehr_sum = 0.0;
 
     auto key_of = [&](int i) -> double { return small ? sh.key[i] : p.cand[cidx(i)].key; };
-    auto site_of = [&](int i) -> int { return small ? sh.site[i] : p.cand[cidx(i)].site; };
-    // below the threshold -> -1, so that from here on a key is valid exactly
-    // when its bit pattern is a positive integer
-    // (compared as integers, as everywhere below: an FP64 comparison takes the FP64 unit
-    // as long as an addition does, and a keyed candidate is no NaN)
-    auto settle = [&](double key) { return above64(key, p.delta_e) ? key : -1.0; };
     int nsel = 0;         // chosen sites (few: in the first warp only)
     bool listed = false;  // the chosen list entries are in sh.idx
     const bool few = n <= 32 && !use_list;
@@ -549,120 +676,9 @@ __device__ __forceinline__ double finish_candidates(const FinalParams &p, S *f, 
             if (lane == 0) sh.nsel = nsel;
         }
     } else {
-        bool owed = false;
-        if (t == 0) {
-            sh.nsel = 0;
-            if (!use_list) sh.valid = 0;
-            sh.count = 0;
-        }
-        if (small) {
-            for (int i = t; i < n; i += kFinThreads) {
-                const Cand c = preloaded && i == t ? first : p.cand[cidx(i)];
-                owed = owed || (kLowPrec && nan64(c.key));
-                sh.key[i] = c.key;
-                sh.site[i] = c.site;
-                sh.ds[i] = nan64(c.key) ? c.ds32 : narrow(c.key);
-            }
-        } else if (kLowPrec && !use_list) {
-            owed = any_owed(p, n);
-        }
-        owed = __syncthreads_or(owed) != 0;
-        if (!use_list) {
-            // FP32 dS pattern below which a candidate cannot be among the k largest; 0
-            // where the FP32 dS of owed keys does not stand for them, and where it would
-            // spare nothing: choose_many goes over all entries of a list that shared
-            // memory does not hold, dropped or not (10^6 keyed candidates of a tube, set
-            // and four steps: 23.6 ms with the bound's passes, 17.1 without)
-            int tlow = 0;
-            if (!owed || sure_delta(p)) {
-                if constexpr (kLowPrec) {
-                    if (owed) mark_unsure<Q, S>(p, n, small, sh);
-                }
-                if (k <= 0)
-                    tlow = 0x7f800000;
-                else if ((small && n > kRank32) || (owed && n > k))
-                    tlow = fp32_bound<S>(p, n, small, !owed, sh);
-            }
-            int nv = 0;  // candidates counted as valid here without a key, then those with one
-            if constexpr (kLowPrec) {
-                if (owed) nv = settle_owed<Q, S>(p, n, small, tlow, sh);
-            }
-            // every candidate is keyed or counted (-1) now
-            if (small) {
-                for (int i = t; i < n; i += kFinThreads) {
-                    double key = settle(sh.key[i]);
-                    nv += (long long)key_bits(key) > 0;
-                    if (__float_as_int(sh.ds[i]) < tlow) key = -1.0;  // counted, out of play
-                    sh.key[i] = key;
-                }
-            } else {
-                nv += settle_many(p, n, tlow);
-            }
-            nv = __reduce_add_sync(kFull, nv);
-            if (lane == 0 && nv) atomicAdd(&sh.valid, nv);
-        }
-        __syncthreads();
+        nsel = choose<Q, S>(p, n, use_list, preloaded, first, sh);
+        listed = nsel <= kCap;
         n_valid = sh.valid;
-        if (k <= 0 || n_valid <= 0) return 0.0;  // the same for the whole block
-
-        // the entries still in play (valid, keyed), compacted: the candidates below
-        // the FP32 bound drop out here
-        int m = n;
-        bool packed = false;
-        if (small) {
-            // who is in play: a ballot per 32 entries (at most 64 of them), the
-            // entries' places from the ballots before theirs
-            static_assert(kCap <= 64 * 32, "two ballots per lane");
-            const int nb = (n + 31) / 32;
-            for (int b = warp; b < nb; b += kFinWarps) {
-                const int i = 32 * b + lane;
-                const unsigned w = __ballot_sync(kFull, i < n && (long long)key_bits(sh.key[i]) > 0);
-                if (lane == 0) sh.hist[b] = w;
-            }
-            __syncthreads();
-            const int c0 = lane < nb ? __popc(sh.hist[lane]) : 0, c1 = lane + 32 < nb ? __popc(sh.hist[lane + 32]) : 0;
-            m = __reduce_add_sync(kFull, c0 + c1);
-            packed = m <= kRankCap;
-            for (int b = warp; b < nb && packed; b += kFinWarps) {
-                const int before = __reduce_add_sync(kFull, (lane < b ? c0 : 0) + (lane + 32 < b ? c1 : 0));
-                const unsigned w = sh.hist[b];
-                if ((w >> lane) & 1u) {
-                    const int at = before + __popc(w & ((1u << lane) - 1u)), i = 32 * b + lane;
-                    sh.rkey[at] = (long long)key_bits(sh.key[i]);
-                    sh.idx[at] = i;
-                }
-            }
-            __syncthreads();
-        }
-        const bool take_all = (long long)n_valid <= k;
-        if (packed) {
-            // each thread ranks its own entry by counting the keys that beat it
-            // (larger dS, or equal dS at a lower site); the rank is its place in the
-            // chosen list, so the list's order does not depend on the recording order
-            int mine = -1, rank = 0;
-            if (t < m) {
-                mine = sh.idx[t];
-                const long long u = sh.rkey[t];
-                int more = 0, same = 0;
-#pragma unroll 4
-                for (int j = 0; j < m; ++j) {  // broadcast reads
-                    const long long v = sh.rkey[j];
-                    more += v > u;
-                    same += v == u;
-                }
-                if (same > 1)  // ties (other than the entry itself)
-                    for (int j = 0; j < m; ++j) more += sh.rkey[j] == u && sh.site[sh.idx[j]] < sh.site[mine];
-                rank = more;
-            }
-            nsel = (int)(k < (long long)m ? k : (long long)m);
-            __syncthreads();
-            if (mine >= 0 && rank < nsel) sh.idx[rank] = mine;
-            if (t == 0) sh.nsel = nsel;
-            __syncthreads();
-        } else {
-            nsel = choose_many<S>(p, n, use_list, small, take_all, sh);
-        }
-        listed = packed || nsel <= kCap;  // the chosen list entries are in sh.idx
     }
     // Ehrenfests' step at each chosen site, in the list's order
     for (int r = t; r < nsel; r += kFinThreads) {
