@@ -52,7 +52,7 @@ typedef enum {
     LBM_ERR_NONFINITE = 4,   /* a site had rho <= 0, f*_k <= 0 or a nonfinite value */
     LBM_ERR_TIMEOUT = 5,     /* a bounded device-side wait gave up: the grid barriers of the tail that
                                 preselects dense Ehrenfests' candidates (lattices of 2^20 sites or
-                                more) and of the resident kernel poll about a second; the pass's results
+                                more) and of the resident kernel poll for a few seconds; the pass's results
                                 are then not to be trusted (re-initialise the state) */
     LBM_ERR_STATE = 6        /* call out of order (e.g. step before init) */
 } lbm_status;
@@ -155,8 +155,10 @@ enum { LBM_PHI_HOMOTHETY = 0, LBM_PHI_ENTROPY = 1 };
 enum {
     LBM_KERNEL_AUTO = 0,    /* the fused D2Q9 cavity kernel or the D1Q3 tube kernel where it applies,
                                else the tiled kernel; small lattices with polynomial f* and no
-                               ensemble-dependent limiter take their steps in one cooperative launch
-                               per call (the same populations, bit for bit) */
+                               ensemble-dependent limiter take many steps in one cooperative launch, a
+                               call's or about 8 ms of them (the same populations, bit for bit); with
+                               live lattices on several streams only where the launch fits its
+                               share of the GPU, so that the streams overlap */
     LBM_KERNEL_TILED = 1,   /* overlapping-tile kernel: every lattice, boundary and precision */
     LBM_KERNEL_FUSED = 2,   /* D2Q9 with LBM_BC_WALLS, FP32/BF16/FP16 storage: row-streaming fused kernel */
     LBM_KERNEL_TUBE = 3     /* D1Q3 with FP32 or FP64 storage, LBM_BC_WALLS or LBM_BC_PERIODIC, no

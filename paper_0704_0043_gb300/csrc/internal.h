@@ -256,12 +256,13 @@ constexpr int kResMaxSteps = 1024;  // steps of one launch
 // Lattices up to these sizes take the resident kernel.  Measured us per step, resident
 // against launch by launch (square cavities with the median filter / with all
 // limiters; tubes with Ehrenfests' steps):
-//   D2Q9 FP32: 256^2 6.2 / 12.0 against 13.4 / 24.9, 384^2 8.1 / 14.2 against 14.2 / 25.8,
-//   512^2 14.9 / 23.2 against 14.5 / 26.7, 640^2 21.0 / 30.0 against 15.9 / 28.1 (16-bit
-//   alike): the fused kernel evaluates two sites a lane and reads each plane once;
-//   D2Q9 FP64: 512^2 149 / 155 against 225 / 235, 640^2 227 / 233 against 324 / 336;
-//   D1Q3 FP32: 2e5 13.2 against 14.5, 1e6 14.9 against 21.3, 1.5e6 28.2 against 26.4;
-//   D1Q3 FP64: 800 13.3 against 17.7, 5e5 102 against 125.
+//   D2Q9 FP32 (16-bit alike): 256^2 6.2 / 12.9 against 13.7 / 27.2, 384^2 8.1 / 15.2
+//   against 15.2 / 29.5, 480^2 10.3 / 17.4 against 16.2 / 29.8.  The limit was set with
+//   lower tiles than round_cost now gives (512^2 14.9 / 23.2 against 14.5 / 26.7): above it
+//   the fused kernel evaluates two sites a lane and reads each plane once;
+//   D2Q9 FP64: 512^2 151 / 156 against 224 / 234, 700^2 261 / 267 against 384 / 396;
+//   D1Q3 FP32: 2e5 9.1 against 15.8, 1e6 15.4 against 20.7;
+//   D1Q3 FP64: 800 9.5 against 13.5, 5e5 100 against 125.
 constexpr long long kResMaxSites = 240000;      // D2Q9, FP32 and 16-bit storage
 constexpr long long kResMaxSites64 = 1ll << 19;  // FP64 storage
 constexpr long long kResMaxSites3 = 1ll << 20;   // D1Q3, FP32 storage
@@ -309,8 +310,9 @@ bool resident_grid(const lbm_config &c, int streams, ResGrid *g);
 constexpr double kResLaunchUs = 8000.0;  // about the longest launch
 // The smallest FP32 D2Q9 lattices without Ehrenfests' steps: one thread-block
 // cluster, populations in shared memory (step_cluster.cu).  us per step against
-// the resident kernel, median filter, boundary nodes: 32^2 4.0 / 5.9, 100^2
-// 4.4 / 6.3, 128^2 5.8 / 6.3, 150^2 7.1 / 4.9 (16 SMs against 151).
+// the resident kernel, median filter, boundary nodes: 32^2 3.4 / 6.0, 64^2 3.4 / 6.2,
+// 100^2 3.8 / 6.3, 128^2 5.3 / 6.3; 150^2 7.1 / 4.9 (16 SMs against 95: tiles of eight rows
+// fill the resident grid there, of four below).
 constexpr long long kCluMaxSites = 128 * 128;
 constexpr size_t kCluMaxBytes = 200 * 1024;  // dynamic shared memory of a block
 bool cluster_applies(const lbm_config &c);

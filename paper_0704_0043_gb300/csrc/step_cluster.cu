@@ -14,7 +14,7 @@
 // block barrier (a thread keeps the first of its own and evaluates others again).
 // The step's sums are formed while the barrier completes and recorded one step later
 // by a warp of the first block.  Measured on the 100 x 100 cavity with boundary nodes
-// and the median filter: 4.4 us a step against 6.3 us in L2 and 16 us launch by launch.
+// and the median filter: 3.8 us a step against 6.3 us in L2 and 16 us launch by launch.
 // With Ehrenfests' steps (their selection needs two more barriers), in FP64 (16 SMs
 // have too few FP64 units) and on tubes the resident kernel is as fast or faster.
 // The per-site operations are those of the other kernels: the populations are the

@@ -38,7 +38,7 @@ namespace {
 
 constexpr int kResThreads = kFinThreads;   // the tail block runs the selection of select.cuh
 constexpr int kResWarps = kResThreads / 32;
-constexpr unsigned kTailKeys = 12;         // candidates of a step that the tail keys alone (one round of its warps)
+constexpr unsigned kTailKeys = 12;         // candidates of a step that the tail keys alone (three a warp: a warp on each sub-partition)
 constexpr int kPoller = kResThreads - 32;  // worker thread that waits: its warp seldom has sums to add first
 constexpr unsigned kResSpin = 4u << 20;    // polls of a wait before giving up (0.5 to 1 us each)
 
