@@ -28,6 +28,8 @@ import time
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
+# how the step's statistics are summed: FP32 and 16-bit storage add a lane's or a warp's terms in FP32
+SUMS = {"fp64": "fp64", **dict.fromkeys(("fp32", "bf16", "fp16"), "fp32 terms, totals exact or fp64")}
 BYTES_PER_SITE = {("d2q9", "fp32"): 72, ("d2q9", "bf16"): 36, ("d2q9", "fp16"): 36, ("d2q9", "fp64"): 144, ("d1q3", "fp32"): 24,
                   ("d1q3", "fp64"): 48}
 FALLBACK_HBM_GBS = 6800.0
@@ -660,8 +662,11 @@ def main():
         del fa
         lat.set_populations(f_act)
         develop = 0
+    before = lat.launch_count()
     lat.step(develop + args.warmup)
     lat.synchronize()
+    # a small lattice takes many steps in one launch: sampling steps would break those up
+    many = f_act is None and 0 < lat.launch_count() - before < develop + args.warmup
 
     stream = torch.cuda.current_stream()
     if dist is not None:
@@ -674,7 +679,8 @@ def main():
     # replay is off while they are recorded, so the graph line times the steps alone
     if f_act is not None:
         every = 1  # each timed step is its own launch pair
-    if not args.graph:
+    sample = not args.graph and not many
+    if sample:
         lat.timing(True, every=every)
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     sampler.timed_begin()
@@ -697,7 +703,7 @@ def main():
         launches0 += args.steps  # the reloads are not steps
     sampler.timed_end()
     launches = lat.launch_count() - launches0
-    step_ms, tail_ms, timed = lat.timing_read() if not args.graph else (0.0, 0.0, 0)
+    step_ms, tail_ms, timed = lat.timing_read() if sample else (0.0, 0.0, 0)
     lat.timing(False)
     clocks = sampler.stop()
     st = lat.stats()
@@ -715,15 +721,16 @@ def main():
             bps += 8  # Eq. EntThresh: the dS field written once and read once (FP32)
     if timed:
         kern_s = step_ms / 1e3 / timed
-    else:  # graph replay: the whole step (step kernel + tail) from the run's own events
+    else:  # graph replay, many steps a launch: the whole step from the run's own events
         kern_s = elapsed / args.steps
     achieved = bps * w.sites / kern_s / 1e9
     peak, peak_kind = peaks()
     kname = {lbm.KERNEL_FUSED: "fused", lbm.KERNEL_TUBE: "tube"}.get(lat.step_kernel(), "tiled")
     roof = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "peak_kind": peak_kind,
-            "traffic": traffic_from_profile(f"{kname}_{prec}", w.sites),
-            "kernel": kname if timed else "whole step (graph replay)", "kernel_ms": kern_s * 1e3,
+            "traffic": None if many else traffic_from_profile(f"{kname}_{prec}", w.sites),
+            "kernel": kname if timed else ("whole step (many steps a launch)" if many else "whole step (graph replay)"),
+            "kernel_ms": kern_s * 1e3,
             "tail_kernel_ms": tail_ms / max(timed, 1), "timed_launches": timed, "timed_every": every,
             "bytes_per_site": bps}
     if w.sites * bps < 100e6:
@@ -767,13 +774,13 @@ def main():
     if args.workload == "cavity4096":
         cfg = {"workload": w.name, "nx": w.nx, "ny": w.ny, "reynolds": 7500,
                "u_lid": w.u_lid, "beta": w.beta, "limiters": args.limiters,
-               "delta": 1e-3, "k_max": w.k_max, "storage": prec, "sums": "fp64",
+               "delta": 1e-3, "k_max": w.k_max, "storage": prec, "sums": SUMS[prec],
                "equilibrium": args.equilibrium}
     elif args.workload == "cavity100":
         cfg = {"workload": w.name, "nx": w.nx, "ny": w.ny, "reynolds": 5000, "u_lid": w.u_lid,
                "rho0": w.rho0, "beta": w.beta, "walls": "boundary nodes on the walls, bounce-back",
                "limiters": "median", "delta": w.delta_median,
-               "storage": prec, "sums": "fp64", "equilibrium": args.equilibrium}
+               "storage": prec, "sums": SUMS[prec], "equilibrium": args.equilibrium}
     else:
         cfg = {"workload": w.name if w.nx == 800 else f"shock_tube_d1q3_{w.nx}", "sites": w.nx,
                "density_ratio": "1:2", "nu": 1e-9, "beta": w.beta, "limiters": "ehrenfest",
