@@ -543,7 +543,11 @@ int round_cost(bool fp64, int rows)
 bool resident_grid(const lbm_config &c, int streams, ResGrid *g)
 {
     const bool fp64 = c.precision == LBM_FP64, tube = c.lattice == LBM_D1Q3;
-    const int sms = std::min(sm_count(), kResMaxBlocks), workers = sms - 1;
+    // A cooperative grid starts when all of its blocks have a place, and a block takes the
+    // whole SM.  So one SM is left to whatever else runs for long (a kernel of one block on
+    // another stream would hold up the steps until it ends), and a grid of several rounds
+    // has no more blocks than its rounds need.
+    const int sms = std::min(sm_count(), kResMaxBlocks), workers = std::max(1, sms - 2);
     // warps that carry sites (rows of a tile): the least time of the busiest SM, its rounds
     // times the time of one, rows beyond the lattice left out
     long long best = -1;
@@ -555,7 +559,7 @@ bool resident_grid(const lbm_config &c, int streams, ResGrid *g)
         if (streams > 1 && tiles + 1 > sms / streams) continue;
         if (best >= 0 && cost >= best) continue;
         best = cost;
-        *g = {w, gx, tiles, std::min(workers, tiles) + 1, 0};
+        *g = {w, gx, tiles, (int)((tiles + rounds - 1) / rounds) + 1, 0};
     }
     if (best < 0) return false;
     // units of round_cost: 1/20 us in FP64 (tubes a third), 1/16 us otherwise

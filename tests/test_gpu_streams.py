@@ -76,3 +76,18 @@ def test_populations_on_several_streams(threads):
                 g.step(4)
     for g, f in zip(gs, want):
         np.testing.assert_array_equal(g.get_populations(), f)
+
+
+def test_a_long_kernel_elsewhere_does_not_hold_the_steps():
+    """One block busy on another stream: the steps go on beside it, as launches of their own would."""
+    large = cavity(480, 0)
+    large.step(3)
+    large.synchronize()
+    s, done = torch.cuda.Stream(), torch.cuda.Event()
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(int(3e9))  # a second or two
+        done.record(s)
+    assert launches(large, 20) == 1
+    large.synchronize()
+    assert not done.query()
+    torch.cuda.synchronize()
