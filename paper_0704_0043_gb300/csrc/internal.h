@@ -79,7 +79,8 @@ enum { FX_SUM = 0, FX_SITES = 8, FX_NPOS, FX_NMED, FX_NBAD, FX_BAD };
 
 // Ehrenfests' candidate: FP64 key dS(f') (NaN: not keyed yet), phi of the
 // limiter pass, site index, and dS(f') in FP32 (the key rounded, or the FP32
-// value the candidate was recorded on; within 1/64 of the key).
+// value the candidate was recorded on; within 1/64 of the key where select.cuh's kSureDelta
+// and kSureFlow say so).
 struct Cand {
     double key;
     double phi;
